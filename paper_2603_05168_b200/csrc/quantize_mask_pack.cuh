@@ -68,7 +68,7 @@ __host__ __device__ inline uint32_t qmp_sample_units(uint32_t num_units) {
     return num_units < want ? num_units : want;
 }
 
-struct QmpSlot {                 // one per CTA, 16 B
+struct __align__(16) QmpSlot {   // one per CTA, 16 B: the stream kernel writes and reads it as one 128-bit word
     unsigned long long nonce;    // tag of the execution that wrote `partial`
     double partial;              // this CTA's sum |W|
 };
@@ -118,15 +118,13 @@ __device__ __forceinline__ float ternary_threshold(float scale) {
 //   min(a2,a3) >  max(a0,a1)  ->  columns 2,3   (and hence > here)
 __device__ __forceinline__ uint32_t select_pair(const float4 w, float& v0, float& v1) {
     const float a0 = fabsf(w.x), a1 = fabsf(w.y), a2 = fabsf(w.z), a3 = fabsf(w.w);
-    const bool c01 = a0 >= a1, c23 = a2 >= a3;
     const bool both01 = fminf(a0, a1) >= fmaxf(a2, a3);
     const bool both23 = fminf(a2, a3) > fmaxf(a0, a1);
-    v0 = c01 ? w.x : w.y;
-    v1 = c23 ? w.z : w.w;
-    uint32_t nib = (c01 ? 0u : 1u) | (c23 ? 8u : 12u);
-    if (both01) { v0 = w.x; v1 = w.y; nib = 4u; }
-    if (both23) { v0 = w.z; v1 = w.w; nib = 14u; }
-    return nib;
+    const bool first0 = a0 >= a1 || both01;
+    const bool second2 = a2 >= a3 && !both23;
+    v0 = both23 ? w.z : (first0 ? w.x : w.y);
+    v1 = both01 ? w.y : (second2 ? w.z : w.w);
+    return (both23 ? 2u : (first0 ? 0u : 1u)) | (both01 ? 4u : (second2 ? 8u : 12u));
 }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {

@@ -43,29 +43,53 @@ namespace sbn {
 constexpr int kQmpStreamWarps = kQmpWarps - 2;             // 30 compute, warp 30 loads, warp 31 finishes
 constexpr int kQmpLoaderWarp = kQmpWarps - 2;
 constexpr int kQmpLists = 3;
-constexpr int kQmpStreamListCap = 4096;                    // undecided entries per CTA and matrix (see qmp_bracket_from)
-constexpr int kQmpStageUnits = 2 * kQmpStreamWarps;        // a half-warp per unit
+constexpr int kQmpWarpListCap = 138;                       // undecided entries per computing warp and matrix, three lists in use
+constexpr int kQmpListEntries = kQmpStreamWarps * kQmpWarpListCap;
+// A launch of one or two matrices uses one or two of the three lists, each that much larger.
+__host__ __device__ inline uint32_t qmp_list_cap(int count) {
+    return static_cast<uint32_t>(count >= kQmpLists ? kQmpWarpListCap : kQmpLists * kQmpWarpListCap / count);
+}
+constexpr int kQmpTeams = 2;                               // the computing warps' two halves take alternate stages
+constexpr int kQmpTeamWarps = kQmpStreamWarps / kQmpTeams;
+constexpr int kQmpStepUnits = 4 * kQmpTeamWarps;           // one unit per quarter-warp: what a team takes in one step
 constexpr int kQmpStages = 4;
-constexpr int kQmpStageBytes = kQmpStageUnits * 512;       // fp32 units; bf16 units fill half of a stage
-constexpr int kQmpStreamSmemBytes = kQmpStages * kQmpStageBytes + kQmpLists * kQmpStreamListCap * 8;
+constexpr int kQmpStageBytes = kQmpStepUnits * 512;        // one step of fp32 units, or two of bf16 units
+constexpr int kQmpStreamSmemBytes = kQmpStages * kQmpStageBytes + kQmpLists * kQmpListEntries * 8;
 constexpr int kQmpMaxBatch = 1024;                         // thresholds of put-off second passes live in shared memory
+constexpr int kQmpJobs = 4;                                // matrices m - 1 .. m + 2 have a job on chip
+
+// What the computing warps need to know about a matrix, in shared memory (a field of the kernel parameters or
+// of a descriptor in global memory is a miss of its own, and all of a CTA's warps would wait for it).
+struct QmpJob {
+    unsigned char* vals;
+    uint8_t* meta;
+    const uint8_t* prev;                                   // or null
+    uint32_t KB;
+    uint32_t units;                                        // of this CTA's range
+    uint32_t n0, kb0;                                      // row and 128-column block of its first unit
+    uint32_t rep_n, rep_kb;                                // kQmpStepUnits units further (bf16: the stage's second step)
+    uint32_t next_n, next_kb;                              // from the last step of a stage to the first of the team's next one
+    uint32_t bf16;
+    float lo, hi;                                          // bracket around the threshold
+};
 
 struct QmpStreamShared {
-    double warp_sum[kQmpLists][kQmpWarps];
-    unsigned int warp_flips[kQmpLists][kQmpWarps];
-    unsigned long long flip_total[kQmpLists];
-    unsigned int arrived[kQmpLists];                       // streaming warps done with the matrix in this slot
-    unsigned int list_count[kQmpLists];
-    float bracket[4][2];                                   // [matrix % 4][lo, hi]
-    int bracket_upto;                                      // brackets exist for matrices < bracket_upto
+    double warp_sum[kQmpLists][kQmpStreamWarps];
+    unsigned int warp_flips[kQmpLists][kQmpStreamWarps];
+    unsigned int warp_listed[kQmpLists][kQmpStreamWarps];  // entries of each warp's list (may exceed its capacity)
+    QmpJob job[kQmpJobs];
+    int bracket_upto;                                      // jobs (and brackets) exist for matrices < bracket_upto
     int fixed_upto;                                        // matrices < fixed_upto are finished: their list slot is free
     int abort;
     float thr_tail;
-    float thr_second_pass[kQmpMaxBatch];                   // >= 0: this matrix needs the exact second pass with this threshold
+    int tail_second_pass;
+    float sample[kQmpWarps];
     unsigned long long bar_full[kQmpStages];               // a stage's bytes have landed
     unsigned long long bar_empty[kQmpStages];              // the computing warps are done with a stage
+    unsigned long long bar_done[kQmpLists];                // the computing warps are done with the matrix in this slot
     uint32_t ring_issued, ring_used;                       // the loader's copies of this launch, and its ring position
     unsigned long long bar_sample;                         // the finisher's sample has landed
+    float thr_second_pass[kQmpMaxBatch];                   // >= 0: this matrix needs the exact second pass with this threshold
 };
 
 // mbarrier and bulk-copy wrappers of the stage ring
@@ -195,8 +219,10 @@ __device__ __forceinline__ bool qmp_hint(const QmpDesc& d, float& g) {
     return qmp_hint_usable(g);
 }
 
-// qmp_sample_gamma in two halves, so that something can be started between asking for the sample and using
-// it: all of a thread's sample loads are issued (into v), later they are added up over the CTA.
+// gamma_est of the first matrix: mean |w| over qmp_sample_units units scattered over it (the same units in every
+// CTA; a multiplicative hash keeps them off any row / column-block period).  In two halves, so that something can
+// be started between asking for the sample and using it: all of a thread's sample loads are issued (into v), later
+// they are added up over the CTA -- one barrier, after which every warp adds the 32 partial sums itself.
 constexpr int kQmpSamplePerWarp = kQmpSampleUnits / kQmpWarps;
 __device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[kQmpSamplePerWarp]) {
     const int lane = threadIdx.x & 31;
@@ -211,12 +237,18 @@ __device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[k
         if (sidx < n_s) v[i] = d.w_bf16 ? qmp_load_group<true>(d.W, u, lane) : qmp_load_group<false>(d.W, u, lane);
     }
 }
-__device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float4 (&v)[kQmpSamplePerWarp], double* s_warp) {
+__device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float4 (&v)[kQmpSamplePerWarp], float* s_sample) {
     float acc = 0.0f;
 #pragma unroll
     for (int i = 0; i < kQmpSamplePerWarp; ++i) acc += (fabsf(v[i].x) + fabsf(v[i].y)) + (fabsf(v[i].z) + fabsf(v[i].w));
-    const double total = qmp_block_sum(static_cast<double>(acc), s_warp);
-    return static_cast<float>(total / (static_cast<double>(qmp_sample_units(d.num_units)) * 128.0));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if ((threadIdx.x & 31) == 0) s_sample[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    float t = s_sample[threadIdx.x & 31];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    return t / (static_cast<float>(qmp_sample_units(d.num_units)) * 128.0f);
 }
 
 // gamma_est by ONE warp (the finisher, for matrices 1, 2, ... of a batch without hints): the first
@@ -225,7 +257,7 @@ __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float
 // The smaller sample gets the wider bracket (qmp_bracket_from, `wide`).  Returns a negative number if the
 // copies did not land within the wait limit (the CTA is then aborting).
 constexpr int kQmpSampleUnitsWarp = kQmpSampleUnitsSmall;
-static_assert(kQmpSampleUnitsWarp * 512 <= kQmpStreamListCap * 8, "the sample fits a list");
+static_assert(kQmpSampleUnitsWarp * 512 <= kQmpListEntries * 8, "the sample fits a list");
 __device__ __forceinline__ float qmp_sample_gamma_warp(const QmpDesc& d, int lane, unsigned char* buf, uint32_t bar, uint32_t& bar_phase,
                                                        volatile int* abort_flag) {
     const uint32_t unit_bytes = d.w_bf16 ? 256u : 512u;
@@ -288,125 +320,280 @@ __device__ __forceinline__ bool qmp_loader_issue(QmpLoader& L, const QmpBatch& b
         if (max_copies == 0u) return true;
         --max_copies;
         if (!qmp_mbar_wait(bar_empty0 + 8u * L.ring.stage(), L.ring.phase() ^ 1u, abort_flag)) return false;
-        const uint32_t bytes = min(L.u_end - L.u, static_cast<uint32_t>(kQmpStageUnits)) * L.unit_bytes;
+        const uint32_t units = min(L.u_end - L.u, static_cast<uint32_t>(kQmpStageBytes) / L.unit_bytes);
+        const uint32_t bytes = units * L.unit_bytes;
         qmp_mbar_expect_tx(bar_full0 + 8u * L.ring.stage(), bytes);
         qmp_bulk_load_once(ring_base + L.ring.stage() * kQmpStageBytes, L.W + static_cast<size_t>(L.u) * L.unit_bytes, bytes, bar_full0 + 8u * L.ring.stage(),
                            L.policy);
         ++L.issued;
         L.ring.advance();
-        L.u += kQmpStageUnits;
+        L.u += units;
         if (L.u >= L.u_end) { L.open = false; ++L.m; }
     }
 }
 
-// One lane's two groups (32 B of a row) of pass 1: sum |W|, metadata, provisional values, undecided list,
-// flip count, as in quantize_mask_pack.cuh.  `meta_row` / `vals_row` point at this lane's byte / word of the
-// unit's row inside the metadata and value tiles; `v_off` is the word's byte offset in vals (for the list).
-struct QmpPass1Consts {
-    float thr_lo, thr_hi, mid, half;
-    QmpEntry* list;
-    unsigned int* list_count;
-};
-__device__ __forceinline__ void qmp_pass1_groups(const float4 va, const float4 vb, const QmpPass1Consts& c, uint8_t* meta_row,
-                                                 const uint8_t* prev_row, uint32_t* vals_row, uint32_t v_off, double& acc, unsigned int& flips) {
-    acc += abs_sum4(va) + abs_sum4(vb);
-    float k[4];
-    const uint32_t nib0 = select_pair(va, k[0], k[1]);
-    const uint32_t nib1 = select_pair(vb, k[2], k[3]);
-    if (prev_row != nullptr) {
-        const uint32_t prev = *prev_row;
-        flips += __popc((nibble_to_mask(nib0) | (nibble_to_mask(nib1) << 4)) ^
-                        (nibble_to_mask(prev & 15u) | (nibble_to_mask(prev >> 4) << 4)));
-    }
-    *meta_row = static_cast<uint8_t>(nib0 | (nib1 << 4));
-    *vals_row = ternary_bytes4(k[0], k[1], k[2], k[3], c.thr_hi);
-    const float far = fminf(fminf(fabsf(fabsf(k[0]) - c.mid), fabsf(fabsf(k[1]) - c.mid)),
-                            fminf(fabsf(fabsf(k[2]) - c.mid), fabsf(fabsf(k[3]) - c.mid)));
-    if (far <= c.half) qmp_list_undecided<kQmpStreamListCap>(k, c.thr_lo, c.thr_hi, v_off, c.list, c.list_count);
+// The job of matrix d for this CTA (everything but the bracket).
+__device__ __forceinline__ void qmp_make_job(const QmpDesc& d, QmpJob& jb) {
+    const QmpRange rg = qmp_range(d);
+    jb.vals = reinterpret_cast<unsigned char*>(d.vals);
+    jb.meta = d.meta;
+    jb.prev = d.prev_meta;
+    jb.KB = d.KB;
+    jb.units = rg.u_end - rg.u_begin;
+    jb.n0 = rg.u_begin / d.KB;
+    jb.kb0 = rg.u_begin - jb.n0 * d.KB;
+    jb.rep_n = kQmpStepUnits / d.KB;
+    jb.rep_kb = kQmpStepUnits % d.KB;
+    const uint32_t next = (d.w_bf16 ? 3u : 2u) * kQmpStepUnits;
+    jb.next_n = next / d.KB;
+    jb.next_kb = next % d.KB;
+    jb.bf16 = d.w_bf16;
 }
 
-// Pass 1 of one matrix for a computing warp: its two units of every stage of the CTA's range (a half-warp
-// per unit, a lane two adjacent groups).  Returns the thread's sum |W|; `ok` turns false if a wait ran out.
-template <bool BF16>
-__device__ __forceinline__ double qmp_stream_pass1(const QmpDesc& d, const QmpRange rg, const float thr_lo, const float thr_hi,
-                                                   QmpEntry* list, unsigned int* list_count, unsigned int& flips,
-                                                   QmpRing& ring, uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0,
-                                                   volatile int* abort_flag, bool& ok) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const uint32_t l16 = lane & 15;
-    const uint32_t KB = d.KB;
-    constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
-    const uint32_t step_n = kQmpStageUnits / KB, step_kb = kQmpStageUnits % KB;
-    // |k| in [thr_lo, thr_hi) implies | |k| - mid | <= half (the subtraction is exact, thr_hi < 2 thr_lo;
-    // `half` is rounded up by far more than the rounding of `mid`): a cheap test with no false negatives
-    const QmpPass1Consts c{thr_lo, thr_hi, 0.5f * (thr_lo + thr_hi), fmaf(thr_hi - thr_lo, 0.50005f, thr_hi * 2.4e-7f), list, list_count};
-    double acc = 0.0;
-    const uint32_t in_stage = 2u * warp + (lane >> 4);               // this half-warp's unit of every stage
-    const uint32_t u_first = rg.u_begin + in_stage;
-    uint32_t n_cur = u_first / KB;
-    uint32_t kb_cur = u_first - n_cur * KB;
-    const uint32_t src_off = ring_base + in_stage * kUnitBytes + l16 * (kUnitBytes / 16u);
-    // this lane's place in a row of a metadata tile (byte l16 of 16) and of a value tile (word l16 & 3 of the
-    // 16-byte chunk (l16 >> 2) ^ ((row >> 1) & 3), see layouts.cuh)
-    uint8_t* const meta_lane = d.meta + l16;
-    const uint8_t* const prev_lane = d.prev_meta != nullptr ? d.prev_meta + l16 : nullptr;
-    unsigned char* const vals_lane = reinterpret_cast<unsigned char*>(d.vals) + 4u * (l16 & 3u);
-    const uint32_t chunk = l16 >> 2;
-    const uint32_t range = rg.u_end - rg.u_begin;
-    const uint32_t n_stages = (range + kQmpStageUnits - 1) / kQmpStageUnits;
-    const uint32_t last_units = range - (n_stages - 1u) * kQmpStageUnits;          // units of the last stage (range > 0)
-    for (uint32_t st = 0; st < n_stages; ++st) {
-        const uint32_t stage = ring.stage();
-        if (!qmp_mbar_wait(bar_full0 + 8u * stage, ring.phase(), abort_flag)) { ok = false; break; }
-        const bool mine = st + 1u < n_stages || in_stage < last_units;
-        float4 va, vb;
-        {
-            // a lane without a unit (last stage only) reads what is there: finite or not, it is not used
-            const uint32_t src = src_off + stage * kQmpStageBytes;
-            if constexpr (BF16) {
-                const float4 raw = qmp_lds128(src);
-                const uint32_t r0 = __float_as_uint(raw.x), r1 = __float_as_uint(raw.y), r2 = __float_as_uint(raw.z), r3 = __float_as_uint(raw.w);
-                va = make_float4(bf16lo_to_f32(r0), bf16hi_to_f32(r0), bf16lo_to_f32(r1), bf16hi_to_f32(r1));
-                vb = make_float4(bf16lo_to_f32(r2), bf16hi_to_f32(r2), bf16lo_to_f32(r3), bf16hi_to_f32(r3));
-            } else {
-                va = qmp_lds128(src);
-                vb = qmp_lds128(src + 16u);
-            }
+__device__ __forceinline__ uint32_t qmp_lanes_below() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// A computing warp's list of undecided kept values; the count is the same in every lane.
+struct QmpWarpList {
+    QmpEntry* entries;
+    uint32_t cap, n;
+};
+// Appends the lanes' undecided values: bit j of `und` = value j of this lane, at byte `off(j)` of vals with weight
+// `value(j)`.  Whole warp.  No atomics: the lanes' places come from ballots (mostly one round: few lanes have two).
+template <typename Off, typename Value>
+__device__ __forceinline__ void qmp_list_append(QmpWarpList& list, uint32_t und, Off off, Value value) {
+    for (uint32_t who = __ballot_sync(0xFFFFFFFFu, und != 0u); who != 0u; who = __ballot_sync(0xFFFFFFFFu, und != 0u)) {
+        if (und != 0u) {
+            const int j = __ffs(static_cast<int>(und)) - 1;
+            const uint32_t at = list.n + __popc(who & qmp_lanes_below());
+            if (at < list.cap) { list.entries[at].byte_off = off(j); list.entries[at].w = value(j); }
+            und &= und - 1u;
         }
+        list.n += __popc(who);
+    }
+}
+
+// Mask bits that differ between two metadata words of four groups, halved: two kept pairs of a group are the same
+// (xor 0), share one column (2 bits differ) or none (4); the last happens exactly for the xors 5 and 10.
+__device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
+    const uint32_t any = (x | (x >> 1) | (x >> 2) | (x >> 3)) & 0x11111111u;
+    const uint32_t same = ~(x ^ (x >> 2));                            // bits 0 / 1 of a nibble equal its bits 2 / 3
+    const uint32_t none = same & (same >> 1) & (x ^ (x >> 1)) & 0x11111111u;
+    return __popc(any | (none << 1));
+}
+
+// Pass 1 of one matrix for a computing warp: its four units of every stage of its team (a quarter-warp per unit, a
+// lane 16 weights = four groups).  `g0` counts the ring's stages up to this matrix.  Returns the thread's
+// sum |W|; `ok` turns false if a wait ran out.
+//
+// The instructions are what this pass costs: the memory delivers 256 weights per SM every 44 clocks (fp32), and
+// selection, signs, comparisons and the fp64 sum of 256 weights alone take 24 (8 more are their shared-memory
+// reads).  An earlier form with 8 weights per lane spent 231 warp instructions on them, more than half beside that
+// core.  So: 16 weights per lane and iteration (one 8-byte store of values, one 2-byte store of metadata, one
+// barrier wait, one look at the previous metadata); the selection's predicates are folded into the compares;
+// "|k| >= thr" and "is |k| undecided" come from ONE subtraction, e = pred(thr_hi) - |k| (its sign bit is the first
+// answer, e <= pred(thr_hi) - thr_lo as an unsigned compare of the bits the second, and four sign bits become four
+// byte masks by byte permutes); the undecided are appended with ballots instead of atomics; flips are counted
+// for four groups at a time from the xor of the metadata.
+//
+// A lane's 64 B (fp32) are read as 16-byte pieces in rotated order, (i + l8 / 2) mod 4, so that the eight lanes of a
+// unit hit different banks; the rotation is undone on the 8 + 2 result bytes (two byte permutes, one shift).
+template <bool BF16>
+__device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t ring_base,
+                                                   uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp = threadIdx.x >> 5;
+    const uint32_t team = warp >= kQmpTeamWarps ? 1u : 0u;
+    const uint32_t l8 = lane & 7;
+    constexpr int REP = BF16 ? 2 : 1;                                 // steps per stage
+    constexpr int PIECES = BF16 ? 2 : 4;                              // 16-byte pieces per lane
+    constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
+    const uint32_t KB = jb.KB;
+    // kept is +-1 iff |k| > thr_pred, undecided iff 0 <= thr_pred - |k| <= width.  The subtraction is exact near the
+    // threshold and monotone everywhere: a value wrongly taken for undecided can only lie below thr_lo, and the
+    // fix-up decides it like any other.
+    const float thr_pred = __uint_as_float(__float_as_uint(jb.hi) - 1u);
+    const uint32_t width = __float_as_uint(thr_pred - jb.lo);
+    const uint32_t n_stages = (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
+    const uint32_t st0 = (team ^ g0) & 1u;                            // the team's first stage of this matrix
+    double acc = 0.0;
+    const uint32_t in_step = 4u * (warp - team * kQmpTeamWarps) + (lane >> 3);   // this quarter-warp's unit of every step
+    uint32_t n, kb;
+    {
+        const uint32_t k0 = jb.kb0 + st0 * (REP * kQmpStepUnits) + in_step;
+        const uint32_t dn = k0 / KB;
+        n = jb.n0 + dn;
+        kb = k0 - dn * KB;
+    }
+    int left = static_cast<int>(jb.units) - static_cast<int>(st0 * (REP * kQmpStepUnits) + in_step);   // > 0: this quarter-warp has a unit in the step
+    const uint32_t turn = BF16 ? (l8 >> 2) : (l8 >> 1);               // rotation of the pieces ...
+    const uint32_t rot = BF16 ? 2u * turn : turn;                     // ... and of the groups
+    uint32_t src[PIECES];
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) src[i] = ring_base + in_step * kUnitBytes + l8 * (kUnitBytes / 8u) + 16u * ((i + turn) & (PIECES - 1u));
+    // result bytes 2 p, 2 p + 1 (p = group of the unit's row) come from the group read as number (p - rot) mod 4
+    uint32_t sel_lo = 0u, sel_hi = 0u;
+#pragma unroll
+    for (uint32_t p = 0; p < 2; ++p) {
+        const uint32_t i_lo = (p - rot) & 3u, i_hi = (p + 2u - rot) & 3u;
+        sel_lo |= ((2u * i_lo) | ((2u * i_lo + 1u) << 4)) << (8u * p);
+        sel_hi |= ((2u * i_hi) | ((2u * i_hi + 1u) << 4)) << (8u * p);
+    }
+    uint8_t* const meta_lane = jb.meta + 2u * l8;
+    const uint8_t* const prev_lane = jb.prev != nullptr ? jb.prev + 2u * l8 : nullptr;
+    const uint32_t chunk = l8 >> 1;
+    // row index in the tiled order: 16 B of metadata and 64 B of values each (layouts.cuh)
+    auto tiled_row = [&](uint32_t nn, uint32_t kk) { return (((nn >> 7) * KB + kk) << 7) + (nn & 127u); };
+    uint32_t q = tiled_row(n, kb);
+    uint32_t prev = 0u;
+    if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
+    for (uint32_t st = st0; st < n_stages; st += 2u) {
+        const uint32_t g = g0 + st;
+        const uint32_t stage = g & (kQmpStages - 1u);
+        if (!qmp_mbar_wait(bar_full0 + 8u * stage, (g / kQmpStages) & 1u, abort_flag)) { ok = false; break; }
+        float4 raw[REP * PIECES];
+        // a lane without a unit (last stage only) reads what is there: it is not used
+#pragma unroll
+        for (int i = 0; i < REP * PIECES; ++i)
+            raw[i] = qmp_lds128(src[i % PIECES] + stage * kQmpStageBytes + (i / PIECES) * (kQmpStepUnits * kUnitBytes));
         __syncwarp();
         if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);           // the values are in registers: the stage may be refilled
-        ring.advance();
-        const uint32_t tile_idx = (n_cur >> 7) * KB + kb_cur;
-        const uint32_t rr = n_cur & 127u;
-        n_cur += step_n;
-        kb_cur += step_kb;
-        if (kb_cur >= KB) { kb_cur -= KB; ++n_cur; }
-        if (mine) {
-            const size_t m_off = static_cast<size_t>(tile_idx) * 2048u + (rr << 4);
-            const size_t v_off = static_cast<size_t>(tile_idx) * 8192u + ((rr << 6) + ((chunk ^ ((rr >> 1) & 3u)) << 4));
-            qmp_pass1_groups(va, vb, c, meta_lane + m_off, prev_lane != nullptr ? prev_lane + m_off : nullptr,
-                             reinterpret_cast<uint32_t*>(vals_lane + v_off), static_cast<uint32_t>(v_off) + 4u * (l16 & 3u), acc, flips);
+#pragma unroll
+        for (int rep = 0; rep < REP; ++rep) {
+            const bool mine = left > 0;
+            const uint32_t q_cur = q, prev_cur = prev;
+            const uint32_t v8 = q_cur * 8u + 2u * (chunk ^ ((n >> 1) & 3u)) + (l8 & 1u);       // 8-byte piece of the values
+            n += rep + 1 < REP ? jb.rep_n : jb.next_n;
+            kb += rep + 1 < REP ? jb.rep_kb : jb.next_kb;
+            if (kb >= KB) { kb -= KB; ++n; }
+            left -= rep + 1 < REP ? kQmpStepUnits : (BF16 ? 3 : 2) * kQmpStepUnits;
+            q = tiled_row(n, kb);
+            if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
+            float k[8];
+            uint32_t nibbles = 0u;
+            double sum = 0.0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float4 w;
+                if constexpr (BF16) {
+                    const float4 r4 = raw[rep * PIECES + (i >> 1)];
+                    const uint32_t r0 = __float_as_uint((i & 1) ? r4.z : r4.x), r1 = __float_as_uint((i & 1) ? r4.w : r4.y);
+                    w = make_float4(bf16lo_to_f32(r0), bf16hi_to_f32(r0), bf16lo_to_f32(r1), bf16hi_to_f32(r1));
+                } else {
+                    w = raw[i];
+                }
+                sum += abs_sum4(w);
+                nibbles |= select_pair(w, k[2 * i], k[2 * i + 1]) << (4 * i);
+            }
+            const uint32_t word = ((nibbles * 0x10001u) >> (16u - 4u * rot)) & 0xFFFFu;        // nibble i to its place, (i + rot) mod 4
+            uint32_t e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(thr_pred - fabsf(k[i]));
+            uint32_t t[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t keep = prmt(prmt(e[4 * h], e[4 * h + 1], 0x00FBu), prmt(e[4 * h + 2], e[4 * h + 3], 0x00FBu), 0x5410u);
+                const uint32_t sign = prmt(prmt(__float_as_uint(k[4 * h]), __float_as_uint(k[4 * h + 1]), 0x00FBu),
+                                           prmt(__float_as_uint(k[4 * h + 2]), __float_as_uint(k[4 * h + 3]), 0x00FBu), 0x5410u);
+                t[h] = (sign | 0x01010101u) & keep;
+            }
+            uint32_t und = 0u;
+            if (mine) {
+                acc += sum;
+                *reinterpret_cast<uint16_t*>(meta_lane + static_cast<size_t>(q_cur) * 16u) = static_cast<uint16_t>(word);
+                *reinterpret_cast<uint2*>(jb.vals + static_cast<size_t>(v8) * 8u) = make_uint2(prmt(t[0], t[1], sel_lo), prmt(t[0], t[1], sel_hi));
+                if (prev_lane != nullptr) flips += qmp_flip_pairs(word ^ prev_cur);
+                if (min(min(min(e[0], e[1]), min(e[2], e[3])), min(min(e[4], e[5]), min(e[6], e[7]))) <= width) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
+                }
+            }
+            qmp_list_append(list, und, [&](int j) { return v8 * 8u + 2u * (((j >> 1) + rot) & 3u) + (j & 1u); },
+                            [&](int j) {
+                                const float a = j & 1 ? k[1] : k[0], b = j & 1 ? k[3] : k[2], c = j & 1 ? k[5] : k[4], d = j & 1 ? k[7] : k[6];
+                                return j & 4 ? (j & 2 ? d : c) : (j & 2 ? b : a);
+                            });
         }
     }
+    g0 += n_stages;
+    flips *= 2u;
     return acc;
 }
 
-// What the exact gamma decides for a matrix whose pass 1 is complete: true if the listed values were
-// all that had to be redone (and `fix` should run), false if the whole range must be ternarised again.
-__device__ __forceinline__ bool qmp_bracket_holds(const QmpDesc& d, float thr, float lo, float hi, unsigned int listed) {
-    return lo <= thr && thr <= hi && listed <= static_cast<unsigned int>(kQmpStreamListCap) && d.dense_q == nullptr &&
+// {tag, partial sum} of a CTA as one 128-bit word: whoever sees the tag has the sum (no fence, one trip).
+__device__ __forceinline__ void qmp_slot_store(QmpSlot* slot, unsigned long long tag, double partial) {
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
+                 ::"l"(slot), "l"(tag), "l"(__double_as_longlong(partial)) : "memory");
+}
+__device__ __forceinline__ bool qmp_slot_load(const QmpSlot* slot, unsigned long long tag, double& partial) {
+    unsigned long long t;
+    long long v;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(t), "=l"(v) : "l"(slot) : "memory");
+    if (t != tag) return false;
+    partial = __longlong_as_double(v);
+    return true;
+}
+
+// The sum of all CTAs' partial sums of a matrix by one warp, in a fixed order: the same bits in every CTA.  A lane
+// looks after the slots lane, lane + 32, ..., all of them polled together.  False if the wait ran out.
+__device__ __forceinline__ bool qmp_exchange(const QmpSlot* base, unsigned long long tag, int lane, volatile int* abort_flag, double& sum) {
+    constexpr int kPerLane = (kQmpMaxCtas + 31) / 32;
+    double part[kPerLane];
+    uint32_t missing = 0u;
+#pragma unroll
+    for (int j = 0; j < kPerLane; ++j) {
+        part[j] = 0.0;
+        if (lane + 32u * j < gridDim.x) missing |= 1u << j;
+    }
+    unsigned long long t0 = 0ull;
+    unsigned int spins = 0;
+    bool ok = true;
+    while (missing != 0u) {
+#pragma unroll
+        for (int j = 0; j < kPerLane; ++j)
+            if (((missing >> j) & 1u) != 0u && qmp_slot_load(&base[lane + 32 * j], tag, part[j])) missing &= ~(1u << j);
+        if (missing != 0u && ((++spins & 0xFFu) == 0u)) {
+            if (*abort_flag) { ok = false; break; }
+            const unsigned long long now = global_timer_ns_qmp();
+            if (t0 == 0ull) t0 = now;
+            else if (now - t0 > *reinterpret_cast<volatile unsigned long long*>(&g_wait_limit_ns)) { ok = false; break; }
+        }
+    }
+    ok = __all_sync(0xFFFFFFFFu, ok);
+    if (!ok) {
+        if (lane == 0) { *abort_flag = 1; atomicExch(&g_device_status, static_cast<int>(SBN_ERR_TIMEOUT)); }
+        return false;
+    }
+    sum = 0.0;
+#pragma unroll
+    for (int j = 0; j < kPerLane; ++j) sum += part[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    return true;
+}
+
+// Do the listed values suffice, or must the whole range be ternarised again with the exact threshold?
+__device__ __forceinline__ bool qmp_bracket_holds(const QmpDesc& d, float thr, const QmpJob& jb, unsigned int longest_list, uint32_t list_cap) {
+    return jb.lo <= thr && thr <= jb.hi && longest_list <= list_cap && d.dense_q == nullptr &&
            d.num_units <= (1u << 26);                        // listed byte offsets are 32-bit
+}
+__device__ __forceinline__ void qmp_fix_entry(uint8_t* vals, const QmpEntry e, float thr) {
+    vals[e.byte_off] = static_cast<uint8_t>(fabsf(e.w) >= thr ? (e.w < 0.0f ? 0xFFu : 0x01u) : 0u);
 }
 
 __global__ void __launch_bounds__(kQmpThreads, 1)
 quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, const QmpDesc* __restrict__ rest, int count,
                                  QmpSlot* slots, unsigned long long* generation, unsigned long long call_nonce,
                                  int test_withhold_slot, QmpMemo* memo) {
-    extern __shared__ __align__(128) unsigned char s_dyn[];   // [kQmpStages][kQmpStageBytes] ring, then [kQmpLists][kQmpStreamListCap] entries
+    extern __shared__ __align__(128) unsigned char s_dyn[];   // [kQmpStages][kQmpStageBytes] ring, then kQmpLists * kQmpListEntries entries
     QmpEntry* const s_list = reinterpret_cast<QmpEntry*>(s_dyn + kQmpStages * kQmpStageBytes);
+    const uint32_t list_cap = qmp_list_cap(count);
+    auto list_of = [&](int slot, int w) { return s_list + static_cast<uint32_t>(slot * kQmpStreamWarps + w) * list_cap; };
     __shared__ QmpStreamShared sh;
-    __shared__ double s_warp[kQmpWarps];
 
     const QmpBatch batch{inl, rest};
     const QmpDesc& first = inl.d[0];
@@ -416,90 +603,89 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     volatile int* const abort_flag = &sh.abort;
     const uint32_t ring_base = qmp_smem_u32(s_dyn);
     const uint32_t bar_full0 = qmp_smem_u32(&sh.bar_full[0]), bar_empty0 = qmp_smem_u32(&sh.bar_empty[0]);
+    const uint32_t bar_done0 = qmp_smem_u32(&sh.bar_done[0]);
     if (threadIdx.x == 0) {
-        sh.bracket_upto = 0;
         sh.fixed_upto = 0;
         sh.abort = 0;
+        sh.tail_second_pass = 0;
         sh.ring_issued = 0u; sh.ring_used = 0u;
-        for (int i = 0; i < kQmpLists; ++i) { sh.arrived[i] = 0u; sh.list_count[i] = 0u; sh.flip_total[i] = 0ull; }
+        for (int i = 0; i < kQmpLists; ++i) qmp_mbar_init(bar_done0 + 8u * i, kQmpStreamWarps);
         for (int i = 0; i < kQmpStages; ++i) {
             qmp_mbar_init(bar_full0 + 8u * i, 1u);                     // the loader's expect_tx
-            qmp_mbar_init(bar_empty0 + 8u * i, kQmpStreamWarps);       // one arrival per computing warp
+            qmp_mbar_init(bar_empty0 + 8u * i, kQmpTeamWarps);         // one arrival per computing warp of the stage's team
         }
         qmp_mbar_init(qmp_smem_u32(&sh.bar_sample), 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < kQmpMaxBatch; i += kQmpThreads) sh.thr_second_pass[i] = -1.0f;
+    if (threadIdx.x == 32) qmp_make_job(first, sh.job[0]);
+    if (threadIdx.x == 64 && count > 1) qmp_make_job(second, sh.job[1]);
+    for (int i = threadIdx.x; i < count; i += kQmpThreads) sh.thr_second_pass[i] = -1.0f;
     __syncthreads();
     // No early signal to the next kernel of the stream: this kernel writes packed weights, and the
     // GEMM kernels fetch weights before their own dependency wait (see sbn_common.cuh).
     pdl_wait();
-    const unsigned long long gen0 = *reinterpret_cast<volatile unsigned long long*>(generation);
-    const unsigned long long tag = qmp_tag(call_nonce, gen0);
 
     // ---- What the first bracket needs is asked for BEFORE the loader fills the ring: the hints of matrices
-    // 0 and 1 (4-byte reads) or, without a usable hint, the sample of matrix 0 (all threads, one round
-    // trip).  Issued together with the ring's first copies they queue behind the 17 MB that the loaders of
-    // all CTAs ask for at the same moment (up to 3.5 us measured, and the CTA that is served last finishes
-    // last); so the loader waits for the hints to be there, or for the sample loads to be on their way.
-    float g01[2];                                            // both reads in flight before either is looked at
+    // 0 and 1 (4-byte reads), and without a hint of the caller's the sample of matrix 0 (all threads, one round
+    // trip) together with what an earlier call may have left.  Issued with the ring's first copies they queue
+    // behind the 17 MB that the loaders of all CTAs ask for at the same moment (up to 3.5 us measured, and the
+    // CTA that is served last finishes last).
+    float g01[2];
     g01[0] = first.gamma_hint != nullptr ? *reinterpret_cast<const volatile float*>(first.gamma_hint) : 0.0f;
     g01[1] = (count > 1 && second.gamma_hint != nullptr) ? *reinterpret_cast<const volatile float*>(second.gamma_hint) : 0.0f;
-    if (memo != nullptr && first.gamma_hint == nullptr) {
-        // a single matrix without a hint: what the previous call on this workspace left, if it was this matrix
-        // (two 16-byte reads in flight together, not four dependent ones)
-        unsigned long long m_tag, m_w;
-        uint32_t m_units, m_scale;
-        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(m_tag), "=l"(m_w) : "l"(memo));
-        asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];" : "=r"(m_units), "=r"(m_scale) : "l"(&memo->num_units));
+    float4 sample0[kQmpSamplePerWarp];
+    const bool sample_early = first.gamma_hint == nullptr;
+    if (sample_early) {
+        unsigned long long m_tag = 0ull, m_w = 0ull;
+        uint32_t m_units = 0u, m_scale = 0u;
+        if (memo != nullptr) {
+            // a single matrix without a hint: what the previous call on this workspace left, if it was this matrix
+            asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(m_tag), "=l"(m_w) : "l"(memo));
+            asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];" : "=r"(m_units), "=r"(m_scale) : "l"(&memo->num_units));
+        }
+        qmp_sample_issue(first, sample0);
         if (m_tag == kQmpMemoMagic && m_w == reinterpret_cast<unsigned long long>(first.W) && m_units == first.num_units)
             g01[0] = __uint_as_float(m_scale);
     }
     const bool hinted01[2] = {qmp_hint_usable(g01[0]), qmp_hint_usable(g01[1])};
-    float4 sample0[kQmpSamplePerWarp];
-    if (!hinted01[0]) qmp_sample_issue(first, sample0);
+    if (!sample_early && !hinted01[0]) qmp_sample_issue(first, sample0);
     QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, qmp_policy_evict_first()};
     const bool is_loader = warp == kQmpLoaderWarp && lane == 0;
     if (is_loader) qmp_loader_issue(loader, batch, count, kQmpStages, ring_base, bar_full0, bar_empty0, abort_flag);
-    if (!hinted01[0]) g01[0] = qmp_sample_finish(first, sample0, s_warp);
+    if (!hinted01[0]) g01[0] = qmp_sample_finish(first, sample0, sh.sample);
     if (threadIdx.x == 0) {
-        qmp_bracket_from(g01[0], first.num_units, hinted01[0], sh.bracket[0][0], sh.bracket[0][1]);
+        qmp_bracket_from(g01[0], first.num_units, hinted01[0], sh.job[0].lo, sh.job[0].hi);
         // matrix 1: from its hint here; without one the finisher samples it while matrix 0 streams
-        if (hinted01[1]) qmp_bracket_from(g01[1], second.num_units, true, sh.bracket[1][0], sh.bracket[1][1]);
+        if (hinted01[1]) qmp_bracket_from(g01[1], second.num_units, true, sh.job[1].lo, sh.job[1].hi);
         sh.bracket_upto = hinted01[1] ? 2 : 1;
     }
     __syncthreads();
 
     if (warp < kQmpStreamWarps) {
         // ------------------------------------------------------------------ computing warps
-        QmpRing ring{0u};
+        uint32_t stages = 0u;                                // of the matrices so far
         for (int m = 0; m < count; ++m) {
             const int slot = m % kQmpLists;
             if (!qmp_wait_ge(&sh.bracket_upto, m + 1, abort_flag)) break;
             if (!qmp_wait_ge(&sh.fixed_upto, m - (kQmpLists - 1), abort_flag)) break;
-            const QmpDesc d = qmp_desc_of(batch, m);
-            const QmpRange rg = qmp_range(d);
-            const float lo = *reinterpret_cast<volatile float*>(&sh.bracket[m & 3][0]);
-            const float hi = *reinterpret_cast<volatile float*>(&sh.bracket[m & 3][1]);
+            __threadfence_block();
+            const QmpJob jb = sh.job[m & (kQmpJobs - 1)];
             unsigned int flips = 0;
             bool ok = true;
-            double mine = d.w_bf16 ? qmp_stream_pass1<true>(d, rg, lo, hi, s_list + slot * kQmpStreamListCap, &sh.list_count[slot], flips,
-                                                            ring, ring_base, bar_full0, bar_empty0, abort_flag, ok)
-                                   : qmp_stream_pass1<false>(d, rg, lo, hi, s_list + slot * kQmpStreamListCap, &sh.list_count[slot], flips,
-                                                             ring, ring_base, bar_full0, bar_empty0, abort_flag, ok);
+            QmpWarpList list{list_of(slot, warp), list_cap, 0u};
+            double mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, ring_base, bar_full0, bar_empty0, abort_flag, ok)
+                                  : qmp_stream_pass1<false>(jb, list, flips, stages, ring_base, bar_full0, bar_empty0, abort_flag, ok);
             if (!ok) break;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
-                flips += __shfl_xor_sync(0xFFFFFFFFu, flips, o);
-            }
+            for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
+            if (jb.prev != nullptr) flips = __reduce_add_sync(0xFFFFFFFFu, flips);
             __syncwarp();                                    // every lane's list entries are written
             if (lane == 0) {
                 sh.warp_sum[slot][warp] = mine;
                 sh.warp_flips[slot][warp] = flips;
-                __threadfence_block();                       // the sums, and this warp's list entries, before the count
-                atomicAdd(&sh.arrived[slot], 1u);
+                sh.warp_listed[slot][warp] = list.n;
+                qmp_mbar_arrive(bar_done0 + 8u * slot);      // release: the sums, and this warp's list entries, before the count
             }
             __syncwarp();
         }
@@ -513,33 +699,39 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         __syncwarp();
     } else {
         // ------------------------------------------------------------------ the finisher (warp 31)
+        const unsigned long long gen0 = *reinterpret_cast<volatile unsigned long long*>(generation);
+        const unsigned long long tag = qmp_tag(call_nonce, gen0);
         bool ok = true;
         uint32_t sample_phase = 0u;
         if (count > 1 && !hinted01[1]) {
             // bracket of matrix 1 from a sample into its own (still unused) list, while matrix 0 streams
-            const float g = qmp_sample_gamma_warp(second, lane, reinterpret_cast<unsigned char*>(s_list + 1 * kQmpStreamListCap),
+            const float g = qmp_sample_gamma_warp(second, lane, reinterpret_cast<unsigned char*>(list_of(1, 0)),
                                                   qmp_smem_u32(&sh.bar_sample), sample_phase, abort_flag);
             if (g < 0.0f) {
                 ok = false;
             } else {
                 if (lane == 0) {
-                    qmp_bracket_from(g, second.num_units, false, sh.bracket[1][0], sh.bracket[1][1], true);
+                    qmp_bracket_from(g, second.num_units, false, sh.job[1].lo, sh.job[1].hi, true);
                     __threadfence_block();
                     *reinterpret_cast<volatile int*>(&sh.bracket_upto) = 2;
                 }
                 __syncwarp();
             }
         }
-        for (int m = 0; ok && m < count; ++m) {
-            const int slot = m % kQmpLists;
-            // bracket of matrix m + 2 from the caller's hint, well before the computing warps ask for it
+        // step m: publish matrix m, then exchange and finish matrix m - 1; step `count` finishes the last matrix
+        // (its fix-up is left to all warps)
+        unsigned int flips_prev = 0u;
+        for (int m = 0; ok && m <= count; ++m) {
+            // job and, from the caller's hint, bracket of matrix m + 2, well before the computing warps ask for it
             bool sample_next = false;
             if (m + 2 < count) {
                 const QmpDesc d2 = qmp_desc_of(batch, m + 2);
+                QmpJob& jb = sh.job[(m + 2) & (kQmpJobs - 1)];
+                if (lane == 0) qmp_make_job(d2, jb);
                 float g;
                 if (qmp_hint(d2, g)) {
                     if (lane == 0) {
-                        qmp_bracket_from(g, d2.num_units, true, sh.bracket[(m + 2) & 3][0], sh.bracket[(m + 2) & 3][1]);
+                        qmp_bracket_from(g, d2.num_units, true, jb.lo, jb.hi);
                         __threadfence_block();
                         *reinterpret_cast<volatile int*>(&sh.bracket_upto) = m + 3;
                     }
@@ -548,116 +740,85 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
                     sample_next = true;
                 }
             }
-            // matrix m: every streaming warp has arrived -> this CTA's partial sum, published
-            if (!qmp_wait_ge(reinterpret_cast<volatile int*>(&sh.arrived[slot]), kQmpStreamWarps, abort_flag)) { ok = false; break; }
-            __threadfence_block();
-            const QmpDesc d = qmp_desc_of(batch, m);
-            {
+            unsigned int flips_cur = 0u;
+            if (m < count) {
+                // matrix m: every computing warp has arrived -> this CTA's partial sum, published
+                const int slot = m % kQmpLists;
+                const QmpDesc d = qmp_desc_of(batch, m);
+                // zeroed well before any CTA can add to it (they add once they have seen this CTA's slot)
+                if (blockIdx.x == 0 && lane == 0 && d.flip_bits != nullptr) { *d.flip_bits = 0ull; __threadfence(); }
+                if (!qmp_mbar_wait(bar_done0 + 8u * slot, static_cast<uint32_t>(m / kQmpLists) & 1u, abort_flag)) { ok = false; break; }
                 double v = lane < kQmpStreamWarps ? *reinterpret_cast<volatile double*>(&sh.warp_sum[slot][lane]) : 0.0;
-                unsigned int f = lane < kQmpStreamWarps ? *reinterpret_cast<volatile unsigned int*>(&sh.warp_flips[slot][lane]) : 0u;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-                    f += __shfl_xor_sync(0xFFFFFFFFu, f, o);
-                }
-                if (lane == 0) {
-                    sh.flip_total[slot] = f;
-                    if (blockIdx.x == 0 && d.flip_bits != nullptr) *d.flip_bits = 0ull;
-                    QmpSlot* sl = slots + static_cast<size_t>(m) * gridDim.x + blockIdx.x;
-                    sl->partial = v;
-                    __threadfence();
-                    if (!(test_withhold_slot && blockIdx.x == gridDim.x - 1))
-                        *reinterpret_cast<volatile unsigned long long*>(&sl->nonce) = tag;
-                }
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+                if (lane == 0 && !(test_withhold_slot && blockIdx.x == gridDim.x - 1))
+                    qmp_slot_store(slots + static_cast<size_t>(m) * gridDim.x + blockIdx.x, tag, v);
+                if (d.flip_bits != nullptr)
+                    flips_cur = __reduce_add_sync(0xFFFFFFFFu, lane < kQmpStreamWarps ? *reinterpret_cast<volatile unsigned int*>(&sh.warp_flips[slot][lane]) : 0u);
                 __syncwarp();
             }
             // matrix m - 1: exchange, exact threshold, fix-up
             if (m >= 1) {
                 const int pslot = (m - 1) % kQmpLists;
                 const QmpDesc dp = qmp_desc_of(batch, m - 1);
-                const QmpSlot* base = slots + static_cast<size_t>(m - 1) * gridDim.x;
-                // a lane looks after the slots lane, lane + 32, ...: all its flags are polled together, then all
-                // its partial sums are read together (two round trips in all, not two per slot)
-                constexpr int kPerLane = (kQmpMaxCtas + 31) / 32;
-                {
-                    unsigned long long t0 = 0ull;
-                    unsigned int spins = 0;
-                    bool seen = false;
-                    while (!seen) {
-                        seen = true;
-#pragma unroll
-                        for (int j = 0; j < kPerLane; ++j) {
-                            const unsigned int i = lane + 32u * j;
-                            if (i < gridDim.x) seen = seen && (*reinterpret_cast<const volatile unsigned long long*>(&base[i].nonce) == tag);
-                        }
-                        if (!seen && ((++spins & 0xFFu) == 0u)) {
-                            if (*abort_flag) break;
-                            const unsigned long long now = global_timer_ns_qmp();
-                            if (t0 == 0ull) t0 = now;
-                            else if (now - t0 > *reinterpret_cast<volatile unsigned long long*>(&g_wait_limit_ns)) break;
-                        }
-                    }
-                    if (!seen) ok = false;
-                }
-                ok = __all_sync(0xFFFFFFFFu, ok);
-                if (!ok) {
-                    if (lane == 0) { *abort_flag = 1; atomicExch(&g_device_status, static_cast<int>(SBN_ERR_TIMEOUT)); }
-                    break;
-                }
-                __threadfence();
-                double part[kPerLane];
-#pragma unroll
-                for (int j = 0; j < kPerLane; ++j) {
-                    const unsigned int i = lane + 32u * j;
-                    part[j] = i < gridDim.x ? *reinterpret_cast<const volatile double*>(&base[i].partial) : 0.0;
-                }
-                double sum = 0.0;
-#pragma unroll
-                for (int j = 0; j < kPerLane; ++j) sum += part[j];                 // a lane's slots in increasing order
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);    // the same order in every CTA
+                double sum;
+                ok = qmp_exchange(slots + static_cast<size_t>(m - 1) * gridDim.x, tag, lane, abort_flag, sum);
+                if (!ok) break;
                 const float gamma = static_cast<float>(sum / (static_cast<double>(dp.num_units) * 128.0));
                 const float scale = fmaxf(gamma, kEps);
-                float thr = 0.0f;
-                if (lane == 0) {
-                    thr = ternary_threshold(scale);
-                    if (blockIdx.x == 0) *dp.w_scale = scale;
-                    if (dp.flip_bits != nullptr && sh.flip_total[pslot] != 0ull) atomicAdd(dp.flip_bits, sh.flip_total[pslot]);
-                }
-                thr = __shfl_sync(0xFFFFFFFFu, thr, 0);
-                const unsigned int listed = *reinterpret_cast<volatile unsigned int*>(&sh.list_count[pslot]);
-                if (qmp_bracket_holds(dp, thr, sh.bracket[(m - 1) & 3][0], sh.bracket[(m - 1) & 3][1], listed)) {
-                    const QmpEntry* list = s_list + pslot * kQmpStreamListCap;
+                const float thr = ternary_threshold(scale);
+                const unsigned int longest = __reduce_max_sync(0xFFFFFFFFu, lane < kQmpStreamWarps ? *reinterpret_cast<volatile unsigned int*>(&sh.warp_listed[pslot][lane]) : 0u);
+                const bool holds = qmp_bracket_holds(dp, thr, sh.job[(m - 1) & (kQmpJobs - 1)], longest, list_cap);
+                if (m == count) {
+                    if (lane == 0) { sh.thr_tail = thr; sh.tail_second_pass = holds ? 0 : 1; }
+                } else if (holds) {
                     uint8_t* vb = reinterpret_cast<uint8_t*>(dp.vals);
-                    for (unsigned int e = lane; e < listed; e += 32u) {
-                        const float w = list[e].w;
-                        vb[list[e].byte_off] = static_cast<uint8_t>(fabsf(w) >= thr ? (w < 0.0f ? 0xFFu : 0x01u) : 0u);
+                    for (int w = 0; w < kQmpStreamWarps; ++w) {
+                        const QmpEntry* list = list_of(pslot, w);
+                        const unsigned int listed = sh.warp_listed[pslot][w];
+                        for (unsigned int i = lane; i < listed; i += 32u) qmp_fix_entry(vb, list[i], thr);
                     }
                 } else if (lane == 0) {
                     sh.thr_second_pass[m - 1] = thr;
                 }
                 __syncwarp();
                 if (lane == 0) {
-                    sh.arrived[pslot] = 0u;
-                    sh.list_count[pslot] = 0u;
                     __threadfence_block();
                     *reinterpret_cast<volatile int*>(&sh.fixed_upto) = m;
+                    if (blockIdx.x == 0) *dp.w_scale = scale;
+                    if (dp.flip_bits != nullptr && flips_prev != 0u) {
+                        __threadfence();                     // after CTA 0's zero: its slot has been seen
+                        atomicAdd(dp.flip_bits, static_cast<unsigned long long>(flips_prev));
+                    }
                 }
                 __syncwarp();
             }
+            flips_prev = flips_cur;
             // bracket of matrix m + 2 from a sample, if it has no hint: a whole matrix before the computing warps
             // ask for it.  The sample lands in the list that matrix m - 1 has just given back (the one m + 2 will use).
             if (sample_next) {
                 const QmpDesc d2 = qmp_desc_of(batch, m + 2);
-                const float g = qmp_sample_gamma_warp(d2, lane, reinterpret_cast<unsigned char*>(s_list + ((m + 2) % kQmpLists) * kQmpStreamListCap),
+                const float g = qmp_sample_gamma_warp(d2, lane, reinterpret_cast<unsigned char*>(list_of((m + 2) % kQmpLists, 0)),
                                                       qmp_smem_u32(&sh.bar_sample), sample_phase, abort_flag);
                 if (g < 0.0f) { ok = false; break; }
                 if (lane == 0) {
-                    qmp_bracket_from(g, d2.num_units, false, sh.bracket[(m + 2) & 3][0], sh.bracket[(m + 2) & 3][1], true);
+                    QmpJob& jb = sh.job[(m + 2) & (kQmpJobs - 1)];
+                    qmp_bracket_from(g, d2.num_units, false, jb.lo, jb.hi, true);
                     __threadfence_block();
                     *reinterpret_cast<volatile int*>(&sh.bracket_upto) = m + 3;
                 }
                 __syncwarp();
+            }
+        }
+        if (ok && blockIdx.x == 0 && lane == 0) {
+            // CTA 0 has read the last slots of all CTAs, so all of them have read the generation and the memo
+            *reinterpret_cast<volatile unsigned long long*>(generation) = gen0 + 1ull;
+            if (memo != nullptr) {
+                memo->W = first.W;
+                memo->num_units = first.num_units;
+                memo->scale = *reinterpret_cast<volatile float*>(first.w_scale);     // written by this thread above
+                __threadfence();
+                memo->magic = kQmpMemoMagic;
             }
         }
     }
@@ -676,60 +837,25 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         return;
     }
 
-    // ---- tail: the last matrix, all threads
+    // ---- tail: fix-up (or second pass) of the last matrix, all warps; then the second passes that were put off
     {
         const int m = count - 1;
         const int slot = m % kQmpLists;
-        const QmpDesc d = qmp_desc_of(batch, m);
-        const QmpRange rg = qmp_range(d);
-        const QmpSlot* base = slots + static_cast<size_t>(m) * gridDim.x;
-        double other = 0.0;
-        if (threadIdx.x < gridDim.x) {
-            const volatile unsigned long long* flag = &base[threadIdx.x].nonce;
-            unsigned long long t0 = 0ull;
-            unsigned int spins = 0;
-            bool seen = (*flag == tag);
-            while (!seen) {
-                seen = (*flag == tag);
-                if (!seen && ((++spins & 0xFFu) == 0u)) {
-                    const unsigned long long now = global_timer_ns_qmp();
-                    if (t0 == 0ull) t0 = now;
-                    else if (now - t0 > *reinterpret_cast<volatile unsigned long long*>(&g_wait_limit_ns)) break;
-                }
-            }
-            if (seen) {
-                __threadfence();
-                other = *reinterpret_cast<const volatile double*>(&base[threadIdx.x].partial);
-            } else {
-                sh.abort = 1;
-                atomicExch(&g_device_status, static_cast<int>(SBN_ERR_TIMEOUT));
-            }
-        }
-        const double S = qmp_block_sum(other, s_warp);          // fixed order: the same bits in every CTA
-        if (sh.abort) return;                                    // a peer never arrived: give up cleanly
-        if (threadIdx.x == 0 && d.flip_bits != nullptr && sh.flip_total[slot] != 0ull) atomicAdd(d.flip_bits, sh.flip_total[slot]);
-        const float gamma = static_cast<float>(S / (static_cast<double>(d.num_units) * 128.0));
-        const float scale = fmaxf(gamma, kEps);
-        if (threadIdx.x == 0) {
-            sh.thr_tail = ternary_threshold(scale);
-            if (blockIdx.x == 0) *d.w_scale = scale;
-        }
-        __syncthreads();
         const float thr = sh.thr_tail;
-        const unsigned int listed = sh.list_count[slot];
-        if (qmp_bracket_holds(d, thr, sh.bracket[m & 3][0], sh.bracket[m & 3][1], listed)) {
-            const QmpEntry* list = s_list + slot * kQmpStreamListCap;
-            uint8_t* vb = reinterpret_cast<uint8_t*>(d.vals);
-            for (unsigned int e = threadIdx.x; e < listed; e += kQmpThreads) {
-                const float w = list[e].w;
-                vb[list[e].byte_off] = static_cast<uint8_t>(fabsf(w) >= thr ? (w < 0.0f ? 0xFFu : 0x01u) : 0u);
+        if (sh.tail_second_pass == 0) {
+            if (warp < kQmpStreamWarps) {
+                uint8_t* vb = sh.job[m & (kQmpJobs - 1)].vals;
+                const QmpEntry* list = list_of(slot, warp);
+                const unsigned int listed = sh.warp_listed[slot][warp];
+                for (unsigned int i = lane; i < listed; i += 32u) qmp_fix_entry(vb, list[i], thr);
             }
         } else {
+            const QmpDesc d = qmp_desc_of(batch, m);
+            const QmpRange rg = qmp_range(d);
             if (d.w_bf16) qmp_pass2_full<true>(d, rg, thr);
             else qmp_pass2_full<false>(d, rg, thr);
         }
     }
-    // ---- the second passes that were put off
     for (int m = 0; m + 1 < count; ++m) {
         const float thr = sh.thr_second_pass[m];
         if (thr >= 0.0f) {
@@ -737,18 +863,6 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
             const QmpRange rg = qmp_range(d);
             if (d.w_bf16) qmp_pass2_full<true>(d, rg, thr);
             else qmp_pass2_full<false>(d, rg, thr);
-        }
-    }
-    // every CTA has published its last slot (CTA 0 has just read them all), hence has read the generation
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *reinterpret_cast<volatile unsigned long long*>(generation) = gen0 + 1ull;
-        if (memo != nullptr) {
-            // every CTA has read the memo by now (they have all published since)
-            memo->W = first.W;
-            memo->num_units = first.num_units;
-            memo->scale = *reinterpret_cast<volatile float*>(first.w_scale);     // written by this thread above
-            __threadfence();
-            memo->magic = kQmpMemoMagic;
         }
     }
 }
