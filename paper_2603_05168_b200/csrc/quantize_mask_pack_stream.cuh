@@ -7,29 +7,32 @@
 // matrix, a third of a batch of 2B-shaped matrices and more for small ones.  Here none of that stops
 // the stream:
 //
-//   warp 30       the loader: one lane copies the CTA's range of matrix 0, 1, 2, ... into a ring of shared-
-//                 memory stages (60 units = 30 KB of fp32 weights each, four stages) with bulk copies that
-//                 count their bytes on a stage's `full` barrier; it refills a stage as soon as the 30
-//                 computing warps have released it (`empty` barrier).  Three stages are always in flight,
-//                 whatever the computing warps are busy with: the loads cost no registers and no issue slots.
-//   warps 0..29   pass 1 of matrix 0, 1, 2, ... back to back, stage by stage: a warp takes two units of a
-//                 stage (a half-warp per unit, a lane two adjacent groups), always the same ones (fixed order
-//                 of additions: the partial sums are reproducible bit for bit); no CTA-wide barrier between
-//                 matrices.  A warp leaves its sum |W| and flip count of matrix m in shared memory and
-//                 counts itself on `arrived`.
-//   warp 31       the finisher.  For matrix m, in this order:
-//                   wait until the 30 computing warps have arrived for m, add their sums in a fixed
+//   warp 28       the loader: one lane copies the CTA's range of matrix 0, 1, 2, ... into a ring of shared-
+//                 memory stages (28 KB = 56 units of fp32 or 112 of bf16 weights each, four stages) with bulk
+//                 copies that count their bytes on a stage's `full` barrier; it refills a stage as soon as the
+//                 warps that use it have released it (`empty` barrier).  The loads cost no registers and no
+//                 issue slots, and run ahead across matrices.
+//   warps 0..27   pass 1 of matrix 0, 1, 2, ... back to back: two teams of 14 warps take the stages in turn
+//                 (fixed order of additions: the partial sums are reproducible bit for bit); no CTA-wide barrier
+//                 between matrices.  A warp leaves its sum |W| and flip count of matrix m in shared memory and
+//                 arrives on the list slot's `done` barrier.  (Seven teams of four warps were tried, to keep more
+//                 warps busy while some are between two matrices: their 8 KB copies stream fp32 weights at
+//                 3.3 TB/s, 28 KB ones at 4.7.)
+//   warp 29       the finisher.  For matrix m, in this order:
+//                   wait until the 28 computing warps have arrived for m, add their sums in a fixed
 //                   order, publish {tag, partial} in the workspace;
 //                   exchange of matrix m - 1 (published by every CTA one matrix ago, so the slots are
 //                   there already), exact gamma, scale, threshold; fix-up of the listed values of
-//                   m - 1, or a note that m - 1 needs the exact second pass; its list becomes free;
-//                   bracket of matrix m + 2 (from the caller's hint, or from a sample of the matrix that
-//                   bulk copies drop into the list just freed).
+//                   m - 1, or a note that m - 1 needs the exact second pass; its list becomes free.
 //                 All of it runs under pass 1 of the following matrices.
-//   three lists   matrix m - 1 is being fixed up while m waits and m + 1 is being written; a streaming
-//                 warp starts matrix m only once m - 3 is fixed (its list slot is free) and the bracket
+//   warps 30, 31  the scouts take turns to prepare the matrices ahead: descriptor, what the computing warps need
+//                 to know (`job`), bracket from the caller's hint or from a sample of the matrix.  Up to seven
+//                 matrices ahead, so neither is ever waited for.  When the finisher did this too it took 7 us per
+//                 matrix, and small matrices (1 us of streaming) waited for it.
+//   three lists   matrix m - 1 is being fixed up while m waits and m + 1 is being written; a computing
+//                 warp starts matrix m only once m - 3 is fixed (its list slot is free) and the job
 //                 of m exists -- both normally long done.
-//   tail          after the last matrix every warp joins: exchange and fix-up of the last matrix, then
+//   tail          after the last matrix every warp joins: fix-up of the last matrix, then
 //                 the exact second passes that were put off (bracket missed, list overflow, or the
 //                 dense W_q wanted), all threads working.
 //
@@ -40,23 +43,30 @@
 
 namespace sbn {
 
-constexpr int kQmpStreamWarps = kQmpWarps - 2;             // 30 compute, warp 30 loads, warp 31 finishes
-constexpr int kQmpLoaderWarp = kQmpWarps - 2;
+constexpr int kQmpStreamWarps = 28;                        // 28 compute, then the loader, the finisher and two scouts
+constexpr int kQmpLoaderWarp = kQmpStreamWarps;
+constexpr int kQmpFinisherWarp = kQmpStreamWarps + 1;
+constexpr int kQmpScoutWarp = kQmpStreamWarps + 2;
+constexpr int kQmpScouts = kQmpWarps - kQmpScoutWarp;
 constexpr int kQmpLists = 3;
-constexpr int kQmpWarpListCap = 138;                       // undecided entries per computing warp and matrix, three lists in use
+constexpr int kQmpWarpListCap = 160;                       // undecided entries per computing warp and matrix, three lists in use
 constexpr int kQmpListEntries = kQmpStreamWarps * kQmpWarpListCap;
 // A launch of one or two matrices uses one or two of the three lists, each that much larger.
 __host__ __device__ inline uint32_t qmp_list_cap(int count) {
     return static_cast<uint32_t>(count >= kQmpLists ? kQmpWarpListCap : kQmpLists * kQmpWarpListCap / count);
 }
-constexpr int kQmpTeams = 2;                               // the computing warps' two halves take alternate stages
+constexpr int kQmpTeams = 2;
 constexpr int kQmpTeamWarps = kQmpStreamWarps / kQmpTeams;
+static_assert(kQmpTeams * kQmpTeamWarps == kQmpStreamWarps && kQmpScouts >= 1, "who does what");
 constexpr int kQmpStepUnits = 4 * kQmpTeamWarps;           // one unit per quarter-warp: what a team takes in one step
-constexpr int kQmpStages = 4;
+// Whole turns of the teams: a slot always belongs to the same team.  A team that comes to a slot's next use has then
+// itself seen the use before land, so the parity of the slot's barrier says which use it is.  (With slots that
+// wander from team to team a use could be taken for landed while the one before, another team's, was still on its way.)
+constexpr int kQmpStages = 2 * kQmpTeams;
 constexpr int kQmpStageBytes = kQmpStepUnits * 512;        // one step of fp32 units, or two of bf16 units
 constexpr int kQmpStreamSmemBytes = kQmpStages * kQmpStageBytes + kQmpLists * kQmpListEntries * 8;
-constexpr int kQmpMaxBatch = 1024;                         // thresholds of put-off second passes live in shared memory
-constexpr int kQmpJobs = 4;                                // matrices m - 1 .. m + 2 have a job on chip
+constexpr int kQmpMaxBatch = 512;                          // thresholds of put-off second passes live in shared memory
+constexpr int kQmpJobs = 8;                                // matrices m - 1 .. m + 6 have a job on chip
 
 // What the computing warps need to know about a matrix, in shared memory (a field of the kernel parameters or
 // of a descriptor in global memory is a miss of its own, and all of a CTA's warps would wait for it).
@@ -65,32 +75,33 @@ struct QmpJob {
     uint8_t* meta;
     const uint8_t* prev;                                   // or null
     uint32_t KB;
+    uint32_t kb_magic;                                     // x / KB = umulhi(x, kb_magic) for the small x of a range's start; 0: KB = 1
     uint32_t units;                                        // of this CTA's range
     uint32_t n0, kb0;                                      // row and 128-column block of its first unit
-    uint32_t rep_n, rep_kb;                                // kQmpStepUnits units further (bf16: the stage's second step)
+    uint32_t rep_n, rep_kb;                                // kQmpStepUnits units further (next step of a stage)
     uint32_t next_n, next_kb;                              // from the last step of a stage to the first of the team's next one
     uint32_t bf16;
     float lo, hi;                                          // bracket around the threshold
+    int ready;                                             // m + 1 once the rest is that of matrix m
 };
 
 struct QmpStreamShared {
-    double warp_sum[kQmpLists][kQmpStreamWarps];
+    double warp_sum[kQmpLists][kQmpStreamWarps][8];
     unsigned int warp_flips[kQmpLists][kQmpStreamWarps];
     unsigned int warp_listed[kQmpLists][kQmpStreamWarps];  // entries of each warp's list (may exceed its capacity)
     QmpJob job[kQmpJobs];
-    int bracket_upto;                                      // jobs (and brackets) exist for matrices < bracket_upto
     int fixed_upto;                                        // matrices < fixed_upto are finished: their list slot is free
     int abort;
     float thr_tail;
     int tail_second_pass;
     float sample[kQmpWarps];
     unsigned long long bar_full[kQmpStages];               // a stage's bytes have landed
-    unsigned long long bar_empty[kQmpStages];              // the computing warps are done with a stage
+    unsigned long long bar_empty[kQmpStages];              // the team's warps are done with a stage
     unsigned long long bar_done[kQmpLists];                // the computing warps are done with the matrix in this slot
     uint32_t ring_issued, ring_used;                       // the loader's copies of this launch, and its ring position
-    unsigned long long bar_sample;                         // the finisher's sample has landed
     float thr_second_pass[kQmpMaxBatch];                   // >= 0: this matrix needs the exact second pass with this threshold
 };
+static_assert(kQmpStreamSmemBytes + sizeof(QmpStreamShared) <= 232448, "shared memory overflow");
 
 // mbarrier and bulk-copy wrappers of the stage ring
 __device__ __forceinline__ uint32_t qmp_smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -133,11 +144,7 @@ __device__ __forceinline__ bool qmp_mbar_wait(uint32_t bar, uint32_t parity, vol
     }
     return true;
 }
-__device__ __forceinline__ void qmp_bulk_load(uint32_t smem_dst, const void* gmem_src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_dst), "l"(gmem_src), "r"(bytes), "r"(bar) : "memory");
-}
-// The same for data that is read once (the master weights of pass 1): the lines are the first to leave the
+// The copies of data that is read once (the master weights of pass 1) carry an L2 policy: the lines are the first to leave the
 // L2 again, so the stream does not push out what the kernels after this one will read (the packed weights
 // this kernel writes, the activations).
 __device__ __forceinline__ unsigned long long qmp_policy_evict_first() {
@@ -154,11 +161,10 @@ __device__ __forceinline__ float4 qmp_lds128(uint32_t addr) {
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
     return v;
 }
-// Position in the ring: the number of stages used so far gives the stage and the parity of its current use.
-static_assert((kQmpStages & (kQmpStages - 1)) == 0, "stage = count mod kQmpStages by masking");
+// The loader's position in the ring: the number of stages used so far gives the slot and the parity of its current use.
 struct QmpRing {
     uint32_t used;
-    __device__ __forceinline__ uint32_t stage() const { return used & (kQmpStages - 1); }
+    __device__ __forceinline__ uint32_t stage() const { return used % kQmpStages; }
     __device__ __forceinline__ uint32_t phase() const { return (used / kQmpStages) & 1u; }
     __device__ __forceinline__ void advance() { ++used; }
 };
@@ -223,6 +229,18 @@ __device__ __forceinline__ bool qmp_hint(const QmpDesc& d, float& g) {
 // CTA; a multiplicative hash keeps them off any row / column-block period).  In two halves, so that something can
 // be started between asking for the sample and using it: all of a thread's sample loads are issued (into v), later
 // they are added up over the CTA -- one barrier, after which every warp adds the 32 partial sums itself.
+// The values stay as loaded (bf16: two words) until they are added up: a conversion next to the load makes every
+// load of a thread wait for the one before (64 trips in a row, 60 us, for a warp's sample of a bf16 matrix).
+__device__ __forceinline__ float4 qmp_load_group_raw(const QmpDesc& d, uint32_t u, int lane) {
+    if (d.w_bf16 == 0u) return __ldg(static_cast<const float4*>(d.W) + static_cast<size_t>(u) * 32 + lane);
+    const float2 v = __ldg(static_cast<const float2*>(d.W) + static_cast<size_t>(u) * 32 + lane);
+    return make_float4(v.x, v.y, 0.0f, 0.0f);
+}
+__device__ __forceinline__ float qmp_abs_sum_raw(const QmpDesc& d, const float4 v) {
+    if (d.w_bf16 == 0u) return (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
+    const uint32_t a = __float_as_uint(v.x), b = __float_as_uint(v.y);
+    return (fabsf(bf16lo_to_f32(a)) + fabsf(bf16hi_to_f32(a))) + (fabsf(bf16lo_to_f32(b)) + fabsf(bf16hi_to_f32(b)));
+}
 constexpr int kQmpSamplePerWarp = kQmpSampleUnits / kQmpWarps;
 __device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[kQmpSamplePerWarp]) {
     const int lane = threadIdx.x & 31;
@@ -234,13 +252,13 @@ __device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[k
         const uint32_t sidx = warp + i * kQmpWarps;
         const uint32_t u = sidx * stride + ((sidx * 2654435761u) >> 8) % stride;
         v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (sidx < n_s) v[i] = d.w_bf16 ? qmp_load_group<true>(d.W, u, lane) : qmp_load_group<false>(d.W, u, lane);
+        if (sidx < n_s) v[i] = qmp_load_group_raw(d, u, lane);
     }
 }
 __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float4 (&v)[kQmpSamplePerWarp], float* s_sample) {
     float acc = 0.0f;
 #pragma unroll
-    for (int i = 0; i < kQmpSamplePerWarp; ++i) acc += (fabsf(v[i].x) + fabsf(v[i].y)) + (fabsf(v[i].z) + fabsf(v[i].w));
+    for (int i = 0; i < kQmpSamplePerWarp; ++i) acc += qmp_abs_sum_raw(d, v[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
     if ((threadIdx.x & 31) == 0) s_sample[threadIdx.x >> 5] = acc;
@@ -251,44 +269,29 @@ __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float
     return t / (static_cast<float>(qmp_sample_units(d.num_units)) * 128.0f);
 }
 
-// gamma_est by ONE warp (the finisher, for matrices 1, 2, ... of a batch without hints): the first
-// kQmpSampleUnitsSmall of qmp_sample_gamma's scattered units, fetched by bulk copies into `buf` (a list that
-// is free at that moment) -- all of them in flight at once, one round trip instead of one per eight units.
-// The smaller sample gets the wider bracket (qmp_bracket_from, `wide`).  Returns a negative number if the
-// copies did not land within the wait limit (the CTA is then aborting).
-constexpr int kQmpSampleUnitsWarp = kQmpSampleUnitsSmall;
-static_assert(kQmpSampleUnitsWarp * 512 <= kQmpListEntries * 8, "the sample fits a list");
-__device__ __forceinline__ float qmp_sample_gamma_warp(const QmpDesc& d, int lane, unsigned char* buf, uint32_t bar, uint32_t& bar_phase,
-                                                       volatile int* abort_flag) {
-    const uint32_t unit_bytes = d.w_bf16 ? 256u : 512u;
+// gamma_est by ONE warp (a scout, for matrices 1, 2, ... of a batch without hints) from the first
+// kQmpSampleUnitsSmall of qmp_sample_issue's scattered units, eight in flight at a time.  The smaller sample gets the
+// wider bracket (qmp_bracket_from, `wide`).
+__device__ __forceinline__ float qmp_sample_gamma_warp(const QmpDesc& d, int lane) {
     const uint32_t n_full = qmp_sample_units(d.num_units);
     const uint32_t stride = d.num_units / n_full;
-    const uint32_t n_s = min(n_full, static_cast<uint32_t>(kQmpSampleUnitsWarp));
-    auto unit_of = [&](uint32_t sidx) { return sidx * stride + ((sidx * 2654435761u) >> 8) % stride; };
-    const uint32_t buf_u32 = qmp_smem_u32(buf);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // the list's earlier (generic) use before the copies
-    if (lane == 0) qmp_mbar_expect_tx(bar, n_s * unit_bytes);
-    __syncwarp();
-    for (uint32_t sidx = lane; sidx < n_s; sidx += 32u)
-        qmp_bulk_load(buf_u32 + sidx * unit_bytes, static_cast<const char*>(d.W) + static_cast<size_t>(unit_of(sidx)) * unit_bytes, unit_bytes, bar);
-    const bool landed = qmp_mbar_wait(bar, bar_phase, abort_flag, true);  // sees its own copies land even if the CTA aborts
-    bar_phase ^= 1u;
-    if (!landed) return -1.0f;
+    const uint32_t n_s = min(n_full, static_cast<uint32_t>(kQmpSampleUnitsSmall));
     float acc = 0.0f;
-    const uint32_t chunks = n_s * unit_bytes / 16u;
-    for (uint32_t c = lane; c < chunks; c += 32u) {
-        const float4 v = qmp_lds128(buf_u32 + c * 16u);
-        if (d.w_bf16) {
-            const uint32_t r0 = __float_as_uint(v.x), r1 = __float_as_uint(v.y), r2 = __float_as_uint(v.z), r3 = __float_as_uint(v.w);
-            acc += ((fabsf(bf16lo_to_f32(r0)) + fabsf(bf16hi_to_f32(r0))) + (fabsf(bf16lo_to_f32(r1)) + fabsf(bf16hi_to_f32(r1)))) +
-                   ((fabsf(bf16lo_to_f32(r2)) + fabsf(bf16hi_to_f32(r2))) + (fabsf(bf16lo_to_f32(r3)) + fabsf(bf16hi_to_f32(r3))));
-        } else {
-            acc += (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
+#pragma unroll 1
+    for (uint32_t s0 = 0; s0 < n_s; s0 += 8u) {
+        float4 v[8];
+#pragma unroll
+        for (uint32_t i = 0; i < 8u; ++i) {
+            const uint32_t sidx = s0 + i;
+            const uint32_t u = sidx * stride + ((sidx * 2654435761u) >> 8) % stride;
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (sidx < n_s) v[i] = qmp_load_group_raw(d, u, lane);
         }
+#pragma unroll
+        for (uint32_t i = 0; i < 8u; ++i) acc += qmp_abs_sum_raw(d, v[i]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    __syncwarp();
     return acc / (static_cast<float>(n_s) * 128.0f);
 }
 
@@ -339,12 +342,14 @@ __device__ __forceinline__ void qmp_make_job(const QmpDesc& d, QmpJob& jb) {
     jb.meta = d.meta;
     jb.prev = d.prev_meta;
     jb.KB = d.KB;
+    jb.kb_magic = d.KB > 1u ? 0xFFFFFFFFu / d.KB + 1u : 0u;         // exact: x * KB < 2^32 for x < KB + a turn of the teams
     jb.units = rg.u_end - rg.u_begin;
     jb.n0 = rg.u_begin / d.KB;
     jb.kb0 = rg.u_begin - jb.n0 * d.KB;
     jb.rep_n = kQmpStepUnits / d.KB;
     jb.rep_kb = kQmpStepUnits % d.KB;
-    const uint32_t next = (d.w_bf16 ? 3u : 2u) * kQmpStepUnits;
+    const uint32_t reps = kQmpStageBytes / (kQmpStepUnits * (d.w_bf16 ? 256u : 512u));
+    const uint32_t next = (kQmpTeams * reps - reps + 1u) * kQmpStepUnits;
     jb.next_n = next / d.KB;
     jb.next_kb = next % d.KB;
     jb.bf16 = d.w_bf16;
@@ -385,15 +390,15 @@ __device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
     return __popc(any | (none << 1));
 }
 
-// Pass 1 of one matrix for a computing warp: its four units of every stage of its team (a quarter-warp per unit, a
-// lane 16 weights = four groups).  `g0` counts the ring's stages up to this matrix.  Returns the thread's
-// sum |W|; `ok` turns false if a wait ran out.
+// Pass 1 of one matrix for a computing warp: its four units of every step of its team's stages (a quarter-warp per
+// unit, a lane 16 weights = four groups).  The matrix's stages are the ring's g0 .. g0 + n - 1, the team's next one is
+// `next_stage`.  Returns the thread's sum |W|; `ok` turns false if a wait ran out.
 //
 // The instructions are what this pass costs: the memory delivers 256 weights per SM every 44 clocks (fp32), and
 // selection, signs, comparisons and the fp64 sum of 256 weights alone take 24 (8 more are their shared-memory
 // reads).  An earlier form with 8 weights per lane spent 231 warp instructions on them, more than half beside that
-// core.  So: 16 weights per lane and iteration (one 8-byte store of values, one 2-byte store of metadata, one
-// barrier wait, one look at the previous metadata); the selection's predicates are folded into the compares;
+// core.  So: 16 weights per lane and step (one 8-byte store of values, one 2-byte store of metadata, one
+// look at the previous metadata); the selection's predicates are folded into the compares;
 // "|k| >= thr" and "is |k| undecided" come from ONE subtraction, e = pred(thr_hi) - |k| (its sign bit is the first
 // answer, e <= pred(thr_hi) - thr_lo as an unsigned compare of the bits the second, and four sign bits become four
 // byte masks by byte permutes); the undecided are appended with ballots instead of atomics; flips are counted
@@ -402,15 +407,14 @@ __device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
 // A lane's 64 B (fp32) are read as 16-byte pieces in rotated order, (i + l8 / 2) mod 4, so that the eight lanes of a
 // unit hit different banks; the rotation is undone on the 8 + 2 result bytes (two byte permutes, one shift).
 template <bool BF16>
-__device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t ring_base,
-                                                   uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok) {
+__device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
+                                                   uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = threadIdx.x >> 5;
-    const uint32_t team = warp >= kQmpTeamWarps ? 1u : 0u;
     const uint32_t l8 = lane & 7;
-    constexpr int REP = BF16 ? 2 : 1;                                 // steps per stage
-    constexpr int PIECES = BF16 ? 2 : 4;                              // 16-byte pieces per lane
     constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
+    constexpr uint32_t REP = kQmpStageBytes / (kQmpStepUnits * kUnitBytes);    // steps per stage
+    constexpr int PIECES = BF16 ? 2 : 4;                              // 16-byte pieces per lane
     const uint32_t KB = jb.KB;
     // kept is +-1 iff |k| > thr_pred, undecided iff 0 <= thr_pred - |k| <= width.  The subtraction is exact near the
     // threshold and monotone everywhere: a value wrongly taken for undecided can only lie below thr_lo, and the
@@ -418,17 +422,18 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     const float thr_pred = __uint_as_float(__float_as_uint(jb.hi) - 1u);
     const uint32_t width = __float_as_uint(thr_pred - jb.lo);
     const uint32_t n_stages = (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
-    const uint32_t st0 = (team ^ g0) & 1u;                            // the team's first stage of this matrix
+    const uint32_t g_end = g0 + n_stages;
     double acc = 0.0;
-    const uint32_t in_step = 4u * (warp - team * kQmpTeamWarps) + (lane >> 3);   // this quarter-warp's unit of every step
+    const uint32_t in_step = 4u * (warp % kQmpTeamWarps) + (lane >> 3);          // this quarter-warp's unit of every step
+    const uint32_t u0 = (next_stage - g0) * (REP * kQmpStepUnits) + in_step;     // ... of its first one here, from the range's start
     uint32_t n, kb;
     {
-        const uint32_t k0 = jb.kb0 + st0 * (REP * kQmpStepUnits) + in_step;
-        const uint32_t dn = k0 / KB;
+        const uint32_t k0 = jb.kb0 + u0;
+        const uint32_t dn = jb.kb_magic != 0u ? __umulhi(k0, jb.kb_magic) : k0;
         n = jb.n0 + dn;
         kb = k0 - dn * KB;
     }
-    int left = static_cast<int>(jb.units) - static_cast<int>(st0 * (REP * kQmpStepUnits) + in_step);   // > 0: this quarter-warp has a unit in the step
+    int left = static_cast<int>(jb.units) - static_cast<int>(u0);     // > 0: this quarter-warp has a unit in the step
     const uint32_t turn = BF16 ? (l8 >> 2) : (l8 >> 1);               // rotation of the pieces ...
     const uint32_t rot = BF16 ? 2u * turn : turn;                     // ... and of the groups
     uint32_t src[PIECES];
@@ -450,26 +455,26 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     uint32_t q = tiled_row(n, kb);
     uint32_t prev = 0u;
     if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
-    for (uint32_t st = st0; st < n_stages; st += 2u) {
-        const uint32_t g = g0 + st;
-        const uint32_t stage = g & (kQmpStages - 1u);
-        if (!qmp_mbar_wait(bar_full0 + 8u * stage, (g / kQmpStages) & 1u, abort_flag)) { ok = false; break; }
-        float4 raw[REP * PIECES];
-        // a lane without a unit (last stage only) reads what is there: it is not used
+    for (; next_stage < g_end; next_stage += kQmpTeams) {
+        const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
+        if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
 #pragma unroll
-        for (int i = 0; i < REP * PIECES; ++i)
-            raw[i] = qmp_lds128(src[i % PIECES] + stage * kQmpStageBytes + (i / PIECES) * (kQmpStepUnits * kUnitBytes));
-        __syncwarp();
-        if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);           // the values are in registers: the stage may be refilled
+        for (uint32_t rep = 0; rep < REP; ++rep) {
+            float4 raw[PIECES];
+            // a lane without a unit (last stage only) reads what is there: it is not used
 #pragma unroll
-        for (int rep = 0; rep < REP; ++rep) {
+            for (int i = 0; i < PIECES; ++i) raw[i] = qmp_lds128(src[i] + stage * kQmpStageBytes + rep * (kQmpStepUnits * kUnitBytes));
+            if (rep + 1 == REP) {
+                __syncwarp();
+                if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);   // the values are in registers: the stage may be refilled
+            }
             const bool mine = left > 0;
             const uint32_t q_cur = q, prev_cur = prev;
             const uint32_t v8 = q_cur * 8u + 2u * (chunk ^ ((n >> 1) & 3u)) + (l8 & 1u);       // 8-byte piece of the values
             n += rep + 1 < REP ? jb.rep_n : jb.next_n;
             kb += rep + 1 < REP ? jb.rep_kb : jb.next_kb;
             if (kb >= KB) { kb -= KB; ++n; }
-            left -= rep + 1 < REP ? kQmpStepUnits : (BF16 ? 3 : 2) * kQmpStepUnits;
+            left -= static_cast<int>((rep + 1 < REP ? 1u : (kQmpTeams * REP - REP + 1u)) * kQmpStepUnits);
             q = tiled_row(n, kb);
             if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
             float k[8];
@@ -479,7 +484,7 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
             for (int i = 0; i < 4; ++i) {
                 float4 w;
                 if constexpr (BF16) {
-                    const float4 r4 = raw[rep * PIECES + (i >> 1)];
+                    const float4 r4 = raw[i >> 1];
                     const uint32_t r0 = __float_as_uint((i & 1) ? r4.z : r4.x), r1 = __float_as_uint((i & 1) ? r4.w : r4.y);
                     w = make_float4(bf16lo_to_f32(r0), bf16hi_to_f32(r0), bf16lo_to_f32(r1), bf16hi_to_f32(r1));
                 } else {
@@ -518,7 +523,7 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
                             });
         }
     }
-    g0 += n_stages;
+    g0 = g_end;
     flips *= 2u;
     return acc;
 }
@@ -576,6 +581,13 @@ __device__ __forceinline__ bool qmp_exchange(const QmpSlot* base, unsigned long 
     return true;
 }
 
+// ternary_threshold by a whole warp: lane i tries the i-th float from 8 below scale / 2, the lowest that passes is it.
+__device__ __forceinline__ float qmp_threshold_warp(float scale, int lane) {
+    const float a = __uint_as_float(__float_as_uint(0.5f * scale) - 8u + lane);
+    const uint32_t passes = __ballot_sync(0xFFFFFFFFu, __fdiv_rn(a, scale) > 0.5f);
+    return __shfl_sync(0xFFFFFFFFu, a, __ffs(static_cast<int>(passes)) - 1);
+}
+
 // Do the listed values suffice, or must the whole range be ternarised again with the exact threshold?
 __device__ __forceinline__ bool qmp_bracket_holds(const QmpDesc& d, float thr, const QmpJob& jb, unsigned int longest_list, uint32_t list_cap) {
     return jb.lo <= thr && thr <= jb.hi && longest_list <= list_cap && d.dense_q == nullptr &&
@@ -597,7 +609,6 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
 
     const QmpBatch batch{inl, rest};
     const QmpDesc& first = inl.d[0];
-    const QmpDesc& second = inl.d[1];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     volatile int* const abort_flag = &sh.abort;
@@ -609,31 +620,27 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         sh.abort = 0;
         sh.tail_second_pass = 0;
         sh.ring_issued = 0u; sh.ring_used = 0u;
+        for (int i = 0; i < kQmpJobs; ++i) sh.job[i].ready = 0;
         for (int i = 0; i < kQmpLists; ++i) qmp_mbar_init(bar_done0 + 8u * i, kQmpStreamWarps);
         for (int i = 0; i < kQmpStages; ++i) {
             qmp_mbar_init(bar_full0 + 8u * i, 1u);                     // the loader's expect_tx
             qmp_mbar_init(bar_empty0 + 8u * i, kQmpTeamWarps);         // one arrival per computing warp of the stage's team
         }
-        qmp_mbar_init(qmp_smem_u32(&sh.bar_sample), 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (threadIdx.x == 32) qmp_make_job(first, sh.job[0]);
-    if (threadIdx.x == 64 && count > 1) qmp_make_job(second, sh.job[1]);
     for (int i = threadIdx.x; i < count; i += kQmpThreads) sh.thr_second_pass[i] = -1.0f;
     __syncthreads();
     // No early signal to the next kernel of the stream: this kernel writes packed weights, and the
     // GEMM kernels fetch weights before their own dependency wait (see sbn_common.cuh).
     pdl_wait();
 
-    // ---- What the first bracket needs is asked for BEFORE the loader fills the ring: the hints of matrices
-    // 0 and 1 (4-byte reads), and without a hint of the caller's the sample of matrix 0 (all threads, one round
-    // trip) together with what an earlier call may have left.  Issued with the ring's first copies they queue
-    // behind the 17 MB that the loaders of all CTAs ask for at the same moment (up to 3.5 us measured, and the
-    // CTA that is served last finishes last).
-    float g01[2];
-    g01[0] = first.gamma_hint != nullptr ? *reinterpret_cast<const volatile float*>(first.gamma_hint) : 0.0f;
-    g01[1] = (count > 1 && second.gamma_hint != nullptr) ? *reinterpret_cast<const volatile float*>(second.gamma_hint) : 0.0f;
+    // ---- What the first bracket needs is asked for BEFORE the loader fills the ring: the hint of matrix 0 (a 4-byte
+    // read), or without a hint of the caller's its sample (all threads, one round trip) together with what an
+    // earlier call may have left.  Issued with the ring's first copies they queue behind the 17 MB that the loaders
+    // of all CTAs ask for at the same moment (up to 3.5 us measured, and the CTA that is served last finishes last).
+    float gamma0 = first.gamma_hint != nullptr ? *reinterpret_cast<const volatile float*>(first.gamma_hint) : 0.0f;
     float4 sample0[kQmpSamplePerWarp];
     const bool sample_early = first.gamma_hint == nullptr;
     if (sample_early) {
@@ -646,140 +653,131 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         }
         qmp_sample_issue(first, sample0);
         if (m_tag == kQmpMemoMagic && m_w == reinterpret_cast<unsigned long long>(first.W) && m_units == first.num_units)
-            g01[0] = __uint_as_float(m_scale);
+            gamma0 = __uint_as_float(m_scale);
     }
-    const bool hinted01[2] = {qmp_hint_usable(g01[0]), qmp_hint_usable(g01[1])};
-    if (!sample_early && !hinted01[0]) qmp_sample_issue(first, sample0);
+    const bool hinted0 = qmp_hint_usable(gamma0);
+    if (!sample_early && !hinted0) qmp_sample_issue(first, sample0);
     QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, qmp_policy_evict_first()};
     const bool is_loader = warp == kQmpLoaderWarp && lane == 0;
     if (is_loader) qmp_loader_issue(loader, batch, count, kQmpStages, ring_base, bar_full0, bar_empty0, abort_flag);
-    if (!hinted01[0]) g01[0] = qmp_sample_finish(first, sample0, sh.sample);
+    if (!hinted0) gamma0 = qmp_sample_finish(first, sample0, sh.sample);
     if (threadIdx.x == 0) {
-        qmp_bracket_from(g01[0], first.num_units, hinted01[0], sh.job[0].lo, sh.job[0].hi);
-        // matrix 1: from its hint here; without one the finisher samples it while matrix 0 streams
-        if (hinted01[1]) qmp_bracket_from(g01[1], second.num_units, true, sh.job[1].lo, sh.job[1].hi);
-        sh.bracket_upto = hinted01[1] ? 2 : 1;
+        qmp_bracket_from(gamma0, first.num_units, hinted0, sh.job[0].lo, sh.job[0].hi);
+        sh.job[0].ready = 1;
+        if (blockIdx.x == 0 && first.flip_bits != nullptr) *first.flip_bits = 0ull;      // published with this CTA's first slot
     }
     __syncthreads();
 
     if (warp < kQmpStreamWarps) {
         // ------------------------------------------------------------------ computing warps
         uint32_t stages = 0u;                                // of the matrices so far
+        uint32_t next_stage = static_cast<uint32_t>(warp) / kQmpTeamWarps;       // this team's
         for (int m = 0; m < count; ++m) {
             const int slot = m % kQmpLists;
-            if (!qmp_wait_ge(&sh.bracket_upto, m + 1, abort_flag)) break;
+            const QmpJob& jb = sh.job[m & (kQmpJobs - 1)];
+            if (!qmp_wait_ge(const_cast<int*>(&jb.ready), m + 1, abort_flag)) break;
             if (!qmp_wait_ge(&sh.fixed_upto, m - (kQmpLists - 1), abort_flag)) break;
             __threadfence_block();
-            const QmpJob jb = sh.job[m & (kQmpJobs - 1)];
             unsigned int flips = 0;
             bool ok = true;
             QmpWarpList list{list_of(slot, warp), list_cap, 0u};
-            double mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, ring_base, bar_full0, bar_empty0, abort_flag, ok)
-                                  : qmp_stream_pass1<false>(jb, list, flips, stages, ring_base, bar_full0, bar_empty0, abort_flag, ok);
+            double mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok)
+                                  : qmp_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok);
             if (!ok) break;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
+            mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 16);
+            mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 8);
+            if (lane < 8) sh.warp_sum[slot][warp][lane] = mine;
             if (jb.prev != nullptr) flips = __reduce_add_sync(0xFFFFFFFFu, flips);
-            __syncwarp();                                    // every lane's list entries are written
             if (lane == 0) {
-                sh.warp_sum[slot][warp] = mine;
                 sh.warp_flips[slot][warp] = flips;
                 sh.warp_listed[slot][warp] = list.n;
-                qmp_mbar_arrive(bar_done0 + 8u * slot);      // release: the sums, and this warp's list entries, before the count
             }
-            __syncwarp();
+            __syncwarp();                                    // every lane's list entries and sums are written
+            if (lane == 0) qmp_mbar_arrive(bar_done0 + 8u * slot);               // release: all of it before the count
         }
     } else if (warp == kQmpLoaderWarp) {
-        // ------------------------------------------------------------------ the loader (warp 30, one lane)
+        // ------------------------------------------------------------------ the loader (one lane)
         if (is_loader) {
             qmp_loader_issue(loader, batch, count, 0xFFFFFFFFu, ring_base, bar_full0, bar_empty0, abort_flag);
             sh.ring_issued = loader.issued;                  // for the drain, should the CTA abort
             sh.ring_used = loader.ring.used;
         }
         __syncwarp();
+    } else if (warp >= kQmpScoutWarp) {
+        // ------------------------------------------------------------------ the scouts
+        for (int m = 1 + (warp - kQmpScoutWarp); m < count; m += kQmpScouts) {
+            const QmpDesc d = qmp_desc_of(batch, m);
+            float g;
+            const bool hinted = qmp_hint(d, g);
+            if (!hinted) g = qmp_sample_gamma_warp(d, lane);
+            // the job's place: matrix m - kQmpJobs is finished
+            if (!qmp_wait_ge(&sh.fixed_upto, m - (kQmpJobs - 1), abort_flag)) break;
+            if (lane == 0) {
+                // zeroed well before any CTA can add to it (they add once they have seen this CTA's slot)
+                if (blockIdx.x == 0 && d.flip_bits != nullptr) { *d.flip_bits = 0ull; __threadfence(); }
+                QmpJob& jb = sh.job[m & (kQmpJobs - 1)];
+                qmp_make_job(d, jb);
+                qmp_bracket_from(g, d.num_units, hinted, jb.lo, jb.hi, true);
+                __threadfence_block();
+                *reinterpret_cast<volatile int*>(&jb.ready) = m + 1;
+            }
+            __syncwarp();
+        }
     } else {
-        // ------------------------------------------------------------------ the finisher (warp 31)
+        // ------------------------------------------------------------------ the finisher
         const unsigned long long gen0 = *reinterpret_cast<volatile unsigned long long*>(generation);
         const unsigned long long tag = qmp_tag(call_nonce, gen0);
         bool ok = true;
-        uint32_t sample_phase = 0u;
-        if (count > 1 && !hinted01[1]) {
-            // bracket of matrix 1 from a sample into its own (still unused) list, while matrix 0 streams
-            const float g = qmp_sample_gamma_warp(second, lane, reinterpret_cast<unsigned char*>(list_of(1, 0)),
-                                                  qmp_smem_u32(&sh.bar_sample), sample_phase, abort_flag);
-            if (g < 0.0f) {
-                ok = false;
-            } else {
-                if (lane == 0) {
-                    qmp_bracket_from(g, second.num_units, false, sh.job[1].lo, sh.job[1].hi, true);
-                    __threadfence_block();
-                    *reinterpret_cast<volatile int*>(&sh.bracket_upto) = 2;
-                }
-                __syncwarp();
-            }
-        }
         // step m: publish matrix m, then exchange and finish matrix m - 1; step `count` finishes the last matrix
         // (its fix-up is left to all warps)
         unsigned int flips_prev = 0u;
-        for (int m = 0; ok && m <= count; ++m) {
-            // job and, from the caller's hint, bracket of matrix m + 2, well before the computing warps ask for it
-            bool sample_next = false;
-            if (m + 2 < count) {
-                const QmpDesc d2 = qmp_desc_of(batch, m + 2);
-                QmpJob& jb = sh.job[(m + 2) & (kQmpJobs - 1)];
-                if (lane == 0) qmp_make_job(d2, jb);
-                float g;
-                if (qmp_hint(d2, g)) {
-                    if (lane == 0) {
-                        qmp_bracket_from(g, d2.num_units, true, jb.lo, jb.hi);
-                        __threadfence_block();
-                        *reinterpret_cast<volatile int*>(&sh.bracket_upto) = m + 3;
-                    }
-                    __syncwarp();
-                } else {
-                    sample_next = true;
-                }
-            }
+        QmpDesc dp = first;                                  // of matrix m - 1
+        for (int m = 0; m <= count; ++m) {
             unsigned int flips_cur = 0u;
+            QmpDesc d = dp;
             if (m < count) {
                 // matrix m: every computing warp has arrived -> this CTA's partial sum, published
                 const int slot = m % kQmpLists;
-                const QmpDesc d = qmp_desc_of(batch, m);
-                // zeroed well before any CTA can add to it (they add once they have seen this CTA's slot)
-                if (blockIdx.x == 0 && lane == 0 && d.flip_bits != nullptr) { *d.flip_bits = 0ull; __threadfence(); }
+                if (m > 0) d = qmp_desc_of(batch, m);        // on its way while the warps are waited for
                 if (!qmp_mbar_wait(bar_done0 + 8u * slot, static_cast<uint32_t>(m / kQmpLists) & 1u, abort_flag)) { ok = false; break; }
-                double v = lane < kQmpStreamWarps ? *reinterpret_cast<volatile double*>(&sh.warp_sum[slot][lane]) : 0.0;
+                double v = 0.0;
+#pragma unroll
+                for (int i = 0; i < 8 * kQmpStreamWarps / 32; ++i) v += (&sh.warp_sum[slot][0][0])[lane + 32 * i];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-                if (lane == 0 && !(test_withhold_slot && blockIdx.x == gridDim.x - 1))
-                    qmp_slot_store(slots + static_cast<size_t>(m) * gridDim.x + blockIdx.x, tag, v);
-                if (d.flip_bits != nullptr)
-                    flips_cur = __reduce_add_sync(0xFFFFFFFFu, lane < kQmpStreamWarps ? *reinterpret_cast<volatile unsigned int*>(&sh.warp_flips[slot][lane]) : 0u);
+                if (lane == 0) {
+                    if (blockIdx.x == 0 && d.flip_bits != nullptr) __threadfence();      // the zeroed flip count before the slot
+                    if (!(test_withhold_slot && blockIdx.x == gridDim.x - 1))
+                        qmp_slot_store(slots + static_cast<size_t>(m) * gridDim.x + blockIdx.x, tag, v);
+                }
+                if (d.flip_bits != nullptr) flips_cur = __reduce_add_sync(0xFFFFFFFFu, lane < kQmpStreamWarps ? sh.warp_flips[slot][lane] : 0u);
                 __syncwarp();
             }
             // matrix m - 1: exchange, exact threshold, fix-up
             if (m >= 1) {
                 const int pslot = (m - 1) % kQmpLists;
-                const QmpDesc dp = qmp_desc_of(batch, m - 1);
                 double sum;
                 ok = qmp_exchange(slots + static_cast<size_t>(m - 1) * gridDim.x, tag, lane, abort_flag, sum);
                 if (!ok) break;
                 const float gamma = static_cast<float>(sum / (static_cast<double>(dp.num_units) * 128.0));
                 const float scale = fmaxf(gamma, kEps);
-                const float thr = ternary_threshold(scale);
-                const unsigned int longest = __reduce_max_sync(0xFFFFFFFFu, lane < kQmpStreamWarps ? *reinterpret_cast<volatile unsigned int*>(&sh.warp_listed[pslot][lane]) : 0u);
+                const float thr = qmp_threshold_warp(scale, lane);
+                const unsigned int mine = lane < kQmpStreamWarps ? sh.warp_listed[pslot][lane] : 0u;     // of warp `lane`'s list
+                const unsigned int longest = __reduce_max_sync(0xFFFFFFFFu, mine);
                 const bool holds = qmp_bracket_holds(dp, thr, sh.job[(m - 1) & (kQmpJobs - 1)], longest, list_cap);
+                uint8_t* const vb = reinterpret_cast<uint8_t*>(dp.vals);
                 if (m == count) {
                     if (lane == 0) { sh.thr_tail = thr; sh.tail_second_pass = holds ? 0 : 1; }
-                } else if (holds) {
-                    uint8_t* vb = reinterpret_cast<uint8_t*>(dp.vals);
+                } else if (!holds) {
+                    if (lane == 0) sh.thr_second_pass[m - 1] = thr;
+                } else if (longest <= 16u) {
+                    // short lists (a hint): a lane per list
+                    for (unsigned int i = 0; i < mine; ++i) qmp_fix_entry(vb, list_of(pslot, lane)[i], thr);
+                } else {
                     for (int w = 0; w < kQmpStreamWarps; ++w) {
-                        const QmpEntry* list = list_of(pslot, w);
-                        const unsigned int listed = sh.warp_listed[pslot][w];
-                        for (unsigned int i = lane; i < listed; i += 32u) qmp_fix_entry(vb, list[i], thr);
+                        const unsigned int listed = __shfl_sync(0xFFFFFFFFu, mine, w);
+                        for (unsigned int i = lane; i < listed; i += 32u) qmp_fix_entry(vb, list_of(pslot, w)[i], thr);
                     }
-                } else if (lane == 0) {
-                    sh.thr_second_pass[m - 1] = thr;
                 }
                 __syncwarp();
                 if (lane == 0) {
@@ -794,21 +792,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
                 __syncwarp();
             }
             flips_prev = flips_cur;
-            // bracket of matrix m + 2 from a sample, if it has no hint: a whole matrix before the computing warps
-            // ask for it.  The sample lands in the list that matrix m - 1 has just given back (the one m + 2 will use).
-            if (sample_next) {
-                const QmpDesc d2 = qmp_desc_of(batch, m + 2);
-                const float g = qmp_sample_gamma_warp(d2, lane, reinterpret_cast<unsigned char*>(list_of((m + 2) % kQmpLists, 0)),
-                                                      qmp_smem_u32(&sh.bar_sample), sample_phase, abort_flag);
-                if (g < 0.0f) { ok = false; break; }
-                if (lane == 0) {
-                    QmpJob& jb = sh.job[(m + 2) & (kQmpJobs - 1)];
-                    qmp_bracket_from(g, d2.num_units, false, jb.lo, jb.hi, true);
-                    __threadfence_block();
-                    *reinterpret_cast<volatile int*>(&sh.bracket_upto) = m + 3;
-                }
-                __syncwarp();
-            }
+            dp = d;
         }
         if (ok && blockIdx.x == 0 && lane == 0) {
             // CTA 0 has read the last slots of all CTAs, so all of them have read the generation and the memo
