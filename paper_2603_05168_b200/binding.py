@@ -1,4 +1,5 @@
-"""Thin ctypes binding over libsbn.so -- argument marshalling only.
+"""Thin binding over libsbn.so -- argument marshalling only.  The calls of a decode loop go through a CPython
+extension (csrc/binding_native.cpp), which a call costs 1 us instead of ctypes' 8; the others through ctypes.
 
 Function names match the C ABI in ``include/sbn.h``.  Tensors are torch CUDA tensors used purely
 as device buffers (``data_ptr()``), the stream is torch's current stream.  Nothing here computes:
@@ -8,6 +9,8 @@ import of this module's functions fails loudly -- there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional
 
@@ -15,6 +18,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libsbn.so")
+NATIVE_PATH = os.path.join(_PKG, "_sbn_native.so")
 
 SBN_OK = 0
 OUT_F32, OUT_BF16 = 0, 1
@@ -29,6 +33,7 @@ EXPORTS = [
 ]
 
 _lib = None
+_native = None
 
 
 class SbnError(RuntimeError):
@@ -118,7 +123,29 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    torch.cuda.init()
+    # what torch.cuda.current_stream() asks, without the Stream object around it (3 us)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+
+
+_NATIVE_CALLS = ["sbn_quant_act", "sbn_quant_act_expand68", "sbn_norm_quant_act", "sbn_norm_quant_act_expand68", "sbn_sparse_bitlinear",
+                 "sbn_bitlinear", "sbn_sparse_bitlinear_packed", "sbn_quant_act_sparse_bitlinear", "sbn_quant_act_bitlinear"]
+
+
+def _load_native():
+    """The extension, bound to the functions of the library that lib() has loaded; raises if either is missing."""
+    global _native
+    L = lib()
+    if not os.path.exists(NATIVE_PATH):
+        raise RuntimeError(f"{NATIVE_PATH} not found: build it with `python -m paper_2603_05168_b200.build`")
+    torch.cuda.init()
+    loader = importlib.machinery.ExtensionFileLoader("_sbn_native", NATIVE_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_sbn_native", loader))
+    loader.exec_module(mod)
+    addresses = {name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_CALLS}
+    mod.bind(addresses, torch.bfloat16, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    _native = mod
+    return mod
 
 
 def _check(code: int, where: str):
@@ -190,14 +217,11 @@ def sbn_quantize_mask_pack_batched(job_array, ws):
 
 
 def sbn_quant_act(x_bf16, xq, a_scale):
-    T, K = x_bf16.shape
-    _check(lib().sbn_quant_act(_ptr(x_bf16), T, K, _ptr(xq), _ptr(a_scale), _stream()), "sbn_quant_act")
+    _check((_native or _load_native()).quant_act(x_bf16, xq, a_scale, False), "sbn_quant_act")
 
 
 def sbn_quant_act_expand68(x_bf16, xq, a_scale):
-    T, K = x_bf16.shape
-    _check(lib().sbn_quant_act_expand68(_ptr(x_bf16), T, K, _ptr(xq), _ptr(a_scale), _stream()),
-           "sbn_quant_act_expand68")
+    _check((_native or _load_native()).quant_act(x_bf16, xq, a_scale, True), "sbn_quant_act_expand68")
 
 
 def sbn_expanded_k(K: int, n_keep: int, m_group: int) -> int:
@@ -205,10 +229,7 @@ def sbn_expanded_k(K: int, n_keep: int, m_group: int) -> int:
 
 
 def sbn_norm_quant_act(x_bf16, xq, a_scale, gain=None, eps: float = 1e-6, expand68: bool = False):
-    T, K = x_bf16.shape
-    fn = lib().sbn_norm_quant_act_expand68 if expand68 else lib().sbn_norm_quant_act
-    _check(fn(_ptr(x_bf16), T, K, _ptr(gain), ctypes.c_float(eps), _ptr(xq), _ptr(a_scale), _stream()),
-           "sbn_norm_quant_act")
+    _check((_native or _load_native()).norm_quant_act(x_bf16, xq, a_scale, gain, eps, expand68), "sbn_norm_quant_act")
 
 
 def _ws_args(ws):
@@ -218,31 +239,17 @@ def _ws_args(ws):
 
 
 def sbn_sparse_bitlinear(xq, a_scale, vals, meta, w_scale, y, bias=None, acc_out=None, ws=None):
-    T, N = y.shape
-    K = 2 * vals.numel() // N
-    dt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
-    wp, wb = _ws_args(ws)
-    _check(lib().sbn_sparse_bitlinear(_ptr(xq), _ptr(a_scale), T, _ptr(vals), _ptr(meta), _ptr(w_scale),
-                                      N, K, _ptr(bias), _ptr(y), dt, _ptr(acc_out), wp, wb, _stream()),
-           "sbn_sparse_bitlinear")
+    _check((_native or _load_native()).sparse_bitlinear(xq, a_scale, vals, meta, w_scale, y, bias, acc_out, ws), "sbn_sparse_bitlinear")
 
 
 def sbn_quant_act_sparse_bitlinear(x_bf16, vals, meta, w_scale, y, bias=None, acc_out=None, a_scale_out=None):
     """Activation quantiser + sparse GEMM in one kernel (few tokens)."""
-    T, K = x_bf16.shape
-    N = y.shape[1]
-    dt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
-    _check(lib().sbn_quant_act_sparse_bitlinear(_ptr(x_bf16), T, _ptr(vals), _ptr(meta), _ptr(w_scale), N, K, _ptr(bias),
-                                                _ptr(y), dt, _ptr(acc_out), _ptr(a_scale_out), _stream()),
+    _check((_native or _load_native()).quant_act_sparse_bitlinear(x_bf16, vals, meta, w_scale, y, bias, acc_out, a_scale_out),
            "sbn_quant_act_sparse_bitlinear")
 
 
 def sbn_quant_act_bitlinear(x_bf16, dense_q, w_scale, y, bias=None, acc_out=None, a_scale_out=None):
-    T, K = x_bf16.shape
-    N = y.shape[1]
-    dt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
-    _check(lib().sbn_quant_act_bitlinear(_ptr(x_bf16), T, _ptr(dense_q), _ptr(w_scale), N, K, _ptr(bias), _ptr(y), dt,
-                                         _ptr(acc_out), _ptr(a_scale_out), _stream()),
+    _check((_native or _load_native()).quant_act_bitlinear(x_bf16, dense_q, w_scale, y, bias, acc_out, a_scale_out),
            "sbn_quant_act_bitlinear")
 
 
@@ -253,11 +260,7 @@ def sbn_pack_vals2(vals, vals2):
 
 
 def sbn_sparse_bitlinear_packed(xq, a_scale, vals2, meta, w_scale, y, bias=None, acc_out=None):
-    T, N = y.shape
-    K = 8 * vals2.numel() // N
-    dt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
-    _check(lib().sbn_sparse_bitlinear_packed(_ptr(xq), _ptr(a_scale), T, _ptr(vals2), _ptr(meta), _ptr(w_scale), N, K,
-                                             _ptr(bias), _ptr(y), dt, _ptr(acc_out), _stream()),
+    _check((_native or _load_native()).sparse_bitlinear_packed(xq, a_scale, vals2, meta, w_scale, y, bias, acc_out),
            "sbn_sparse_bitlinear_packed")
 
 
@@ -267,13 +270,7 @@ def alloc_vals2(N: int, K: int, device="cuda"):
 
 
 def sbn_bitlinear(xq, a_scale, dense_q, w_scale, y, bias=None, acc_out=None, ws=None):
-    T, N = y.shape
-    K = dense_q.numel() // N
-    dt = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
-    wp, wb = _ws_args(ws)
-    _check(lib().sbn_bitlinear(_ptr(xq), _ptr(a_scale), T, _ptr(dense_q), _ptr(w_scale), N, K,
-                               _ptr(bias), _ptr(y), dt, _ptr(acc_out), wp, wb, _stream()),
-           "sbn_bitlinear")
+    _check((_native or _load_native()).bitlinear(xq, a_scale, dense_q, w_scale, y, bias, acc_out, ws), "sbn_bitlinear")
 
 
 def sbn_layer_forward_host(x_host, x_dev, xq_dev, a_scale_dev, w_scale, y_dev, y_host, vals=None,

@@ -199,3 +199,54 @@ def test_canonical_layout_calls_validate_on_host(L):
         assert fn(p, p, 0, 256, q, q, None) == SHAPE
         assert fn(odd, p, 256, 256, q, q, None) == ALIGN
         assert fn(p, p, 256, 256, p, q, None) == UNSUP                     # in place
+
+
+def test_native_calls_marshal_like_the_abi(L, monkeypatch):
+    """The extension hands every argument of a tensor call to the C ABI where sbn.h has it (fake functions, CPU tensors)."""
+    import torch
+    from paper_2603_05168_b200 import binding as b
+    seen = {}
+
+    def fake(name):
+        argtypes = getattr(L, name).argtypes
+        def f(*args):
+            seen[name] = args
+            return 3
+        return ctypes.CFUNCTYPE(ctypes.c_int, *argtypes)(f)
+
+    fakes = {name: fake(name) for name in b._NATIVE_CALLS}
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 1, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 0x70 + dev, raising=False)
+    monkeypatch.setattr(b, "lib", lambda: type("Fake", (), fakes))
+    monkeypatch.setattr(b, "_native", None)                          # restored afterwards: the next real use binds again
+    monkeypatch.setattr(b, "status_string", lambda code: "")
+    T, N, K = 3, 128, 256
+    t = lambda *shape, dt=torch.int8: torch.zeros(shape, dtype=dt)
+    x, xq, sc, vals, meta, w = t(T, K, dt=torch.bfloat16), t(16 * K), t(T, dt=torch.float32), t(N, K // 2), t(N, K // 8), t(1)
+    y, yf, bias, acc, ws, q = t(T, N, dt=torch.bfloat16), t(T, N, dt=torch.float32), t(N), t(T), t(5, dt=torch.int32), t(N, K)
+    p = lambda v: v.data_ptr()
+    calls = [
+        (lambda: b.sbn_quant_act(x, xq, sc), "sbn_quant_act", (p(x), T, K, p(xq), p(sc))),
+        (lambda: b.sbn_quant_act_expand68(x, xq, sc), "sbn_quant_act_expand68", (p(x), T, K, p(xq), p(sc))),
+        (lambda: b.sbn_norm_quant_act(x, xq, sc, gain=bias, eps=0.5), "sbn_norm_quant_act", (p(x), T, K, p(bias), 0.5, p(xq), p(sc))),
+        (lambda: b.sbn_norm_quant_act(x, xq, sc, expand68=True), "sbn_norm_quant_act_expand68", (p(x), T, K, None, ctypes.c_float(1e-6).value, p(xq), p(sc))),
+        (lambda: b.sbn_sparse_bitlinear(xq, sc, vals, meta, w, y, bias=bias, ws=ws), "sbn_sparse_bitlinear",
+         (p(xq), p(sc), T, p(vals), p(meta), p(w), N, K, p(bias), p(y), b.OUT_BF16, None, p(ws), 20)),
+        (lambda: b.sbn_bitlinear(xq, sc, q, w, yf, acc_out=acc), "sbn_bitlinear",
+         (p(xq), p(sc), T, p(q), p(w), N, K, None, p(yf), b.OUT_F32, p(acc), None, 0)),
+        (lambda: b.sbn_sparse_bitlinear_packed(xq, sc, meta, vals, w, y, acc_out=acc), "sbn_sparse_bitlinear_packed",
+         (p(xq), p(sc), T, p(meta), p(vals), p(w), N, K, None, p(y), b.OUT_BF16, p(acc))),
+        (lambda: b.sbn_quant_act_sparse_bitlinear(x, vals, meta, w, yf, bias=bias, a_scale_out=sc), "sbn_quant_act_sparse_bitlinear",
+         (p(x), T, p(vals), p(meta), p(w), N, K, p(bias), p(yf), b.OUT_F32, None, p(sc))),
+        (lambda: b.sbn_quant_act_bitlinear(x, q, w, y), "sbn_quant_act_bitlinear",
+         (p(x), T, p(q), p(w), N, K, None, p(y), b.OUT_BF16, None, None)),
+    ]
+    for call, name, want in calls:
+        with pytest.raises(b.SbnError) as err:
+            call()
+        assert err.value.code == 3
+        assert seen.pop(name) == want + (0x71,), name
+    with pytest.raises(ValueError):
+        b.sbn_quant_act(xq, xq, sc)                                  # not two-dimensional
+    assert not seen
