@@ -14,7 +14,6 @@
 #include "quant_act.cuh"
 #include "norm_quant_act.cuh"
 #include "quantize_mask_pack.cuh"
-#include "quantize_mask_pack68.cuh"
 #include "quantize_mask_pack_stream.cuh"
 #include "canonical_layout.cuh"
 #include "gemm_tcgen05.cuh"
@@ -592,12 +591,10 @@ static sbn_status quantize_mask_pack_any(const void* W, bool w_bf16, int N, int 
         misaligned(w_scale, 4) || (dense_q && misaligned(dense_q, 16)) ||
         (prev_meta && misaligned(prev_meta, 16)) || (flip_bits && misaligned(flip_bits, 8)))
         return SBN_ERR_ALIGN;
-    if (p68) {
-        const QmpDesc d = qmp_make_desc(W, w_bf16, N, K, vals, meta, w_scale, nullptr, prev_meta, flip_bits);
-        return launch_quantize_mask_pack_batch<68>(d, nullptr, 1, d.num_units, static_cast<QmpWorkspace*>(ws)->slot,
-                                                   &static_cast<QmpWorkspace*>(ws)->generation, static_cast<cudaStream_t>(stream));
-    }
-    return launch_quantize_mask_pack(W, w_bf16, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits,
+    if (p68)
+        return launch_quantize_mask_pack<68>(W, w_bf16, N, K, vals, meta, w_scale, nullptr, prev_meta, flip_bits,
+                                             static_cast<QmpWorkspace*>(ws), static_cast<cudaStream_t>(stream));
+    return launch_quantize_mask_pack<24>(W, w_bf16, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits,
                                      static_cast<QmpWorkspace*>(ws),
                                      static_cast<cudaStream_t>(stream));
 }
@@ -669,7 +666,7 @@ sbn_status sbn_quantize_mask_pack_batched(int count, const sbn_pack_job* jobs, v
             ++g_launch_count;
             if (err != cudaSuccess) return SBN_ERR_CUDA;
         }
-        const sbn_status st = launch_quantize_mask_pack_stream(descs.data() + lo, descs_dev + lo, n_here, max_units,
+        const sbn_status st = launch_quantize_mask_pack_stream<24>(descs.data() + lo, descs_dev + lo, n_here, max_units,
                                                                slots + static_cast<size_t>(lo) * kQmpMaxCtas, generation, s);
         if (st != SBN_OK) return st;
     }
@@ -697,7 +694,7 @@ sbn_status sbn_quantize_mask_pack_static_ws(const float* W, int N, int K, int n_
     void* scratch = static_scratch_for_current_device();
     if (!scratch) return SBN_ERR_CUDA;
     // every slot that is read carries this call's nonce, so stale contents are harmless
-    return launch_quantize_mask_pack(W, false, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits,
+    return launch_quantize_mask_pack<24>(W, false, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits,
                                      static_cast<QmpWorkspace*>(scratch),
                                      static_cast<cudaStream_t>(stream));
 }

@@ -5,8 +5,8 @@
 // rounded correctly from an ESTIMATE of gamma: W_q = sign(w) [ |w| >= thr(gamma) ] and only the
 // few |w| that lie within a few percent of thr depend on its exact value.  One persistent kernel
 // (one 1024-thread CTA per SM) therefore reads W ONCE, for one matrix or a batch of them.  This file
-// holds the building blocks and the phase-by-phase kernel that the 6:8 pattern uses; the 2:4 pattern
-// runs the same phases as one uninterrupted stream (quantize_mask_pack_stream.cuh).  The phases:
+// holds the building blocks; the kernel runs the phases as one uninterrupted stream
+// (quantize_mask_pack_stream.cuh).  The phases:
 //
 //   sample   every CTA adds |w| over the same 256 scattered 512 B units of the matrix (128 KB,
 //            L2-served for all CTAs but the first; 64 units for matrices below 33 M weights)
@@ -52,8 +52,6 @@ namespace sbn {
 constexpr int kQmpThreads = 1024;
 constexpr int kQmpWarps = kQmpThreads / 32;
 constexpr int kQmpMaxCtas = kNumSMs;                       // one CTA per SM, all co-resident
-constexpr int kQmpListCap = 8192;                          // undecided entries per CTA and matrix
-constexpr int kQmpSmemBytes = 2 * kQmpListCap * 8;         // two lists (consecutive matrices of a batch)
 constexpr int kQmpSampleUnits = 256;                       // units in the gamma_est sample of a large matrix
 constexpr float kQmpBracket = 0.03f;                       // gamma_est * (1 -+ this) brackets gamma
 // Matrices below 2^18 units (33.5 M weights) are sampled at a quarter of that with a wider bracket:
@@ -102,14 +100,6 @@ __device__ __forceinline__ unsigned long long global_timer_ns_qmp() {
     return t;
 }
 
-// Smallest fp32 a with fl(a / scale) > 0.5, searched around 0.5 * scale with IEEE divisions.
-__device__ __forceinline__ float ternary_threshold(float scale) {
-    float a = 0.5f * scale;
-    for (int it = 0; it < 8 && __fdiv_rn(a, scale) > 0.5f; ++it) a = __uint_as_float(__float_as_uint(a) - 1u);
-    for (int it = 0; it < 16 && !(__fdiv_rn(a, scale) > 0.5f); ++it) a = __uint_as_float(__float_as_uint(a) + 1u);
-    return a;
-}
-
 // Eq. 2 for one group: the two largest |w| of four (ranking on the fp32 master weights; on equal
 // magnitudes the lower column wins).  Returns the nibble i0 | i1 << 2 (i0 < i1) and the two kept
 // weights in column order.  The winners of the pairs (0,1) and (2,3) are the answer unless the
@@ -151,22 +141,6 @@ __device__ __forceinline__ uint32_t ternary_bytes2(float w0, float w1, float thr
 
 __device__ __forceinline__ uint32_t nibble_to_mask(uint32_t nib) {
     return (1u << (nib & 3u)) | (1u << ((nib >> 2) & 3u));
-}
-
-constexpr int kQmpPrefetchAhead = 3;                       // pass 1 iterations (128 units = 64 KB each) ahead
-
-// Sum of `v` over the CTA in a fixed order; identical in every thread.
-__device__ __forceinline__ double qmp_block_sum(double v, double* s_warp) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) s_warp[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < kQmpWarps; ++w) t += s_warp[w];
-    __syncthreads();
-    return t;
 }
 
 __device__ __forceinline__ double abs_sum4(const float4 v) {
@@ -228,53 +202,6 @@ __device__ __forceinline__ QmpRange qmp_range(const QmpDesc& d) {
     return r;
 }
 
-// gamma_est: mean |w| over kQmpSampleUnits units scattered over the matrix (the same units in every
-// CTA; a multiplicative hash keeps them off any row / column-block period).  fp32 is plenty here.
-template <bool BF16>
-__device__ __forceinline__ float qmp_sample_gamma(const QmpDesc& d, double* s_warp) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const uint32_t n_s = qmp_sample_units(d.num_units);
-    const uint32_t stride = d.num_units / n_s;                        // >= 1
-    float acc = 0.0f;
-    constexpr int kPerWarp = kQmpSampleUnits / kQmpWarps;
-    float4 v[kPerWarp];
-#pragma unroll
-    for (int i = 0; i < kPerWarp; ++i) {                  // all loads of the warp in flight at once
-        const uint32_t sidx = warp + i * kQmpWarps;
-        const uint32_t u = sidx * stride + ((sidx * 2654435761u) >> 8) % stride;
-        v[i] = sidx < n_s ? qmp_load_group<BF16>(d.W, u, lane) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int i = 0; i < kPerWarp; ++i) acc += (fabsf(v[i].x) + fabsf(v[i].y)) + (fabsf(v[i].z) + fabsf(v[i].w));
-    const double total = qmp_block_sum(static_cast<double>(acc), s_warp);
-    return static_cast<float>(total / (static_cast<double>(n_s) * 128.0));
-}
-
-// Appends the undecided ones of four consecutive kept values (bytes byte_off .. byte_off + 3 of vals).
-template <int CAP = kQmpListCap>
-__device__ __forceinline__ void qmp_list_undecided(const float (&k)[4], const float thr_lo, const float thr_hi,
-                                                   const uint32_t byte_off, QmpEntry* list, unsigned int* list_count) {
-    bool und[4];
-    unsigned int cnt = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float a = fabsf(k[i]);
-        und[i] = a >= thr_lo && a < thr_hi;
-        cnt += und[i] ? 1u : 0u;
-    }
-    if (cnt != 0u) {                                       // a few percent of the lanes get here
-        unsigned int at = atomicAdd(list_count, cnt);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (und[i]) {
-                if (at < static_cast<unsigned int>(CAP)) { list[at].byte_off = byte_off + i; list[at].w = k[i]; }
-                ++at;
-            }
-        }
-    }
-}
-
 // Ternarise a whole range again with the exact threshold (the path taken when the bracket missed,
 // the list overflowed or the dense W_q is wanted): a warp per unit, four units at a time, newest
 // first (what pass 1 read last is still in L2).
@@ -321,156 +248,6 @@ __device__ __forceinline__ void qmp_pass2_full(const QmpDesc& d, const QmpRange 
     }
 }
 
-// The pass of the 6:8 pattern (quantize_mask_pack68.cuh; FINAL = values only, exact threshold).
-template <bool BF16, bool FINAL>
-__device__ __forceinline__ double qmp68_pass(const QmpDesc& d, const QmpRange rg, const float thr_lo, const float thr_hi,
-                                             QmpEntry* list, unsigned int* list_count, double* s_warp,
-                                             unsigned int& flips);
-
-// Batch of `count` matrices in one persistent launch, software-pipelined over the matrices:
-//   S+P1(0) | S+P1(1) F(0) | S+P1(2) F(1) | ... | F(count-1)        (S sample, F exchange + fix-up)
-// so by the time a CTA needs gamma of matrix m, every CTA has long published its partial for m,
-// and the per-launch and per-exchange latencies are paid once per batch, not once per matrix.
-// The two undecided lists alternate between consecutive matrices.  `first` is matrix 0 (passed by
-// value), `rest` matrices 1.. in global memory.  PATTERN: 68 (the 2:4 pattern has its own kernel).
-template <int PATTERN>
-__global__ void __launch_bounds__(kQmpThreads, 1)
-quantize_mask_pack_kernel(const QmpDesc first, const QmpDesc* __restrict__ rest, int count,
-                          QmpSlot* slots, unsigned long long* generation, unsigned long long call_nonce,
-                          int test_withhold_slot) {
-    extern __shared__ QmpEntry s_list[];                // [2][kQmpListCap]
-    __shared__ double s_warp[kQmpWarps];
-    __shared__ float s_thr;
-    __shared__ int s_ok;
-    __shared__ unsigned int s_flips[kQmpWarps];
-    __shared__ unsigned long long s_flip_total[2];
-    __shared__ unsigned int s_list_count[2];
-    __shared__ float s_bracket[2][2];                   // [matrix parity][lo, hi]
-
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_ok = 1;
-    __syncthreads();
-    // No early signal to the next kernel of the stream: this kernel writes packed weights, and the
-    // GEMM kernels fetch weights before their own dependency wait (see sbn_common.cuh).
-    pdl_wait();
-    // stable for the whole execution: CTA 0 advances it only after it has seen every CTA's last slot,
-    // and every CTA reads it here, before it publishes anything
-    const unsigned long long gen0 = *reinterpret_cast<volatile unsigned long long*>(generation);
-    const unsigned long long nonce = qmp_tag(call_nonce, gen0);
-
-    QmpDesc d_prev = first;
-    QmpRange rg_prev = {0u, 0u};
-    for (int m = 0; m <= count; ++m) {
-        // ---- sample + pass 1 of matrix m, publish its partial
-        QmpDesc d_cur = first;
-        QmpRange rg_cur = {0u, 0u};
-        if (m < count) {
-            if (m > 0) d_cur = rest[m - 1];
-            rg_cur = qmp_range(d_cur);
-            const int par = m & 1;
-            const float gamma_est = d_cur.w_bf16 ? qmp_sample_gamma<true>(d_cur, s_warp) : qmp_sample_gamma<false>(d_cur, s_warp);
-            if (threadIdx.x == 0) {
-                s_list_count[par] = 0u;
-                // any lo <= hi will do (the exact threshold is checked against them later), so no
-                // divisions here: thr(scale) is 0.5 * scale to within a few ulps
-                const float b = d_cur.num_units < kQmpSmallMatrixUnits ? kQmpBracketSmall : kQmpBracket;
-                s_bracket[par][0] = 0.5f * fmaxf(gamma_est * (1.0f - b), kEps) * (1.0f - 1e-6f);
-                s_bracket[par][1] = 0.5f * fmaxf(gamma_est * (1.0f + b), kEps) * (1.0f + 1e-6f);
-            }
-            __syncthreads();
-            unsigned int flips = 0;
-            double mine;
-            static_assert(PATTERN == 68, "the 2:4 pattern runs in quantize_mask_pack_stream_kernel");
-            mine = d_cur.w_bf16
-                ? qmp68_pass<true, false>(d_cur, rg_cur, s_bracket[par][0], s_bracket[par][1], s_list + par * kQmpListCap,
-                                          &s_list_count[par], s_warp, flips)
-                : qmp68_pass<false, false>(d_cur, rg_cur, s_bracket[par][0], s_bracket[par][1], s_list + par * kQmpListCap,
-                                           &s_list_count[par], s_warp, flips);
-            // this CTA's flip count of matrix m; it is added to the global counter one phase later,
-            // after the exchange has shown that CTA 0 zeroed that counter
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) flips += __shfl_xor_sync(0xFFFFFFFFu, flips, o);
-            if (lane == 0) s_flips[warp] = flips;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned long long t = 0;
-#pragma unroll
-                for (int w2 = 0; w2 < kQmpWarps; ++w2) t += s_flips[w2];
-                s_flip_total[par] = t;
-                if (blockIdx.x == 0 && d_cur.flip_bits != nullptr) *d_cur.flip_bits = 0ull;
-                QmpSlot* sl = slots + static_cast<size_t>(m) * gridDim.x + blockIdx.x;
-                sl->partial = mine;
-                __threadfence();
-                // diagnostics (sbn_set_wait_test): the last CTA keeps its tag to itself, so every CTA's
-                // bounded wait for that slot runs out
-                if (!(test_withhold_slot && blockIdx.x == gridDim.x - 1))
-                    *reinterpret_cast<volatile unsigned long long*>(&sl->nonce) = nonce;
-            }
-            __syncthreads();
-        }
-        // ---- exchange + fix-up of matrix m-1 (published one phase ago by every CTA)
-        if (m >= 1) {
-            const int par = (m - 1) & 1;
-            const QmpSlot* base = slots + static_cast<size_t>(m - 1) * gridDim.x;
-            double other = 0.0;
-            if (threadIdx.x < gridDim.x) {
-                const volatile unsigned long long* flag = &base[threadIdx.x].nonce;
-                const unsigned long long t0 = global_timer_ns_qmp();
-                unsigned int spins = 0;
-                bool seen = (*flag == nonce);
-                while (!seen) {
-                    seen = (*flag == nonce);
-                    if (!seen && ((++spins & 0xFFu) == 0) &&
-                        global_timer_ns_qmp() - t0 > *reinterpret_cast<volatile unsigned long long*>(&g_wait_limit_ns)) break;
-                }
-                if (seen) {
-                    __threadfence();
-                    other = *reinterpret_cast<const volatile double*>(&base[threadIdx.x].partial);
-                } else {
-                    s_ok = 0;
-                    atomicExch(&g_device_status, static_cast<int>(SBN_ERR_TIMEOUT));
-                }
-            }
-            const double S = qmp_block_sum(other, s_warp);      // fixed order: the same bits in every CTA
-            if (!s_ok) return;                                   // a peer never arrived: give up cleanly
-            if (threadIdx.x == 0 && d_prev.flip_bits != nullptr && s_flip_total[par] != 0ull)
-                atomicAdd(d_prev.flip_bits, s_flip_total[par]);
-            const double cnt = static_cast<double>(d_prev.num_units) * 128.0;
-            const float gamma = static_cast<float>(S / cnt);
-            const float scale = fmaxf(gamma, kEps);
-            if (threadIdx.x == 0) {
-                s_thr = ternary_threshold(scale);
-                if (blockIdx.x == 0) *d_prev.w_scale = scale;
-            }
-            __syncthreads();
-            const float thr = s_thr;
-            const unsigned int listed = s_list_count[par];
-            const bool bracket_ok = s_bracket[par][0] <= thr && thr <= s_bracket[par][1] &&
-                                    listed <= static_cast<unsigned int>(kQmpListCap) && d_prev.dense_q == nullptr &&
-                                    d_prev.num_units <= (PATTERN == 68 ? (1u << 25) : (1u << 26));   // listed byte offsets are 32-bit
-            if (bracket_ok) {
-                // every byte not on the list is already final; the listed ones get the exact compare
-                const QmpEntry* list = s_list + par * kQmpListCap;
-                uint8_t* vb = reinterpret_cast<uint8_t*>(d_prev.vals);
-                for (unsigned int e = threadIdx.x; e < listed; e += kQmpThreads) {
-                    const float w = list[e].w;
-                    vb[list[e].byte_off] = static_cast<uint8_t>(fabsf(w) >= thr ? (w < 0.0f ? 0xFFu : 0x01u) : 0u);
-                }
-            } else {
-                unsigned int unused = 0;
-                if (d_prev.w_bf16) qmp68_pass<true, true>(d_prev, rg_prev, thr, thr, nullptr, nullptr, s_warp, unused);
-                else qmp68_pass<false, true>(d_prev, rg_prev, thr, thr, nullptr, nullptr, s_warp, unused);
-            }
-            __syncthreads();                                     // s_thr / this list may be reused
-        }
-        d_prev = d_cur;
-        rg_prev = rg_cur;
-    }
-    // every CTA has published its last slot (CTA 0 has just read them all), hence has read the generation
-    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long*>(generation) = gen0 + 1ull;
-}
-
 // Copies up to kQmpDescChunk job descriptors, passed by value, into the batch workspace: the batched
 // call hands its jobs to the device without a host-side staging copy.
 constexpr int kQmpDescChunk = 48;
@@ -508,28 +285,6 @@ inline QmpDesc qmp_make_desc(const void* W, bool w_bf16, int N, int K, int8_t* v
     d.num_units = static_cast<uint32_t>(static_cast<size_t>(N) * K / 128);
     d.KB = static_cast<uint32_t>(K / 128);
     return d;
-}
-
-// Launch for `count` matrices: `first` by value, the others already copied to `rest_dev`.
-template <int PATTERN>
-inline sbn_status launch_quantize_mask_pack_batch(const QmpDesc& first, const QmpDesc* rest_dev, int count,
-                                                  uint32_t max_units, QmpSlot* slots, unsigned long long* generation,
-                                                  cudaStream_t stream) {
-    const int test_withhold_slot = g_test_break_waits;
-    unsigned long long nonce = qmp_next_nonce();
-    // every CTA must be resident at once (they exchange partial sums): never more CTAs than this
-    // device has SMs, and never more than the workspace has slots
-    const unsigned cap = static_cast<unsigned>(std::min(device_sm_count(), kQmpMaxCtas));
-    const unsigned grid = max_units < cap ? max_units : cap;
-    static_assert(kQmpThreads >= kQmpMaxCtas, "one thread per slot in the exchange");
-    if (!ensure_dynamic_smem<quantize_mask_pack_kernel<PATTERN>>(kQmpSmemBytes)) return SBN_ERR_CUDA;
-    // At most one CTA per SM (1024 threads x 64 registers each) and never more CTAs than SMs, so all
-    // of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
-    // another kernel kept SMs busy for seconds, the bounded wait reports SBN_ERR_TIMEOUT instead.
-    const cudaError_t err = launch_kernel(quantize_mask_pack_kernel<PATTERN>, dim3(grid), dim3(kQmpThreads), kQmpSmemBytes, stream,
-                                          first, rest_dev, count, slots, generation, nonce, test_withhold_slot);
-    ++g_launch_count;
-    return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
 
 }  // namespace sbn

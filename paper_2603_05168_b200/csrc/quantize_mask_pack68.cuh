@@ -12,10 +12,8 @@
 // sparse GEMM runs unchanged at 3/4 of the dense MMA work.  The outputs are the compressed values
 // and metadata of that [N][K'] matrix in the tiled layouts of layouts.cuh.
 //
-// Same single-pass scheme as the 2:4 kernel (sample -> bracket, pass 1 with provisional
-// ternarisation and a list of undecided kept values, exchange of partial sums, fix-up).  A lane
-// owns one group of 8 (32 B of a row): 6 bytes of values (three 2-byte stores) and 12 bits of
-// metadata (a quad of lanes writes its 6 bytes as three 2-byte stores).
+// The pack kernel is the 2:4 one (quantize_mask_pack_stream.cuh) with another pass 1: a group's kept set is
+// an index into a table (in shared memory) that says which columns the windows take, in which order.
 #pragma once
 
 #include "quantize_mask_pack.cuh"
@@ -24,21 +22,29 @@ namespace sbn {
 
 // Eq. 2 for one group of 8: bit j set = column j kept.  The two smallest |w| are dropped; among
 // equal magnitudes the higher column goes first (the lower column wins a tie, as in the 2:4 rule).
+// t2 = the second smallest (a merge network of sorted pairs); what is larger is kept, and unless there is a tie at t2
+// that is all of it.
 __device__ __forceinline__ uint32_t select6of8(const float (&a)[8]) {
-    float m = a[7];
-    int i1 = 7;
+    float lo[4], hi[4];
 #pragma unroll
-    for (int i = 6; i >= 0; --i) {
-        if (a[i] < m) { m = a[i]; i1 = i; }
-    }
-    float m2 = (i1 == 7) ? __int_as_float(0x7F800000) : a[7];
-    int i2 = 7;
+    for (int i = 0; i < 4; ++i) { lo[i] = fminf(a[2 * i], a[2 * i + 1]); hi[i] = fmaxf(a[2 * i], a[2 * i + 1]); }
+    const float l0 = fminf(lo[0], lo[1]), s0 = fminf(fmaxf(lo[0], lo[1]), fminf(hi[0], hi[1]));
+    const float l1 = fminf(lo[2], lo[3]), s1 = fminf(fmaxf(lo[2], lo[3]), fminf(hi[2], hi[3]));
+    const float t2 = fminf(fmaxf(l0, l1), fminf(s0, s1));
+    uint32_t d[8];
 #pragma unroll
-    for (int i = 6; i >= 0; --i) {
-        const float b = (i == i1) ? __int_as_float(0x7F800000) : a[i];
-        if (b < m2) { m2 = b; i2 = i; }
+    for (int i = 0; i < 8; ++i) d[i] = __float_as_uint(t2 - a[i]);            // sign bit set: larger
+    const uint32_t g03 = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u);     // 0xFF per such column
+    const uint32_t g47 = prmt(prmt(d[4], d[5], 0x00FBu), prmt(d[6], d[7], 0x00FBu), 0x5410u);
+    uint32_t S = (((g03 & 0x08040201u) | (g47 & 0x80402010u)) * 0x01010101u) >> 24;
+    int need = 6 - __popc(S);
+    if (need != 0) {                                          // a tie: the lowest of the columns that equal t2
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (need != 0 && a[i] == t2) { S |= 1u << i; --need; }
+        }
     }
-    return 0xFFu ^ (1u << i1) ^ (1u << i2);
+    return S;
 }
 
 // Deals the kept columns S (6 bits set of 8) out to the three windows: 4-bit masks, two bits each.
@@ -59,10 +65,20 @@ __device__ __forceinline__ uint32_t mask4_to_nibble(uint32_t m) {
     constexpr uint32_t kHi = (12u << 4) | (13u << 8) | (14u << 16);     // masks 9, 10, 12
     return (((m & 8u) ? kHi : kLo) >> (4u * (m & 7u))) & 15u;
 }
-// The two kept weights of a window in column order.
-__device__ __forceinline__ void window_values(uint32_t m, float c0, float c1, float c2, float c3, float& v0, float& v1) {
-    v0 = (m & 1u) ? c0 : ((m & 2u) ? c1 : c2);
-    v1 = (m & 8u) ? c3 : ((m & 4u) ? c2 : c1);
+// Table entry of the kept set S: x = columns of the six kept values, a nibble each, window by window (a byte-permute
+// selector for the group's eight value bytes); y = the three windows' metadata nibbles.
+__device__ __forceinline__ uint2 table68_entry(uint32_t S) {
+    if (__popc(S) != 6) return make_uint2(0u, 0u);
+    uint32_t m[3];
+    windows68(S, m[0], m[1], m[2]);
+    uint2 e = make_uint2(0u, 0u);
+#pragma unroll
+    for (uint32_t w = 0; w < 3; ++w) {
+        const uint32_t first = __ffs(static_cast<int>(m[w])) - 1, last = 31 - __clz(static_cast<int>(m[w]));
+        e.x |= ((2u * w + first) | ((2u * w + last) << 4)) << (8u * w);
+        e.y |= mask4_to_nibble(m[w]) << (4u * w);
+    }
+    return e;
 }
 
 // Kept-column mask of a group of 8 from its three metadata nibbles.
@@ -79,111 +95,48 @@ __device__ __forceinline__ size_t vals68_offset(uint32_t n, uint32_t c, uint32_t
     return (static_cast<size_t>(n >> 7) * KBp + (c >> 6)) * 8192u + vals_in_tile(n & 127u, c & 63u);
 }
 
-// Pass over this CTA's range.  FINAL = false: pass 1 (sum |W|, metadata, flip count, provisional
-// values against thr_hi, list of the kept values in [thr_lo, thr_hi)).  FINAL = true: the values
-// again with the exact threshold (thr_hi = thr), nothing else.
-template <bool BF16, bool FINAL>
-__device__ __forceinline__ double qmp68_pass(const QmpDesc& d, const QmpRange rg, const float thr_lo, const float thr_hi,
-                                             QmpEntry* list, unsigned int* list_count, double* s_warp,
-                                             unsigned int& flips) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const uint32_t l16 = lane & 15;
-    const uint32_t quad_lane = l16 & 3u;
-    const uint32_t KB = d.KB;
-    const uint32_t KBp = KB + (KB >> 1);                      // K' / 128
-    constexpr uint32_t kStep = 2 * kQmpWarps;
-    constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
-    const bool count_flips = !FINAL && d.prev_meta != nullptr;
-    uint8_t* vals_b = reinterpret_cast<uint8_t*>(d.vals);
-    double acc = 0.0;
-    const uint32_t u_first = rg.u_begin + 2 * warp + (lane >> 4);
-    const uint32_t step_n = kStep / KB, step_kb = kStep % KB;  // a thread's next unit, without a division
-    uint32_t n = u_first / KB;
-    uint32_t kb = u_first - n * KB;
-    if (threadIdx.x == 0) {
-        for (int j = 1; j < kQmpPrefetchAhead; ++j) {
-            const uint32_t ub = rg.u_begin + j * kStep;
-            if (ub < rg.u_end) prefetch_l2_bulk(static_cast<const char*>(d.W) + static_cast<size_t>(ub) * kUnitBytes, min(rg.u_end - ub, kStep) * kUnitBytes);
-        }
+// Eq. 1 for the eight weights of a group as bytes (+1 -> 0x01, -1 -> 0xFF, 0 -> 0x00), +-1 iff |w| > thr_pred; `e` =
+// the bits of thr_pred - |w|.
+__device__ __forceinline__ void ternary68(const float (&w)[8], const float thr_pred, uint32_t (&e)[8], uint32_t& b03, uint32_t& b47) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(thr_pred - fabsf(w[i]));
+    uint32_t b[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t keep = prmt(prmt(e[4 * h], e[4 * h + 1], 0x00FBu), prmt(e[4 * h + 2], e[4 * h + 3], 0x00FBu), 0x5410u);
+        const uint32_t sign = prmt(prmt(__float_as_uint(w[4 * h]), __float_as_uint(w[4 * h + 1]), 0x00FBu),
+                                   prmt(__float_as_uint(w[4 * h + 2]), __float_as_uint(w[4 * h + 3]), 0x00FBu), 0x5410u);
+        b[h] = (sign | 0x01010101u) & keep;
     }
-    for (uint32_t u0 = rg.u_begin; u0 < rg.u_end; u0 += kStep, n += step_n, kb += step_kb) {
-        if (kb >= KB) { kb -= KB; ++n; }
-        if (threadIdx.x == 0) {
-            const uint32_t ub = u0 + kQmpPrefetchAhead * kStep;
-            if (ub < rg.u_end) prefetch_l2_bulk(static_cast<const char*>(d.W) + static_cast<size_t>(ub) * kUnitBytes, min(rg.u_end - ub, kStep) * kUnitBytes);
-        }
-        const uint32_t uq = u0 + (u_first - rg.u_begin);
-        const bool active = uq < rg.u_end;                     // uniform over a half-warp
-        float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
-        if (active) qmp_load_group_pair<BF16>(d.W, uq, l16, va, vb);
-        if constexpr (!FINAL) acc += abs_sum4(va) + abs_sum4(vb);
-        const uint32_t g_row = kb * 16u + l16;                 // group of 8 within the row
+    b03 = b[0];
+    b47 = b[1];
+}
+
+// Values of this CTA's range again with the exact threshold (what qmp_pass2_full is for 2:4): a half-warp per unit, a lane
+// one group.
+template <bool BF16>
+__device__ __forceinline__ void qmp68_pass2_full(const QmpDesc& d, const QmpRange rg, const float thr, const uint2* table) {
+    const uint32_t l16 = threadIdx.x & 15u;
+    const uint32_t KB = d.KB, KBp = KB + (KB >> 1);           // K' / 128
+    const float thr_pred = __uint_as_float(__float_as_uint(thr) - 1u);
+    uint8_t* const vals = reinterpret_cast<uint8_t*>(d.vals);
+    for (uint32_t u = rg.u_begin + (threadIdx.x >> 4); u < rg.u_end; u += 2u * kQmpWarps) {
+        const uint32_t n = u / KB, kb = u - n * KB;
+        float4 va, vb;
+        qmp_load_group_pair<BF16>(d.W, u, l16, va, vb);
         const float w[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
         float a[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) a[i] = fabsf(w[i]);
-        const uint32_t S = select6of8(a);
-        uint32_t m0, m1, m2;
-        windows68(S, m0, m1, m2);
-        float k[6];
-        window_values(m0, w[0], w[1], w[2], w[3], k[0], k[1]);
-        window_values(m1, w[2], w[3], w[4], w[5], k[2], k[3]);
-        window_values(m2, w[4], w[5], w[6], w[7], k[4], k[5]);
-        if constexpr (!FINAL) {
-            const uint32_t m12 = mask4_to_nibble(m0) | (mask4_to_nibble(m1) << 4) | (mask4_to_nibble(m2) << 8);
-            if (count_flips) {
-                // this group's 12 bits of the previous metadata: bits 12 g .. 12 g + 11 of the row.
-                // meta may be the same buffer as prev_meta: every byte a quad overwrites below is read
-                // here by lanes of that quad only, and the warp barrier orders those reads first.
-                if (active) {
-                    const uint32_t b0 = (3u * g_row) >> 1;
-                    const uint32_t lo = d.prev_meta[meta68_offset(n, b0, KBp)];
-                    const uint32_t hi = d.prev_meta[meta68_offset(n, b0 + 1u, KBp)];
-                    const uint32_t p12 = ((lo | (hi << 8)) >> ((g_row & 1u) * 4u)) & 0xFFFu;
-                    flips += __popc(S ^ mask8_from_meta12(p12));
-                }
-                __syncwarp();
-            }
-            // a quad's 48 bits leave as three 2-byte stores (lanes 0..2 of the quad)
-            const uint32_t nxt = __shfl_down_sync(0xFFFFFFFFu, m12, 1);
-            if (active && quad_lane < 3u) {
-                const uint32_t out = ((m12 >> (4u * quad_lane)) | (nxt << (12u - 4u * quad_lane))) & 0xFFFFu;
-                const size_t m_off = meta68_offset(n, 6u * (g_row >> 2) + 2u * quad_lane, KBp);
-                *reinterpret_cast<uint16_t*>(d.meta + m_off) = static_cast<uint16_t>(out);
-            }
-        }
-        if (active) {
-            uint32_t off[3];
-            unsigned int cnt = 0;
-            bool und[6];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                off[j] = static_cast<uint32_t>(vals68_offset(n, 6u * g_row + 2u * j, KBp));
-                *reinterpret_cast<uint16_t*>(vals_b + off[j]) = static_cast<uint16_t>(ternary_bytes2(k[2 * j], k[2 * j + 1], thr_hi));
-            }
-            if constexpr (!FINAL) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    const float ak = fabsf(k[i]);
-                    und[i] = ak >= thr_lo && ak < thr_hi;
-                    cnt += und[i] ? 1u : 0u;
-                }
-                if (cnt != 0u) {
-                    unsigned int at = atomicAdd(list_count, cnt);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        if (und[i]) {
-                            if (at < static_cast<unsigned int>(kQmpListCap)) { list[at].byte_off = off[i >> 1] + (i & 1); list[at].w = k[i]; }
-                            ++at;
-                        }
-                    }
-                }
-            }
-        }
+        uint32_t e[8], b03, b47;
+        ternary68(w, thr_pred, e, b03, b47);
+        const uint32_t sel = table[select6of8(a)].x;
+        const uint32_t v4 = prmt(b03, b47, sel & 0xFFFFu), v2 = prmt(b03, b47, sel >> 16);
+        const uint32_t c = 96u * kb + 6u * l16;
+        *reinterpret_cast<uint16_t*>(vals + vals68_offset(n, c, KBp)) = static_cast<uint16_t>(v4);
+        *reinterpret_cast<uint16_t*>(vals + vals68_offset(n, c + 2u, KBp)) = static_cast<uint16_t>(v4 >> 16);
+        *reinterpret_cast<uint16_t*>(vals + vals68_offset(n, c + 4u, KBp)) = static_cast<uint16_t>(v2);
     }
-    if constexpr (FINAL) return 0.0;
-    else return qmp_block_sum(acc, s_warp);
 }
 
 }  // namespace sbn

@@ -1,4 +1,4 @@
-// Part 1 (Eq. 1-3, 2:4 pattern) for one matrix or a batch, as ONE uninterrupted stream over the weights.
+// Part 1 (Eq. 1-3) for one matrix or a batch, as ONE uninterrupted stream over the weights; 2:4 and 6:8 patterns.
 //
 // quantize_mask_pack.cuh explains the single-read scheme (bracketed threshold, provisional values,
 // fix-up list, exact fallback).  What costs time beside the stream itself is latency: the sample that
@@ -40,6 +40,7 @@
 #pragma once
 
 #include "quantize_mask_pack.cuh"
+#include "quantize_mask_pack68.cuh"
 
 namespace sbn {
 
@@ -49,7 +50,7 @@ constexpr int kQmpFinisherWarp = kQmpStreamWarps + 1;
 constexpr int kQmpScoutWarp = kQmpStreamWarps + 2;
 constexpr int kQmpScouts = kQmpWarps - kQmpScoutWarp;
 constexpr int kQmpLists = 3;
-constexpr int kQmpWarpListCap = 160;                       // undecided entries per computing warp and matrix, three lists in use
+constexpr int kQmpWarpListCap = 156;                       // undecided entries per computing warp and matrix, three lists in use
 constexpr int kQmpListEntries = kQmpStreamWarps * kQmpWarpListCap;
 // A launch of one or two matrices uses one or two of the three lists, each that much larger.
 __host__ __device__ inline uint32_t qmp_list_cap(int count) {
@@ -101,7 +102,7 @@ struct QmpStreamShared {
     uint32_t ring_issued, ring_used;                       // the loader's copies of this launch, and its ring position
     float thr_second_pass[kQmpMaxBatch];                   // >= 0: this matrix needs the exact second pass with this threshold
 };
-static_assert(kQmpStreamSmemBytes + sizeof(QmpStreamShared) <= 232448, "shared memory overflow");
+static_assert(kQmpStreamSmemBytes + sizeof(QmpStreamShared) + 256 * sizeof(uint2) <= 232448, "shared memory overflow");
 
 // mbarrier and bulk-copy wrappers of the stage ring
 __device__ __forceinline__ uint32_t qmp_smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -390,6 +391,29 @@ __device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
     return __popc(any | (none << 1));
 }
 
+// Where a computing warp is in a matrix: its quarter-warp's unit of the current step of its team's stages.
+template <bool BF16>
+struct QmpWalk {
+    static constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
+    static constexpr uint32_t REP = kQmpStageBytes / (kQmpStepUnits * kUnitBytes);     // steps per stage
+    uint32_t n, kb;                       // row and 128-column block
+    int left;                             // > 0: the quarter-warp has a unit in the step
+    __device__ __forceinline__ QmpWalk(const QmpJob& jb, uint32_t stage_in_matrix, uint32_t in_step) {
+        const uint32_t u0 = stage_in_matrix * (REP * kQmpStepUnits) + in_step;         // from the range's start
+        const uint32_t k0 = jb.kb0 + u0;
+        const uint32_t dn = jb.kb_magic != 0u ? __umulhi(k0, jb.kb_magic) : k0;
+        n = jb.n0 + dn;
+        kb = k0 - dn * jb.KB;
+        left = static_cast<int>(jb.units) - static_cast<int>(u0);
+    }
+    __device__ __forceinline__ void advance(const QmpJob& jb, uint32_t KB, bool in_stage) {
+        n += in_stage ? jb.rep_n : jb.next_n;
+        kb += in_stage ? jb.rep_kb : jb.next_kb;
+        if (kb >= KB) { kb -= KB; ++n; }
+        left -= static_cast<int>((in_stage ? 1u : (kQmpTeams * REP - REP + 1u)) * kQmpStepUnits);
+    }
+};
+
 // Pass 1 of one matrix for a computing warp: its four units of every step of its team's stages (a quarter-warp per
 // unit, a lane 16 weights = four groups).  The matrix's stages are the ring's g0 .. g0 + n - 1, the team's next one is
 // `next_stage`.  Returns the thread's sum |W|; `ok` turns false if a wait ran out.
@@ -412,8 +436,8 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     const int lane = threadIdx.x & 31;
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t l8 = lane & 7;
-    constexpr uint32_t kUnitBytes = BF16 ? 256u : 512u;
-    constexpr uint32_t REP = kQmpStageBytes / (kQmpStepUnits * kUnitBytes);    // steps per stage
+    using Walk = QmpWalk<BF16>;
+    constexpr uint32_t kUnitBytes = Walk::kUnitBytes, REP = Walk::REP;
     constexpr int PIECES = BF16 ? 2 : 4;                              // 16-byte pieces per lane
     const uint32_t KB = jb.KB;
     // kept is +-1 iff |k| > thr_pred, undecided iff 0 <= thr_pred - |k| <= width.  The subtraction is exact near the
@@ -425,15 +449,7 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     const uint32_t g_end = g0 + n_stages;
     double acc = 0.0;
     const uint32_t in_step = 4u * (warp % kQmpTeamWarps) + (lane >> 3);          // this quarter-warp's unit of every step
-    const uint32_t u0 = (next_stage - g0) * (REP * kQmpStepUnits) + in_step;     // ... of its first one here, from the range's start
-    uint32_t n, kb;
-    {
-        const uint32_t k0 = jb.kb0 + u0;
-        const uint32_t dn = jb.kb_magic != 0u ? __umulhi(k0, jb.kb_magic) : k0;
-        n = jb.n0 + dn;
-        kb = k0 - dn * KB;
-    }
-    int left = static_cast<int>(jb.units) - static_cast<int>(u0);     // > 0: this quarter-warp has a unit in the step
+    Walk at(jb, next_stage - g0, in_step);
     const uint32_t turn = BF16 ? (l8 >> 2) : (l8 >> 1);               // rotation of the pieces ...
     const uint32_t rot = BF16 ? 2u * turn : turn;                     // ... and of the groups
     uint32_t src[PIECES];
@@ -452,9 +468,9 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     const uint32_t chunk = l8 >> 1;
     // row index in the tiled order: 16 B of metadata and 64 B of values each (layouts.cuh)
     auto tiled_row = [&](uint32_t nn, uint32_t kk) { return (((nn >> 7) * KB + kk) << 7) + (nn & 127u); };
-    uint32_t q = tiled_row(n, kb);
+    uint32_t q = tiled_row(at.n, at.kb);
     uint32_t prev = 0u;
-    if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
+    if (prev_lane != nullptr && at.left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
@@ -468,15 +484,12 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
                 __syncwarp();
                 if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);   // the values are in registers: the stage may be refilled
             }
-            const bool mine = left > 0;
+            const bool mine = at.left > 0;
             const uint32_t q_cur = q, prev_cur = prev;
-            const uint32_t v8 = q_cur * 8u + 2u * (chunk ^ ((n >> 1) & 3u)) + (l8 & 1u);       // 8-byte piece of the values
-            n += rep + 1 < REP ? jb.rep_n : jb.next_n;
-            kb += rep + 1 < REP ? jb.rep_kb : jb.next_kb;
-            if (kb >= KB) { kb -= KB; ++n; }
-            left -= static_cast<int>((rep + 1 < REP ? 1u : (kQmpTeams * REP - REP + 1u)) * kQmpStepUnits);
-            q = tiled_row(n, kb);
-            if (prev_lane != nullptr && left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
+            const uint32_t v8 = q_cur * 8u + 2u * (chunk ^ ((at.n >> 1) & 3u)) + (l8 & 1u);       // 8-byte piece of the values
+            at.advance(jb, KB, rep + 1 < REP);
+            q = tiled_row(at.n, at.kb);
+            if (prev_lane != nullptr && at.left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
             float k[8];
             uint32_t nibbles = 0u;
             double sum = 0.0;
@@ -525,6 +538,125 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     }
     g0 = g_end;
     flips *= 2u;
+    return acc;
+}
+
+// Pass 1 for the 6:8 pattern.  As above; a lane's 16 weights are two groups of 8, which leave as 12 value bytes (three 4-byte
+// stores) and 24 bits of metadata (a quad of lanes has 12 bytes, its lanes 0..2 store 4 each).  The two groups are read in the
+// order that halves the bank conflicts of the 64 B (fp32; none for bf16) per lane and put in place on the results.
+template <bool BF16>
+__device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
+                                                     uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok,
+                                                     const uint2* table) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp = threadIdx.x >> 5;
+    const uint32_t l8 = lane & 7, quad = l8 & 3u;
+    using Walk = QmpWalk<BF16>;
+    constexpr uint32_t kUnitBytes = Walk::kUnitBytes, REP = Walk::REP;
+    const uint32_t KB = jb.KB, KBp = KB + (KB >> 1);                  // K' / 128
+    const float thr_pred = __uint_as_float(__float_as_uint(jb.hi) - 1u);
+    const uint32_t width = __float_as_uint(thr_pred - jb.lo);
+    const uint32_t g_end = g0 + (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
+    double acc = 0.0;
+    const uint32_t in_step = 4u * (warp % kQmpTeamWarps) + (lane >> 3);
+    Walk at(jb, next_stage - g0, in_step);
+    const uint32_t swap = BF16 ? (l8 >> 2) : ((l8 >> 1) & 1u);        // the second group is read first
+    const uint32_t src0 = ring_base + in_step * kUnitBytes + l8 * (kUnitBytes / 8u);
+    const uint32_t src[2] = {src0 + swap * (kUnitBytes / 16u), src0 + (swap ^ 1u) * (kUnitBytes / 16u)};
+    // this lane's word of its quad's metadata
+    auto meta_at = [&](uint32_t n, uint32_t kb) { return meta68_offset(n, 24u * kb + 12u * (l8 >> 2) + 4u * quad, KBp); };
+    const bool has_prev = jb.prev != nullptr;
+    size_t m_off = quad < 3u ? meta_at(at.n, at.kb) : 0u;
+    uint32_t prev = 0u;
+    if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + m_off);
+    for (; next_stage < g_end; next_stage += kQmpTeams) {
+        const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
+        if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
+#pragma unroll 1
+        for (uint32_t rep = 0; rep < REP; ++rep) {
+            const uint32_t off = stage * kQmpStageBytes + rep * (kQmpStepUnits * kUnitBytes);
+            float4 raw[2][BF16 ? 1 : 2];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                raw[g][0] = qmp_lds128(src[g] + off);
+                if constexpr (!BF16) raw[g][1] = qmp_lds128(src[g] + off + 16u);
+            }
+            if (rep + 1 == REP) {
+                __syncwarp();
+                if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);
+            }
+            const bool mine = at.left > 0;
+            const size_t m_cur = m_off;
+            const uint32_t prev_cur = prev;
+            uint32_t v_word[3];                                       // 4-byte words of vals
+#pragma unroll
+            for (uint32_t i = 0; i < 3; ++i) v_word[i] = static_cast<uint32_t>(vals68_offset(at.n, 96u * at.kb + 12u * l8 + 4u * i, KBp) >> 2);
+            at.advance(jb, KB, rep + 1 < REP);
+            m_off = quad < 3u ? meta_at(at.n, at.kb) : 0u;
+            if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + m_off);
+            uint32_t v4[2], v2[2], m12[2], S[2];
+            double sum = 0.0;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                float w[8], a[8];
+                if constexpr (BF16) {
+                    const float4 r = raw[g][0];
+                    const uint32_t r4[4] = {__float_as_uint(r.x), __float_as_uint(r.y), __float_as_uint(r.z), __float_as_uint(r.w)};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { w[2 * i] = bf16lo_to_f32(r4[i]); w[2 * i + 1] = bf16hi_to_f32(r4[i]); }
+                } else {
+                    w[0] = raw[g][0].x; w[1] = raw[g][0].y; w[2] = raw[g][0].z; w[3] = raw[g][0].w;
+                    w[4] = raw[g][1].x; w[5] = raw[g][1].y; w[6] = raw[g][1].z; w[7] = raw[g][1].w;
+                }
+                sum += abs_sum4(make_float4(w[0], w[1], w[2], w[3])) + abs_sum4(make_float4(w[4], w[5], w[6], w[7]));
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = fabsf(w[i]);
+                S[g] = select6of8(a);
+                const uint2 entry = table[S[g]];
+                uint32_t e[8], b03, b47;
+                ternary68(w, thr_pred, e, b03, b47);
+                v4[g] = prmt(b03, b47, entry.x & 0xFFFFu);
+                v2[g] = prmt(b03, b47, entry.x >> 16) & 0xFFFFu;
+                m12[g] = entry.y;
+                uint32_t und = 0u;
+                if (mine && min(min(min(e[0], e[1]), min(e[2], e[3])), min(min(e[4], e[5]), min(e[6], e[7]))) <= width) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
+                    und &= S[g];
+                }
+                qmp_list_append(list, und,
+                                [&](int j) {
+                                    uint32_t at_byte = 6u * (static_cast<uint32_t>(g) ^ swap);      // of the lane's 12
+                                    uint32_t sel = entry.x;
+                                    for (int i = 0; i < 5 && (sel & 15u) != static_cast<uint32_t>(j); ++i, sel >>= 4) ++at_byte;
+                                    const uint32_t word = at_byte >> 2;
+                                    return (word == 0u ? v_word[0] : (word == 1u ? v_word[1] : v_word[2])) * 4u + (at_byte & 3u);
+                                },
+                                [&](int j) {
+                                    const float x = j & 1 ? w[1] : w[0], y = j & 1 ? w[3] : w[2], z = j & 1 ? w[5] : w[4], u = j & 1 ? w[7] : w[6];
+                                    return j & 4 ? (j & 2 ? u : z) : (j & 2 ? y : x);
+                                });
+            }
+            const uint32_t f4 = swap ? v4[1] : v4[0], f2 = swap ? v2[1] : v2[0], l4 = swap ? v4[0] : v4[1], l2 = swap ? v2[0] : v2[1];
+            const uint32_t m24 = swap ? (m12[1] | (m12[0] << 12)) : (m12[0] | (m12[1] << 12));
+            const uint32_t nxt = __shfl_down_sync(0xFFFFFFFFu, m24, 1);
+            if (has_prev) {
+                // this lane's 24 bits of the previous metadata, from its own and the lane before's word
+                const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, prev_cur, 1);
+                const uint32_t p24 = (quad == 0u ? prev_cur : ((before >> (32u - 8u * quad)) | (prev_cur << (8u * quad)))) & 0xFFFFFFu;
+                if (mine && p24 != m24)
+                    flips += __popc((swap ? S[1] : S[0]) ^ mask8_from_meta12(p24)) + __popc((swap ? S[0] : S[1]) ^ mask8_from_meta12(p24 >> 12));
+            }
+            if (mine) {
+                acc += sum;
+                if (quad < 3u) *reinterpret_cast<uint32_t*>(jb.meta + m_cur) = (m24 >> (8u * quad)) | (nxt << (24u - 8u * quad));
+                reinterpret_cast<uint32_t*>(jb.vals)[v_word[0]] = f4;
+                reinterpret_cast<uint32_t*>(jb.vals)[v_word[1]] = f2 | (l4 << 16);
+                reinterpret_cast<uint32_t*>(jb.vals)[v_word[2]] = (l4 >> 16) | (l2 << 16);
+            }
+        }
+    }
+    g0 = g_end;
     return acc;
 }
 
@@ -589,14 +721,30 @@ __device__ __forceinline__ float qmp_threshold_warp(float scale, int lane) {
 }
 
 // Do the listed values suffice, or must the whole range be ternarised again with the exact threshold?
+template <int PATTERN>
 __device__ __forceinline__ bool qmp_bracket_holds(const QmpDesc& d, float thr, const QmpJob& jb, unsigned int longest_list, uint32_t list_cap) {
     return jb.lo <= thr && thr <= jb.hi && longest_list <= list_cap && d.dense_q == nullptr &&
-           d.num_units <= (1u << 26);                        // listed byte offsets are 32-bit
+           d.num_units <= (PATTERN == 68 ? 1u << 25 : 1u << 26);     // listed byte offsets are 32-bit
 }
 __device__ __forceinline__ void qmp_fix_entry(uint8_t* vals, const QmpEntry e, float thr) {
     vals[e.byte_off] = static_cast<uint8_t>(fabsf(e.w) >= thr ? (e.w < 0.0f ? 0xFFu : 0x01u) : 0u);
 }
 
+// Ternarises this CTA's range of matrix d again with the exact threshold.
+template <int PATTERN>
+__device__ __forceinline__ void qmp_second_pass(const QmpDesc& d, float thr, const uint2* table) {
+    const QmpRange rg = qmp_range(d);
+    if constexpr (PATTERN == 68) {
+        if (d.w_bf16) qmp68_pass2_full<true>(d, rg, thr, table);
+        else qmp68_pass2_full<false>(d, rg, thr, table);
+    } else {
+        if (d.w_bf16) qmp_pass2_full<true>(d, rg, thr);
+        else qmp_pass2_full<false>(d, rg, thr);
+    }
+}
+
+// PATTERN: 24 (2:4) or 68 (6:8).
+template <int PATTERN>
 __global__ void __launch_bounds__(kQmpThreads, 1)
 quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, const QmpDesc* __restrict__ rest, int count,
                                  QmpSlot* slots, unsigned long long* generation, unsigned long long call_nonce,
@@ -606,6 +754,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     const uint32_t list_cap = qmp_list_cap(count);
     auto list_of = [&](int slot, int w) { return s_list + static_cast<uint32_t>(slot * kQmpStreamWarps + w) * list_cap; };
     __shared__ QmpStreamShared sh;
+    __shared__ uint2 s_table[PATTERN == 68 ? 256 : 1];        // by kept set (6:8)
 
     const QmpBatch batch{inl, rest};
     const QmpDesc& first = inl.d[0];
@@ -631,6 +780,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     }
     if (threadIdx.x == 32) qmp_make_job(first, sh.job[0]);
     for (int i = threadIdx.x; i < count; i += kQmpThreads) sh.thr_second_pass[i] = -1.0f;
+    if (PATTERN == 68 && threadIdx.x < 256) s_table[threadIdx.x] = table68_entry(threadIdx.x);
     __syncthreads();
     // No early signal to the next kernel of the stream: this kernel writes packed weights, and the
     // GEMM kernels fetch weights before their own dependency wait (see sbn_common.cuh).
@@ -681,8 +831,13 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
             unsigned int flips = 0;
             bool ok = true;
             QmpWarpList list{list_of(slot, warp), list_cap, 0u};
-            double mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok)
-                                  : qmp_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok);
+            double mine;
+            if constexpr (PATTERN == 68)
+                mine = jb.bf16 ? qmp68_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table)
+                               : qmp68_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table);
+            else
+                mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok)
+                               : qmp_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok);
             if (!ok) break;
             mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 16);
             mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 8);
@@ -764,7 +919,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
                 const float thr = qmp_threshold_warp(scale, lane);
                 const unsigned int mine = lane < kQmpStreamWarps ? sh.warp_listed[pslot][lane] : 0u;     // of warp `lane`'s list
                 const unsigned int longest = __reduce_max_sync(0xFFFFFFFFu, mine);
-                const bool holds = qmp_bracket_holds(dp, thr, sh.job[(m - 1) & (kQmpJobs - 1)], longest, list_cap);
+                const bool holds = qmp_bracket_holds<PATTERN>(dp, thr, sh.job[(m - 1) & (kQmpJobs - 1)], longest, list_cap);
                 uint8_t* const vb = reinterpret_cast<uint8_t*>(dp.vals);
                 if (m == count) {
                     if (lane == 0) { sh.thr_tail = thr; sh.tail_second_pass = holds ? 0 : 1; }
@@ -835,24 +990,21 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
             }
         } else {
             const QmpDesc d = qmp_desc_of(batch, m);
-            const QmpRange rg = qmp_range(d);
-            if (d.w_bf16) qmp_pass2_full<true>(d, rg, thr);
-            else qmp_pass2_full<false>(d, rg, thr);
+            qmp_second_pass<PATTERN>(d, thr, s_table);
         }
     }
     for (int m = 0; m + 1 < count; ++m) {
         const float thr = sh.thr_second_pass[m];
         if (thr >= 0.0f) {
             const QmpDesc d = qmp_desc_of(batch, m);
-            const QmpRange rg = qmp_range(d);
-            if (d.w_bf16) qmp_pass2_full<true>(d, rg, thr);
-            else qmp_pass2_full<false>(d, rg, thr);
+            qmp_second_pass<PATTERN>(d, thr, s_table);
         }
     }
 }
 
 // Launch for `count` (<= kQmpMaxBatch) matrices: the first kQmpInlineDescs of `descs_host` by value, matrices
 // 1, 2, ... already copied to `rest_dev` if there are more than that.
+template <int PATTERN>
 inline sbn_status launch_quantize_mask_pack_stream(const QmpDesc* descs_host, const QmpDesc* rest_dev, int count,
                                                    uint32_t max_units, QmpSlot* slots, unsigned long long* generation,
                                                    cudaStream_t stream, QmpMemo* memo = nullptr) {
@@ -864,23 +1016,24 @@ inline sbn_status launch_quantize_mask_pack_stream(const QmpDesc* descs_host, co
     // device has SMs, and never more than the workspace has slots
     const unsigned cap = static_cast<unsigned>(std::min(device_sm_count(), kQmpMaxCtas));
     const unsigned grid = max_units < cap ? max_units : cap;
-    if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
+    if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel<PATTERN>>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
     // At most one CTA per SM (1024 threads x 64 registers each) and never more CTAs than SMs, so all
     // of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
     // another kernel kept SMs busy for seconds, the bounded wait reports SBN_ERR_TIMEOUT instead.
-    const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
+    const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel<PATTERN>, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
                                           inl, rest_dev, count, slots, generation, nonce, test_withhold_slot, count == 1 ? memo : nullptr);
     ++g_launch_count;
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
 
+template <int PATTERN>
 inline sbn_status launch_quantize_mask_pack(const void* W, bool w_bf16, int N, int K, int8_t* vals,
                                             uint8_t* meta, float* w_scale, int8_t* dense_q,
                                             const uint8_t* prev_meta,
                                             unsigned long long* flip_bits, QmpWorkspace* ws,
                                             cudaStream_t stream) {
     const QmpDesc d = qmp_make_desc(W, w_bf16, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits);
-    return launch_quantize_mask_pack_stream(&d, nullptr, 1, d.num_units, ws->slot, &ws->generation, stream, &ws->memo);
+    return launch_quantize_mask_pack_stream<PATTERN>(&d, nullptr, 1, d.num_units, ws->slot, &ws->generation, stream, &ws->memo);
 }
 
 }  // namespace sbn
