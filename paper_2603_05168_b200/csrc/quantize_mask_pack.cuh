@@ -123,6 +123,16 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
+// Three-input minima (one instruction each on this architecture).
+__device__ __forceinline__ float fmin3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ uint32_t umin8(const uint32_t (&e)[8]) {
+    return __vimin3_u32(__vimin3_u32(e[0], e[1], e[2]), __vimin3_u32(e[3], e[4], e[5]), min(e[6], e[7]));
+}
+
 // Eq. 1 for four elements as four bytes (+1 -> 0x01, -1 -> 0xFF, 0 -> 0x00; thr: see the header),
 // lowest byte = first argument.  The sign bytes come from byte permutes in sign-replication mode.
 __device__ __forceinline__ uint32_t ternary_bytes4(float w0, float w1, float w2, float w3, float thr) {

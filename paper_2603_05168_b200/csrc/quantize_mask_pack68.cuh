@@ -28,9 +28,9 @@ __device__ __forceinline__ uint32_t select6of8(const float (&a)[8]) {
     float lo[4], hi[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) { lo[i] = fminf(a[2 * i], a[2 * i + 1]); hi[i] = fmaxf(a[2 * i], a[2 * i + 1]); }
-    const float l0 = fminf(lo[0], lo[1]), s0 = fminf(fmaxf(lo[0], lo[1]), fminf(hi[0], hi[1]));
-    const float l1 = fminf(lo[2], lo[3]), s1 = fminf(fmaxf(lo[2], lo[3]), fminf(hi[2], hi[3]));
-    const float t2 = fminf(fmaxf(l0, l1), fminf(s0, s1));
+    const float l0 = fminf(lo[0], lo[1]), s0 = fmin3(fmaxf(lo[0], lo[1]), hi[0], hi[1]);
+    const float l1 = fminf(lo[2], lo[3]), s1 = fmin3(fmaxf(lo[2], lo[3]), hi[2], hi[3]);
+    const float t2 = fmin3(fmaxf(l0, l1), s0, s1);
     uint32_t d[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) d[i] = __float_as_uint(t2 - a[i]);            // sign bit set: larger
@@ -66,7 +66,8 @@ __device__ __forceinline__ uint32_t mask4_to_nibble(uint32_t m) {
     return (((m & 8u) ? kHi : kLo) >> (4u * (m & 7u))) & 15u;
 }
 // Table entry of the kept set S: x = columns of the six kept values, a nibble each, window by window (a byte-permute
-// selector for the group's eight value bytes); y = the three windows' metadata nibbles.
+// selector for the group's eight value bytes); y = the three windows' metadata nibbles.  Window by window the columns
+// ascend (window 0 takes the lowest kept ones, window 2 the highest), so column j is kept value popc(S & (2^j - 1)).
 __device__ __forceinline__ uint2 table68_entry(uint32_t S) {
     if (__popc(S) != 6) return make_uint2(0u, 0u);
     uint32_t m[3];

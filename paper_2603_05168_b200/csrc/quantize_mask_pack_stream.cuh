@@ -524,7 +524,7 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
                 *reinterpret_cast<uint16_t*>(meta_lane + static_cast<size_t>(q_cur) * 16u) = static_cast<uint16_t>(word);
                 *reinterpret_cast<uint2*>(jb.vals + static_cast<size_t>(v8) * 8u) = make_uint2(prmt(t[0], t[1], sel_lo), prmt(t[0], t[1], sel_hi));
                 if (prev_lane != nullptr) flips += qmp_flip_pairs(word ^ prev_cur);
-                if (min(min(min(e[0], e[1]), min(e[2], e[3])), min(min(e[4], e[5]), min(e[6], e[7]))) <= width) {
+                if (umin8(e) <= width) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
                 }
@@ -563,12 +563,26 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
     const uint32_t swap = BF16 ? (l8 >> 2) : ((l8 >> 1) & 1u);        // the second group is read first
     const uint32_t src0 = ring_base + in_step * kUnitBytes + l8 * (kUnitBytes / 8u);
     const uint32_t src[2] = {src0 + swap * (kUnitBytes / 16u), src0 + (swap ^ 1u) * (kUnitBytes / 16u)};
-    // this lane's word of its quad's metadata
-    auto meta_at = [&](uint32_t n, uint32_t kb) { return meta68_offset(n, 24u * kb + 12u * (l8 >> 2) + 4u * quad, KBp); };
+    // Column block kb of a row starts at byte 96 kb of its values and 24 kb of its metadata in the [N][K'] form: in tile 3 kb / 2,
+    // for odd kb half a tile in.  With q = the row's index in that tile, a lane's three words of values are at
+    // 64 q + (v ^ the row's swizzle) and its word of its quad's metadata at 16 q + m, v and m constants for even
+    // (low half) and odd (high half) kb.
+    auto tiled_row = [&](uint32_t nn, uint32_t kk) { return (((nn >> 7) * KBp + ((3u * kk) >> 1)) << 7) + (nn & 127u); };
+    uint32_t v_const[3], m_const = 0u;
+#pragma unroll
+    for (uint32_t odd = 0; odd < 2; ++odd) {
+#pragma unroll
+        for (uint32_t i = 0; i < 3; ++i) {
+            const uint32_t y = 12u * l8 + 4u * i + 32u * odd;
+            v_const[i] = (odd ? v_const[i] : 0u) | (((y >> 6) * 8192u + (y & 63u)) << (16u * odd));
+        }
+        const uint32_t y = 12u * (l8 >> 2) + 4u * quad + 8u * odd;
+        m_const |= ((y >> 4) * 2048u + (y & 15u)) << (16u * odd);
+    }
     const bool has_prev = jb.prev != nullptr;
-    size_t m_off = quad < 3u ? meta_at(at.n, at.kb) : 0u;
-    uint32_t prev = 0u;
-    if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + m_off);
+    uint32_t q = tiled_row(at.n, at.kb), prev = 0u;
+    auto meta_at = [&](uint32_t qq, uint32_t kk) { return static_cast<size_t>(qq) * 16u + ((kk & 1u) ? m_const >> 16 : m_const & 0xFFFFu); };
+    if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + meta_at(q, at.kb));
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
@@ -586,14 +600,12 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
                 if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);
             }
             const bool mine = at.left > 0;
-            const size_t m_cur = m_off;
-            const uint32_t prev_cur = prev;
-            uint32_t v_word[3];                                       // 4-byte words of vals
-#pragma unroll
-            for (uint32_t i = 0; i < 3; ++i) v_word[i] = static_cast<uint32_t>(vals68_offset(at.n, 96u * at.kb + 12u * l8 + 4u * i, KBp) >> 2);
+            const uint32_t q_cur = q, odd_cur = at.kb & 1u, prev_cur = prev;
+            const uint32_t half = odd_cur ? 0x4432u : 0x4410u, swizzle = ((at.n >> 1) & 3u) << 4;
             at.advance(jb, KB, rep + 1 < REP);
-            m_off = quad < 3u ? meta_at(at.n, at.kb) : 0u;
-            if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + m_off);
+            q = tiled_row(at.n, at.kb);
+            if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + meta_at(q, at.kb));
+            auto v_off = [&](uint32_t v) { return prmt(v, 0u, half) ^ swizzle; };           // on top of 64 q_cur
             uint32_t v4[2], v2[2], m12[2], S[2];
             double sum = 0.0;
 #pragma unroll
@@ -615,22 +627,19 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
                 const uint2 entry = table[S[g]];
                 uint32_t e[8], b03, b47;
                 ternary68(w, thr_pred, e, b03, b47);
-                v4[g] = prmt(b03, b47, entry.x & 0xFFFFu);
+                v4[g] = prmt(b03, b47, entry.x);
                 v2[g] = prmt(b03, b47, entry.x >> 16) & 0xFFFFu;
                 m12[g] = entry.y;
                 uint32_t und = 0u;
-                if (mine && min(min(min(e[0], e[1]), min(e[2], e[3])), min(min(e[4], e[5]), min(e[6], e[7]))) <= width) {
+                if (mine && umin8(e) <= width) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
                     und &= S[g];
                 }
                 qmp_list_append(list, und,
                                 [&](int j) {
-                                    uint32_t at_byte = 6u * (static_cast<uint32_t>(g) ^ swap);      // of the lane's 12
-                                    uint32_t sel = entry.x;
-                                    for (int i = 0; i < 5 && (sel & 15u) != static_cast<uint32_t>(j); ++i, sel >>= 4) ++at_byte;
-                                    const uint32_t word = at_byte >> 2;
-                                    return (word == 0u ? v_word[0] : (word == 1u ? v_word[1] : v_word[2])) * 4u + (at_byte & 3u);
+                                    const uint32_t at_byte = 6u * (static_cast<uint32_t>(g) ^ swap) + __popc(S[g] & ((1u << j) - 1u));   // of the lane's 12
+                                    return q_cur * 64u + v_off(at_byte < 4u ? v_const[0] : (at_byte < 8u ? v_const[1] : v_const[2])) + (at_byte & 3u);
                                 },
                                 [&](int j) {
                                     const float x = j & 1 ? w[1] : w[0], y = j & 1 ? w[3] : w[2], z = j & 1 ? w[5] : w[4], u = j & 1 ? w[7] : w[6];
@@ -649,10 +658,11 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
             }
             if (mine) {
                 acc += sum;
-                if (quad < 3u) *reinterpret_cast<uint32_t*>(jb.meta + m_cur) = (m24 >> (8u * quad)) | (nxt << (24u - 8u * quad));
-                reinterpret_cast<uint32_t*>(jb.vals)[v_word[0]] = f4;
-                reinterpret_cast<uint32_t*>(jb.vals)[v_word[1]] = f2 | (l4 << 16);
-                reinterpret_cast<uint32_t*>(jb.vals)[v_word[2]] = (l4 >> 16) | (l2 << 16);
+                if (quad < 3u) *reinterpret_cast<uint32_t*>(jb.meta + meta_at(q_cur, odd_cur)) = (m24 >> (8u * quad)) | (nxt << (24u - 8u * quad));
+                unsigned char* const row = jb.vals + static_cast<size_t>(q_cur) * 64u;
+                *reinterpret_cast<uint32_t*>(row + v_off(v_const[0])) = f4;
+                *reinterpret_cast<uint32_t*>(row + v_off(v_const[1])) = f2 | (l4 << 16);
+                *reinterpret_cast<uint32_t*>(row + v_off(v_const[2])) = (l4 >> 16) | (l2 << 16);
             }
         }
     }
