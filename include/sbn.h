@@ -308,10 +308,10 @@ sbn_status sbn_sparse_bitlinear(const int8_t *xq, const float *a_scale, int T,
  * Parts 2 and 3 in one kernel, for few tokens -- Algorithm 2's forward as it stands: the per-token
  * absmax quantiser (Sec. 2.1) and Eq. 4.  Results are those of sbn_quant_act followed by
  * sbn_sparse_bitlinear (resp. sbn_bitlinear), bit for bit; what is saved is a kernel launch.  That
- * pays when launches are plainly serialised (measured 9.8 us against 12.8 us per layer at T = 8);
- * in a stream of this library's own calls, which overlap through programmatic dependent launch,
- * the two separate calls are faster (6.4 us against 7.6 us).  The quantised activations never reach
- * memory.
+ * pays most when launches are plainly serialised; in a stream of this library's own calls, which
+ * overlap through programmatic dependent launch, the two are about equal up to K = 2560 (3.7 us each
+ * at T = 1, 2560 x 2560) and the two separate calls are faster beyond (6912 -> 2560: 5.7 us against
+ * 6.8).  The quantised activations never reach memory.
  *   x_bf16        device, bf16 [T][K], 16-byte aligned, K % 128 == 0
  *   a_scale_out   device out or NULL, fp32 [T]: the per-token scales d / 127
  *   the other arguments as for sbn_sparse_bitlinear / sbn_bitlinear; no workspace
@@ -455,7 +455,9 @@ sbn_status sbn_set_wait_test(int break_waits, unsigned long long wait_limit_us);
  * Used by `bench.py --workload mmaprobe`. */
 void sbn_set_gemm_probe(int flags);
 
-/* Diagnostic: what the dispatcher would run for this shape (host only, launches nothing).
+/* Diagnostic: which tcgen05 kernel the dispatcher picks for this shape (host only, launches nothing).  It runs
+ * with more than 16 tokens, or whenever sbn_set_gemm_tuning or sbn_set_wait_test is in force; otherwise calls of up to 8
+ * tokens, and some sparse ones of up to 16, run the register-fed few-token kernel instead.
  * out4[0] = kernel (0 single-CTA tiles, 1 cluster split-K, 2 CTA pair with 512-feature tiles, 3 CTA
  * pair with 256-feature tiles and double-buffered accumulators), out4[1] = tokens per tile,
  * out4[2] = split-K factor through global memory (1 = none), out4[3] = cluster size (0 = none).

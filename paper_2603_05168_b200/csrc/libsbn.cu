@@ -21,6 +21,7 @@
 #include "gemm_splitk_cluster_tcgen05.cuh"
 #include "gemm_packed_cluster_tcgen05.cuh"
 #include "gemm_fused_act_cluster_tcgen05.cuh"
+#include "gemm_few_tokens_mma.cuh"
 #include "backward_prep.cuh"
 #include "gemm_bf16_pair_tcgen05.cuh"
 
@@ -383,6 +384,27 @@ static sbn_status launch_splitk_cluster(const CUtensorMap& ta, const CUtensorMap
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
 
+// ---- few tokens: register-fed kernel ----------------------------------------------------------------
+static FewParams few_params(int T, int N, int K, const void* xq, const void* x_bf16, const float* a_scale, float* a_scale_out, const void* vals,
+                            const uint8_t* meta, const float* w_scale, const float* bias, void* y, sbn_out_dtype dt, int32_t* acc_out) {
+    FewParams p;
+    p.T = T; p.N = N; p.k_blocks = K / kBK;
+    p.tb8 = static_cast<int>(xq_tb8(T));
+    p.xq = static_cast<const uint8_t*>(xq);
+    p.x_bf16 = static_cast<const uint4*>(x_bf16);
+    p.a_scale = a_scale; p.a_scale_out = a_scale_out;
+    p.vals = static_cast<const uint8_t*>(vals); p.meta = meta;
+    p.w_scale = w_scale; p.bias = bias;
+    p.y = y; p.out_bf16 = (dt == SBN_OUT_BF16);
+    p.acc_out = acc_out;
+    return p;
+}
+template <int WT, bool FUSED>
+static bool use_few_kernel(int T, int N, int K) {
+    if (g_force_token_tile != 0 || g_force_split_k != 0 || g_test_break_waits) return false;   // diagnostics: the tcgen05 kernels as told
+    return few_takes<WT, FUSED>(T, N, K);
+}
+
 static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, int T,
                            const int8_t* wvals, const uint8_t* meta, const float* w_scale,
                            int N, int K, const float* bias, void* y, sbn_out_dtype dt,
@@ -395,6 +417,10 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
         (acc_out && misaligned(acc_out, 4)) || (bias && misaligned(bias, 4)))
         return SBN_ERR_ALIGN;
 
+    if (sparse ? use_few_kernel<kFewSparse, false>(T, N, K) : use_few_kernel<kFewDense, false>(T, N, K)) {
+        const FewParams p = few_params(T, N, K, xq, nullptr, a_scale, nullptr, wvals, meta, w_scale, bias, y, dt, acc_out);
+        return sparse ? launch_few<kFewSparse, false>(p, stream) : launch_few<kFewDense, false>(p, stream);
+    }
     const GemmPlan plan = plan_gemm(sparse, T, N, K);
     if (plan.pair)
         return run_gemm_pair(sparse, xq, a_scale, T, wvals, meta, w_scale, N, K, bias, y, dt, acc_out, plan.bn, plan.mt, stream);
@@ -819,6 +845,10 @@ static sbn_status run_fused_act(bool sparse, const void* x_bf16, int T, const in
         misaligned(w_scale, 4) || (acc_out && misaligned(acc_out, 4)) || (bias && misaligned(bias, 4)) ||
         (a_scale_out && misaligned(a_scale_out, 4)))
         return SBN_ERR_ALIGN;
+    if (sparse ? use_few_kernel<kFewSparse, true>(T, N, K) : use_few_kernel<kFewDense, true>(T, N, K)) {
+        const FewParams p = few_params(T, N, K, nullptr, x_bf16, nullptr, a_scale_out, wvals, meta, w_scale, bias, y, dt, acc_out);
+        return sparse ? launch_few<kFewSparse, true>(p, stream) : launch_few<kFewDense, true>(p, stream);
+    }
     CUtensorMap ta, te;
     bool ok;
     const uint64_t NK = static_cast<uint64_t>(N) * K;
@@ -891,6 +921,10 @@ sbn_status sbn_sparse_bitlinear_packed(const int8_t* xq, const float* a_scale, i
     if (misaligned(xq, 16) || misaligned(vals2, 16) || misaligned(meta, 16) || misaligned(y, 16) || misaligned(a_scale, 4) ||
         misaligned(w_scale, 4) || (acc_out && misaligned(acc_out, 4)) || (bias && misaligned(bias, 4)))
         return SBN_ERR_ALIGN;
+    if (use_few_kernel<kFewPacked, false>(T, N, K)) {
+        const FewParams p = few_params(T, N, K, xq, nullptr, a_scale, nullptr, vals2, meta, w_scale, bias, y, dt, acc_out);
+        return launch_few<kFewPacked, false>(p, static_cast<cudaStream_t>(stream));
+    }
     using Cfg = PackedSplitConfig;
     CUtensorMap tb;
     if (!encode_flat_1k(&tb, xq, xq_tiled_bytes(T, K), Cfg::BN / 8)) return SBN_ERR_CUDA;

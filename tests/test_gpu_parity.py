@@ -1211,3 +1211,44 @@ def test_quantize_mask_pack_scale_left_in_the_workspace_never_changes_the_result
     run_and_check(other, refs["b"])                 # another buffer: the tag does not match
     buf.copy_(torch.from_numpy(Wa).cuda())
     run_and_check(buf, refs["a"])
+
+
+# ---- the register-fed few-token kernel -----------------------------------------------------------------------------
+@pytest.mark.parametrize("T,N,K", [(1, 128, 128), (8, 128, 256), (3, 256, 1152), (5, 4864, 384), (1, 4864, 3328), (9, 640, 1408),
+                                   (16, 2560, 256), (16, 128, 128)])
+def test_few_token_kernel_all_forms(T, N, K):
+    # one token and the last of each group of 8; fewer 128-column blocks than warps, a last round that leaves warps without
+    # a block; more row groups than CTAs (4864 / 16 = 304 on 148 SMs) and fewer.  Accumulators exact, outputs as everywhere.
+    W = inputs.latent_weights(N, K, seed=200 + T)
+    bits = inputs.activations_bf16(T, K, seed=300 + K, token_lognormal_sigma=0.5)
+    bias = np.random.default_rng(N).standard_normal(N).astype(np.float32)
+    r = _oracle_pack(W)
+    xq_ref, s_ref = oracle.quant_act(bits)
+    g = gpu_quantize_mask_pack(W)
+    p = g["dev"]
+    vals2, _ = gpu_pack_vals2(p)
+    xq, a_scale = gpu_quant_act(bits)
+    x, bias_d = bf16_dev(bits), torch.from_numpy(bias).cuda()
+    sparse_ref = oracle.sparse_bitlinear(xq_ref, s_ref, r["vals"], r["meta"], r["scale"], bias)
+    dense_ref = oracle.bitlinear(xq_ref, s_ref, r["dense_q"], r["scale"], bias)
+    calls = [
+        (lambda y, acc: b.sbn_sparse_bitlinear(xq, a_scale, p["vals"], p["meta"], p["w_scale"], y, bias=bias_d, acc_out=acc), sparse_ref),
+        (lambda y, acc: b.sbn_bitlinear(xq, a_scale, p["dense_q"], p["w_scale"], y, bias=bias_d, acc_out=acc), dense_ref),
+    ]
+    if K >= 256:
+        calls += [
+            (lambda y, acc: b.sbn_sparse_bitlinear_packed(xq, a_scale, vals2, p["meta"], p["w_scale"], y, bias=bias_d, acc_out=acc), sparse_ref),
+            (lambda y, acc: b.sbn_quant_act_sparse_bitlinear(x, p["vals"], p["meta"], p["w_scale"], y, bias=bias_d, acc_out=acc), sparse_ref),
+            (lambda y, acc: b.sbn_quant_act_bitlinear(x, p["dense_q"], p["w_scale"], y, bias=bias_d, acc_out=acc), dense_ref),
+        ]
+    for call, (y_ref, acc_ref) in calls:
+        y = torch.full((T, N), float("nan"), dtype=torch.float32, device="cuda")
+        acc = torch.full((T, N), -(2 ** 31), dtype=torch.int32, device="cuda")
+        call(y, acc)
+        b.sbn_check_status()
+        assert np.array_equal(acc.cpu().numpy(), acc_ref)
+        _assert_y(y.cpu().numpy(), y_ref)
+        yb = torch.full((T, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+        call(yb, None)
+        b.sbn_check_status()
+        assert torch.equal(yb, y.to(torch.bfloat16))                # bf16 = the fp32 value rounded to nearest even
