@@ -8,8 +8,15 @@
 // squares, maximum of |xn|, rounding -- and xn is recomputed (two multiplies) instead of stored.
 // HBM-bound like the plain quantiser: 2 B read + 1 B written per element; the normalised
 // activations never exist in memory.  Same persistent-CTA row pipeline and the same tiled xq
-// layout as quant_act.cuh.  The squares of bf16 values are exact in fp32 (16-bit significands); they
-// are added in fp64 in a fixed order (thread-local, then a butterfly, then the warps in order).
+// layout as quant_act.cuh.  The squares of bf16 values are added in fp64 in a fixed order (thread-local, then a
+// butterfly, then the warps in order).
+//
+// Measured in a chain of launches, with a gain (us; HBM time of the bytes in brackets): 1 x 2560 1.50, 16 x 4096 1.73,
+// 201 x 2560 2.0 -- two trips to memory, two barriers and the arithmetic between them; 4096 x 2560 11.8 [4.9],
+// 4096 x 6912 26.4 [13.2], 8192 x 4096 28.5 [15.6], 8192 x 11008 78 [42] -- bound by the instructions per element, of
+// which the plain quantiser (7.4, 16.3, 21.8, 49) needs fewer.  Squares through the conversion instruction, gains
+// fetched before the row, a division for the mean and a clamp: 2.21, 2.10, 3.14, 12.0, 28.2, 31.6 and 82.  One or two
+// warps per row without the prefetch of the next row were slower: 15.7, 31.7, 36.6, 90.
 #pragma once
 
 #include "quant_act.cuh"
@@ -31,18 +38,29 @@ __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
     return d;
 }
 
-__device__ __forceinline__ void bf16x8_to_f32(const uint4& v, float (&f)[8]) {
-    f[0] = bf16lo_to_f32(v.x); f[1] = bf16hi_to_f32(v.x);
-    f[2] = bf16lo_to_f32(v.y); f[3] = bf16hi_to_f32(v.y);
-    f[4] = bf16lo_to_f32(v.z); f[5] = bf16hi_to_f32(v.z);
-    f[6] = bf16lo_to_f32(v.w); f[7] = bf16hi_to_f32(v.w);
+// max(m, |a|, |b|) in one instruction
+__device__ __forceinline__ float max_abs3(float m, float a, float b) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(m), "f"(a), "f"(b));
+    return d;
+}
+// The low bytes of four words, lowest first.
+__device__ __forceinline__ uint32_t low_bytes4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+// |value| of a finite bf16 (its 15 bits) as a double: the exponent moves to the double's bias, the significand to the
+// top of the high word -- two integer instructions; the conversion instruction runs at an eighth of their rate.  Zero and
+// subnormals come out as up to 2^-126 instead; their squares (below 2^-251 each) vanish in the mean's cast to fp32
+// (smallest value 2^-149) either way.
+__device__ __forceinline__ double bf16_abs_to_f64(uint32_t abs15) {
+    return __hiloint2double(static_cast<int>((abs15 << 13) + 0x38000000u), 0);
 }
 
 // G threads per token row, VPT 16-byte vectors per thread (G * VPT >= K / 8).  The gains are copied
 // to shared memory once per CTA (rows differ, channels do not).
 template <int G, int VPT, bool EXPAND68 = false>
 __global__ void __launch_bounds__(kActThreads, (VPT <= 4) ? 3 : 2)
-norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __restrict__ gain, float eps,
+norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __restrict__ gain, float eps, double n, double inv_n,
                       uint2* __restrict__ xq, float* __restrict__ a_scale) {
     constexpr int ROWS = kActThreads / G;
     constexpr int WARPS_PER_ROW = (G + 31) / 32;
@@ -61,18 +79,29 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
     pdl_launch_dependents();             // the next kernel may become resident (and fetch weights) right away
     pdl_wait();
 
-    extern __shared__ float4 s_gain[];                           // [nvec * 2] when a gain is given
-    if (has_gain) {
-        for (int i = threadIdx.x; i < 2 * nvec; i += kActThreads) s_gain[i] = __ldg(gain + i);
-        __syncthreads();
-    }
-
+    // the first row is on its way before the gains are fetched (one after the other they were two trips to memory)
     uint4 cur[VPT], nxt[VPT];
     int row = blockIdx.x * ROWS + r;
 #pragma unroll
     for (int i = 0; i < VPT; ++i) {
         const int idx = g + i * G;
         cur[i] = (row < T && idx < nvec) ? __ldg(x + static_cast<size_t>(row) * nvec + idx) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    // The gains of a thread's columns: in registers up to two vectors, else in shared memory -- the first halves of all
+    // vectors, then the second ones (one after the other the lanes' reads had two-way bank conflicts).
+    constexpr bool GAIN_REGS = VPT <= 2;
+    extern __shared__ float4 s_gain[];                           // [2][nvec] when a gain is given
+    float4 gain_r[GAIN_REGS ? VPT : 1][2];
+    if constexpr (GAIN_REGS) {
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) {
+            const int idx = g + i * G;
+            gain_r[i][0] = gain_r[i][1] = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+            if (has_gain && idx < nvec) { gain_r[i][0] = __ldg(gain + 2 * idx); gain_r[i][1] = __ldg(gain + 2 * idx + 1); }
+        }
+    } else if (has_gain) {
+        for (int i = threadIdx.x; i < 2 * nvec; i += kActThreads) s_gain[(i & 1) * nvec + (i >> 1)] = __ldg(gain + i);
+        __syncthreads();
     }
     for (int it = 0; it < iters; ++it, row += row_stride) {
         const int row_n = row + row_stride;
@@ -85,12 +114,12 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
         double s4[4] = {0.0, 0.0, 0.0, 0.0};                      // four chains: the adds overlap
 #pragma unroll
         for (int i = 0; i < VPT; ++i) {
-            float f[8];
-            bf16x8_to_f32(cur[i], f);
+            const uint32_t w[4] = {cur[i].x, cur[i].y, cur[i].z, cur[i].w};
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {                                   // exact product, one rounding in the add
-                const double dv = static_cast<double>(f[j]);
-                s4[j & 3] = __fma_rn(dv, dv, s4[j & 3]);
+            for (int j = 0; j < 4; ++j) {                                   // exact product, one rounding in the add
+                const double lo = bf16_abs_to_f64(w[j] & 0x7FFFu), hi = bf16_abs_to_f64((w[j] >> 16) & 0x7FFFu);
+                s4[(2 * j) & 3] = __fma_rn(lo, lo, s4[(2 * j) & 3]);
+                s4[(2 * j + 1) & 3] = __fma_rn(hi, hi, s4[(2 * j + 1) & 3]);
             }
         }
         double ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
@@ -105,7 +134,10 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
             for (int w = 0; w < WARPS_PER_ROW; ++w) t += sm[w0 + w];
             ss = t;
         }
-        const float ms = static_cast<float>(ss / static_cast<double>(nvec * 8));
+        // ss / n, correctly rounded, from the rounded reciprocal: quotient, exact remainder, correction (Markstein's theorem
+        // for division with a correctly rounded reciprocal)
+        const double quot = ss * inv_n;
+        const float ms = static_cast<float>(__fma_rn(__fma_rn(-quot, n, ss), inv_n, quot));
         const float rinv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(ms, eps)));
         // ---- xn = (x * r) * g with packed fp32x2 multiplies, and max |xn|.  Up to four vectors per
         // thread the fp32 xn stays in registers for the rounding; longer rows recompute it.
@@ -113,13 +145,14 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
         const uint64_t r2 = pack_f32x2(rinv, rinv);
         uint64_t xn2[KEEP ? VPT : 1][4];
         float amax = 0.0f;
-        auto normalise = [&](const uint4& v, int idx, uint64_t (&out)[4]) {
+        auto normalise = [&](const uint4& v, int i, uint64_t (&out)[4]) {
+            const int idx = g + i * G;
             out[0] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.x), bf16hi_to_f32(v.x)), r2);
             out[1] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.y), bf16hi_to_f32(v.y)), r2);
             out[2] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.z), bf16hi_to_f32(v.z)), r2);
             out[3] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.w), bf16hi_to_f32(v.w)), r2);
             if (has_gain && idx < nvec) {
-                const float4 a = s_gain[2 * idx], b = s_gain[2 * idx + 1];
+                const float4 a = GAIN_REGS ? gain_r[GAIN_REGS ? i : 0][0] : s_gain[idx], b = GAIN_REGS ? gain_r[GAIN_REGS ? i : 0][1] : s_gain[nvec + idx];
                 out[0] = mul_f32x2(out[0], pack_f32x2(a.x, a.y));
                 out[1] = mul_f32x2(out[1], pack_f32x2(a.z, a.w));
                 out[2] = mul_f32x2(out[2], pack_f32x2(b.x, b.y));
@@ -130,12 +163,12 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
         for (int i = 0; i < VPT; ++i) {
             uint64_t tmp[4];
             uint64_t (&o)[4] = KEEP ? xn2[KEEP ? i : 0] : tmp;
-            normalise(cur[i], g + i * G, o);
+            normalise(cur[i], i, o);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 float lo, hi;
                 unpack_f32x2(o[j], lo, hi);
-                amax = fmaxf(amax, fmaxf(fabsf(lo), fabsf(hi)));
+                amax = max_abs3(amax, lo, hi);
             }
         }
         // bit patterns of non-negative floats order like integers: one redux instruction per warp
@@ -159,9 +192,9 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
                 const int idx = g + i * G;
                 if (idx < nvec) {
                     uint64_t tmp[4];
-                    if constexpr (!KEEP) normalise(cur[i], idx, tmp);
+                    if constexpr (!KEEP) normalise(cur[i], i, tmp);
                     const uint64_t (&o)[4] = KEEP ? xn2[KEEP ? i : 0] : tmp;
-                    int q[8];
+                    uint32_t q[8];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         // rint(xn * s_x) for two values: multiply, then add 1.5 * 2^23 -- the adder's round-to-nearest-even
@@ -170,12 +203,14 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
                         // rounding (a fused multiply-add), which breaks exact ties such as 63.5.
                         float lo, hi;
                         unpack_f32x2(mul_f32x2(o[j], s2), lo, hi);
-                        q[2 * j] = static_cast<int>(__float_as_uint(__fadd_rn(lo, 12582912.0f)) - 0x4B400000u);
-                        q[2 * j + 1] = static_cast<int>(__float_as_uint(__fadd_rn(hi, 12582912.0f)) - 0x4B400000u);
+                        q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
+                        q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
                     }
+                    // The method's clamp cannot act: |xn| <= d, so |xn * s_x| <= 127 (1 + 2^-23) and rounds to at most 127.  The
+                    // code is the low byte.
                     uint2 ov;                                      // lowest column in the lowest byte
-                    ov.x = pack_sat_s8x2(q[1], q[0], pack_sat_s8x2(q[3], q[2], 0u));
-                    ov.y = pack_sat_s8x2(q[5], q[4], pack_sat_s8x2(q[7], q[6], 0u));
+                    ov.x = low_bytes4(q[0], q[1], q[2], q[3]);
+                    ov.y = low_bytes4(q[4], q[5], q[6], q[7]);
                     store_codes8<EXPAND68>(xq, row, idx, tb8, ov);     // plain, or expanded for the 6:8 pattern
                 }
             }
@@ -192,9 +227,10 @@ static cudaError_t launch_norm_quant_act_cfg(const uint4* x, int T, int nvec, co
     const int ctas_per_sm = (VPT <= 4) ? 3 : 2;
     int grid = (T + rows - 1) / rows;
     if (grid > kNumSMs * ctas_per_sm) grid = kNumSMs * ctas_per_sm;
-    const size_t smem = gain ? static_cast<size_t>(nvec) * 32 : 0;          // K floats
+    const size_t smem = gain && VPT > 2 ? static_cast<size_t>(nvec) * 32 : 0;   // K floats
     if (!ensure_dynamic_smem<norm_quant_act_kernel<G, VPT, EXPAND68>>(65536)) return cudaErrorUnknown;
-    return launch_kernel(norm_quant_act_kernel<G, VPT, EXPAND68>, dim3(grid), dim3(kActThreads), smem, stream, x, T, nvec, gain, eps, q, a_scale);
+    return launch_kernel(norm_quant_act_kernel<G, VPT, EXPAND68>, dim3(grid), dim3(kActThreads), smem, stream, x, T, nvec, gain, eps,
+                         static_cast<double>(nvec * 8), 1.0 / static_cast<double>(nvec * 8), q, a_scale);
 }
 
 // K up to 16384 (the register-resident row); longer rows are refused by the caller.
@@ -206,7 +242,12 @@ inline sbn_status launch_norm_quant_act(const void* x_bf16, int T, int K, const 
     const float4* g4 = reinterpret_cast<const float4*>(gain);
     uint2* q = reinterpret_cast<uint2*>(xq);
     cudaError_t err;
-    if (nvec <= 32 * 2) err = launch_norm_quant_act_cfg<32, 2, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);
+    // Few rows: one per CTA with all its threads, so that what a thread does between the barriers is short.  With 2560 columns
+    // (us, a whole CTA / two rows per CTA): 1.59 / 2.11 at 16 rows, 2.08 / 2.33 at 222, 2.86 / 3.28 at 444 (every row
+    // resident), 4.17 / 4.12 at 777; narrower rows cross earlier (1280 columns: 1.59 / 1.80 at 148, 1.85 / 1.78 at 222).
+    // Many rows: smaller groups, whose barriers are shared by fewer warps.
+    if (T <= kNumSMs * (nvec > 256 ? 3 : 1) && nvec > 128 && nvec <= 256 * 2) err = launch_norm_quant_act_cfg<256, 2, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);
+    else if (nvec <= 32 * 2) err = launch_norm_quant_act_cfg<32, 2, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);
     else if (nvec <= 64 * 2) err = launch_norm_quant_act_cfg<64, 2, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);
     else if (nvec <= 128 * 2) err = launch_norm_quant_act_cfg<128, 2, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);
     else if (nvec <= 128 * 3) err = launch_norm_quant_act_cfg<128, 3, EXPAND68>(x, T, nvec, g4, eps, q, a_scale, stream);

@@ -86,6 +86,13 @@ def test_norm_quant_act_parity(T, K, with_gain):
     assert np.array_equal(xq_to_numpy(xq, T, K), r["xq"])
 
 
+# around the row counts where a whole CTA per row gives way to two or more rows per CTA; columns that leave the last
+# vectors of a thread empty, and the widest row the whole-CTA form takes.  Whole numbers: equality.
+@pytest.mark.parametrize("T,K", [(1, 1280), (148, 1280), (149, 1280), (1, 2048), (444, 2176), (445, 2176), (444, 4096), (1, 1152)])
+def test_norm_quant_act_rows_per_cta(T, K):
+    test_norm_quant_act_parity(T, K, True)
+
+
 def test_norm_quant_act_edge_rows():
     K = 512
     x = np.zeros((5, K), np.float32)
