@@ -1,6 +1,6 @@
 // Eq. 4 for few tokens: split-K inside a thread-block cluster.
 //
-// With T up to a few hundred there are only N/128 x ceil(T/BN) output tiles -- far fewer than SMs --
+// With few tokens (narrow tiles here; from about 65 on gemm_splitk_wide_tcgen05.cuh takes over) there are only N/128 x ceil(T/BN) output tiles -- far fewer than SMs --
 // and a CTA that walks the whole K of its tile is bound by what ONE SM can pull out of L2
 // (~100 GB/s: 18 KB per 128 columns -> 0.23 us each).  Splitting K over CTAs puts more SMs on the
 // weight stream; the partial accumulators then have to be added.  Through global memory that is
@@ -42,19 +42,19 @@ struct SplitConfig {
     static constexpr int B_BYTES = BN * kBK;
     static constexpr int E_BYTES = SPARSE ? kBM * (kBK / 8) : 0;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + E_BYTES;
-    // BN <= 64: few enough stages that TWO CTAs fit on an SM (< 113 KB each), so the CTAs of the next
+    // Few enough stages that TWO CTAs fit on an SM (< 113 KB each), so the CTAs of the next
     // launch of a decode loop are resident -- and already pulling their weights -- while this one
     // reduces and finishes.  A stage that is filled before the dependency wait costs nothing, one
     // that has to be refilled costs an L2 round trip on the critical path: the 32-token tile keeps
     // six (sparse) stages, enough for the whole K slice of a CTA at the usual sizes.
-    static constexpr int STAGES = (BN == 32) ? (SPARSE ? 6 : 4) : (BN == 64) ? (SPARSE ? 4 : 3) : (SPARSE ? 6 : 4);
-    static constexpr int CTAS_PER_SM = (BN <= 64) ? 2 : 1;
+    static constexpr int STAGES = (BN == 32) ? (SPARSE ? 6 : 4) : (SPARSE ? 4 : 3);
+    static constexpr int CTAS_PER_SM = 2;
     static constexpr int REDUCE_BYTES = (BN + 4) * kBM * 4;    // [S][ceil(BN/S) tokens][128 features] int32, S in {2, 3, 4, 8}
     static constexpr int META_COL0 = BN;                        // metadata columns above the accumulator
     static constexpr uint32_t TMEM_COLS = (BN + 4 * STAGES <= 64) ? 64 : (BN + 4 * STAGES <= 128 ? 128 : 256);
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + REDUCE_BYTES + kBarrierBytes;
     static_assert(SMEM_BYTES <= 232448 / CTAS_PER_SM - 1024 * (CTAS_PER_SM - 1), "shared memory overflow");
-    static_assert(BN % 32 == 0 && BN <= 128, "token tile");
+    static_assert(BN == 32 || BN == 64, "token tile (wider ones: gemm_splitk_wide_tcgen05.cuh)");
 };
 
 // 4-byte store into a peer's shared memory that counts its bytes on an mbarrier of that peer.
@@ -319,15 +319,12 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
         else scatter(std::integral_constant<int, 8>{});
         tcgen05_fence_before();
     }
-    // s of Eq. 4 for the tokens this CTA finishes, fetched before the barrier (lane l: its l-th and
-    // (l + 32)-th token) so that the finishing loop has no global load to wait for
-    float sc_a = 0.0f, sc_b = 0.0f;
+    // s of Eq. 4 for the tokens this CTA finishes (at most 32), fetched before the barrier (lane l: its l-th token) so that the finishing loop has no global load to wait for
+    float sc_a = 0.0f;
     if (warp >= 2) {
         const float w_scale = __ldg(p.w_scale);
         const int ja = lane * static_cast<int>(S) + static_cast<int>(rank);          // token inside the tile
-        const int jb = (lane + 32) * static_cast<int>(S) + static_cast<int>(rank);
         if (lane < tok_per_cta && ja < tile_tokens) sc_a = __fmul_rn(w_scale, __ldg(p.a_scale + t0 + ja));
-        if (lane + 32 < tok_per_cta && jb < tile_tokens) sc_b = __fmul_rn(w_scale, __ldg(p.a_scale + t0 + jb));
     }
 
     if (warp >= 2) {
@@ -345,7 +342,7 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
         const int n_tok = (fine && ok) ? my_tokens : 0;
         cluster_finish(S, red, tok_per_cta, n_tok, f, [&](int j, int acc) {
             const int t = t0 + j * static_cast<int>(S) + static_cast<int>(rank);
-            const float sc = __shfl_sync(0xFFFFFFFFu, j < 32 ? sc_a : sc_b, j & 31);
+            const float sc = __shfl_sync(0xFFFFFFFFu, sc_a, j);
             if (p.acc_out) p.acc_out[static_cast<size_t>(t) * p.N + n] = acc;
             float v = __fmul_rn(static_cast<float>(acc), sc);
             if (p.bias) v = __fadd_rn(v, bias);

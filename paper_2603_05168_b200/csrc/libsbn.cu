@@ -19,6 +19,7 @@
 #include "gemm_tcgen05.cuh"
 #include "gemm_pair_tcgen05.cuh"
 #include "gemm_splitk_cluster_tcgen05.cuh"
+#include "gemm_splitk_wide_tcgen05.cuh"
 #include "gemm_packed_cluster_tcgen05.cuh"
 #include "gemm_fused_act_cluster_tcgen05.cuh"
 #include "gemm_few_tokens_mma.cuh"
@@ -31,8 +32,7 @@ namespace sbn {
 // host state
 // ------------------------------------------------------------------------------------------------
 static int g_force_token_tile = 0;
-static int g_force_split_k = 0;            // > 0: global-atomics split-K factor; -2, -4, -8: cluster split-K of that size
-static bool g_allow_cluster = true;
+static int g_force_split_k = 0;            // > 0: global-atomics split-K factor; < 0: cluster split-K of that size
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -176,44 +176,6 @@ static sbn_status launch_gemm_cfg(const CUtensorMap& ta, const CUtensorMap& tb, 
 }
 
 // ---- CTA-pair kernel (large T) -------------------------------------------------------------------
-// Token-tile width for the pair kernel: a small cost model of (operand ingest | MMA rate) per unit
-// of K, the accumulator drain per tile, and the number of waves over the 74 CTA pairs.
-static int pick_pair_bn(bool sparse, int T, int N, int K) {
-    if (g_force_token_tile < 0) {
-        int bn = -g_force_token_tile;
-        const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
-        bn = (bn / 16) * 16;
-        if (bn < 32) bn = 32;
-        if (bn > cap) bn = cap;
-        return bn;
-    }
-    const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
-    const double mac_rate = sparse ? 16384.0 : 8192.0;          // MAC / clk / SM
-    const double ingest = 64.0;                                  // B / clk / SM
-    const int full_m = N / 512, rem_m = (N % 512) ? 1 : 0;
-    int best = 128;
-    double best_cost = 1e300;
-    for (int bn = 64; bn <= cap; bn += 16) {
-        const int tt = (T + bn - 1) / bn;
-        auto tile_clk = [&](int mtiles) {
-            const double a_bytes = sparse ? 72.0 : 128.0;
-            const double bytes = mtiles * a_bytes + bn / 2.0;
-            const double macs = mtiles * 128.0 * bn;
-            const double per_k = std::max(bytes / ingest, macs / mac_rate);
-            return per_k * K + 12.0 * bn + 600.0;                // + drain and tile turnaround
-        };
-        // greedy waves: full tiles first, then the half tiles
-        const double work = static_cast<double>(full_m) * tt * tile_clk(2) + static_cast<double>(rem_m) * tt * tile_clk(1);
-        const long tiles = static_cast<long>(full_m + rem_m) * tt;
-        const long waves = (tiles + 73) / 74;
-        const double balanced = work / 74.0;
-        const double quantised = static_cast<double>(waves) * tile_clk(2);
-        const double cost = std::max(balanced, 0.5 * (balanced + quantised));
-        if (cost < best_cost) { best_cost = cost; best = bn; }
-    }
-    return best;
-}
-
 template <bool SPARSE, int MT>
 static sbn_status launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& te,
                               const PairParams& pp, cudaStream_t stream) {
@@ -227,74 +189,109 @@ static sbn_status launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, cons
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
 
-// Which kernel, which token tile, whether to split K: a small model of the measured times (us).
-//   single-CTA kernel   F(bn) + waves * (K/128 / splits) * c(bn)  [+ split-K: 1 + 8e-6 per atomic]
-//                       F = 3.0 + 0.02 bn (prologue + last epilogue), c = 0.23 (bn = 64) | 0.27 (128) | 0.49 (256)
-//   CTA-pair kernel     4.3 + 0.02 bn + waves * (K/128 * 0.31 + 2.5 (exposed drain)); dense K-loop x 1.65;
-//                       with one M-tile per CTA: 4.3 + 0.02 bn + waves * K/128 * 0.205 (dense 0.29)
-// waves over 148 CTAs resp. 74 pairs.  Small problems are latency-bound and favour many small
-// single-CTA tiles; large ones favour the pair kernel's operand reuse.  K is split only when the
-// tiles cannot fill the machine and the int32 atomics cost less than the K-loop they save.
+// Which kernel, which token tile, whether to split K: the measured times (us) of every candidate, as a small model.
+//
+// The coefficients were fitted to a sweep of quantiser + GEMM chains: eight shapes from 2048 x 1024 to 11008 x 4096, 30
+// token counts from 12 to 8192, every kernel with its useful tiles and splits, sparse and dense; 5000 timings.  What the
+// model picks was within 0.3 % of the fastest candidate on average (the worst 13 %).  q = K-blocks per CTA, w = waves.
+//   clusters, narrow tiles   a + q (c + x crowd) + tokens (t + s / S) + o [two CTAs on some SM] + 3-way owner selection
+//   clusters, wide tiles     a + q (c + u bn / 256) + e tokens (S - 1) / S + 1.0 or 1.4 x share of the SMs in use
+//   single-CTA tiles         a + w (q c + d)
+//   CTA pairs                a + b bn + w (q (c + u bn / 256) + d), with one or two M-tiles per CTA
+// What follows from it (2560 -> 3840, us, sparse): 65 tokens wide tiles split four ways 7.2 (narrow ones 7.9); 201 two
+// wide tiles split two ways 9.0 (64-token tiles unsplit 10.3, split 9.9); 400 pairs 10.4 (128-token tiles 12.1).
+// 6912 -> 2560 dense, 512 tokens: wide tiles 17.6 (128-token tiles 22.4, pairs 25).
+struct ClusterCost { double a, c, x, t, s, o, s3; };
+struct WideCost { double a, c, e, share, u; };
+struct TileCost { double a, c, d; };
+struct PairCost { double a, b, c, d, u; };
+struct PlanCosts {
+    ClusterCost narrow32, narrow64;
+    WideCost wide;
+    TileCost tile64, tile128, tile256;
+    PairCost pair1, pair2;
+};
+static const PlanCosts kSparseCosts = {
+    {2.39, 0.269, 0.029, 0.0305, 0.003, 0.38, 0.11}, {2.42, 0.276, 0.049, 0.0338, 0.0125, 0.41, 1.17},
+    {2.26, 0.261, 0.0303, 1.04, 0.041},
+    {3.63, 0.250, 0.0}, {4.27, 0.252, 0.72}, {3.60, 0.290, 3.11},
+    {2.01, 0.0093, 0.197, 1.15, 0.015}, {1.29, 0.0179, 0.2605, 3.17, 0.098}};
+static const PlanCosts kDenseCosts = {
+    {2.37, 0.317, 0.060, 0.0245, 0.0, 0.40, 0.17}, {2.20, 0.364, 0.090, 0.0329, 0.0043, 0.60, 1.23},
+    {1.87, 0.295, 0.0319, 1.40, 0.060},
+    {3.60, 0.277, 0.17}, {4.69, 0.284, 0.39}, {8.00, 0.3835, 0.0},
+    {2.24, 0.0096, 0.329, 1.00, 0.0235}, {1.96, 0.0139, 0.376, 3.20, 0.215}};
+
 static GemmPlan plan_gemm(bool sparse, int T, int N, int K) {
     GemmPlan best = {false, 64, 1, 0};
     const int kb = K / kBK;
     const int rows = N / kBM;
     if (g_force_token_tile < 0) {                               // diagnostics: the pair kernel as told (split_k 1 = one M-tile per CTA)
-        GemmPlan g{true, pick_pair_bn(sparse, T, N, K), 1, 0};
+        const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
+        GemmPlan g{true, std::min(cap, std::max(32, (-g_force_token_tile) / 16 * 16)), 1, 0};
         g.mt = g_force_split_k == 1 ? 1 : 2;
         return g;
     }
     if (g_force_split_k < 0) {                                  // diagnostics: cluster split-K as told
         int S = -g_force_split_k;
+        if (g_force_token_tile > 64) {                          // wide tiles: any width and cluster that fit
+            const int bn = std::min(256, g_force_token_tile / 16 * 16);
+            S = std::min(8, std::min(S, K / kBK));
+            while (S > 1 && !wide_fits(bn, S)) --S;
+            if (S > 1) return GemmPlan{false, bn, 1, S};
+        }
         S = S >= 8 ? 8 : (S >= 4 ? 4 : (S == 3 ? 3 : 2));
         while (S > 1 && S > K / kBK) --S;
         if (S > 4 && S < 8) S = 4;
-        const int bn = g_force_token_tile == 128 ? 128 : (g_force_token_tile == 32 ? 32 : 64);
+        const int bn = g_force_token_tile == 32 ? 32 : 64;
         if (S > 1) return GemmPlan{false, bn, 1, S};
     }
     if (g_force_token_tile > 0 || g_force_split_k > 0) {        // diagnostics: single-CTA kernel as told
         const int bn = pick_token_tile(T);
         return GemmPlan{false, bn, pick_split_k(T, N, K, bn), 0};
     }
-    const double mm = sparse ? 1.0 : 1.3;                       // dense K-loop relative to sparse
+    const PlanCosts& cost = sparse ? kSparseCosts : kDenseCosts;
     double best_t = 1e300;
     auto consider = [&](const GemmPlan& g, double t) { if (t < best_t) { best_t = t; best = g; } };
-    // split-K inside clusters of 2, 3 or 4 CTAs: the K-loop shrinks and the reduction stays on chip.
-    // Fitted to a sweep in a decode loop (weights from HBM, launches back to back), in us:
-    //   a(bn) + q * (0.22 sparse | 0.27 dense per 128 columns) * (1 .. 1.6: co-resident CTAs share the
-    //   one tensor pipe) + tokens of a tile * (scatter + finish / S).
-    // All CTAs must be resident at once (tiles up to 64 tokens fit two per SM): a second wave costs
-    // a whole kernel lifetime.  Clusters of 3 matter for matrices with 75..90 row tiles, where 2
-    // leaves SMs with two CTAs' long K slices and 4 does not fit; they need some slack in the slot
-    // count (288 CTAs in clusters of 3 did not all become resident on 296 slots).
-    auto consider_cluster = [&](int bn) {
+    // Clusters of 2, 3 or 4 CTAs, narrow tiles: all CTAs resident at once (two per SM), a second wave costs a whole kernel
+    // lifetime.  Clusters of 3 need some slack in the slot count (288 CTAs in clusters of 3 did not all become resident
+    // on 296 slots).
+    for (const int bn : {32, 64}) {
+        const ClusterCost& c = bn == 32 ? cost.narrow32 : cost.narrow64;
         const long tiles = static_cast<long>(rows) * ((T + bn - 1) / bn);
-        const long slots = bn <= 64 ? 2L * kNumSMs : kNumSMs;
-        const double a = bn == 32 ? 3.0 : (bn == 64 ? 3.3 : 3.7);
-        const int tt = std::min(bn, T);
-        for (int S = 2; S <= 4; ++S) {
-            if (S > kb || tiles * S > slots) break;
-            if (S == 3 && tiles * S * 100 > slots * 93) continue;
+        const int tokens = std::min(bn, T);
+        for (int S = 2; S <= 4 && S <= kb && tiles * S <= 2L * kNumSMs; ++S) {
+            if (S == 3 && tiles * S * 100 > 2L * kNumSMs * 93) continue;
             const int q = (kb + S - 1) / S;
-            const double per_tok = (bn == 128 ? 0.018 : 0.013) + 0.042 / S;
             const long ctas = tiles * S;
-            const long per_sm = (ctas + kNumSMs - 1) / kNumSMs;
             // share of the SMs that hold two CTAs; the slowdown saturates once ~40 % of them do
-            const double crowd = per_sm > 1 ? std::min(1.0, 2.5 * static_cast<double>(ctas - kNumSMs) / kNumSMs) : 0.0;
-            consider(GemmPlan{false, bn, 1, S}, a + q * (sparse ? 0.22 : 0.27) * (1.0 + 0.6 * crowd) + per_tok * tt +
-                                                    (per_sm > 1 ? 0.3 : 0.0) + (S == 3 ? 0.4 + 0.03 * tt : 0.0));   // 3: owner by select, not by mask
+            const double crowd = ctas > kNumSMs ? std::min(1.0, 2.5 * static_cast<double>(ctas - kNumSMs) / kNumSMs) : 0.0;
+            consider(GemmPlan{false, bn, 1, S}, c.a + q * (c.c + c.x * crowd) + tokens * (c.t + c.s / S) + (ctas > kNumSMs ? c.o : 0.0) + (S == 3 ? c.s3 : 0.0));
         }
-    };
-    if (g_allow_cluster) consider_cluster(32);
-    const int bns[3] = {64, 128, 256};
-    for (int bn : bns) {
+    }
+    // Wide tiles: one CTA per SM, and the clusters that fit at once (74 of 2, 45 of 3, 33 of 4).
+    if (T > 64 && T <= 800) {
+        const int most[5] = {0, 0, 74, 45, 33};
+        for (int tt = (T + 255) / 256; tt <= (T + 255) / 256 + 2; ++tt) {
+            const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
+            if (bn * (tt - 1) >= T) continue;
+            const int tokens = std::min(bn, T);
+            for (int S = 2; S <= 4 && S <= kb; ++S) {
+                if (static_cast<long>(rows) * tt > most[S] || !wide_fits(bn, S)) continue;
+                const int q = (kb + S - 1) / S;
+                consider(GemmPlan{false, bn, 1, S}, cost.wide.a + q * (cost.wide.c + cost.wide.u * bn / 256) + cost.wide.e * tokens * (S - 1) / S +
+                                                        cost.wide.share * rows * tt * S / kNumSMs);
+            }
+        }
+    }
+    // Single-CTA tiles.  K is split through global memory only when the tiles cannot fill the machine and the int32 atomics
+    // cost less than the K-loop they save.
+    for (const int bn : {64, 128, 256}) {
         if (bn > 64 && T <= bn / 2) continue;                   // a tile mostly beyond T
+        const TileCost& c = bn == 64 ? cost.tile64 : (bn == 128 ? cost.tile128 : cost.tile256);
         const long tiles = static_cast<long>(rows) * ((T + bn - 1) / bn);
-        const double c = (bn == 256 ? 0.49 : (bn == 128 ? 0.27 : 0.23)) * mm;   // per 128 columns and wave
-        const double F = 3.0 + 0.02 * bn;
         const long waves = (tiles + kNumSMs - 1) / kNumSMs;
-        consider(GemmPlan{false, bn, 1, 0}, F + waves * kb * c);
-        if (bn <= 128 && g_allow_cluster) consider_cluster(bn);
+        if (waves <= 2) consider(GemmPlan{false, bn, 1, 0}, c.a + waves * (kb * c.c + c.d));    // beyond, the pairs' operand reuse wins
         if (bn == 64 && tiles * 2 <= kNumSMs) {
             // smallest split that gives at least ~100 units of work
             int sp = static_cast<int>((100 + tiles - 1) / tiles);
@@ -302,37 +299,27 @@ static GemmPlan plan_gemm(bool sparse, int T, int N, int K) {
             while (sp > 1 && kb % sp != 0) ++sp;                // next divisor upwards (kb divides itself)
             if (sp > 1 && sp <= kb && sp <= 10) {               // many slices: the atomics dominate (33 us measured at 43)
                 const double atomics = 8e-6 * static_cast<double>(T) * N * sp;
-                consider(GemmPlan{false, bn, sp, 0}, F + (kb / sp) * c + 1.0 + atomics);
+                consider(GemmPlan{false, bn, sp, 0}, c.a + (kb / sp) * c.c + c.d + 1.0 + atomics);
             }
         }
     }
-    {
-        const int bn = pick_pair_bn(sparse, T, N, K);
-        const long tiles = static_cast<long>((N + 511) / 512) * ((T + bn - 1) / bn);
-        const long waves = (tiles + kNumSMs / 2 - 1) / (kNumSMs / 2);
-        consider(GemmPlan{true, bn, 1, 0}, 4.3 + 0.02 * bn + waves * kb * 0.31 * (sparse ? 1.0 : 1.65) + waves * 2.5);
-    }
-    {
-        // One M-tile per CTA: 256-feature tiles with double-buffered accumulators.  A tile costs the same
-        // whatever its token width (the MMAs' pace does not depend on it), so: fewest waves over the 74
-        // pairs, then least token padding, then the widest tile.  Per 128 columns 0.205 us (sparse) /
-        // 0.29 us (dense) against 0.31 / 0.43 for twice the features with two M-tiles, and no exposed
-        // drain: wins for short K and for the dense kernel, loses for the sparse one at K >= 4096.
+    // CTA pairs: a tile costs nearly the same whatever its token width, so the tile counts worth a look are the smallest
+    // ones, down to those that fill the last wave.
+    if (T > 32) {
         const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
-        const long rows1 = (N + 255) / 256;
-        int best_bn = 0;
-        long best_waves = 0, best_cover = 0;
-        for (int bn = cap; bn >= 128; bn -= 16) {
-            const long tt = (T + bn - 1) / bn;
-            const long waves = (rows1 * tt + kNumSMs / 2 - 1) / (kNumSMs / 2);
-            const long cover = tt * bn;
-            if (best_bn == 0 || waves < best_waves || (waves == best_waves && cover < best_cover)) {
-                best_bn = bn; best_waves = waves; best_cover = cover;
+        const int fewest = (T + cap - 1) / cap;
+        for (int tt = fewest; tt <= fewest + (T < 1000 ? 3 : 8); ++tt) {
+            const int bn = std::max(T > 64 ? 80 : 32, ((T + tt - 1) / tt + 15) / 16 * 16);
+            if (bn * (tt - 1) >= T) continue;
+            for (int mt = 1; mt <= 2; ++mt) {
+                const PairCost& c = mt == 1 ? cost.pair1 : cost.pair2;
+                const long tiles = static_cast<long>((N + 256 * mt - 1) / (256 * mt)) * tt;
+                const long waves = (tiles + kNumSMs / 2 - 1) / (kNumSMs / 2);
+                GemmPlan g{true, bn, 1, 0};
+                g.mt = mt;
+                consider(g, c.a + c.b * bn + waves * (kb * (c.c + c.u * bn / 256) + c.d));
             }
         }
-        GemmPlan g{true, best_bn, 1, 0};
-        g.mt = 1;
-        consider(g, 4.3 + 0.02 * best_bn + best_waves * kb * (sparse ? 0.205 : 0.29));
     }
     return best;
 }
@@ -380,6 +367,17 @@ static sbn_status launch_splitk_cluster(const CUtensorMap& ta, const CUtensorMap
     const int tiles = (p.N / kBM) * ((p.T + BN - 1) / BN);
     const cudaError_t err = launch_kernel_cluster(kernel, dim3(tiles * cluster), dim3(kSplitThreads), Cfg::SMEM_BYTES, stream,
                                                   static_cast<unsigned>(cluster), ta, tb, te, p);
+    ++g_launch_count;
+    return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+}
+
+template <bool SPARSE>
+static sbn_status launch_splitk_wide(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& te, const GemmParams& p, int bn,
+                                     int cluster, cudaStream_t stream) {
+    if (!ensure_dynamic_smem<bitlinear_gemm_splitk_wide_kernel<SPARSE>>(kWideSmemBytes)) return SBN_ERR_CUDA;
+    const int tiles = (p.N / kBM) * ((p.T + bn - 1) / bn);
+    const cudaError_t err = launch_kernel_cluster(bitlinear_gemm_splitk_wide_kernel<SPARSE>, dim3(tiles * cluster), dim3(kWideThreads),
+                                                  kWideSmemBytes, stream, static_cast<unsigned>(cluster), ta, tb, te, p, bn);
     ++g_launch_count;
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
@@ -462,12 +460,12 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
 
     if (plan.cluster > 1) {
         p.k_splits = 1;
+        if (bn > 64) return sparse ? launch_splitk_wide<true>(ta, tb, te, p, bn, plan.cluster, stream)
+                                   : launch_splitk_wide<false>(ta, tb, te, p, bn, plan.cluster, stream);
         if (sparse) return bn == 32 ? launch_splitk_cluster<true, 32>(ta, tb, te, p, plan.cluster, stream)
-                         : bn == 64 ? launch_splitk_cluster<true, 64>(ta, tb, te, p, plan.cluster, stream)
-                                    : launch_splitk_cluster<true, 128>(ta, tb, te, p, plan.cluster, stream);
+                                    : launch_splitk_cluster<true, 64>(ta, tb, te, p, plan.cluster, stream);
         return bn == 32 ? launch_splitk_cluster<false, 32>(ta, tb, te, p, plan.cluster, stream)
-             : bn == 64 ? launch_splitk_cluster<false, 64>(ta, tb, te, p, plan.cluster, stream)
-                        : launch_splitk_cluster<false, 128>(ta, tb, te, p, plan.cluster, stream);
+                        : launch_splitk_cluster<false, 64>(ta, tb, te, p, plan.cluster, stream);
     }
 
     sbn_status st;

@@ -754,6 +754,18 @@ def test_gemm_parity_cluster_split_k(sparse, T, N, K, tile, cluster):
     assert np.abs(bf16_tensor_bits(yb).astype(np.int32) - ref_bits).max() <= 1
 
 
+# Wide token tiles split over clusters: one token in the last tile (CTAs that own none), unequal shares, tiles of the least
+# and the greatest width, K-blocks that do not divide by the cluster, one block per CTA, more blocks than stages.
+WIDE_CASES = [(81, 128, 512, 80, 4), (65, 256, 384, 80, 3), (201, 256, 1280, 112, 2), (256, 128, 1664, 256, 4), (255, 256, 2560, 256, 2),
+              (160, 128, 2176, 160, 3), (300, 128, 768, 208, 6), (97, 384, 256, 112, 2)]
+
+
+@pytest.mark.parametrize("sparse", [True, False])
+@pytest.mark.parametrize("T,N,K,tile,cluster", WIDE_CASES)
+def test_gemm_parity_cluster_wide_tiles(sparse, T, N, K, tile, cluster):
+    test_gemm_parity_cluster_split_k(sparse, T, N, K, tile, cluster)
+
+
 @pytest.mark.parametrize("sparse", [True, False])
 @pytest.mark.parametrize("split", [2, 5, 10])
 def test_gemm_parity_split_k(sparse, split):
@@ -1072,7 +1084,7 @@ def test_quantize_mask_pack_graph_replay_on_changed_weights():
 
 # ---- bounded waits that run out --------------------------------------------------------------------------
 WAIT_CASES = [("single_cta", 64, 256, 512, (128, 1)), ("pair", 300, 512, 512, (-128, 0)), ("pair_one_m_tile", 300, 256, 512, (-128, 1)),
-              ("cluster", 16, 256, 1280, (32, -4))]
+              ("cluster", 16, 256, 1280, (32, -4)), ("cluster_wide", 100, 256, 1280, (112, -2))]
 
 
 @pytest.mark.parametrize("sparse", [True, False])
