@@ -1,15 +1,17 @@
 // Operands of the backward GEMMs (dual straight-through estimator, Sec. 2.3, Eq. 5; Algorithm 2's
 // backward) in bf16, as the tensor-core kernel of gemm_bf16_pair_tcgen05.cuh reads them:
 //
-//   dX[t][k] = sum_n dY[t][n] * w_masked[n][k]   contraction over n: A = dY [T][N] as it is (K-major),
-//                                                 B = W_eff^T [K][N] (weff_t_bf16_kernel: a 128 x 128 tile
-//                                                 transposed through shared memory, written as 256 B rows)
-//   dW[n][k] = sum_t dY[t][n] * x_q[t][k]        contraction over t: A = dY [T][N] and B = x_q [T][K]
-//                                                 (xq_bf16_kernel), both as they lie in memory; the MMA
-//                                                 reads them MN-major, so nothing is transposed
+//   dX[t][k] = sum_n dY[t][n] * w_masked[n][k]   contraction over n: B = W_eff [N][K]
+//   dW[n][k] = sum_t dY[t][n] * x_q[t][k]        contraction over t: B = x_q [T][K]
 //
+// Both are row-major with the contraction down the rows; the MMA reads them MN-major, so nothing is transposed.
 // x_q[t][k] = bf16(x~[t][k] * a_scale[t]) are the fake-quantised activations as a bf16 training run holds
 // them; W_eff is written as +-1.0 / 0.0 and its scale is applied once in the GEMM's epilogue.
+//
+// The work is cut into items of 128 threads, memory-bound (2.6 and 3 bytes per element): 8 lanes per row, so that a warp
+// reads whole rows of a tile and every lane writes a full 32-byte sector; both operands in one launch.
+// 2560 -> 3840 at 4096 tokens 9.7 us (two launches, W_eff transposed through shared memory: 16.6), 2560 -> 6912 11.4 (20.6),
+// 6912 -> 2560 21 (31).
 #pragma once
 
 #include "sbn_common.cuh"
@@ -17,82 +19,101 @@
 
 namespace sbn {
 
-constexpr int kPrepThreads = 256;
-constexpr int kPrepTile = 128;
-constexpr int kPrepRowBytes = kPrepTile * 2 + 16;            // bf16 row of the transposed tile, padded (keeps 16 B alignment)
+constexpr int kPrepThreads = 128;                              // one item at a time
+constexpr int kPrepItemTokens = 64;                            // x_q item: 64 tokens x 128 columns; W_eff item: 128 x 128
 
-__device__ __forceinline__ uint16_t bf16_bits_of(float f) { return static_cast<uint16_t>(f32_to_bf16_rne(f)); }
+struct PrepJob {
+    const uint8_t* vals;                                       // W_eff from the compressed 2:4 form (tiled)
+    const uint8_t* meta;
+    uint16_t* w_out;
+    const uint8_t* xq;                                         // x_q from the tiled int8 activations and their scales
+    const float* a_scale;
+    uint16_t* x_out;
+    int T, N, K;
+    int w_items, x_items;                                      // 0: not wanted
+};
 
-// Writes the transposed tile (128 rows x 128 bf16) from shared memory: row j goes to dst + j * ld
-// (elements), columns [0, 128); rows >= rows_valid and 16-byte chunks beyond cols_valid are skipped.
-__device__ __forceinline__ void prep_store_tile(const unsigned char* s_t, uint16_t* dst, size_t ld, int rows_valid, int cols_valid) {
-    const int chunk = threadIdx.x & 15;                        // 16 B = 8 elements
-    for (int j = threadIdx.x >> 4; j < kPrepTile; j += kPrepThreads / 16) {
-        if (j < rows_valid && chunk * 8 < cols_valid) {
-            const uint4 v = *reinterpret_cast<const uint4*>(s_t + j * kPrepRowBytes + chunk * 16);
-            *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * ld + chunk * 8) = v;
-        }
-    }
+__device__ __forceinline__ void st_global_32b(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
 }
 
-// W_eff^T [K][N] in bf16 (+-1, 0) from the compressed 2:4 form (tiled vals / meta).
-__global__ void __launch_bounds__(kPrepThreads)
-weff_t_bf16_kernel(const uint8_t* __restrict__ vals, const uint8_t* __restrict__ meta, int N, int K, uint16_t* __restrict__ Wt) {
-    __shared__ __align__(16) unsigned char s_t[kPrepTile * kPrepRowBytes];
-    pdl_wait();
-    const int KB = K >> 7;
-    const int kb = blockIdx.x % KB, nb = blockIdx.x / KB;
-    const size_t tile = static_cast<size_t>(nb) * KB + kb;
-    const int r = threadIdx.x >> 1, half = threadIdx.x & 1;    // weight row inside the tile, half of its 32 groups
-    const uint2 m8 = *reinterpret_cast<const uint2*>(meta + tile * 2048 + r * 16 + half * 8);
-    const uint4 v0 = *reinterpret_cast<const uint4*>(vals + tile * 8192 + vals_in_tile(r, 32u * half));
-    const uint4 v1 = *reinterpret_cast<const uint4*>(vals + tile * 8192 + vals_in_tile(r, 32u * half + 16u));
-    const uint32_t vw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    const uint32_t mw[2] = {m8.x, m8.y};
-#pragma unroll
-    for (int g = 0; g < 16; ++g) {                             // group g of this half: columns 64 half + 4 g ..
-        const uint32_t nib = (mw[g >> 3] >> (4 * (g & 7))) & 15u;
-        const uint32_t pair = (vw[g >> 1] >> (16 * (g & 1))) & 0xFFFFu;
-        const int8_t a = static_cast<int8_t>(pair & 0xFFu), b = static_cast<int8_t>(pair >> 8);
-        const uint32_t i0 = nib & 3u, i1 = nib >> 2;
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) {
-            const int q = (j == i0) ? a : ((j == i1) ? b : 0);
-            const uint16_t bits = q > 0 ? 0x3F80u : (q < 0 ? 0xBF80u : 0u);      // +1.0, -1.0, 0.0
-            *reinterpret_cast<uint16_t*>(s_t + (64 * half + 4 * g + j) * kPrepRowBytes + r * 2) = bits;
-        }
-    }
-    __syncthreads();
-    prep_store_tile(s_t, Wt + (static_cast<size_t>(kb) * 128) * N + static_cast<size_t>(nb) * 128, static_cast<size_t>(N), kPrepTile, kPrepTile);
-}
+// +-1.0, 0.0 in bf16 from the byte of a ternary value
+__device__ __forceinline__ uint32_t ternary_bf16(uint32_t byte) { return (byte & 1u) * 0x3F80u | ((byte & 0x80u) << 8); }
 
-// x_q [T][K] in bf16 (token-major, as the activations themselves) from the tiled int8 activations and their
-// per-token scales: the B operand of the weight-gradient GEMM when it reads MN-major operands.  A thread
-// converts 16 codes (one 16 B chunk) into 32 B of output.
-__global__ void __launch_bounds__(kPrepThreads)
-xq_bf16_kernel(const uint8_t* __restrict__ xq, const float* __restrict__ a_scale, int T, int K, uint16_t* __restrict__ X) {
-    pdl_wait();
-    const size_t tb8 = xq_tb8(T);
-    const int chunks_per_row = K >> 4;
-    const size_t total = static_cast<size_t>(T) * chunks_per_row;
-    for (size_t i = static_cast<size_t>(blockIdx.x) * kPrepThreads + threadIdx.x; i < total; i += static_cast<size_t>(gridDim.x) * kPrepThreads) {
-        const int t = static_cast<int>(i / chunks_per_row), ch = static_cast<int>(i % chunks_per_row);
-        const int kb = ch >> 3, c8 = ch & 7;
-        const float s = __ldg(a_scale + t);
-        const uint4 c = *reinterpret_cast<const uint4*>(xq + (static_cast<size_t>(kb) * tb8 + (static_cast<uint32_t>(t) >> 3)) * 1024 + (t & 7) * 128 +
-                                                        ((c8 ^ (t & 7)) << 4));
-        const uint32_t w[4] = {c.x, c.y, c.z, c.w};
+// Item of W_eff: 128 rows x 128 columns, `tid` of 128 threads.
+__device__ __forceinline__ void prep_w_item(const PrepJob& j, int item, int tid) {
+    const int KB = j.K >> 7;
+    const int kb = item % KB, nb = item / KB;
+    const uint32_t r0 = static_cast<uint32_t>(tid) >> 3, c = static_cast<uint32_t>(tid) & 7u;     // 8 value bytes = 4 groups = 16 columns
+    const uint8_t* vt = j.vals + static_cast<size_t>(item) * 8192;
+    const uint8_t* mt = j.meta + static_cast<size_t>(item) * 2048;
+    uint16_t* out = j.w_out + (static_cast<size_t>(nb) * 128) * j.K + static_cast<size_t>(kb) * 128 + c * 16;
+    uint2 v[8];
+    uint32_t m[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t r = r0 + 16u * i;
+        v[i] = __ldg(reinterpret_cast<const uint2*>(vt + vals_in_tile(r, 8u * c)));
+        m[i] = __ldg(reinterpret_cast<const unsigned short*>(mt + r * 16 + c * 2));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
         uint32_t o[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int q0 = static_cast<int8_t>((w[j >> 1] >> (16 * (j & 1))) & 0xFFu);
-            const int q1 = static_cast<int8_t>((w[j >> 1] >> (16 * (j & 1) + 8)) & 0xFFu);
-            o[j] = static_cast<uint32_t>(bf16_bits_of(__fmul_rn(static_cast<float>(q0), s))) |
-                   (static_cast<uint32_t>(bf16_bits_of(__fmul_rn(static_cast<float>(q1), s))) << 16);
+        for (int g = 0; g < 4; ++g) {
+            const uint32_t pair = (g < 2 ? v[i].x : v[i].y) >> (16 * (g & 1));
+            const uint32_t nib = m[i] >> (4 * g);
+            const unsigned long long q = (static_cast<unsigned long long>(ternary_bf16(pair & 0xFFu)) << (16 * (nib & 3u))) |
+                                         (static_cast<unsigned long long>(ternary_bf16((pair >> 8) & 0xFFu)) << (16 * ((nib >> 2) & 3u)));
+            o[2 * g] = static_cast<uint32_t>(q);
+            o[2 * g + 1] = static_cast<uint32_t>(q >> 32);
         }
-        uint4* dst = reinterpret_cast<uint4*>(X + static_cast<size_t>(t) * K + static_cast<size_t>(ch) * 16);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        st_global_32b(out + static_cast<size_t>(r0 + 16u * i) * j.K, o);
+    }
+}
+
+// Item of x_q: 64 tokens x 128 columns.
+__device__ __forceinline__ void prep_x_item(const PrepJob& j, int item, int tid) {
+    const int KB = j.K >> 7;
+    const int kb = item % KB, t0 = (item / KB) * kPrepItemTokens;
+    const int r0 = tid >> 3, c = tid & 7;                      // 16 codes
+    const size_t tb8 = xq_tb8(j.T);
+    uint4 v[4];
+    float s[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int t = t0 + r0 + 16 * i;
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        s[i] = 0.0f;
+        if (t < j.T) {
+            v[i] = __ldg(reinterpret_cast<const uint4*>(j.xq + (static_cast<size_t>(kb) * tb8 + (static_cast<uint32_t>(t) >> 3)) * 1024 + (t & 7) * 128 + ((c ^ (t & 7)) << 4)));
+            s[i] = __ldg(j.a_scale + t);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int t = t0 + r0 + 16 * i;
+        const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        uint32_t o[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            const float q0 = static_cast<float>(static_cast<int8_t>((w[p >> 1] >> (16 * (p & 1))) & 0xFFu));
+            const float q1 = static_cast<float>(static_cast<int8_t>((w[p >> 1] >> (16 * (p & 1) + 8)) & 0xFFu));
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(o[p]) : "f"(__fmul_rn(q1, s[i])), "f"(__fmul_rn(q0, s[i])));
+        }
+        if (t < j.T) st_global_32b(j.x_out + static_cast<size_t>(t) * j.K + static_cast<size_t>(kb) * 128 + c * 16, o);
+    }
+}
+
+__global__ void __launch_bounds__(kPrepThreads)
+backward_prep_kernel(const PrepJob j) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int items = j.w_items + j.x_items;
+    for (int i = blockIdx.x; i < items; i += gridDim.x) {
+        if (i < j.w_items) prep_w_item(j, i, threadIdx.x);
+        else prep_x_item(j, i - j.w_items, threadIdx.x);
     }
 }
 

@@ -1,24 +1,32 @@
-// D[M][Nn] = A[M][Kc] * B[Nn][Kc]^T in bf16 with fp32 accumulation on the 5th-generation tensor cores --
-// the two contractions of the layer's backward pass (Sec. 2.3, Eq. 5: dX = dY w_masked with K-major
-// operands, dW = dY^T x_q with MN-major ones; backward_prep.cuh makes the bf16 operands).
+// The two contractions of a layer's backward pass (Sec. 2.3, Eq. 5) in bf16 with fp32 accumulation on the 5th-generation
+// tensor cores, in ONE persistent launch:
 //
-// Same skeleton as the int8 CTA-pair kernel (gemm_pair_tcgen05.cuh): two CTAs of a cluster issue one
-// `tcgen05.mma.cta_group::2.kind::f16` (M = 256: each CTA supplies 128 rows of A and half of the B tile
-// and keeps its 128 x BN slice of the accumulator in its own tensor memory), persistent over output tiles
-// of 256 x BN (BN runtime, multiple of 16, <= 256), operands fetched by TMA (plain row-major tensors,
-// 128-byte swizzle: a box of 64 bf16 x rows IS the K-major shared-memory image), the full barrier of a
-// stage lives in the leader CTA and collects both CTAs' bytes, `tcgen05.commit ... multicast::cluster`
-// releases stages and publishes accumulators in both CTAs.  The two 256-column halves of tensor memory
-// alternate as accumulators, so the epilogue of a tile (8 warps: TMEM -> registers -> optional scale ->
-// row-major fp32 or bf16 stores; a thread owns an output row and writes 128 B or 64 B runs of it) runs
-// under the next tile's MMAs.  No TMA multicast.  All waits are bounded.
+//   part 0   dW [N][K] = dY^T x_q      contraction over the tokens; A = dY [T][N] read MN-major
+//   part 1   dX [T][K] = dY W_eff      contraction over the features; A = dY [T][N] read K-major; times bf16(w_scale)
+//
+// B (x_q [T][K] resp. W_eff [N][K], backward_prep.cuh) is read MN-major in both.  Two CTAs of a cluster issue one
+// `tcgen05.mma.cta_group::2.kind::f16` (M = 256: each CTA supplies 128 rows of A and half of the B tile and keeps its
+// 128 x BN slice of the accumulator in its own tensor memory).  Operands come by TMA from plain row-major tensors, six
+// stages of 64 contraction steps; the full barrier of a stage lives in the leader CTA and collects both CTAs' bytes,
+// `tcgen05.commit ... multicast::cluster` releases stages and publishes accumulators in both CTAs.  The two 256-column
+// halves of tensor memory alternate as accumulators, so the epilogue of a tile (a thread owns an output row and writes
+// 128 B or 64 B runs of it) runs under the next tile's MMAs.  No TMA multicast.  All waits are bounded.
 //
 //   warps        0 TMA producer (both CTAs), 1 MMA issuer (leader CTA only; both allocate TMEM),
 //                2..9 epilogue: warp w reads TMEM lane quarter w % 4, the even (w < 6) or odd 32-column chunks
-//   per stage    A 128 rows x 128 B (16 KB) | B BN/2 rows x 128 B (<= 16 KB): K step of 64 elements,
-//                four MMAs of K = 16
+//   per stage    A 128 rows x 128 B (16 KB) | B BN/2 rows x 128 B (<= 16 KB): K step of 64 elements, four MMAs of K = 16
+//
+// Bound by the tensor cores under the power cap: 256 x 256 x 64 takes 0.36 us per pair, 1.7 PFLOP/s while all pairs work.
+// Both gradients, preparation included, calls back to back at 4096 tokens (us, two launches with their own waves and
+// separate preparation kernels before): 2560 -> 3840 135 -> 119, 2560 -> 2560 110 -> 80, 2560 -> 6912 246 -> 207,
+// 6912 -> 2560 234 -> 209.  Converting one operand on spare warps of this kernel, under the other part's tiles, was slower
+// (138, 110, 228, 247): the conversion's loads and stores cost the main loop more than the launch they save.
+//
+// Tiles are 256 x 256, or halves of 256 x 128 where those even out the pairs (backward_plan.h): every pair has a list of
+// its own, made so that all end at about the same time although the two parts' tiles differ in length.
 #pragma once
 
+#include "backward_plan.h"
 #include "gemm_pair_tcgen05.cuh"
 
 namespace sbn {
@@ -28,26 +36,20 @@ constexpr int kBf16Threads = 32 * (2 + kBf16EpiWarps);
 constexpr int kBf16StageA = 128 * 128;                      // bytes
 constexpr int kBf16StageB = 128 * 128;                      // bytes reserved (BN/2 <= 128 rows)
 constexpr int kBf16StageBytes = kBf16StageA + kBf16StageB;
-constexpr int kBf16Stages = 6;
+constexpr int kBf16Stages = 7;
 constexpr int kBf16SmemBytes = kBf16Stages * kBf16StageBytes + kBarrierBytes;
 static_assert(kBf16SmemBytes <= 232448, "shared memory overflow");
 
-struct Bf16GemmParams {
-    int M, Nn, Kc;               // output rows, output columns, contraction length (elements)
-    int bn;                      // output columns per tile
-    void* out;                   // [M][Nn] row-major, fp32 or bf16
-    int out_bf16;
+struct Bf16Part {
+    int M, Kc;                   // output rows, contraction length
+    void* out;                   // [M][K] row-major
+    int out_bf16;                // else fp32
     const float* scale;          // device, one fp32, or null: the result is multiplied by bf16(scale)
-    // Two launches of this kernel that do not depend on each other (dW and dX of one backward call) share
-    // the machine at the seam: the first one's last wave leaves pairs idle, the second one's CTAs move in as
-    // soon as pairs are free instead of waiting for the whole grid.
-    //   first launch:  signal_after_wait -- it lets its dependents go only after its own dependency wait, so
-    //                  that whatever it waited for is complete for them too;
-    //   second launch: wait_at_end -- no dependency wait before its work (its inputs are complete by the rule
-    //                  above), but one before it exits: it is not complete before the first launch is, and the
-    //                  kernels after it in the stream see both results.
-    int signal_after_wait = 0;
-    int wait_at_end = 0;
+};
+struct Bf16GemmParams {
+    Bf16Part part[2];            // dW, dX
+    int Nn;                      // output columns of both (K)
+    BackwardPlan plan;
 };
 
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar_cluster_addr) {
@@ -64,27 +66,37 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, u
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// Instruction descriptor for kind::f16: D = fp32, A = B = bf16; both K-major, or both MN-major (the
-// contraction index is the SLOW index of the operands in memory: bits 15 / 16).
-__host__ __device__ constexpr uint32_t make_idesc_bf16(int mma_m, int mma_n, bool mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? ((1u << 15) | (1u << 16)) : 0u) |
+// Instruction descriptor for kind::f16: D = fp32, A = B = bf16; A K-major or MN-major (bit 15), B MN-major (bit 16).
+__host__ __device__ constexpr uint32_t make_idesc_bf16(int mma_m, int mma_n, bool a_mn_major) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major ? (1u << 15) : 0u) | (1u << 16) |
            (static_cast<uint32_t>(mma_n >> 3) << 17) | (static_cast<uint32_t>(mma_m >> 4) << 24);
 }
 
-// MN = false (K-major operands):  tmap_a: [M][Kc] bf16, box {64, 128};  tmap_b: [Nn][Kc] bf16, box {64, bn / 2}.
-// MN = true (MN-major operands: A is stored [Kc][M], B is stored [Kc][Nn], i.e. D = A^T B without a
-// transposed copy of either):  tmap_a: [Kc][M], box {64 of M, 64 of Kc};  tmap_b: [Kc][Nn], box {64, 64};
-// bn must be 128 or 256.  A box of 64 contraction rows x 128 B is the MN-major shared-memory image of a
-// block of 64 output rows (or columns): 8-row groups 1 KB apart along the contraction (the stride offset),
-// blocks 8 KB apart (the leading offset); an MMA of K = 16 starts 2 KB further per step.
-template <bool MN>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBf16Threads, 1)
-gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, const Bf16GemmParams p) {
-    constexpr int STAGES = kBf16Stages;
-    const int BN = p.bn;
-    const int half_bn = BN >> 1;
+struct Bf16Tile { int part, m0, n0, bn; };
+// Entry `i` of this pair in segment `g` (backward_plan.h).
+__device__ __forceinline__ Bf16Tile bf16_tile(const Bf16GemmParams& p, int g, int pair, int i) {
+    const BackwardSegment& sg = p.plan.seg[g];
+    const int u = sg.index(pair, i);
+    const int tiles_m = (p.part[sg.part].M + 255) / 256;
+    const int tile = sg.half ? sg.first_tile + (u >> 1) : u;
+    return Bf16Tile{sg.part, (tile % tiles_m) * 256, (tile / tiles_m) * 256 + (sg.half ? (u & 1) * 128 : 0), sg.half ? 128 : 256};
+}
 
-    if (!p.signal_after_wait) pdl_launch_dependents();
+// Tensor maps.  MN-major operands are fetched as 3-D boxes {64 columns, 64 contraction rows, 1 or 2 blocks of 64 columns}:
+// a block of 64 rows x 128 B is the MN-major shared-memory image of 64 output rows (or columns) -- 8-row groups 1 KB apart
+// along the contraction (the stride offset), blocks 8 KB apart (the leading offset); an MMA of K = 16 starts 2 KB further per
+// step.  One instruction per operand and stage: TMA takes about 64 ns per instruction and 2.8 ns per KB, so that with one
+// instruction per block (four per stage) the loads, 0.35 us per stage, paced the loop, not the MMAs (0.28).
+struct Bf16Maps {
+    CUtensorMap aw;              // dY [T][N] for dW: two blocks
+    CUtensorMap ax;              // dY [T][N] for dX: K-major, box {64 of N, 128 tokens}
+    CUtensorMap b[2][2];         // x_q [T][K], W_eff [N][K]: two blocks, one block (half tiles)
+};
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBf16Threads, 1)
+backward_gemm_kernel(const __grid_constant__ Bf16Maps maps, const __grid_constant__ Bf16GemmParams p) {
+    constexpr int STAGES = kBf16Stages;
+
+    pdl_launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = smem_u32(smem_raw);
     if (smem_base & 1023u) {          // swizzled tiles need 1 KB alignment; identical in every CTA
@@ -103,11 +115,6 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair_id = blockIdx.x >> 1;
-    const int num_pairs = gridDim.x >> 1;
-    const int tiles_m = (p.M + 255) / 256;
-    const int tiles_n = (p.Nn + BN - 1) / BN;
-    const int num_tiles = tiles_m * tiles_n;
-    const int k_stages = (p.Kc + 63) / 64;
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
@@ -129,72 +136,78 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
     __syncthreads();
     cluster_sync_all();
     tcgen05_fence_after();
-    if (!p.wait_at_end) pdl_wait();      // nothing above touches global memory
-    if (p.signal_after_wait) pdl_launch_dependents();
+    pdl_wait();                       // nothing above touches global memory
     uint32_t tmem_base;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            tma_prefetch_desc(&tmap_a);
-            tma_prefetch_desc(&tmap_b);
-            const uint32_t bytes_per_cta = static_cast<uint32_t>(kBf16StageA + half_bn * 128);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
-                const int m0 = (tile % tiles_m) * 256 + static_cast<int>(rank) * 128;
-                const int n0 = (tile / tiles_m) * BN + static_cast<int>(rank) * half_bn;
-                for (int ks = 0; ks < k_stages; ++ks) {
-                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t full_leader = map_to_cta(bar_full + 8 * stage, 0);
-                    if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, 2 * bytes_per_cta);
-                    const uint32_t st = smem_base + stage * kBf16StageBytes;
-                    // rows or columns beyond the tensors are zero-filled by the hardware and still count their full size
-                    if constexpr (MN) {
-                        tma_load_2d_pair(st, &tmap_a, m0, ks * 64, full_leader);
-                        tma_load_2d_pair(st + 8192, &tmap_a, m0 + 64, ks * 64, full_leader);
-                        for (int j = 0; j < half_bn / 64; ++j)
-                            tma_load_2d_pair(st + kBf16StageA + j * 8192, &tmap_b, n0 + 64 * j, ks * 64, full_leader);
-                    } else {
-                        tma_load_2d_pair(st, &tmap_a, ks * 64, m0, full_leader);
-                        tma_load_2d_pair(st + kBf16StageA, &tmap_b, ks * 64, n0, full_leader);
+            for (int g = 0; ok && g < p.plan.segments; ++g) {
+                for (int i = 0; ok && i < p.plan.seg[g].count(pair_id); ++i) {
+                    const Bf16Tile t = bf16_tile(p, g, pair_id, i);
+                    const int half_bn = t.bn >> 1;
+                    const uint32_t bytes_per_cta = static_cast<uint32_t>(kBf16StageA + half_bn * 128);
+                    const int m0 = t.m0 + static_cast<int>(rank) * 128;
+                    const int n0 = t.n0 + static_cast<int>(rank) * half_bn;
+                    const int k_stages = (p.part[t.part].Kc + 63) / 64;
+                    const CUtensorMap* tb = &maps.b[t.part][t.bn == 128];
+                    for (int ks = 0; ks < k_stages; ++ks) {
+                        if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
+                        const uint32_t full_leader = map_to_cta(bar_full + 8 * stage, 0);
+                        if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, 2 * bytes_per_cta);
+                        const uint32_t st = smem_base + stage * kBf16StageBytes;
+                        // rows or columns beyond the tensors are zero-filled by the hardware and still count their full size
+                        if (t.part == 0) {
+                            tma_load_3d_pair(st, &maps.aw, 0, ks * 64, m0 >> 6, full_leader);
+                        } else {
+                            tma_load_2d_pair(st, &maps.ax, ks * 64, m0, full_leader);
+                        }
+                        tma_load_3d_pair(st + kBf16StageA, tb, 0, ks * 64, n0 >> 6, full_leader);
+                        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     }
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader)
         if (rank == 0 && lane == 0) {
-            const uint32_t idesc = make_idesc_bf16(256, BN, MN);
             int stage = 0;
             uint32_t phase = 0;
             uint32_t acc_iter = 0;
             bool ok = true;
-            for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
-                const uint32_t buf = acc_iter & 1u;
-                const uint32_t acc_phase = (acc_iter >> 1) & 1u;
-                if (!mbar_wait(bar_acc_empty + 8 * buf, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-                tcgen05_fence_after();
-                const uint32_t d_tmem = tmem_base + buf * 256u;
-                for (int ks = 0; ks < k_stages; ++ks) {
-                    if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { ok = false; break; }
+            for (int g = 0; ok && g < p.plan.segments; ++g) {
+                const int part = p.plan.seg[g].part;
+                const uint32_t idesc = make_idesc_bf16(256, p.plan.seg[g].half ? 128 : 256, part == 0);
+                const int k_stages = (p.part[part].Kc + 63) / 64;
+                // K = 16 elements per instruction: 16 rows of an MN-major operand, 32 B along a row of a K-major one
+                const uint64_t a_step = part == 0 ? (2048 >> 4) : (32 >> 4);
+                const uint32_t a_lbo = part == 0 ? 8192 : 16;
+                for (int i = 0; ok && i < p.plan.seg[g].count(pair_id); ++i) {
+                    const uint32_t buf = acc_iter & 1u;
+                    const uint32_t acc_phase = (acc_iter >> 1) & 1u;
+                    if (!mbar_wait(bar_acc_empty + 8 * buf, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                     tcgen05_fence_after();
-                    const uint32_t st = smem_base + stage * kBf16StageBytes;
-                    const uint64_t a_desc = MN ? make_smem_desc(st, 8192, 1024, kSwz128) : make_smem_desc(st, 16, 1024, kSwz128);
-                    const uint64_t b_desc = MN ? make_smem_desc(st + kBf16StageA, 8192, 1024, kSwz128) : make_smem_desc(st + kBf16StageA, 16, 1024, kSwz128);
-                    constexpr uint64_t kStep = MN ? (2048 >> 4) : (32 >> 4);      // K = 16 elements per instruction: 16 rows, or 32 B along a row
+                    const uint32_t d_tmem = tmem_base + buf * 256u;
+                    for (int ks = 0; ks < k_stages; ++ks) {
+                        if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                        tcgen05_fence_after();
+                        const uint32_t st = smem_base + stage * kBf16StageBytes;
+                        const uint64_t a_desc = make_smem_desc(st, a_lbo, 1024, kSwz128);
+                        const uint64_t b_desc = make_smem_desc(st + kBf16StageA, 8192, 1024, kSwz128);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        mma_bf16_pair(d_tmem, a_desc + kStep * q, b_desc + kStep * q, idesc, (ks | q) != 0 ? 1u : 0u);
-                    tcgen05_commit_pair(bar_empty + 8 * stage);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                        for (int q = 0; q < 4; ++q)
+                            mma_bf16_pair(d_tmem, a_desc + a_step * q, b_desc + (2048u >> 4) * q, idesc, (ks | q) != 0 ? 1u : 0u);
+                        tcgen05_commit_pair(bar_empty + 8 * stage);
+                        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    }
+                    if (!ok) break;
+                    tcgen05_commit_pair(bar_acc_full + 8 * buf);
+                    ++acc_iter;
                 }
-                if (!ok) break;
-                tcgen05_commit_pair(bar_acc_full + 8 * buf);
-                ++acc_iter;
             }
         }
     } else {
@@ -202,55 +215,48 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         const int quarter = warp & 3;                     // TMEM lane quarter this warp may read
         const int parity = (warp - 2) >> 2;               // even or odd 32-column chunks
         const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
-        float scale = 1.0f;
-        if (p.scale != nullptr) scale = __uint_as_float(f32_to_bf16_rne(__ldg(p.scale)) << 16);    // the scale as a bf16 run holds it
         uint32_t acc_iter = 0;
         bool ok = true;
-        for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
-            const int m = (tile % tiles_m) * 256 + static_cast<int>(rank) * 128 + quarter * 32 + lane;
-            const int n_tile = (tile / tiles_m) * BN;
-            const uint32_t buf = acc_iter & 1u;
-            const uint32_t acc_phase = (acc_iter >> 1) & 1u;
-            const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty + 8 * buf, 0);
-            if (!mbar_wait(bar_acc_full + 8 * buf, acc_phase, abort_flag)) { ok = false; break; }
-            tcgen05_fence_after();
-            const uint32_t t_addr = tmem_base + lane_base + buf * 256u;
-            const int chunks = (BN + 31) >> 5;            // a last chunk of 16 columns when BN % 32 == 16
-            int my_last = -1;
-            for (int c = parity; c < chunks; c += 2) my_last = c;
-            if (my_last < 0) {
-                tcgen05_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
-            }
+        for (int g = 0; ok && g < p.plan.segments; ++g) {
+            const Bf16Part& pt = p.part[p.plan.seg[g].part];
+            float scale = 1.0f;
+            if (pt.scale != nullptr) scale = __uint_as_float(f32_to_bf16_rne(__ldg(pt.scale)) << 16);    // the scale as a bf16 run holds it
+            for (int i = 0; i < p.plan.seg[g].count(pair_id); ++i) {
+                const Bf16Tile t = bf16_tile(p, g, pair_id, i);
+                const int m = t.m0 + static_cast<int>(rank) * 128 + quarter * 32 + lane;
+                const uint32_t buf = acc_iter & 1u;
+                const uint32_t acc_phase = (acc_iter >> 1) & 1u;
+                const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty + 8 * buf, 0);
+                if (!mbar_wait(bar_acc_full + 8 * buf, acc_phase, abort_flag)) { ok = false; break; }
+                tcgen05_fence_after();
+                const uint32_t t_addr = tmem_base + lane_base + buf * 256u;
+                const int chunks = t.bn >> 5;
 #pragma unroll 1
-            for (int c = parity; c < chunks; c += 2) {
-                const int width = min(32, BN - c * 32);   // 32 or 16
+                for (int c = parity; c < chunks; c += 2) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (h * 16 < width) {
+                    for (int h = 0; h < 2; ++h) {
                         uint32_t r[16];
                         tmem_ld_32x32b_x16(t_addr + static_cast<uint32_t>(c * 32 + h * 16), r);
                         tmem_ld_wait();
-                        if (c == my_last && (h == 1 || width == 16)) {
+                        if (c + 2 >= chunks && h == 1) {
                             tcgen05_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
                         }
-                        const int n = n_tile + c * 32 + h * 16;
-                        if (m < p.M && n < p.Nn) {        // Nn % 16 == 0: a run of 16 columns is in or out as a whole
-                            if (p.out_bf16) {
+                        const int n = t.n0 + c * 32 + h * 16;
+                        if (m < pt.M && n < p.Nn) {       // Nn % 16 == 0: a run of 16 columns is in or out as a whole
+                            if (pt.out_bf16) {
                                 uint32_t pk[8];
 #pragma unroll
                                 for (int j = 0; j < 8; ++j) {
                                     const float v0 = __fmul_rn(__uint_as_float(r[2 * j]), scale), v1 = __fmul_rn(__uint_as_float(r[2 * j + 1]), scale);
                                     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(v1), "f"(v0));
                                 }
-                                uint4* o = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.Nn + n);
+                                uint4* o = reinterpret_cast<uint4*>(static_cast<uint16_t*>(pt.out) + static_cast<size_t>(m) * p.Nn + n);
                                 o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                                 o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
                             } else {
-                                float4* o = reinterpret_cast<float4*>(static_cast<float*>(p.out) + static_cast<size_t>(m) * p.Nn + n);
+                                float4* o = reinterpret_cast<float4*>(static_cast<float*>(pt.out) + static_cast<size_t>(m) * p.Nn + n);
 #pragma unroll
                                 for (int j = 0; j < 4; ++j)
                                     o[j] = make_float4(__fmul_rn(__uint_as_float(r[4 * j]), scale), __fmul_rn(__uint_as_float(r[4 * j + 1]), scale),
@@ -259,8 +265,8 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                         }
                     }
                 }
+                ++acc_iter;
             }
-            ++acc_iter;
         }
     }
 
@@ -273,7 +279,6 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         tcgen05_fence_after();
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
-    if (p.wait_at_end) pdl_wait();
 }
 
 }  // namespace sbn

@@ -113,6 +113,20 @@ static bool encode_2d_bf16_sw128(CUtensorMap* map, const void* base, uint64_t in
     return r == CUDA_SUCCESS;
 }
 
+// Row-major bf16 matrix [rows][cols], cols % 64 == 0, fetched as `blocks` blocks of 64 columns x 64 rows, block by block.
+static bool encode_3d_bf16_blocks(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t blocks) {
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {64, rows, cols / 64};
+    cuuint64_t strides[2] = {cols * 2, 128};
+    cuuint32_t box[3] = {64, 64, blocks};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 static inline bool misaligned(const void* p, size_t a) {
     return (reinterpret_cast<uintptr_t>(p) & (a - 1)) != 0;
 }
@@ -481,68 +495,50 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
 }
 
 // ---- backward GEMMs (bf16) -------------------------------------------------------------------------
-struct BackwardWs {                    // W_eff^T [K][N] and x_q [T][K], both bf16
-    size_t wt_off, xq_off, total;
+struct BackwardWs {                    // W_eff [N][K] and x_q [T][K], both bf16
+    size_t w_off, xq_off, total;
 };
 static BackwardWs backward_ws_layout(int T, int N, int K) {
     BackwardWs w;
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
-    w.wt_off = 0;
+    w.w_off = 0;
     w.xq_off = up(static_cast<size_t>(K) * N * 2);
     w.total = w.xq_off + up(static_cast<size_t>(T) * K * 2);
     return w;
 }
 
-// Output columns per tile: fewest waves over the 74 CTA pairs, weighted by what a tile costs (the A part of a
-// stage is fixed, the B part grows with the tile's width).
-static int pick_bf16_bn(int M, int Nn) {
-    const long tiles_m = (M + 255) / 256;
-    int best = 256;
-    double best_cost = 1e300;
-    for (int bn = 256; bn >= 128; bn -= 16) {
-        const long tiles = tiles_m * ((Nn + bn - 1) / bn);
-        const long waves = (tiles + kNumSMs / 2 - 1) / (kNumSMs / 2);
-        const double cost = static_cast<double>(waves) * (256.0 + bn);
-        if (cost < best_cost) { best_cost = cost; best = bn; }
-    }
-    return best;
-}
-
-// D[M][Nn] = A[M][Kc] B[Nn][Kc]^T (bf16 in, fp32 accumulation), optionally times bf16(*scale).
-// mn_major: A is stored [Kc][M] (row stride lda) and B [Kc][Nn] (row stride ldb): D = A^T B.
-static sbn_status run_gemm_bf16(bool mn_major, const void* A, int M, uint64_t lda, const void* B, int Nn, uint64_t ldb, int Kc,
-                                void* out, bool out_bf16, const float* scale, cudaStream_t stream,
-                                bool signal_after_wait = false, bool wait_at_end = false) {
+static sbn_status run_backward(const void* dY, int T, const int8_t* xq, const float* a_scale, const int8_t* vals, const uint8_t* meta,
+                               const float* w_scale, int N, int K, void* dX, float* dW, void* ws, cudaStream_t stream) {
+    const BackwardWs lay = backward_ws_layout(T, N, K);
+    char* base = static_cast<char*>(ws);
+    const int KB = K / kBK, tiles_k = (K + 255) / 256;
+    const int w_items = dX ? KB * (N / kBM) : 0;
+    const int x_items = dW ? KB * ((T + kPrepItemTokens - 1) / kPrepItemTokens) : 0;
+    const int tiles[2] = {dW ? (N + 255) / 256 * tiles_k : 0, dX ? (T + 255) / 256 * tiles_k : 0};
+    const int stages[2] = {(T + 63) / 64, N / 64};
     Bf16GemmParams p;
-    p.signal_after_wait = signal_after_wait ? 1 : 0;
-    p.wait_at_end = wait_at_end ? 1 : 0;
-    p.M = M; p.Nn = Nn; p.Kc = Kc;
-    p.bn = g_force_token_tile < 0 ? std::min(256, std::max(64, (-g_force_token_tile) / 16 * 16)) : pick_bf16_bn(M, Nn);
-    if (mn_major) p.bn = p.bn > 128 ? 256 : 128;                // whole 64-column blocks per CTA
-    p.out = out; p.out_bf16 = out_bf16 ? 1 : 0;
-    p.scale = scale;
-    CUtensorMap ta, tb;
-    bool ok;
-    if (mn_major) {
-        ok = encode_2d_bf16_sw128(&ta, A, static_cast<uint64_t>(M), static_cast<uint64_t>(Kc), lda, 64) &&
-             encode_2d_bf16_sw128(&tb, B, static_cast<uint64_t>(Nn), static_cast<uint64_t>(Kc), ldb, 64);
-    } else {
-        ok = encode_2d_bf16_sw128(&ta, A, static_cast<uint64_t>(Kc), static_cast<uint64_t>(M), lda, 128) &&
-             encode_2d_bf16_sw128(&tb, B, static_cast<uint64_t>(Kc), static_cast<uint64_t>(Nn), ldb, static_cast<uint32_t>(p.bn / 2));
-    }
+    p.part[0] = Bf16Part{N, T, dW, 0, nullptr};
+    p.part[1] = Bf16Part{T, N, dX, 1, w_scale};
+    p.Nn = K;
+    const PrepJob job{reinterpret_cast<const uint8_t*>(vals), meta, reinterpret_cast<uint16_t*>(base + lay.w_off),
+                      reinterpret_cast<const uint8_t*>(xq), a_scale, reinterpret_cast<uint16_t*>(base + lay.xq_off), T, N, K, w_items, x_items};
+    p.plan = plan_backward(tiles, stages, 0, g_force_token_tile < 0 ? (-g_force_token_tile <= 128 ? 1 : 0) : -1, nullptr);
+
+    const uint64_t t = static_cast<uint64_t>(T), n = static_cast<uint64_t>(N), k = static_cast<uint64_t>(K);
+    Bf16Maps maps;
+    bool ok = encode_3d_bf16_blocks(&maps.aw, dY, n, t, 2) && encode_2d_bf16_sw128(&maps.ax, dY, n, t, n, 128);
+    for (int blocks = 1; ok && blocks <= 2; ++blocks)
+        ok = encode_3d_bf16_blocks(&maps.b[0][2 - blocks], base + lay.xq_off, k, t, blocks) &&
+             encode_3d_bf16_blocks(&maps.b[1][2 - blocks], base + lay.w_off, k, n, blocks);
     if (!ok) return SBN_ERR_CUDA;
-    const int tiles = ((M + 255) / 256) * ((Nn + p.bn - 1) / p.bn);
-    const int pairs = tiles < kNumSMs / 2 ? tiles : kNumSMs / 2;
-    cudaError_t err;
-    if (mn_major) {
-        if (!ensure_dynamic_smem<gemm_bf16_pair_kernel<true>>(kBf16SmemBytes)) return SBN_ERR_CUDA;
-        err = launch_kernel(gemm_bf16_pair_kernel<true>, dim3(2 * pairs), dim3(kBf16Threads), kBf16SmemBytes, stream, ta, tb, p);
-    } else {
-        if (!ensure_dynamic_smem<gemm_bf16_pair_kernel<false>>(kBf16SmemBytes)) return SBN_ERR_CUDA;
-        err = launch_kernel(gemm_bf16_pair_kernel<false>, dim3(2 * pairs), dim3(kBf16Threads), kBf16SmemBytes, stream, ta, tb, p);
-    }
+    if (!ensure_dynamic_smem<backward_gemm_kernel>(kBf16SmemBytes)) return SBN_ERR_CUDA;
+    const int blocks = std::max(1, std::min(w_items + x_items, 16 * device_sm_count()));
+    if (launch_kernel(backward_prep_kernel, dim3(blocks), dim3(kPrepThreads), 0, stream, job) != cudaSuccess) return SBN_ERR_CUDA;
     ++g_launch_count;
-    return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+    if (launch_kernel(backward_gemm_kernel, dim3(2 * kBackwardPairs), dim3(kBf16Threads), kBf16SmemBytes, stream, maps, p) != cudaSuccess)
+        return SBN_ERR_CUDA;
+    ++g_launch_count;
+    return SBN_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -980,39 +976,7 @@ sbn_status sbn_bitlinear_backward(const void* dY_bf16, int T, const int8_t* xq, 
         (dW && (misaligned(dW, 16) || misaligned(xq, 16) || misaligned(a_scale, 4))))
         return SBN_ERR_ALIGN;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    char* base = static_cast<char*>(ws);
-    uint16_t* Wt = reinterpret_cast<uint16_t*>(base + lay.wt_off);
-    uint16_t* XT = reinterpret_cast<uint16_t*>(base + lay.xq_off);
-    const int KB = K / kBK, NB = N / kBM;
-    // Operands first (two small memory-bound kernels), then the GEMMs.  With both gradients wanted the
-    // weight-gradient GEMM goes first and the input-gradient GEMM moves into the pairs its last wave
-    // leaves idle (Bf16GemmParams: signal_after_wait / wait_at_end): the two do not depend on each other.
-    const bool both = dX_bf16 != nullptr && dW != nullptr;
-    if (dX_bf16) {
-        if (launch_kernel(weff_t_bf16_kernel, dim3(KB * NB), dim3(kPrepThreads), 0, s, reinterpret_cast<const uint8_t*>(vals), meta, N, K, Wt) != cudaSuccess)
-            return SBN_ERR_CUDA;
-        ++g_launch_count;
-    }
-    if (dW) {
-        const unsigned blocks = static_cast<unsigned>(std::min<size_t>((static_cast<size_t>(T) * (K / 16) + kPrepThreads - 1) / kPrepThreads,
-                                                                           static_cast<size_t>(device_sm_count()) * 8));
-        if (launch_kernel(xq_bf16_kernel, dim3(blocks), dim3(kPrepThreads), 0, s, reinterpret_cast<const uint8_t*>(xq), a_scale, T, K, XT) != cudaSuccess)
-            return SBN_ERR_CUDA;
-        ++g_launch_count;
-        // dW[n][k] = sum_t dY[t][n] x_q[t][k]
-        // both operands as they lie in memory, token-major: dY [T][N] and x_q [T][K] (bf16 copy of the
-        // fake-quantised activations); the MMA reads them MN-major, the contraction runs down the rows
-        const sbn_status st = run_gemm_bf16(true, dY_bf16, N, static_cast<uint64_t>(N), XT, K, static_cast<uint64_t>(K), T, dW, false, nullptr, s,
-                                            both, false);
-        if (st != SBN_OK) return st;
-    }
-    if (dX_bf16) {
-        // dX[t][k] = bf16(scale) * sum_n dY[t][n] W_eff[n][k]: A = dY [T][N], B = W_eff^T [K][N]
-        const sbn_status st = run_gemm_bf16(false, dY_bf16, T, static_cast<uint64_t>(N), Wt, K, static_cast<uint64_t>(N), N, dX_bf16, true, w_scale, s,
-                                            false, both);
-        if (st != SBN_OK) return st;
-    }
-    return SBN_OK;
+    return run_backward(dY_bf16, T, xq, a_scale, vals, meta, w_scale, N, K, dX_bf16, dW, ws, s);
 }
 
 sbn_status sbn_check_status(void* stream) {

@@ -99,6 +99,16 @@ def test_backward_parity_every_tile_width(bn):
     _assert_dx(c, dX)
 
 
+# More tiles than CTA pairs: rounds of all pairs, remainders, half tiles of either gradient, a last tile of 128 columns, one
+# gradient whose tiles are too few to go round, the last tokens of a tile missing.
+@pytest.mark.parametrize("T,N,K", [(300, 2560, 2176), (1100, 1280, 2560), (64, 1280, 6912), (2050, 1024, 1152)])
+def test_backward_parity_tile_lists(T, N, K):
+    c = _case(T, N, K, seed=300 + T + N + K)
+    dX, dW = _gpu_backward(c)
+    _assert_dw(c, dW)
+    _assert_dx(c, dX)
+
+
 def test_backward_weight_gradient_reaches_pruned_weights():
     # Eq. 5: the mask is transparent -- a mask-gated gradient is the negative control
     c = _case(200, 256, 512, seed=270)
