@@ -375,7 +375,7 @@ sbn_status sbn_bitlinear(const int8_t *xq, const float *a_scale, int T,
  *   dX_bf16   device out, bf16 [T][K], or NULL to skip
  *   dW        device out, fp32 [N][K], or NULL to skip (overwritten, not accumulated)
  *   ws        device workspace of sbn_workspace_bytes(SBN_OP_BACKWARD, T, N, K) bytes, 256-byte aligned
- *             (W_eff^T [K][N] and x_q [T][K] in bf16); no initialisation needed
+ *             (W_eff [N][K] and x_q [T][K] in bf16); no initialisation needed
  * The bias gradient (a column sum of dY) is not computed here.
  */
 sbn_status sbn_bitlinear_backward(const void *dY_bf16, int T, const int8_t *xq, const float *a_scale,
@@ -431,9 +431,11 @@ const char *sbn_status_string(sbn_status s);
 /* Tuning/diagnostic knob (host state, not thread-safe).  token_tile: 0 = automatic; 64, 128 or
  * 256 = force the single-CTA kernel with that token-tile width; a negative value -BN = force the
  * CTA-pair kernel with BN tokens per tile (rounded to a multiple of 16, capped at 240 sparse /
- * 256 dense; with split_k = 1 its variant with one M-tile per CTA).  split_k: 0 = automatic; k > 0 = split K k ways through int32 atomics in the
+ * 256 dense; with split_k = 1 its variant with one M-tile per CTA) and the backward GEMMs with tiles of 128 (BN <= 128) or
+ * 256 columns.  split_k: 0 = automatic; k > 0 = split K k ways through int32 atomics in the
  * workspace (single-CTA kernel); -2, -3, -4, -8 = split K inside thread-block clusters of that many
- * CTAs (token tile 64, or 32 / 128 if token_tile says so; no workspace; -2, -3, -4 also set the
+ * CTAs (token tile 64, or 32 if token_tile says so; a token_tile above 64 selects the wide-tile kernel with that width,
+ * a multiple of 16 up to 256, and clusters of 2 to 8; no workspace; -2, -3, -4 also set the
  * cluster size of sbn_sparse_bitlinear_packed and of the sbn_quant_act_*bitlinear kernels).  Results do not depend on
  * it. */
 void sbn_set_gemm_tuning(int token_tile, int split_k);

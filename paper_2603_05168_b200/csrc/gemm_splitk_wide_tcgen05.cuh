@@ -16,10 +16,10 @@
 //   finish        own partials + S - 1 slots, dequantised (+ bias), stored; a warp stores 32 features of a token
 //
 // Measured (time stamps, 2560 -> 3840, 201 tokens in two tiles of 112, S = 2, 120 CTAs): dependency wait to last MMA 3.0 us
-// for 10 K-blocks, peers' half of P 0.3, exchange 0.75, finish 0.5; chained with the quantiser 9.0 us, against 10.3 unsplit
-// in 64-token tiles and 9.9 with one store per partial sum.  What the exchange costs is per token and peer: 0.03 us x
-// tokens x (S - 1) / S, mostly the copies between the SMs (about 38 GB/s each way per SM), so S stays at 2 to 4.
-// 6912 -> 2560 at 201 tokens 14.4 -> 11.8, 11008 -> 4096 21.3 -> 17.0; dense at 512 tokens 22.4 -> 17.6 and 38.4 -> 27.0.
+// for 10 K-blocks (one per stage), peers' half of P 0.3, exchange 0.75, finish 0.5; chained with the quantiser 8.4 us, against
+// 10.3 unsplit in 64-token tiles and 9.9 with one store per partial sum.  What the exchange costs is per token and peer:
+// 0.03 us x tokens x (S - 1) / S, mostly the copies between the SMs (about 38 GB/s each way per SM), so S stays at 2 to 4.
+// 6912 -> 2560 at 201 tokens 14.4 -> 10.6, 11008 -> 4096 21.3 -> 16.2; dense at 512 tokens 22.4 -> 17.6 and 38.4 -> 26.8.
 //
 // No CTA leaves before all have received everything (cluster barrier): the sources of the copies stay in place.  All
 // mbarrier waits are bounded.
@@ -38,7 +38,12 @@ static_assert(kWideSmemBytes + 1024 + 64 <= 232448, "shared memory overflow");
 constexpr uint32_t kWideTmemCols = 512;                     // accumulator up to 256, metadata above it
 constexpr int kWideMetaCol0 = 256;
 
-__host__ __device__ constexpr int wide_stage_bytes(bool sparse, int bn) { return (sparse ? kBM * (kBK / 2 + kBK / 8) : kBM * kBK) + bn * kBK; }
+__host__ __device__ constexpr int wide_block_bytes(bool sparse, int bn) { return (sparse ? kBM * (kBK / 2 + kBK / 8) : kBM * kBK) + bn * kBK; }
+// K-blocks per stage.  TMA takes about 64 ns per instruction and 2.8 ns per KB, so a stage has two blocks fetched with one
+// instruction per operand -- where three such stages fit (sparse up to 208 tokens, dense up to 160).  Quantiser + GEMM, us,
+// one block / two: 6912 -> 2560 256 tokens in tiles of 128 13.1 / 11.7, 4096 -> 4096 11.9 / 10.5, 11008 -> 4096 201 tokens in
+// one tile 17.1 / 16.2; with room for two stages of two only, tiles of 256 19.0 / 20.3, dense tiles of 208 24.0 / 27.5.
+__host__ __device__ constexpr int wide_group(bool sparse, int bn) { return 6 * wide_block_bytes(sparse, bn) <= kWideDataBytes ? 2 : 1; }
 // Does the exchange fit (P and S - 1 slots of ceil(bn / S) tokens, 512 B per token)?
 __host__ __device__ constexpr bool wide_fits(int bn, int S) { return (bn + (S - 1) * ((bn + S - 1) / S)) * kBM * 4 <= kWideDataBytes; }
 
@@ -47,8 +52,15 @@ __device__ __forceinline__ void bulk_copy_to_cta(uint32_t dst_cluster, uint32_t 
                  ::"r"(dst_cluster), "r"(src_cta), "r"(bytes), "r"(bar_cluster) : "memory");
 }
 
-// tmap_a / tmap_e: weight tiles and metadata as rows of 1 KB; tmap_b: xq as rows of 1 KB, box of bn / 8 rows.
-template <bool SPARSE>
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
+}
+
+// tmap_a / tmap_e: weight tiles and metadata as rows of 1 KB, boxes of G tiles; tmap_b: xq as rows of 1 KB, box of bn / 8
+// (G = 1), or as [K / 128][atoms][1 KB], box of 2 x bn / 8 atoms.  A stage holds G = wide_group K-blocks: weights of all, metadata of all, activations of all.  The
+// second block of a slice of odd length is loaded and not used (beyond the arrays the hardware fills in zeros).
+template <bool SPARSE, int G>
 __global__ void __launch_bounds__(kWideThreads, 1)
 bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                   const __grid_constant__ CUtensorMap tmap_b,
@@ -56,7 +68,7 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                   const GemmParams p, const int bn) {
     constexpr int A_BYTES = SPARSE ? kBM * (kBK / 2) : kBM * kBK;
     constexpr int E_BYTES = SPARSE ? kBM * (kBK / 8) : 0;
-    const int stage_bytes = wide_stage_bytes(SPARSE, bn);
+    const int stage_bytes = G * wide_block_bytes(SPARSE, bn);
     const int stages = min(kWideMaxStages, kWideDataBytes / stage_bytes);
 
     extern __shared__ uint8_t smem_raw[];
@@ -111,15 +123,16 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
     cluster_arrive();                                        // peers' barriers are touched after the matching wait only
     // The weights of the first stages before the dependency wait: no kernel that writes packed weights signals its
     // dependents early (sbn_common.cuh).
-    const int n_pre = min(stages, kb1 - kb0);
-    auto load_weights = [&](int stage, int kb) {
+    const int n_stages = (kb1 - kb0 + G - 1) / G;                // of this CTA's slice
+    const int n_pre = min(stages, n_stages);
+    auto load_weights = [&](int stage, int kb) {             // blocks kb .. kb + G - 1
         const uint32_t full = bar_full + 8 * stage;
         const uint32_t st = smem_base + stage * stage_bytes;
         const int wt = mt * p.k_blocks_total + kb;
         mbar_expect_tx(full, static_cast<uint32_t>(stage_bytes));
         if constexpr (SPARSE) {
             tma_load_2d(st, &tmap_a, 0, wt * 8, full);
-            tma_load_2d(st + A_BYTES, &tmap_e, 0, wt * 2, full);
+            tma_load_2d(st + G * A_BYTES, &tmap_e, 0, wt * 2, full);
         } else {
             tma_load_2d(st, &tmap_a, 0, wt * 16, full);
         }
@@ -128,11 +141,12 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
         tma_prefetch_desc(&tmap_a);
         tma_prefetch_desc(&tmap_b);
         if constexpr (SPARSE) tma_prefetch_desc(&tmap_e);
-        for (int i = 0; i < n_pre; ++i) load_weights(i, kb0 + i);
-        if (kb1 - kb0 > n_pre) {                             // the rest of the slice goes to L2
-            const size_t wt0 = static_cast<size_t>(mt) * p.k_blocks_total + kb0 + n_pre;
-            prefetch_l2_bulk(static_cast<const char*>(p.w_vals) + wt0 * p.w_tile_bytes, static_cast<uint32_t>((kb1 - kb0 - n_pre) * p.w_tile_bytes));
-            if (p.w_meta) prefetch_l2_bulk(static_cast<const char*>(p.w_meta) + wt0 * 2048, static_cast<uint32_t>((kb1 - kb0 - n_pre) * 2048));
+        for (int i = 0; i < n_pre; ++i) load_weights(i, kb0 + G * i);
+        const int rest = kb1 - kb0 - G * n_pre;              // the rest of the slice goes to L2
+        if (rest > 0) {
+            const size_t wt0 = static_cast<size_t>(mt) * p.k_blocks_total + kb0 + G * n_pre;
+            prefetch_l2_bulk(static_cast<const char*>(p.w_vals) + wt0 * p.w_tile_bytes, static_cast<uint32_t>(rest * p.w_tile_bytes));
+            if (p.w_meta) prefetch_l2_bulk(static_cast<const char*>(p.w_meta) + wt0 * 2048, static_cast<uint32_t>(rest * 2048));
         }
     }
     pdl_wait();
@@ -144,12 +158,14 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
         if (lane == 0 && !p.test_skip_loads) {
             int stage = 0;
             uint32_t phase = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (kb - kb0 >= n_pre) {
+            for (int i = 0; i < n_stages; ++i) {
+                if (i >= n_pre) {
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag)) break;
-                    load_weights(stage, kb);
+                    load_weights(stage, kb0 + G * i);
                 }
-                tma_load_2d(smem_base + stage * stage_bytes + A_BYTES + E_BYTES, &tmap_b, 0, kb * p.tb8 + (t0 >> 3), bar_full + 8 * stage);
+                const uint32_t b_dst = smem_base + stage * stage_bytes + G * (A_BYTES + E_BYTES);
+                if constexpr (G == 1) tma_load_2d(b_dst, &tmap_b, 0, (kb0 + i) * p.tb8 + (t0 >> 3), bar_full + 8 * stage);
+                else tma_load_3d(b_dst, &tmap_b, 0, t0 >> 3, kb0 + G * i, bar_full + 8 * stage);
                 if (++stage == stages) { stage = 0; phase ^= 1u; }
             }
         }
@@ -162,27 +178,32 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
             int stage = 0;
             uint32_t phase = 0;
             bool good = true;
-            for (int kb = kb0; kb < kb1; ++kb) {
+            for (int kb = kb0; kb < kb1; kb += G) {
                 if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { good = false; break; }
                 tcgen05_fence_after();
-                const uint32_t a_addr = smem_base + stage * stage_bytes;
-                const uint32_t b_addr = a_addr + A_BYTES + E_BYTES;
-                const uint32_t first = (kb == kb0) ? 0u : 1u;
-                const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
-                if constexpr (SPARSE) {
-                    const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(kWideMetaCol0 + 4 * stage);
-                    tcgen05_cp_128x128b(e_tmem, make_smem_desc(a_addr + A_BYTES, 128, 128, kSwzNone));
-                    const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
+                const uint32_t st = smem_base + stage * stage_bytes;
 #pragma unroll
-                    for (int j = 0; j < kBK / 64; ++j)
-                        mma_i8_sparse(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(4 * j),
-                                      e_tmem + 2 * j, idesc, j == 0 ? first : 1u);
-                } else {
-                    const uint64_t a_desc = make_smem_desc(a_addr, 16, 1024, kSwz128);
+                for (int h = 0; h < G; ++h) {
+                    if (h > 0 && kb + h >= kb1) break;
+                    const uint32_t a_addr = st + h * A_BYTES;
+                    const uint32_t b_addr = st + G * (A_BYTES + E_BYTES) + h * bn * kBK;
+                    const uint32_t first = (kb + h == kb0) ? 0u : 1u;
+                    const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
+                    if constexpr (SPARSE) {
+                        const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(kWideMetaCol0 + 8 * stage + 4 * h);
+                        tcgen05_cp_128x128b(e_tmem, make_smem_desc(st + G * A_BYTES + h * E_BYTES, 128, 128, kSwzNone));
+                        const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
 #pragma unroll
-                    for (int j = 0; j < kBK / 32; ++j)
-                        mma_i8_dense(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(2 * j),
-                                     idesc, j == 0 ? first : 1u);
+                        for (int j = 0; j < kBK / 64; ++j)
+                            mma_i8_sparse(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(4 * j),
+                                          e_tmem + 2 * j, idesc, j == 0 ? first : 1u);
+                    } else {
+                        const uint64_t a_desc = make_smem_desc(a_addr, 16, 1024, kSwz128);
+#pragma unroll
+                        for (int j = 0; j < kBK / 32; ++j)
+                            mma_i8_dense(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(2 * j),
+                                         idesc, j == 0 ? first : 1u);
+                    }
                 }
                 tcgen05_commit(bar_empty + 8 * stage);
                 if (++stage == stages) { stage = 0; phase ^= 1u; }

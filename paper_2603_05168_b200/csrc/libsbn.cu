@@ -213,10 +213,10 @@ static sbn_status launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, cons
 //   single-CTA tiles         a + w (q c + d)
 //   CTA pairs                a + b bn + w (q (c + u bn / 256) + d), with one or two M-tiles per CTA
 // What follows from it (2560 -> 3840, us, sparse): 65 tokens wide tiles split four ways 7.2 (narrow ones 7.9); 201 two
-// wide tiles split two ways 9.0 (64-token tiles unsplit 10.3, split 9.9); 400 pairs 10.4 (128-token tiles 12.1).
+// wide tiles split two ways 8.4 (64-token tiles unsplit 10.3, split 9.9); 400 pairs 10.4 (128-token tiles 12.1).
 // 6912 -> 2560 dense, 512 tokens: wide tiles 17.6 (128-token tiles 22.4, pairs 25).
 struct ClusterCost { double a, c, x, t, s, o, s3; };
-struct WideCost { double a, c, e, share, u; };
+struct WideCost { double a, c, e, share, u, c2, u2; };      // c2, u2: stages of two K-blocks
 struct TileCost { double a, c, d; };
 struct PairCost { double a, b, c, d, u; };
 struct PlanCosts {
@@ -227,12 +227,12 @@ struct PlanCosts {
 };
 static const PlanCosts kSparseCosts = {
     {2.39, 0.269, 0.029, 0.0305, 0.003, 0.38, 0.11}, {2.42, 0.276, 0.049, 0.0338, 0.0125, 0.41, 1.17},
-    {2.26, 0.261, 0.0303, 1.04, 0.041},
+    {2.26, 0.261, 0.0303, 1.04, 0.041, 0.15, 0.125},
     {3.63, 0.250, 0.0}, {4.27, 0.252, 0.72}, {3.60, 0.290, 3.11},
     {2.01, 0.0093, 0.197, 1.15, 0.015}, {1.29, 0.0179, 0.2605, 3.17, 0.098}};
 static const PlanCosts kDenseCosts = {
     {2.37, 0.317, 0.060, 0.0245, 0.0, 0.40, 0.17}, {2.20, 0.364, 0.090, 0.0329, 0.0043, 0.60, 1.23},
-    {1.87, 0.295, 0.0319, 1.40, 0.060},
+    {1.87, 0.295, 0.0319, 1.40, 0.060, 0.20, 0.11},
     {3.60, 0.277, 0.17}, {4.69, 0.284, 0.39}, {8.00, 0.3835, 0.0},
     {2.24, 0.0096, 0.329, 1.00, 0.0235}, {1.96, 0.0139, 0.376, 3.20, 0.215}};
 
@@ -290,10 +290,11 @@ static GemmPlan plan_gemm(bool sparse, int T, int N, int K) {
             const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
             if (bn * (tt - 1) >= T) continue;
             const int tokens = std::min(bn, T);
+            const double c = wide_group(sparse, bn) == 2 ? cost.wide.c2 + cost.wide.u2 * bn / 256 : cost.wide.c + cost.wide.u * bn / 256;
             for (int S = 2; S <= 4 && S <= kb; ++S) {
                 if (static_cast<long>(rows) * tt > most[S] || !wide_fits(bn, S)) continue;
                 const int q = (kb + S - 1) / S;
-                consider(GemmPlan{false, bn, 1, S}, cost.wide.a + q * (cost.wide.c + cost.wide.u * bn / 256) + cost.wide.e * tokens * (S - 1) / S +
+                consider(GemmPlan{false, bn, 1, S}, cost.wide.a + q * c + cost.wide.e * tokens * (S - 1) / S +
                                                         cost.wide.share * rows * tt * S / kNumSMs);
             }
         }
@@ -385,15 +386,21 @@ static sbn_status launch_splitk_cluster(const CUtensorMap& ta, const CUtensorMap
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
 }
 
-template <bool SPARSE>
-static sbn_status launch_splitk_wide(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& te, const GemmParams& p, int bn,
-                                     int cluster, cudaStream_t stream) {
-    if (!ensure_dynamic_smem<bitlinear_gemm_splitk_wide_kernel<SPARSE>>(kWideSmemBytes)) return SBN_ERR_CUDA;
+template <bool SPARSE, int G>
+static sbn_status launch_splitk_wide_cfg(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& te, const GemmParams& p, int bn,
+                                         int cluster, cudaStream_t stream) {
+    if (!ensure_dynamic_smem<bitlinear_gemm_splitk_wide_kernel<SPARSE, G>>(kWideSmemBytes)) return SBN_ERR_CUDA;
     const int tiles = (p.N / kBM) * ((p.T + bn - 1) / bn);
-    const cudaError_t err = launch_kernel_cluster(bitlinear_gemm_splitk_wide_kernel<SPARSE>, dim3(tiles * cluster), dim3(kWideThreads),
+    const cudaError_t err = launch_kernel_cluster(bitlinear_gemm_splitk_wide_kernel<SPARSE, G>, dim3(tiles * cluster), dim3(kWideThreads),
                                                   kWideSmemBytes, stream, static_cast<unsigned>(cluster), ta, tb, te, p, bn);
     ++g_launch_count;
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+}
+template <bool SPARSE>
+static sbn_status launch_splitk_wide(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& te, const GemmParams& p, int bn,
+                                     int cluster, cudaStream_t stream) {
+    return wide_group(SPARSE, bn) == 2 ? launch_splitk_wide_cfg<SPARSE, 2>(ta, tb, te, p, bn, cluster, stream)
+                                       : launch_splitk_wide_cfg<SPARSE, 1>(ta, tb, te, p, bn, cluster, stream);
 }
 
 // ---- few tokens: register-fed kernel ----------------------------------------------------------------
@@ -474,6 +481,12 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
 
     if (plan.cluster > 1) {
         p.k_splits = 1;
+        if (bn > 64) {                                          // boxes of wide_group K-blocks
+            const uint32_t G = static_cast<uint32_t>(wide_group(sparse, bn));
+            ok = (sparse ? encode_flat_1k(&ta, wvals, NK / 2, 8 * G) && encode_flat_1k(&te, meta, NK / 8, 2 * G) : encode_flat_1k(&ta, wvals, NK, 16 * G)) &&
+                 (G == 1 || encode_3d_1k(&tb, xq, xq_tb8(T), static_cast<uint64_t>(K) / kBK, static_cast<uint32_t>(bn / 8), G));   // G = 1: tb as it is
+            if (!ok) return SBN_ERR_CUDA;
+        }
         if (bn > 64) return sparse ? launch_splitk_wide<true>(ta, tb, te, p, bn, plan.cluster, stream)
                                    : launch_splitk_wide<false>(ta, tb, te, p, bn, plan.cluster, stream);
         if (sparse) return bn == 32 ? launch_splitk_cluster<true, 32>(ta, tb, te, p, plan.cluster, stream)
