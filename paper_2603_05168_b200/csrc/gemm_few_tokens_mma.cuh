@@ -359,15 +359,15 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     for FUSED with K > 3072 (4096 -> 11008 10.0 against 9.5).
 //   9 to 16 tokens    only while two CTAs per SM take all row groups (4096 -> 11008 10.6 / 9.1: every CTA reads all activations,
 //                     the cluster kernel's 128-row tiles read them less often).  Packed weights then always (7B MLPs, whole pass,
-//                     47 / 52), int8-held ones up to K = 8192 (2B layers 107 / 110; 7B MLPs with 11008 -> 4096 here 50 / 45, although
-//                     that GEMM alone takes 9.8 / 11.2: its CTAs leave the next kernel's no room to start early).  Dense: not
+//                     47 / 52), int8-held ones up to K = 3328 (quantiser + GEMM at 16 tokens: 2560 -> 2560 4.85 / 5.12, 2560 -> 3840
+//                     4.97 / 5.18, 4096 -> 4096 5.95 / 5.74, 6912 -> 2560 7.6 / 6.7).  Dense: not
 //                     (2B layers 63.5 / 59.3).  FUSED: not (6912 -> 2560 13.6 / 11.1).
 inline bool few_wide(const FewParams& p) { return p.N / 16 > 2 * device_sm_count(); }
 template <int WT, bool FUSED>
 inline bool few_takes(int T, int N, int K) {
     if (T <= 8) return true;
     if (T > 16 || FUSED || WT == kFewDense || N / 16 > 2 * device_sm_count()) return false;
-    return WT == kFewPacked || K <= 8192;
+    return WT == kFewPacked || K <= 3328;
 }
 template <int WT, bool FUSED>
 inline sbn_status launch_few(const FewParams& p, cudaStream_t stream) {

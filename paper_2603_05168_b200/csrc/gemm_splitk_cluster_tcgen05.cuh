@@ -1,6 +1,7 @@
 // Eq. 4 for few tokens: split-K inside a thread-block cluster.
 //
-// With few tokens (narrow tiles here; from about 65 on gemm_splitk_wide_tcgen05.cuh takes over) there are only N/128 x ceil(T/BN) output tiles -- far fewer than SMs --
+// With few tokens (narrow tiles here; from about 65 on gemm_splitk_wide_tcgen05.cuh takes over) there are only
+// N/128 x ceil(T/BN) output tiles -- far fewer than SMs --
 // and a CTA that walks the whole K of its tile is bound by what ONE SM can pull out of L2
 // (~100 GB/s: 18 KB per 128 columns -> 0.23 us each).  Splitting K over CTAs puts more SMs on the
 // weight stream; the partial accumulators then have to be added.  Through global memory that is
@@ -41,22 +42,30 @@ struct SplitConfig {
     static constexpr int A_BYTES = SPARSE ? kBM * (kBK / 2) : kBM * kBK;
     static constexpr int B_BYTES = BN * kBK;
     static constexpr int E_BYTES = SPARSE ? kBM * (kBK / 8) : 0;
-    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + E_BYTES;
+    // K-blocks per stage: two, fetched with one TMA instruction (about 64 ns each) per operand, where three such stages fit.
+    // Quantiser + GEMM at 32 tokens, us, one block / two: 2560 -> 3840 6.2 / 5.9, 6912 -> 2560 8.2 / 7.2, 11008 -> 4096 11.0 / 9.8.
+    static constexpr int G = (SPARSE && BN == 32) ? 2 : 1;
+    static constexpr int STAGE_BYTES = G * (A_BYTES + B_BYTES + E_BYTES);
     // Few enough stages that TWO CTAs fit on an SM (< 113 KB each), so the CTAs of the next
     // launch of a decode loop are resident -- and already pulling their weights -- while this one
     // reduces and finishes.  A stage that is filled before the dependency wait costs nothing, one
     // that has to be refilled costs an L2 round trip on the critical path: the 32-token tile keeps
-    // six (sparse) stages, enough for the whole K slice of a CTA at the usual sizes.
-    static constexpr int STAGES = (BN == 32) ? (SPARSE ? 6 : 4) : (SPARSE ? 4 : 3);
+    // three stages of two (sparse), enough for the whole K slice of a CTA at the usual sizes.
+    static constexpr int STAGES = (BN == 32) ? (SPARSE ? 3 : 4) : (SPARSE ? 4 : 3);
     static constexpr int CTAS_PER_SM = 2;
     static constexpr int REDUCE_BYTES = (BN + 4) * kBM * 4;    // [S][ceil(BN/S) tokens][128 features] int32, S in {2, 3, 4, 8}
     static constexpr int META_COL0 = BN;                        // metadata columns above the accumulator
-    static constexpr uint32_t TMEM_COLS = (BN + 4 * STAGES <= 64) ? 64 : (BN + 4 * STAGES <= 128 ? 128 : 256);
+    static constexpr uint32_t TMEM_COLS = (BN + 4 * G * STAGES <= 64) ? 64 : 128;
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + REDUCE_BYTES + kBarrierBytes;
     static_assert(SMEM_BYTES <= 232448 / CTAS_PER_SM - 1024 * (CTAS_PER_SM - 1), "shared memory overflow");
     static_assert(BN == 32 || BN == 64, "token tile (wider ones: gemm_splitk_wide_tcgen05.cuh)");
 };
 
+// 3-D box load of this CTA.
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
+}
 // 4-byte store into a peer's shared memory that counts its bytes on an mbarrier of that peer.
 __device__ __forceinline__ void st_async_cluster_u32(uint32_t cluster_addr, uint32_t v, uint32_t cluster_bar) {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];"
@@ -108,15 +117,15 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
                                      const __grid_constant__ CUtensorMap tmap_e,
                                      const GemmParams p) {
     using Cfg = SplitConfig<SPARSE, BN>;
-    constexpr int STAGES = Cfg::STAGES;
+    constexpr int STAGES = Cfg::STAGES, G = Cfg::G;
 
     extern __shared__ uint8_t smem_raw[];
     // 1 KB alignment: required by the 128 B swizzle atoms; the offset is the same in every CTA of
     // the cluster (same kernel, same static shared memory), so peers' buffers sit at the same offset
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t smem_a = smem_base;
-    const uint32_t smem_b = smem_a + STAGES * Cfg::A_BYTES;
-    const uint32_t smem_e = smem_b + STAGES * Cfg::B_BYTES;
+    const uint32_t smem_b = smem_a + STAGES * G * Cfg::A_BYTES;
+    const uint32_t smem_e = smem_b + STAGES * G * Cfg::B_BYTES;
     const uint32_t smem_red = smem_base + STAGES * Cfg::STAGE_BYTES;
     const uint32_t bar_base = smem_red + Cfg::REDUCE_BYTES;
     const uint32_t bar_full = bar_base;
@@ -172,7 +181,8 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
     // finishing.  This is safe because no kernel that WRITES packed weights signals its dependents
     // early (see sbn_common.cuh): a kernel that is running implies every earlier weight producer
     // has completed.  The activations (written by the kernel right before this one) wait.
-    const int n_pre = min(STAGES, kb1 - kb0);
+    const int n_stages = (kb1 - kb0 + G - 1) / G;               // a slice of odd length: the last block is loaded and not used
+    const int n_pre = min(STAGES, n_stages);
     if (threadIdx.x == 0) {
         tma_prefetch_desc(&tmap_a);
         tma_prefetch_desc(&tmap_b);
@@ -180,19 +190,20 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
         for (int i = 0; i < n_pre; ++i) {
             const uint32_t full = bar_full + 8 * i;
             mbar_expect_tx(full, Cfg::STAGE_BYTES);
-            const int wt = mt * p.k_blocks_total + kb0 + i;
+            const int wt = mt * p.k_blocks_total + kb0 + G * i;
             if constexpr (SPARSE) {
-                tma_load_2d(smem_a + i * Cfg::A_BYTES, &tmap_a, 0, wt * 8, full);
-                tma_load_2d(smem_e + i * Cfg::E_BYTES, &tmap_e, 0, wt * 2, full);
+                tma_load_2d(smem_a + i * G * Cfg::A_BYTES, &tmap_a, 0, wt * 8, full);
+                tma_load_2d(smem_e + i * G * Cfg::E_BYTES, &tmap_e, 0, wt * 2, full);
             } else {
-                tma_load_2d(smem_a + i * Cfg::A_BYTES, &tmap_a, 0, wt * 16, full);
+                tma_load_2d(smem_a + i * G * Cfg::A_BYTES, &tmap_a, 0, wt * 16, full);
             }
         }
         // the rest of this CTA's slice goes to L2 (the point of coherence: nothing can go stale there)
-        if (kb1 - kb0 > n_pre) {
-            const size_t wt0 = static_cast<size_t>(mt) * p.k_blocks_total + kb0 + n_pre;
-            prefetch_l2_bulk(static_cast<const char*>(p.w_vals) + wt0 * p.w_tile_bytes, static_cast<uint32_t>((kb1 - kb0 - n_pre) * p.w_tile_bytes));
-            if (p.w_meta) prefetch_l2_bulk(static_cast<const char*>(p.w_meta) + wt0 * 2048, static_cast<uint32_t>((kb1 - kb0 - n_pre) * 2048));
+        const int rest = kb1 - kb0 - G * n_pre;
+        if (rest > 0) {
+            const size_t wt0 = static_cast<size_t>(mt) * p.k_blocks_total + kb0 + G * n_pre;
+            prefetch_l2_bulk(static_cast<const char*>(p.w_vals) + wt0 * p.w_tile_bytes, static_cast<uint32_t>(rest * p.w_tile_bytes));
+            if (p.w_meta) prefetch_l2_bulk(static_cast<const char*>(p.w_meta) + wt0 * 2048, static_cast<uint32_t>(rest * 2048));
         }
     }
     pdl_wait();
@@ -205,20 +216,22 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
         if (lane == 0 && !p.test_skip_loads) {
             int stage = 0;
             uint32_t phase = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
+            for (int i = 0; i < n_stages; ++i) {
                 const uint32_t full = bar_full + 8 * stage;
-                if (kb - kb0 >= n_pre) {                                 // the first n_pre stages got their weights above
+                const int kb = kb0 + G * i;
+                if (i >= n_pre) {                                 // the first n_pre stages got their weights above
                     if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag)) break;
                     mbar_expect_tx(full, Cfg::STAGE_BYTES);
                     const int wt = mt * p.k_blocks_total + kb;            // weight tile index
                     if constexpr (SPARSE) {
-                        tma_load_2d(smem_a + stage * Cfg::A_BYTES, &tmap_a, 0, wt * 8, full);
-                        tma_load_2d(smem_e + stage * Cfg::E_BYTES, &tmap_e, 0, wt * 2, full);
+                        tma_load_2d(smem_a + stage * G * Cfg::A_BYTES, &tmap_a, 0, wt * 8, full);
+                        tma_load_2d(smem_e + stage * G * Cfg::E_BYTES, &tmap_e, 0, wt * 2, full);
                     } else {
-                        tma_load_2d(smem_a + stage * Cfg::A_BYTES, &tmap_a, 0, wt * 16, full);
+                        tma_load_2d(smem_a + stage * G * Cfg::A_BYTES, &tmap_a, 0, wt * 16, full);
                     }
                 }
-                tma_load_2d(smem_b + stage * Cfg::B_BYTES, &tmap_b, 0, kb * p.tb8 + (t0 >> 3), full);
+                if constexpr (G == 1) tma_load_2d(smem_b + stage * Cfg::B_BYTES, &tmap_b, 0, kb * p.tb8 + (t0 >> 3), full);
+                else tma_load_3d(smem_b + stage * G * Cfg::B_BYTES, &tmap_b, 0, t0 >> 3, kb, full);
                 if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
         }
@@ -231,29 +244,33 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
             int stage = 0;
             uint32_t phase = 0;
             bool good = true;
-            for (int kb = kb0; kb < kb1; ++kb) {
+            for (int kb = kb0; kb < kb1; kb += G) {
                 if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { good = false; break; }
                 tcgen05_fence_after();
-                const uint32_t a_addr = smem_a + stage * Cfg::A_BYTES;
-                const uint32_t b_addr = smem_b + stage * Cfg::B_BYTES;
-                const uint32_t first = (kb == kb0) ? 0u : 1u;
-                if constexpr (SPARSE) {
-                    const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(Cfg::META_COL0 + 4 * stage);
-                    const uint64_t e_desc = make_smem_desc(smem_e + stage * Cfg::E_BYTES, 128, 128, kSwzNone);
-                    tcgen05_cp_128x128b(e_tmem, e_desc);
-                    const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
-                    const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
 #pragma unroll
-                    for (int j = 0; j < kBK / 64; ++j)
-                        mma_i8_sparse(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(4 * j),
-                                      e_tmem + 2 * j, idesc, j == 0 ? first : 1u);
-                } else {
-                    const uint64_t a_desc = make_smem_desc(a_addr, 16, 1024, kSwz128);
-                    const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
+                for (int h = 0; h < G; ++h) {
+                    if (h > 0 && kb + h >= kb1) break;
+                    const uint32_t a_addr = smem_a + (stage * G + h) * Cfg::A_BYTES;
+                    const uint32_t b_addr = smem_b + (stage * G + h) * Cfg::B_BYTES;
+                    const uint32_t first = (kb + h == kb0) ? 0u : 1u;
+                    if constexpr (SPARSE) {
+                        const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(Cfg::META_COL0 + 4 * (stage * G + h));
+                        const uint64_t e_desc = make_smem_desc(smem_e + (stage * G + h) * Cfg::E_BYTES, 128, 128, kSwzNone);
+                        tcgen05_cp_128x128b(e_tmem, e_desc);
+                        const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
+                        const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
 #pragma unroll
-                    for (int j = 0; j < kBK / 32; ++j)
-                        mma_i8_dense(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(2 * j),
-                                     idesc, j == 0 ? first : 1u);
+                        for (int j = 0; j < kBK / 64; ++j)
+                            mma_i8_sparse(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(4 * j),
+                                          e_tmem + 2 * j, idesc, j == 0 ? first : 1u);
+                    } else {
+                        const uint64_t a_desc = make_smem_desc(a_addr, 16, 1024, kSwz128);
+                        const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
+#pragma unroll
+                        for (int j = 0; j < kBK / 32; ++j)
+                            mma_i8_dense(tmem_base, a_desc + static_cast<uint64_t>(2 * j), b_desc + static_cast<uint64_t>(2 * j),
+                                         idesc, j == 0 ? first : 1u);
+                    }
                 }
                 tcgen05_commit(bar_empty + 8 * stage);
                 if (++stage == STAGES) { stage = 0; phase ^= 1u; }

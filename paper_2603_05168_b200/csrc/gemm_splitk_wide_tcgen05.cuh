@@ -52,11 +52,6 @@ __device__ __forceinline__ void bulk_copy_to_cta(uint32_t dst_cluster, uint32_t 
                  ::"r"(dst_cluster), "r"(src_cta), "r"(bytes), "r"(bar_cluster) : "memory");
 }
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
-}
-
 // tmap_a / tmap_e: weight tiles and metadata as rows of 1 KB, boxes of G tiles; tmap_b: xq as rows of 1 KB, box of bn / 8
 // (G = 1), or as [K / 128][atoms][1 KB], box of 2 x bn / 8 atoms.  A stage holds G = wide_group K-blocks: weights of all, metadata of all, activations of all.  The
 // second block of a slice of odd length is loaded and not used (beyond the arrays the hardware fills in zeros).

@@ -226,7 +226,7 @@ struct PlanCosts {
     PairCost pair1, pair2;
 };
 static const PlanCosts kSparseCosts = {
-    {2.39, 0.269, 0.029, 0.0305, 0.003, 0.38, 0.11}, {2.42, 0.276, 0.049, 0.0338, 0.0125, 0.41, 1.17},
+    {2.39, 0.205, 0.029, 0.0305, 0.003, 0.38, 0.11}, {2.42, 0.276, 0.049, 0.0338, 0.0125, 0.41, 1.17},
     {2.26, 0.261, 0.0303, 1.04, 0.041, 0.15, 0.125},
     {3.63, 0.250, 0.0}, {4.27, 0.252, 0.72}, {3.60, 0.290, 3.11},
     {2.01, 0.0093, 0.197, 1.15, 0.015}, {1.29, 0.0179, 0.2605, 3.17, 0.098}};
@@ -489,6 +489,12 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
         }
         if (bn > 64) return sparse ? launch_splitk_wide<true>(ta, tb, te, p, bn, plan.cluster, stream)
                                    : launch_splitk_wide<false>(ta, tb, te, p, bn, plan.cluster, stream);
+        if (sparse && bn == 32) {                               // two K-blocks per stage
+            static_assert(SplitConfig<true, 32>::G == 2 && SplitConfig<true, 64>::G == 1 && SplitConfig<false, 32>::G == 1, "boxes");
+            if (!encode_flat_1k(&ta, wvals, NK / 2, 16) || !encode_flat_1k(&te, meta, NK / 8, 4) ||
+                !encode_3d_1k(&tb, xq, xq_tb8(T), static_cast<uint64_t>(K) / kBK, 4, 2))
+                return SBN_ERR_CUDA;
+        }
         if (sparse) return bn == 32 ? launch_splitk_cluster<true, 32>(ta, tb, te, p, plan.cluster, stream)
                                     : launch_splitk_cluster<true, 64>(ta, tb, te, p, plan.cluster, stream);
         return bn == 32 ? launch_splitk_cluster<false, 32>(ta, tb, te, p, plan.cluster, stream)
