@@ -33,6 +33,19 @@ def test_header_symbols_are_exported(L):
     assert sorted(binding.EXPORTS) == names
 
 
+def test_every_included_source_triggers_a_rebuild():
+    """Whatever libsbn.cu includes from csrc is among the files whose change makes build() compile again."""
+    known, todo, seen = set(sbn_build.sources()), ["libsbn.cu"], set()
+    while todo:
+        name = todo.pop()
+        if name in seen or not os.path.exists(os.path.join(sbn_build.CSRC, name)):
+            continue
+        seen.add(name)
+        todo += re.findall(r'#include "([^"]+)"', open(os.path.join(sbn_build.CSRC, name)).read())
+    assert len(seen) > 15
+    assert {os.path.join(sbn_build.CSRC, n) for n in seen} <= known
+
+
 def test_status_strings(L):
     from paper_2603_05168_b200 import binding
     seen = {binding.status_string(i) for i in range(8)}
