@@ -1043,7 +1043,9 @@ inline sbn_status launch_quantize_mask_pack(const void* W, bool w_bf16, int N, i
                                             unsigned long long* flip_bits, QmpWorkspace* ws,
                                             cudaStream_t stream) {
     const QmpDesc d = qmp_make_desc(W, w_bf16, N, K, vals, meta, w_scale, dense_q, prev_meta, flip_bits);
-    return launch_quantize_mask_pack_stream<PATTERN>(&d, nullptr, 1, d.num_units, ws->slot, &ws->generation, stream, &ws->memo);
+    // the scale a call leaves behind is for the next 2:4 call only; 6:8 always samples (its tag names neither pattern nor dtype)
+    return launch_quantize_mask_pack_stream<PATTERN>(&d, nullptr, 1, d.num_units, ws->slot, &ws->generation, stream,
+                                                     PATTERN == 24 ? &ws->memo : nullptr);
 }
 
 }  // namespace sbn

@@ -1232,6 +1232,33 @@ def test_quantize_mask_pack_scale_left_in_the_workspace_never_changes_the_result
     run_and_check(buf, refs["a"])
 
 
+def test_quantize_mask_pack_68_starts_from_a_sample():
+    # The scale left in the workspace belongs to the 2:4 calls: a 6:8 call neither takes one that a 2:4 call on the same
+    # buffer left (here useless: the weights have changed since) nor leaves its own.
+    N, K = 256, 1024
+    Wa, Wb = inputs.latent_weights(N, K, seed=420), inputs.latent_weights(N, K, seed=421, sigma=0.31)
+    buf = dev(Wa)
+    bufs = b.alloc_packed(N, K, n_keep=6, m_group=8)
+    b24 = b.alloc_packed(N, K)
+    slots_and_generation = 148 * 16 + 8
+
+    def pack68(W):
+        b.sbn_quantize_mask_pack(buf, bufs["vals"], bufs["meta"], bufs["w_scale"], bufs["ws"], n_keep=6, m_group=8)
+        b.sbn_check_status()
+        vals, meta = gpu_unpack_canonical(bufs, N, b.sbn_expanded_k(K, 6, 8))
+        _assert_pack68(W, dict(vals=vals, meta=meta, scale=np.float32(bufs["w_scale"].cpu().numpy()[0])))
+
+    bufs["ws"].fill_(0xA5)
+    pack68(Wa)
+    assert bool((bufs["ws"][slots_and_generation:] == 0xA5).all())
+    b.sbn_quantize_mask_pack(buf, b24["vals"], b24["meta"], b24["w_scale"], bufs["ws"])
+    left = bufs["ws"][slots_and_generation:].clone()
+    assert bool((left != 0xA5).any())                               # the 2:4 call did leave one
+    buf.copy_(torch.from_numpy(Wb).cuda())
+    pack68(Wb)
+    assert torch.equal(bufs["ws"][slots_and_generation:], left)
+
+
 # ---- the register-fed few-token kernel -----------------------------------------------------------------------------
 @pytest.mark.parametrize("T,N,K", [(1, 128, 128), (8, 128, 256), (3, 256, 1152), (5, 4864, 384), (1, 4864, 3328), (9, 640, 1408),
                                    (16, 2560, 256), (16, 128, 128)])
