@@ -56,6 +56,30 @@ __device__ __forceinline__ double bf16_abs_to_f64(uint32_t abs15) {
     return __hiloint2double(static_cast<int>((abs15 << 13) + 0x38000000u), 0);
 }
 
+// Codes of a finite row whose xn is not finite: mean square 0 with eps = 0 (rinv infinite), or a gain that takes xn out of range
+// (s_x = 0).  The product is NaN where xn is infinite or NaN: code 127, as a saturating conversion gives; else 0.  The row is read
+// again and its codes stored over the ones before: a call that is never made, 1 % of the kernel (code for it inside the loop
+// 2 to 4 %, a minimum per code 3 to 8 %).
+template <int G, bool EXPAND68>
+__device__ __noinline__ void odd_row_codes(const uint4* x, const float4* gain, float rinv, int row, int nvec, int g, uint2* xq, size_t tb8) {
+#pragma unroll 1
+    for (int idx = g; idx < nvec; idx += G) {
+        const uint4 v = __ldg(x + static_cast<size_t>(row) * nvec + idx);
+        uint32_t code[2];
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t w0 = h ? v.z : v.x, w1 = h ? v.w : v.y;
+            const float4 gn = gain != nullptr ? __ldg(gain + 2 * idx + h) : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+            const float xn[4] = {bf16lo_to_f32(w0) * rinv * gn.x, bf16hi_to_f32(w0) * rinv * gn.y, bf16lo_to_f32(w1) * rinv * gn.z, bf16hi_to_f32(w1) * rinv * gn.w};
+            uint32_t c = 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c |= fabsf(xn[j]) < __int_as_float(0x7F800000) ? 0u : 0x7Fu << (8 * j);
+            if (h) code[1] = c; else code[0] = c;
+        }
+        store_codes8<EXPAND68>(xq, row, idx, tb8, make_uint2(code[0], code[1]));
+    }
+}
+
 // G threads per token row, VPT 16-byte vectors per thread (G * VPT >= K / 8).  The gains are copied
 // to shared memory once per CTA (rows differ, channels do not).
 template <int G, int VPT, bool EXPAND68 = false>
@@ -206,7 +230,7 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
                         q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
                         q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
                     }
-                    // The method's clamp cannot act: |xn| <= d, so |xn * s_x| <= 127 (1 + 2^-23) and rounds to at most 127.  The
+                    // The method's clamp cannot act: |xn| <= d (finite), so |xn * s_x| <= 127 (1 + 2^-23) and rounds to at most 127.  The
                     // code is the low byte.
                     uint2 ov;                                      // lowest column in the lowest byte
                     ov.x = low_bytes4(q[0], q[1], q[2], q[3]);
@@ -214,6 +238,8 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
                     store_codes8<EXPAND68>(xq, row, idx, tb8, ov);     // plain, or expanded for the 6:8 pattern
                 }
             }
+            if (fmaxf(d, rinv) == __int_as_float(0x7F800000))              // for the whole group of threads, so for whole warps
+                odd_row_codes<G, EXPAND68>(x, gain, rinv, row, nvec, g, xq, tb8);
         }
 #pragma unroll
         for (int i = 0; i < VPT; ++i) cur[i] = nxt[i];

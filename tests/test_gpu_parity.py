@@ -93,6 +93,36 @@ def test_norm_quant_act_rows_per_cta(T, K):
     test_norm_quant_act_parity(T, K, True)
 
 
+# Finite inputs whose normalised row is not finite: no scale brings such a value into range, and its code is 127 (the saturated
+# end), as for every width of the kernel; with eps > 0 and finite products nothing changes.
+@pytest.mark.parametrize("T,K", [(5, 256), (5, 1280), (600, 1280), (600, 2560), (5, 4096), (600, 6912), (600, 11008), (5, 16384)])
+def test_norm_quant_act_rows_that_overflow(T, K):
+    x = np.random.default_rng(K).standard_normal((T, K)).astype(np.float32)
+    x[0] = 0.0                                        # mean square 0: r is infinite, 0 * r is not a number
+    x[1] *= 1e-30                                     # squares vanish in fp32: r is infinite, x * r too
+    x[2] = 0.0
+    x[2, K // 2] = -1e-30
+    bits = inputs.f32_to_bf16_bits(x)
+    xq, s = gpu_norm_quant_act(bits, None, 0.0)
+    codes = xq_to_numpy(xq, T, K)
+    s = s.cpu().numpy()
+    assert (codes[:3] == 127).all()
+    assert s[0] == np.float32(1e-5) / np.float32(127.0) and np.isinf(s[1:3]).all()
+    r = oracle.norm_quant_act(bits, None, 1e-6)
+    xq, s = gpu_norm_quant_act(bits, None, 1e-6)
+    ok = ~r["near_tie"]
+    assert np.array_equal(xq_to_numpy(xq, T, K)[ok], r["xq"][ok])
+    gain = np.full(K, 1e30, np.float32)
+    gain[::7] = 3e38                                  # |xn| > 1.14 times this is out of range
+    xn = np.abs(oracle.norm_quant_act(bits, None, 1e-6, want_xn=True)["xn"][3]) * gain.astype(np.float64)
+    out_of_range = xn > 3.5e38
+    close = np.abs(xn - 3.4e38) < 0.1e38
+    assert out_of_range.any()
+    xq, s = gpu_norm_quant_act(bits, gain, 1e-6)
+    row = xq_to_numpy(xq, T, K)[3]
+    assert np.array_equal(row[~close], np.where(out_of_range, 127, 0)[~close]) and np.isinf(s.cpu().numpy()[3])
+
+
 def test_norm_quant_act_edge_rows():
     K = 512
     x = np.zeros((5, K), np.float32)
