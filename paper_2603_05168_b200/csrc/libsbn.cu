@@ -541,14 +541,15 @@ static sbn_status run_backward(const void* dY, int T, const int8_t* xq, const fl
     p.Nn = K;
     const PrepJob job{reinterpret_cast<const uint8_t*>(vals), meta, reinterpret_cast<uint16_t*>(base + lay.w_off),
                       reinterpret_cast<const uint8_t*>(xq), a_scale, reinterpret_cast<uint16_t*>(base + lay.xq_off), T, N, K, w_items, x_items};
-    p.plan = plan_backward(tiles, stages, 0, g_force_token_tile < 0 ? (-g_force_token_tile <= 128 ? 1 : 0) : -1, nullptr);
+    p.plan = plan_backward(tiles, stages, g_force_token_tile < 0 ? (-g_force_token_tile <= 128 ? 1 : 0) : -1);
 
     const uint64_t t = static_cast<uint64_t>(T), n = static_cast<uint64_t>(N), k = static_cast<uint64_t>(K);
-    Bf16Maps maps;
-    bool ok = encode_3d_bf16_blocks(&maps.aw, dY, n, t, 2) && encode_2d_bf16_sw128(&maps.ax, dY, n, t, n, 128);
-    for (int blocks = 1; ok && blocks <= 2; ++blocks)
-        ok = encode_3d_bf16_blocks(&maps.b[0][2 - blocks], base + lay.xq_off, k, t, blocks) &&
-             encode_3d_bf16_blocks(&maps.b[1][2 - blocks], base + lay.w_off, k, n, blocks);
+    Bf16Maps maps;                                              // only those that the plan reads are filled in
+    bool ok = (!dW || encode_3d_bf16_blocks(&maps.aw, dY, n, t, 2)) && (!dX || encode_2d_bf16_sw128(&maps.ax, dY, n, t, n, 128));
+    for (int g = 0; ok && g < p.plan.segments; ++g) {
+        const int part = p.plan.seg[g].part, half = p.plan.seg[g].half;
+        ok = encode_3d_bf16_blocks(&maps.b[part][half], base + (part == 0 ? lay.xq_off : lay.w_off), k, part == 0 ? t : n, half ? 1 : 2);
+    }
     if (!ok) return SBN_ERR_CUDA;
     if (!ensure_dynamic_smem<backward_gemm_kernel>(kBf16SmemBytes)) return SBN_ERR_CUDA;
     const int blocks = std::max(1, std::min(w_items + x_items, 16 * device_sm_count()));
