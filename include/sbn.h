@@ -91,8 +91,8 @@ typedef enum {
 /* Host, pure.  Bytes of the tiled int8 activation buffer xq for T tokens of K columns. */
 size_t sbn_xq_bytes(int T, int K);
 
-/* Host, pure.  Bytes of device workspace the given call needs for these sizes (0 if none).
- * T is ignored by SBN_OP_QUANTIZE_MASK_PACK. */
+/* Host, pure.  Bytes of device workspace the given call takes for these sizes (0 if none; the
+ * forward GEMMs also run without).  T is ignored by SBN_OP_QUANTIZE_MASK_PACK. */
 size_t sbn_workspace_bytes(int op, int T, int N, int K);
 
 /*
@@ -295,9 +295,10 @@ sbn_status sbn_norm_quant_act_expand68(const void *x_bf16, int T, int K, const f
  *   y             device out, [T][N] of `dt`
  *   acc_out       device out or NULL, int32 [T][N]: the raw accumulators (for parity checks)
  *   ws, ws_bytes  device workspace of sbn_workspace_bytes(SBN_OP_SPARSE_BITLINEAR, T, N, K)
- *                 bytes (may be NULL when that is 0).  It must be zero-filled before its first
- *                 use; every call that completes leaves it zero-filled again (split-K sums for
- *                 small T live there), so it can be reused without clearing
+ *                 bytes.  It must be zero-filled before its first use; every call that completes
+ *                 leaves it zero-filled again (split-K sums for small T live there), so it can be
+ *                 reused without clearing.  NULL or fewer bytes: the same result from the fastest
+ *                 kernel that needs none (SBN_ERR_WORKSPACE only if sbn_set_gemm_tuning asks for the split)
  */
 sbn_status sbn_sparse_bitlinear(const int8_t *xq, const float *a_scale, int T,
                                 const int8_t *vals, const uint8_t *meta, const float *w_scale,

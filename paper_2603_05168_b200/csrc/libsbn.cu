@@ -166,14 +166,17 @@ struct GemmPlan {
     int cluster;    // > 1: split-K inside clusters of this many CTAs (reduction in shared memory)
     int mt = 2;     // CTA-pair kernel: M-tiles per CTA (2: 512-feature tiles; 1: 256-feature tiles, double-buffered accumulators)
 };
-static GemmPlan plan_gemm(bool sparse, int T, int N, int K);
+static GemmPlan plan_gemm(bool sparse, int T, int N, int K, bool may_split = true);
+template <int WT, bool FUSED> static bool use_few_kernel(int T, int N, int K);
 
+// Scratch of a plan that splits K through global memory: int32 [T][N] + one counter per output tile.
+static size_t split_workspace_bytes(const GemmPlan& plan, int T, int N) {
+    if (plan.pair || plan.splits <= 1) return 0;
+    return split_acc_bytes(T, N) + static_cast<size_t>(N / kBM) * ((T + plan.bn - 1) / plan.bn) * sizeof(unsigned int);
+}
 static size_t gemm_workspace_bytes(bool sparse, int T, int N, int K) {
-    // split-K scratch: int32 [T][N] + one counter per output tile; only the small-T regime splits
-    const GemmPlan plan = plan_gemm(sparse, T, N, K);
-    if (!plan.pair && plan.splits > 1)
-        return split_acc_bytes(T, N) + static_cast<size_t>(N / kBM) * ((T + plan.bn - 1) / plan.bn) * sizeof(unsigned int);
-    return 0;
+    if (sparse ? use_few_kernel<kFewSparse, false>(T, N, K) : use_few_kernel<kFewDense, false>(T, N, K)) return 0;
+    return split_workspace_bytes(plan_gemm(sparse, T, N, K), T, N);
 }
 
 template <bool SPARSE, int BN>
@@ -236,7 +239,7 @@ static const PlanCosts kDenseCosts = {
     {3.60, 0.277, 0.17}, {4.69, 0.284, 0.39}, {8.00, 0.3835, 0.0},
     {2.24, 0.0096, 0.329, 1.00, 0.0235}, {1.96, 0.0139, 0.376, 3.20, 0.215}};
 
-static GemmPlan plan_gemm(bool sparse, int T, int N, int K) {
+static GemmPlan plan_gemm(bool sparse, int T, int N, int K, bool may_split) {
     GemmPlan best = {false, 64, 1, 0};
     const int kb = K / kBK;
     const int rows = N / kBM;
@@ -307,7 +310,7 @@ static GemmPlan plan_gemm(bool sparse, int T, int N, int K) {
         const long tiles = static_cast<long>(rows) * ((T + bn - 1) / bn);
         const long waves = (tiles + kNumSMs - 1) / kNumSMs;
         if (waves <= 2) consider(GemmPlan{false, bn, 1, 0}, c.a + waves * (kb * c.c + c.d));    // beyond, the pairs' operand reuse wins
-        if (bn == 64 && tiles * 2 <= kNumSMs) {
+        if (may_split && bn == 64 && tiles * 2 <= kNumSMs) {
             // smallest split that gives at least ~100 units of work
             int sp = static_cast<int>((100 + tiles - 1) / tiles);
             if (sp > kb) sp = kb;
@@ -440,18 +443,22 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
         const FewParams p = few_params(T, N, K, xq, nullptr, a_scale, nullptr, wvals, meta, w_scale, bias, y, dt, acc_out);
         return sparse ? launch_few<kFewSparse, false>(p, stream) : launch_few<kFewDense, false>(p, stream);
     }
-    const GemmPlan plan = plan_gemm(sparse, T, N, K);
+    GemmPlan plan = plan_gemm(sparse, T, N, K);
+    if (plan.splits > 1) {
+        // scratch is zero on entry (caller's duty before the first use) and the kernel re-zeroes it.  Without it: the
+        // fastest plan that needs none, unless this one was asked for
+        if (!ws || ws_bytes < split_workspace_bytes(plan, T, N)) {
+            if (g_force_token_tile != 0 || g_force_split_k != 0) return SBN_ERR_WORKSPACE;
+            plan = plan_gemm(sparse, T, N, K, false);
+        } else if (misaligned(ws, 16)) {
+            return SBN_ERR_ALIGN;
+        }
+    }
     if (plan.pair)
         return run_gemm_pair(sparse, xq, a_scale, T, wvals, meta, w_scale, N, K, bias, y, dt, acc_out, plan.bn, plan.mt, stream);
 
     const int bn = plan.bn;
     const int splits = plan.splits;
-    if (splits > 1) {
-        // scratch is zero on entry (caller's duty before the first use) and the kernel re-zeroes it
-        const size_t need = gemm_workspace_bytes(sparse, T, N, K);
-        if (!ws || ws_bytes < need) return SBN_ERR_WORKSPACE;
-        if (misaligned(ws, 16)) return SBN_ERR_ALIGN;
-    }
 
     CUtensorMap ta, tb, te, ty;
     bool ok;

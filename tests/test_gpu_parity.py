@@ -1328,3 +1328,26 @@ def test_few_token_kernel_all_forms(T, N, K):
         call(yb, None)
         b.sbn_check_status()
         assert torch.equal(yb, y.to(torch.bfloat16))                # bf16 = the fp32 value rounded to nearest even
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_gemm_without_the_workspace_its_split_would_use(dtype):
+    # K through global memory is the fastest plan here; a caller without a workspace (or with too little) gets the fastest
+    # other one, bit for bit the same
+    T, N, K = 9, 2304, 24576
+    need = b.sbn_workspace_bytes(b.OP_BITLINEAR, T, N, K)
+    assert need > 0
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randint(-1, 2, (N, K), generator=gen, device="cuda", dtype=torch.int8)
+    x = torch.randn((T, K), generator=gen, device="cuda").to(torch.bfloat16)
+    xq, a_scale, w_scale = b.alloc_xq(T, K), torch.empty(T, device="cuda"), torch.full((1,), 0.02, device="cuda")
+    b.sbn_quant_act(x, xq, a_scale)
+    ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
+    ys = []
+    for w in (ws, None, ws[:256]):
+        y = torch.full((T, N), float("nan"), dtype=dtype, device="cuda")
+        b.sbn_bitlinear(xq, a_scale, q, w_scale, y, ws=w)
+        b.sbn_check_status()
+        ys.append(y)
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
+    assert int(ws.count_nonzero()) == 0                             # zero-kept
