@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <mutex>
 #include <vector>
 
@@ -166,7 +167,7 @@ struct GemmPlan {
     int cluster;    // > 1: split-K inside clusters of this many CTAs (reduction in shared memory)
     int mt = 2;     // CTA-pair kernel: M-tiles per CTA (2: 512-feature tiles; 1: 256-feature tiles, double-buffered accumulators)
 };
-static GemmPlan plan_gemm(bool sparse, int T, int N, int K, bool may_split = true);
+static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool may_split = true);
 template <int WT, bool FUSED> static bool use_few_kernel(int T, int N, int K);
 
 // Scratch of a plan that splits K through global memory: int32 [T][N] + one counter per output tile.
@@ -176,7 +177,7 @@ static size_t split_workspace_bytes(const GemmPlan& plan, int T, int N) {
 }
 static size_t gemm_workspace_bytes(bool sparse, int T, int N, int K) {
     if (sparse ? use_few_kernel<kFewSparse, false>(T, N, K) : use_few_kernel<kFewDense, false>(T, N, K)) return 0;
-    return split_workspace_bytes(plan_gemm(sparse, T, N, K), T, N);
+    return std::max(split_workspace_bytes(plan_gemm(sparse, false, T, N, K), T, N), split_workspace_bytes(plan_gemm(sparse, true, T, N, K), T, N));
 }
 
 template <bool SPARSE, int BN>
@@ -208,38 +209,57 @@ static sbn_status launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, cons
 
 // Which kernel, which token tile, whether to split K: the measured times (us) of every candidate, as a small model.
 //
-// The coefficients were fitted to a sweep of quantiser + GEMM chains: eight shapes from 2048 x 1024 to 11008 x 4096, 30
-// token counts from 12 to 8192, every kernel with its useful tiles and splits, sparse and dense; 5000 timings.  What the
-// model picks was within 0.3 % of the fastest candidate on average (the worst 13 %).  q = K-blocks per CTA, w = waves.
-//   clusters, narrow tiles   a + q (c + x crowd) + tokens (t + s / S) + o [two CTAs on some SM] + 3-way owner selection
-//   clusters, wide tiles     a + q (c + u bn / 256) + e tokens (S - 1) / S + 1.0 or 1.4 x share of the SMs in use
-//   single-CTA tiles         a + w (q c + d)
-//   CTA pairs                a + b bn + w (q (c + u bn / 256) + d), with one or two M-tiles per CTA
-// What follows from it (2560 -> 3840, us, sparse): 65 tokens wide tiles split four ways 7.2 (narrow ones 7.9); 201 two
-// wide tiles split two ways 8.4 (64-token tiles unsplit 10.3, split 9.9); 400 pairs 10.4 (128-token tiles 12.1).
-// 6912 -> 2560 dense, 512 tokens: wide tiles 17.6 (128-token tiles 22.4, pairs 25).
-struct ClusterCost { double a, c, x, t, s, o, s3; };
-struct WideCost { double a, c, e, share, u, c2, u2; };      // c2, u2: stages of two K-blocks
-struct TileCost { double a, c, d; };
-struct PairCost { double a, b, c, d, u; };
+// The coefficients were fitted to quantiser + GEMM chains (weights from memory): 43 shapes from 640 x 1280 to 65536 x 2560 and
+// 2048 x 65536 (K x N), 30 token counts from 9 to 8192, every kernel with its useful tiles and splits, sparse and dense, bf16 and
+// fp32 outputs; 43000 timings.  What the model picks is within 0.5 % of the fastest candidate on average (the worst 13 %), and on
+// 16 shapes and 24 token counts that the fit has not seen within 0.6 % (12 %).  q = K-blocks per CTA, w = waves.
+//   clusters, narrow tiles   a + q (c + x crowd + x2 share of SMs with two CTAs) + tokens (t + s / S) + o crowd min(1, q / 3) + 3-way
+//                            owner selection
+//   clusters, wide tiles     a + q (c + u bn / 256) + e tokens (S - 1) / S + (share + z q) x share of the SMs in use
+//   single-CTA tiles         a + (w q c or m MB) + w d; K split through global memory: a + q c + atomics T N S
+//   CTA pairs                a + b bn + (w q (c + u bn / 256) or m MB) + w d, with one or two M-tiles per CTA
+// "or": whichever is longer, smoothed (fourth powers); MB = megabytes of weights and outputs.
+// The output type matters to the pairs: with two M-tiles the accumulator waits for the stores of fp32 outputs (5 us per tile, bf16
+// ones leave through registers in 2.5), with one it does not.  2560 -> 6912 sparse, 6000 tokens, fp32: two M-tiles 86 us, one 75.
+struct ClusterCost { double a, c, x, t, s, o, s3, x2; };
+struct WideCost { double a, c, e, share, u, c2, u2, z; };   // c2, u2: stages of two K-blocks
+struct TileCost { double a, c, d, m; };
+struct PairCost { double a, b, c, d, u, m; };
 struct PlanCosts {
     ClusterCost narrow32, narrow64;
     WideCost wide;
     TileCost tile64, tile128, tile256;
     PairCost pair1, pair2;
 };
-static const PlanCosts kSparseCosts = {
-    {2.39, 0.205, 0.029, 0.0305, 0.003, 0.38, 0.11}, {2.42, 0.276, 0.049, 0.0338, 0.0125, 0.41, 1.17},
-    {2.26, 0.261, 0.0303, 1.04, 0.041, 0.15, 0.125},
-    {3.63, 0.250, 0.0}, {4.27, 0.252, 0.72}, {3.60, 0.290, 3.11},
-    {2.01, 0.0093, 0.197, 1.15, 0.015}, {1.29, 0.0179, 0.2605, 3.17, 0.098}};
-static const PlanCosts kDenseCosts = {
-    {2.37, 0.317, 0.060, 0.0245, 0.0, 0.40, 0.17}, {2.20, 0.364, 0.090, 0.0329, 0.0043, 0.60, 1.23},
-    {1.87, 0.295, 0.0319, 1.40, 0.060, 0.20, 0.11},
-    {3.60, 0.277, 0.17}, {4.69, 0.284, 0.39}, {8.00, 0.3835, 0.0},
-    {2.24, 0.0096, 0.329, 1.00, 0.0235}, {1.96, 0.0139, 0.376, 3.20, 0.215}};
+static const PlanCosts kPlanCosts[2][2] = {                 // [sparse][fp32 outputs or raw accumulators]
+    {{{5.2724, 0.2689, 0.003, 0.002, 0.01, 0.4005, 0.0371, 0.0685}, {5.0562, 0.3367, 0.0157, 0.0225, 0.0051, 0.4646, 1.2385, 0.0819},
+      {4.5917, 0.1501, 0.0295, 0.5418, 0.1432, 0.1242, 0.1469, 0.0775},
+      {5.2199, 0.2497, 0.5009, 0.07}, {6.0228, 0.2653, 0.7606, 0.1161}, {9.2108, 0.3821, -0.3368, 0.1839}, {4.8432, 0.0053, 0.2966, 0.6719, 0.0509, 0.0002}, {3.4272, 0.0134, 0.3953, 2.9039, 0.1588, 0.1106}},
+     {{5.2688, 0.2675, 0.0064, 0.0018, 0.0081, 0.4248, 0.0791, 0.0575}, {5.073, 0.3341, 0.0095, 0.0212, 0.0044, 0.5437, 1.4758, 0.0795},
+      {4.5868, 0.1448, 0.0292, 0.5865, 0.1469, 0.1255, 0.1402, 0.0747},
+      {5.2396, 0.2516, 0.3646, 0.0725}, {5.8416, 0.2673, 0.4823, 0.1166}, {7.6558, 0.395, 0.0374, 0.1638}, {5.1877, 0.01, 0.2932, 0.8005, 0.0524, 0.0007}, {1.9177, 0.0179, 0.366, 5.1005, 0.2111, 0.1001}}},
+    {{{4.757, 0.1929, 0.013, 0.023, 0.0004, 0.2915, 0.0598, 0.0471}, {4.8582, 0.2677, 0.0395, 0.0317, 0.0021, 0.1165, 1.1535, 0.0332},
+      {4.7161, 0.2772, 0.0299, 0.2317, -0.0365, 0.1183, 0.0977, 0.0818},
+      {5.3343, 0.2414, 0.2205, 0.1108}, {6.2223, 0.2463, 0.546, 0.1228}, {5.3179, 0.2778, 3.487, 0.1858}, {4.8079, 0.0054, 0.1838, 0.6455, 0.0348, 0.0992}, {3.8719, 0.0136, 0.2539, 2.458, 0.1053, 0.1233}},
+     {{4.8398, 0.1906, 0.0118, 0.0169, 0.0021, 0.3432, 0.1063, 0.0447}, {4.8808, 0.2655, 0.0342, 0.029, 0.0022, 0.2248, 1.3655, 0.0341},
+      {4.6456, 0.2668, 0.03, 0.3028, -0.0285, 0.117, 0.0944, 0.0807},
+      {5.1138, 0.2422, 0.2679, 0.126}, {5.9491, 0.2478, 0.3353, 0.1469}, {5.3549, 0.282, 2.349, 0.157}, {4.9998, 0.0107, 0.1749, 0.8473, 0.0446, 0.1231}, {2.7183, 0.0176, 0.233, 4.2553, 0.1481, 0.1171}}}};
 
-static GemmPlan plan_gemm(bool sparse, int T, int N, int K, bool may_split) {
+// Clusters of S with two CTAs per SM that were all resident at once; one more waited for a whole kernel lifetime (12288 -> 2304,
+// 128 tokens: 72 clusters of 4 19.5 us, other plans 13.1; clusters of 3: 88 were, 90 not always).
+constexpr int kNarrowClusters[5] = {0, 0, 148, 88, 70};
+// The same with one CTA per SM (wide tiles; 45 clusters of 3 were not: 5376 -> 1920, 230 tokens: 14.8 us, 33 or fewer of 4 9.9).
+constexpr int kWideClusters[5] = {0, 0, 74, 44, 33};
+
+static double narrow_cost(const ClusterCost& c, int kb, long tiles, int tokens, int S) {
+    const int q = (kb + S - 1) / S;
+    // SMs that hold two CTAs: part of the slowdown grows with their share, part is all there once 40 % of them do
+    const double two = std::max(0.0, static_cast<double>(tiles * S - kNumSMs) / kNumSMs), crowd = std::min(1.0, 2.5 * two);
+    return c.a + q * (c.c + c.x * crowd + c.x2 * two) + tokens * (c.t + c.s / S) + c.o * crowd * std::min(1.0, q / 3.0) + (S == 3 ? c.s3 : 0.0);
+}
+
+// out_wide: four bytes per output or more (fp32, or the raw accumulators as well).  may_split: a plan may need a workspace.
+static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool may_split) {
     GemmPlan best = {false, 64, 1, 0};
     const int kb = K / kBK;
     const int rows = N / kBM;
@@ -267,76 +287,66 @@ static GemmPlan plan_gemm(bool sparse, int T, int N, int K, bool may_split) {
         const int bn = pick_token_tile(T);
         return GemmPlan{false, bn, pick_split_k(T, N, K, bn), 0};
     }
-    const PlanCosts& cost = sparse ? kSparseCosts : kDenseCosts;
+    const PlanCosts& cost = kPlanCosts[sparse][out_wide];
+    const double megabytes = 1e-6 * N * ((sparse ? 0.625 : 1.0) * K + (out_wide ? 4.0 : 2.0) * T);
+    auto longer = [](double x, double y) { return std::sqrt(std::sqrt(x * x * x * x + y * y * y * y)); };
     double best_t = 1e300;
     auto consider = [&](const GemmPlan& g, double t) { if (t < best_t) { best_t = t; best = g; } };
-    // Clusters of 2, 3 or 4 CTAs, narrow tiles: all CTAs resident at once (two per SM), a second wave costs a whole kernel
-    // lifetime.  Clusters of 3 need some slack in the slot count (288 CTAs in clusters of 3 did not all become resident
-    // on 296 slots).
+    // Clusters of 2, 3 or 4 CTAs, narrow tiles: all of them resident at once, two CTAs per SM.
     for (const int bn : {32, 64}) {
-        const ClusterCost& c = bn == 32 ? cost.narrow32 : cost.narrow64;
         const long tiles = static_cast<long>(rows) * ((T + bn - 1) / bn);
-        const int tokens = std::min(bn, T);
-        for (int S = 2; S <= 4 && S <= kb && tiles * S <= 2L * kNumSMs; ++S) {
-            if (S == 3 && tiles * S * 100 > 2L * kNumSMs * 93) continue;
-            const int q = (kb + S - 1) / S;
-            const long ctas = tiles * S;
-            // share of the SMs that hold two CTAs; the slowdown saturates once ~40 % of them do
-            const double crowd = ctas > kNumSMs ? std::min(1.0, 2.5 * static_cast<double>(ctas - kNumSMs) / kNumSMs) : 0.0;
-            consider(GemmPlan{false, bn, 1, S}, c.a + q * (c.c + c.x * crowd) + tokens * (c.t + c.s / S) + (ctas > kNumSMs ? c.o : 0.0) + (S == 3 ? c.s3 : 0.0));
-        }
+        for (int S = 2; S <= 4 && S <= kb; ++S)
+            if (tiles <= kNarrowClusters[S])
+                consider(GemmPlan{false, bn, 1, S}, narrow_cost(bn == 32 ? cost.narrow32 : cost.narrow64, kb, tiles, std::min(bn, T), S));
     }
-    // Wide tiles: one CTA per SM, and the clusters that fit at once (74 of 2, 45 of 3, 33 of 4).
-    if (T > 64 && T <= 800) {
-        const int most[5] = {0, 0, 74, 45, 33};
-        for (int tt = (T + 255) / 256; tt <= (T + 255) / 256 + 2; ++tt) {
+    // Wide tiles: one CTA per SM.  (8192 -> 1024 dense, 1000 tokens: 21.3 us, narrow clusters 22.7.)
+    if (T > 64 && T <= 2048) {
+        const int fewest = (T + 255) / 256;
+        for (int tt = fewest; tt <= fewest + (T > 512 ? 4 : 2); ++tt) {
             const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
             if (bn * (tt - 1) >= T) continue;
             const int tokens = std::min(bn, T);
             const double c = wide_group(sparse, bn) == 2 ? cost.wide.c2 + cost.wide.u2 * bn / 256 : cost.wide.c + cost.wide.u * bn / 256;
             for (int S = 2; S <= 4 && S <= kb; ++S) {
-                if (static_cast<long>(rows) * tt > most[S] || !wide_fits(bn, S)) continue;
+                if (static_cast<long>(rows) * tt > kWideClusters[S] || !wide_fits(bn, S)) continue;
                 const int q = (kb + S - 1) / S;
                 consider(GemmPlan{false, bn, 1, S}, cost.wide.a + q * c + cost.wide.e * tokens * (S - 1) / S +
-                                                        cost.wide.share * rows * tt * S / kNumSMs);
+                                                        (cost.wide.share + cost.wide.z * q) * rows * tt * S / kNumSMs);
             }
         }
     }
-    // Single-CTA tiles.  K is split through global memory only when the tiles cannot fill the machine and the int32 atomics
-    // cost less than the K-loop they save.
+    // Single-CTA tiles: one token tile in any number of waves, else up to two, with short K (1024 -> 2560: 15.0 us for 2048
+    // tokens dense, pairs 15.9) up to four; beyond, the pairs' operand reuse wins.
     for (const int bn : {64, 128, 256}) {
         if (bn > 64 && T <= bn / 2) continue;                   // a tile mostly beyond T
         const TileCost& c = bn == 64 ? cost.tile64 : (bn == 128 ? cost.tile128 : cost.tile256);
         const long tiles = static_cast<long>(rows) * ((T + bn - 1) / bn);
         const long waves = (tiles + kNumSMs - 1) / kNumSMs;
-        if (waves <= 2) consider(GemmPlan{false, bn, 1, 0}, c.a + waves * (kb * c.c + c.d));    // beyond, the pairs' operand reuse wins
-        if (may_split && bn == 64 && tiles * 2 <= kNumSMs) {
-            // smallest split that gives at least ~100 units of work
+        if (T <= 64 || waves <= (kb <= 12 && bn < 256 ? 4 : 2)) consider(GemmPlan{false, bn, 1, 0}, c.a + longer(waves * kb * c.c, c.m * megabytes) + waves * c.d);
+        // K through global memory: dense weights of very long rows only (24576 -> 2304, 9 tokens: 19.1 us, clusters 20.9; at
+        // K = 16384 it was slower, sparse weights never faster).  One wave, at least ~100 units of work.
+        if (may_split && !sparse && bn == 64 && K >= 24576 && tiles * 2 <= kNumSMs) {
             int sp = static_cast<int>((100 + tiles - 1) / tiles);
-            if (sp > kb) sp = kb;
-            while (sp > 1 && kb % sp != 0) ++sp;                // next divisor upwards (kb divides itself)
-            if (sp > 1 && sp <= kb && sp <= 10) {               // many slices: the atomics dominate (33 us measured at 43)
-                const double atomics = 8e-6 * static_cast<double>(T) * N * sp;
-                consider(GemmPlan{false, bn, sp, 0}, c.a + (kb / sp) * c.c + c.d + 1.0 + atomics);
-            }
+            while (sp > 1 && sp <= 10 && kb % sp != 0) ++sp;
+            if (sp > 1 && sp <= 10 && tiles * sp <= kNumSMs)
+                consider(GemmPlan{false, bn, sp, 0}, 7.6 + kb / sp * 0.269 + 7.2e-6 * T * N * sp);
         }
     }
     // CTA pairs: a tile costs nearly the same whatever its token width, so the tile counts worth a look are the smallest
-    // ones, down to those that fill the last wave.
-    if (T > 32) {
-        const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
-        const int fewest = (T + cap - 1) / cap;
-        for (int tt = fewest; tt <= fewest + (T < 1000 ? 3 : 8); ++tt) {
-            const int bn = std::max(T > 64 ? 80 : 32, ((T + tt - 1) / tt + 15) / 16 * 16);
-            if (bn * (tt - 1) >= T) continue;
-            for (int mt = 1; mt <= 2; ++mt) {
-                const PairCost& c = mt == 1 ? cost.pair1 : cost.pair2;
-                const long tiles = static_cast<long>((N + 256 * mt - 1) / (256 * mt)) * tt;
-                const long waves = (tiles + kNumSMs / 2 - 1) / (kNumSMs / 2);
-                GemmPlan g{true, bn, 1, 0};
-                g.mt = mt;
-                consider(g, c.a + c.b * bn + waves * (kb * (c.c + c.u * bn / 256) + c.d));
-            }
+    // ones, down to those that fill the last wave.  For few tokens too: they have more places than the clusters (4096 -> 20480
+    // sparse, 16 tokens: 17.6 us, single-CTA tiles 23.2).
+    const int cap = sparse ? kPairMaxBnSparse : kPairMaxBnDense;
+    const int fewest = (T + cap - 1) / cap;
+    for (int tt = fewest; tt <= fewest + (T < 1000 ? 3 : 8); ++tt) {
+        const int bn = std::max(T > 64 ? 80 : 32, ((T + tt - 1) / tt + 15) / 16 * 16);
+        if (bn * (tt - 1) >= T) continue;
+        for (int mt = 1; mt <= 2; ++mt) {
+            const PairCost& c = mt == 1 ? cost.pair1 : cost.pair2;
+            const long tiles = static_cast<long>((N + 256 * mt - 1) / (256 * mt)) * tt;
+            const long waves = (tiles + kNumSMs / 2 - 1) / (kNumSMs / 2);
+            GemmPlan g{true, bn, 1, 0};
+            g.mt = mt;
+            consider(g, c.a + c.b * bn + longer(waves * kb * (c.c + c.u * bn / 256), c.m * megabytes) + waves * c.d);
         }
     }
     return best;
@@ -443,13 +453,14 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
         const FewParams p = few_params(T, N, K, xq, nullptr, a_scale, nullptr, wvals, meta, w_scale, bias, y, dt, acc_out);
         return sparse ? launch_few<kFewSparse, false>(p, stream) : launch_few<kFewDense, false>(p, stream);
     }
-    GemmPlan plan = plan_gemm(sparse, T, N, K);
+    const bool out_wide = dt == SBN_OUT_F32 || acc_out != nullptr;
+    GemmPlan plan = plan_gemm(sparse, out_wide, T, N, K);
     if (plan.splits > 1) {
         // scratch is zero on entry (caller's duty before the first use) and the kernel re-zeroes it.  Without it: the
         // fastest plan that needs none, unless this one was asked for
         if (!ws || ws_bytes < split_workspace_bytes(plan, T, N)) {
             if (g_force_token_tile != 0 || g_force_split_k != 0) return SBN_ERR_WORKSPACE;
-            plan = plan_gemm(sparse, T, N, K, false);
+            plan = plan_gemm(sparse, out_wide, T, N, K, false);
         } else if (misaligned(ws, 16)) {
             return SBN_ERR_ALIGN;
         }
@@ -493,9 +504,9 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
             ok = (sparse ? encode_flat_1k(&ta, wvals, NK / 2, 8 * G) && encode_flat_1k(&te, meta, NK / 8, 2 * G) : encode_flat_1k(&ta, wvals, NK, 16 * G)) &&
                  (G == 1 || encode_3d_1k(&tb, xq, xq_tb8(T), static_cast<uint64_t>(K) / kBK, static_cast<uint32_t>(bn / 8), G));   // G = 1: tb as it is
             if (!ok) return SBN_ERR_CUDA;
+            return sparse ? launch_splitk_wide<true>(ta, tb, te, p, bn, plan.cluster, stream)
+                          : launch_splitk_wide<false>(ta, tb, te, p, bn, plan.cluster, stream);
         }
-        if (bn > 64) return sparse ? launch_splitk_wide<true>(ta, tb, te, p, bn, plan.cluster, stream)
-                                   : launch_splitk_wide<false>(ta, tb, te, p, bn, plan.cluster, stream);
         if (sparse && bn == 32) {                               // two K-blocks per stage
             static_assert(SplitConfig<true, 32>::G == 2 && SplitConfig<true, 64>::G == 1 && SplitConfig<false, 32>::G == 1, "boxes");
             if (!encode_flat_1k(&ta, wvals, NK / 2, 16) || !encode_flat_1k(&te, meta, NK / 8, 4) ||
@@ -1037,7 +1048,7 @@ void sbn_plan_gemm(int sparse, int T, int N, int K, int* out4) {
     if (!out4) return;
     out4[0] = out4[1] = out4[2] = out4[3] = 0;
     if (T <= 0 || N <= 0 || K <= 0 || N % kBM != 0 || K % kBK != 0) return;
-    const GemmPlan g = plan_gemm(sparse != 0, T, N, K);
+    const GemmPlan g = plan_gemm(sparse != 0, false, T, N, K);
     out4[0] = g.pair ? (g.mt == 1 ? 3 : 2) : (g.cluster > 1 ? 1 : 0);
     out4[1] = g.bn;
     out4[2] = g.splits;

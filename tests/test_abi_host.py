@@ -263,3 +263,33 @@ def test_native_calls_marshal_like_the_abi(L, monkeypatch):
     with pytest.raises(ValueError):
         b.sbn_quant_act(xq, xq, sc)                                  # not two-dimensional
     assert not seen
+
+
+def test_plans_never_ask_for_more_clusters_than_fit(L):
+    """The split-K clusters of a plan are resident all at once: 148 / 88 / 70 of 2 / 3 / 4 CTAs at two per SM (narrow tiles),
+    74 / 44 / 33 at one (wide tiles)."""
+    import random
+    from paper_2603_05168_b200 import binding as b
+    rng = random.Random(3)
+    seen = set()
+    for _ in range(20000):
+        T, N, K = round(2 ** rng.uniform(0, 12)), 128 * round(2 ** rng.uniform(0, 7)), 128 * round(2 ** rng.uniform(1, 7.5))
+        kernel, bn, split, cluster = b.sbn_plan_gemm(rng.random() < 0.5, T, N, K)
+        assert bn % 16 == 0 and 32 <= bn <= 256
+        if kernel == 1:
+            tiles = N // 128 * -(-T // bn)
+            assert tiles <= ({2: 148, 3: 88, 4: 70} if bn <= 64 else {2: 74, 3: 44, 4: 33})[cluster], (T, N, K)
+            assert cluster <= K // 128
+        seen.add((kernel, cluster, bn > 64))
+    assert len(seen) >= 9                                             # tiles, both pairs, every cluster size in both widths
+
+
+def test_wide_matrices_run_on_pairs_and_long_dense_rows_may_split(L):
+    from paper_2603_05168_b200 import binding as b
+    assert b.sbn_plan_gemm(True, 16, 20480, 4096)[0] in (2, 3)        # 160 row tiles: more than the clusters have places
+    assert b.sbn_plan_gemm(False, 9, 2304, 24576)[2] > 1              # K through global memory, with a workspace
+    assert b.sbn_workspace_bytes(b.OP_BITLINEAR, 9, 2304, 24576) > 0
+    assert b.sbn_workspace_bytes(b.OP_BITLINEAR, 8, 2304, 24576) == 0  # the register-fed kernel needs none
+    for T in (9, 16, 64, 201, 777):
+        assert b.sbn_workspace_bytes(b.OP_SPARSE_BITLINEAR, T, 2304, 24576) == 0
+        assert b.sbn_workspace_bytes(b.OP_BITLINEAR, T, 2304, 12288) == 0
