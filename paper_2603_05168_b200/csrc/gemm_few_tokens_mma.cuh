@@ -362,12 +362,23 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     47 / 52), int8-held ones up to K = 3328 (quantiser + GEMM at 16 tokens: 2560 -> 2560 4.85 / 5.12, 2560 -> 3840
 //                     4.97 / 5.18, 4096 -> 4096 5.95 / 5.74, 6912 -> 2560 7.6 / 6.7).  Dense: not
 //                     (2B layers 63.5 / 59.3).  FUSED: not (6912 -> 2560 13.6 / 11.1).
+//   Not where a second round of CTAs would be barely filled: it costs as much as a full one, and the clusters have none.
+//                     Three CTAs per SM: int8-held 2:4 from K = 2560 on, a second round of up to a third (2560 -> 8192 6.6 / 5.7, 6912 -> 7424
+//                     10.8 / 9.2; 2048 -> 8192 4.8 / 5.4), a third one likewise around K = 2560 (2560 -> 16384 8.6 / 7.5, 3072 -> 16384
+//                     even); dense around K = 3072, up to a fifth (2560 -> 8704 6.9 / 6.4, 4096 -> 8704 8.7 / 9.2).  Two per SM
+//                     (FUSED): long rows, up to a half (6912 -> 5120 dense, 8 tokens 15.1 / 12.1).  Packed: a second round of up to
+//                     a half, K from 2560 on (8192 -> 8704 12.2 / 11.2, 4096 -> 11008 8.9 / 8.8; 2048 -> 8192 5.0 / 5.5).
 inline bool few_wide(const FewParams& p) { return p.N / 16 > 2 * device_sm_count(); }
 template <int WT, bool FUSED>
 inline bool few_takes(int T, int N, int K) {
-    if (T <= 8) return true;
-    if (T > 16 || FUSED || WT == kFewDense || N / 16 > 2 * device_sm_count()) return false;
-    return WT == kFewPacked || K <= 3328;
+    const double per_sm = static_cast<double>(N / 16) / device_sm_count();
+    if (T > 8) return T <= 16 && !FUSED && WT != kFewDense && per_sm <= 2.0 && (WT == kFewPacked || K <= 3328);
+    if (FUSED && K > 3072)
+        return !(per_sm > 2.0 && per_sm <= (T > 4 ? 3.25 : 3.0) && (K >= 6144 || (WT == kFewDense && T > 4 && K >= 4096)));
+    if (WT == kFewDense) return !(per_sm > 3.0 && per_sm <= 3.7 && K >= 2560 && K <= 3584 && (!FUSED || T > 4));
+    if (WT == kFewSparse && !FUSED) return !((per_sm > 3.0 && per_sm <= 4.0 && K >= 2560) || (per_sm > 6.0 && per_sm <= 7.0 && K >= 2560 && K < 3072));
+    if (WT == kFewPacked) return !(per_sm > 3.1 && per_sm <= 4.7 && K >= 2560);
+    return true;
 }
 template <int WT, bool FUSED>
 inline sbn_status launch_few(const FewParams& p, cudaStream_t stream) {
