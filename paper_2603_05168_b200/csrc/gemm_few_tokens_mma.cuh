@@ -367,7 +367,8 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     10.8 / 9.2; 2048 -> 8192 4.8 / 5.4), a third one likewise around K = 2560 (2560 -> 16384 8.6 / 7.5, 3072 -> 16384
 //                     even); dense around K = 3072, up to a fifth (2560 -> 8704 6.9 / 6.4, 4096 -> 8704 8.7 / 9.2).  Two per SM
 //                     (FUSED): long rows, up to a half (6912 -> 5120 dense, 8 tokens 15.1 / 12.1).  Packed: a second round of up to
-//                     a half, K from 2560 on (8192 -> 8704 12.2 / 11.2, 4096 -> 11008 8.9 / 8.8; 2048 -> 8192 5.0 / 5.5).
+//                     a third, K from 2560 on (8192 -> 8704 12.2 / 11.2; 2048 -> 8192 5.0 / 5.5), of up to a half, long rows (6912 ->
+//                     11008 13.1 / 12.1; 4096 -> 11008 8.9 / 8.8, but 2 % slower among other matrices).
 inline bool few_wide(const FewParams& p) { return p.N / 16 > 2 * device_sm_count(); }
 template <int WT, bool FUSED>
 inline bool few_takes(int T, int N, int K) {
@@ -377,7 +378,7 @@ inline bool few_takes(int T, int N, int K) {
         return !(per_sm > 2.0 && per_sm <= (T > 4 ? 3.25 : 3.0) && (K >= 6144 || (WT == kFewDense && T > 4 && K >= 4096)));
     if (WT == kFewDense) return !(per_sm > 3.0 && per_sm <= 3.7 && K >= 2560 && K <= 3584 && (!FUSED || T > 4));
     if (WT == kFewSparse && !FUSED) return !((per_sm > 3.0 && per_sm <= 4.0 && K >= 2560) || (per_sm > 6.0 && per_sm <= 7.0 && K >= 2560 && K < 3072));
-    if (WT == kFewPacked) return !(per_sm > 3.1 && per_sm <= 4.7 && K >= 2560);
+    if (WT == kFewPacked) return !((per_sm > 3.1 && per_sm <= 4.0 && K >= 2560) || (per_sm > 4.0 && per_sm <= 4.7 && K >= 6144));
     return true;
 }
 template <int WT, bool FUSED>
