@@ -106,10 +106,13 @@ struct BackwardRuns {
 inline BackwardPlan plan_backward(const int (&tiles)[2], const int (&stages)[2], int split_hint) {
     const int lng = (tiles[1] > 0 && (tiles[0] == 0 || stages[1] >= stages[0])) ? 1 : 0;
     const int sht = tiles[1 - lng] > 0 ? 1 - lng : lng;                     // a single part is both
-    // In stages (0.36 us): a tile's loads and MMAs, or its output if that takes longer (256 KB in fp32 resp. 128 KB in bf16 at
-    // the 47 GB/s per pair that the memory takes), and the turnaround.
-    auto full = [&](int part) { return std::max(stages[part] * 1.0, part == 0 ? 15.0 : 7.5) + 3.0; };
-    auto half = [&](int part) { return std::max(stages[part] * 0.65, part == 0 ? 7.5 : 3.75) + 3.0; };
+    // In stages (0.36 us): a tile's loads and MMAs, or its output if that takes longer, and the turnaround.  256 KB in fp32 resp.
+    // 128 KB in bf16 take 15 resp. 7.5 at the 47 GB/s per pair that the memory takes; beside dW's fp32 its loads take half their
+    // time again (with 15 alone the pairs that write most ended last: 54 sizes of 256 to 2048 tokens 3.5 % slower, 11008 x 4096 at 777
+    // 208 us against 186).
+    const double out_w = 15.0 + 0.5 * stages[0];
+    auto full = [&](int part) { return std::max(stages[part] * 1.0, part == 0 ? out_w : 7.5) + 3.0; };
+    auto half = [&](int part) { return std::max(stages[part] * 0.65, part == 0 ? 0.5 * out_w : 3.75) + 3.0; };
     const bool long_cut = split_hint >= 0 ? split_hint != 0 : 2 * tiles[lng] <= kBackwardPairs;   // too few to go round: all in halves
     BackwardRuns long_placed;
     if (sht != lng) long_placed.spread(0, long_cut ? 2 * tiles[lng] : tiles[lng], long_cut ? half(lng) : full(lng));
