@@ -458,9 +458,10 @@ sbn_status sbn_set_wait_test(int break_waits, unsigned long long wait_limit_us);
  * Used by `bench.py --workload mmaprobe`. */
 void sbn_set_gemm_probe(int flags);
 
-/* Diagnostic: which tcgen05 kernel the dispatcher picks for this shape (host only, launches nothing).  It runs
- * with more than 16 tokens, or whenever sbn_set_gemm_tuning or sbn_set_wait_test is in force; otherwise calls of up to 8
- * tokens, and some sparse ones of up to 16, run the register-fed few-token kernel instead.
+/* Diagnostic: which tcgen05 kernel the dispatcher picks for this shape and bf16 outputs, with a workspace (host only,
+ * launches nothing; fp32 outputs and raw accumulators have costs of their own).  It runs with more than 16 tokens, or
+ * whenever sbn_set_gemm_tuning or sbn_set_wait_test is in force; most calls of up to 8 tokens, and some sparse ones of up
+ * to 16, run the register-fed few-token kernel instead.
  * out4[0] = kernel (0 single-CTA tiles, 1 cluster split-K, 2 CTA pair with 512-feature tiles, 3 CTA
  * pair with 256-feature tiles and double-buffered accumulators), out4[1] = tokens per tile,
  * out4[2] = split-K factor through global memory (1 = none), out4[3] = cluster size (0 = none).

@@ -6,7 +6,7 @@
 //
 // B (x_q [T][K] resp. W_eff [N][K], backward_prep.cuh) is read MN-major in both.  Two CTAs of a cluster issue one
 // `tcgen05.mma.cta_group::2.kind::f16` (M = 256: each CTA supplies 128 rows of A and half of the B tile and keeps its
-// 128 x BN slice of the accumulator in its own tensor memory).  Operands come by TMA from plain row-major tensors, six
+// 128 x BN slice of the accumulator in its own tensor memory).  Operands come by TMA from plain row-major tensors, seven
 // stages of 64 contraction steps; the full barrier of a stage lives in the leader CTA and collects both CTAs' bytes,
 // `tcgen05.commit ... multicast::cluster` releases stages and publishes accumulators in both CTAs.  The two 256-column
 // halves of tensor memory alternate as accumulators, so the epilogue of a tile (a thread owns an output row and writes

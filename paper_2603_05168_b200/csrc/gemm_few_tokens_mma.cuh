@@ -352,7 +352,7 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 
 // Which calls run here, with what split.  All times in us for quantiser + GEMM in a decode loop (weights from HBM), this
 // kernel / the cluster kernel of tcgen05 instructions at its best cluster size.
-//   up to 8 tokens    always.  1 token: 2560 -> 2560 3.7 / 5.0, 2560 -> 6912 4.6 / 5.6, 6912 -> 2560 5.7 / 7.5,
+//   up to 8 tokens    all but the places at the end.  1 token: 2560 -> 2560 3.7 / 5.0, 2560 -> 6912 4.6 / 5.6, 6912 -> 2560 5.7 / 7.5,
 //                     4096 -> 11008 7.8 / 8.5, 11008 -> 4096 8.4 / 10.6.
 //                     With more row groups than two CTAs per SM take at once, three CTAs per SM with fewer blocks in flight
 //                     each (4.6 against 5.4 for 2560 -> 6912; but 6.4 against 5.7 for 6912 -> 2560, which fits two).  Not

@@ -11,10 +11,10 @@
 // layout as quant_act.cuh.  The squares of bf16 values are added in fp64 in a fixed order (thread-local, then a
 // butterfly, then the warps in order).
 //
-// Measured in a chain of launches, with a gain (us; HBM time of the bytes in brackets): 1 x 2560 1.50, 16 x 4096 1.73,
-// 201 x 2560 2.0 -- two trips to memory, two barriers and the arithmetic between them; 4096 x 2560 11.8 [4.9],
-// 4096 x 6912 26.4 [13.2], 8192 x 4096 28.5 [15.6], 8192 x 11008 78 [42] -- bound by the instructions per element, of
-// which the plain quantiser (7.4, 16.3, 21.8, 49) needs fewer.  Squares through the conversion instruction, gains
+// Measured in a chain of launches, with a gain (us; HBM time of the bytes in brackets): 1 x 2560 1.57, 16 x 4096 1.8,
+// 201 x 2560 2.5 -- two trips to memory, two barriers and the arithmetic between them; 4096 x 2560 11.8 [4.9],
+// 4096 x 6912 26.8 [13.2], 8192 x 4096 29.7 [15.6], 8192 x 11008 76 [42] -- bound by the instructions, 22.7 per element
+// (73 % of the issue slots busy); the plain quantiser (7.4, 16.3, 21.8, 49) needs fewer.  Squares through the conversion instruction, gains
 // fetched before the row, a division for the mean and a clamp: 2.21, 2.10, 3.14, 12.0, 28.2, 31.6 and 82.  One or two
 // warps per row without the prefetch of the next row were slower: 15.7, 31.7, 36.6, 90.
 #pragma once
@@ -58,8 +58,8 @@ __device__ __forceinline__ double bf16_abs_to_f64(uint32_t abs15) {
 
 // Codes of a finite row whose xn is not finite: mean square 0 with eps = 0 (rinv infinite), or a gain that takes xn out of range
 // (s_x = 0).  The product is NaN where xn is infinite or NaN: code 127, as a saturating conversion gives; else 0.  The row is read
-// again and its codes stored over the ones before: a call that is never made, 1 % of the kernel (code for it inside the loop
-// 2 to 4 %, a minimum per code 3 to 8 %).
+// again and its codes stored over the ones before: a call that is never made, 1 % of the kernel's time on average (5 % for 8192 rows
+// of 4096; code for it inside the loop 2 to 4 % on average, a minimum per code 3 to 8 %).
 template <int G, bool EXPAND68>
 __device__ __noinline__ void odd_row_codes(const uint4* x, const float4* gain, float rinv, int row, int nvec, int g, uint2* xq, size_t tb8) {
 #pragma unroll 1
