@@ -123,6 +123,28 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
+// 0xFF where the word is negative, a byte per word (byte permutes in sign-replication mode).
+__device__ __forceinline__ uint32_t sign_bytes4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return prmt(prmt(a, b, 0x00FBu), prmt(c, d, 0x00FBu), 0x5410u);
+}
+__device__ __forceinline__ uint32_t sign_bytes4(float a, float b, float c, float d) {
+    return sign_bytes4(__float_as_uint(a), __float_as_uint(b), __float_as_uint(c), __float_as_uint(d));
+}
+// Eight byte masks -> eight bits.
+__device__ __forceinline__ uint32_t qmp_byte_bits(uint32_t lo, uint32_t hi) {
+    return (((lo & 0x08040201u) | (hi & 0x80402010u)) * 0x01010101u) >> 24;
+}
+// Two bf16 in a word: magnitudes, sign bits, the permute that turns the four sign bits of two words into four byte masks (low half
+// of the first word first).
+constexpr uint32_t kAbs2 = 0x7FFF7FFFu, kGuard2 = 0x80008000u, kSign2 = 0xFDB9u;
+// |a| - |b| for two bf16 at once: only the sign bits (15 and 31) are used -- rounding cannot change them, and equal magnitudes
+// give +0.  It runs on the FMA pipe, where nothing else waits: pass 1 is bound by the ALU pipe.
+__device__ __forceinline__ uint32_t sub_abs_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("{\n\t.reg .b32 x, y;\n\tabs.bf16x2 x, %1;\n\tabs.bf16x2 y, %2;\n\tsub.rn.bf16x2 %0, x, y;\n\t}" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
 // Three-input minima (one instruction each on this architecture).
 __device__ __forceinline__ float fmin3(float a, float b, float c) {
     float d;
@@ -170,7 +192,18 @@ struct QmpDesc {
     uint32_t num_units;                // N * K / 128
     uint32_t KB;                       // K / 128
     uint32_t w_bf16;                   // master weights are bf16 (Sec. 2.2 keeps them "e.g. in bf16")
+    uint32_t kb_magic;                 // qmp_magic(KB)
 };
+// Division by a number the host knows: a 32-bit division is 25 dependent instructions, and one thread's chain of them
+// is what a short call waits for at its start.
+__host__ __device__ inline uint32_t qmp_magic(uint32_t d) { return d > 1u ? 0xFFFFFFFFu / d + 1u : 0u; }
+// x / d and its remainder: magic / 2^32 lies above 1 / d by less than 2^-32, so the estimate is at most one too large.
+__device__ __forceinline__ uint32_t qmp_div(uint32_t x, uint32_t d, uint32_t magic, uint32_t& rem) {
+    uint32_t q = magic != 0u ? __umulhi(x, magic) : x;
+    rem = x - q * d;
+    if (rem >= d) { --q; rem += d; }
+    return q;
+}
 
 struct QmpRange {                      // this CTA's share of one matrix
     uint32_t u_begin, u_end;
@@ -204,9 +237,10 @@ __device__ __forceinline__ void qmp_load_group_pair(const void* W, size_t u, uin
     }
 }
 
-__device__ __forceinline__ QmpRange qmp_range(const QmpDesc& d) {
+__device__ __forceinline__ QmpRange qmp_range(const QmpDesc& d, uint32_t grid_magic) {
     QmpRange r;
-    const uint32_t per = (d.num_units + gridDim.x - 1) / gridDim.x;
+    uint32_t rem;
+    const uint32_t per = qmp_div(d.num_units + gridDim.x - 1u, gridDim.x, grid_magic, rem);
     r.u_begin = min(d.num_units, blockIdx.x * per);
     r.u_end = min(d.num_units, r.u_begin + per);
     return r;
@@ -294,6 +328,7 @@ inline QmpDesc qmp_make_desc(const void* W, bool w_bf16, int N, int K, int8_t* v
     d.flip_bits = prev_meta ? flip_bits : nullptr;
     d.num_units = static_cast<uint32_t>(static_cast<size_t>(N) * K / 128);
     d.KB = static_cast<uint32_t>(K / 128);
+    d.kb_magic = qmp_magic(d.KB);
     return d;
 }
 

@@ -31,12 +31,7 @@ __device__ __forceinline__ uint32_t select6of8(const float (&a)[8]) {
     const float l0 = fminf(lo[0], lo[1]), s0 = fmin3(fmaxf(lo[0], lo[1]), hi[0], hi[1]);
     const float l1 = fminf(lo[2], lo[3]), s1 = fmin3(fmaxf(lo[2], lo[3]), hi[2], hi[3]);
     const float t2 = fmin3(fmaxf(l0, l1), s0, s1);
-    uint32_t d[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) d[i] = __float_as_uint(t2 - a[i]);            // sign bit set: larger
-    const uint32_t g03 = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u);     // 0xFF per such column
-    const uint32_t g47 = prmt(prmt(d[4], d[5], 0x00FBu), prmt(d[6], d[7], 0x00FBu), 0x5410u);
-    uint32_t S = (((g03 & 0x08040201u) | (g47 & 0x80402010u)) * 0x01010101u) >> 24;
+    uint32_t S = qmp_byte_bits(sign_bytes4(t2 - a[0], t2 - a[1], t2 - a[2], t2 - a[3]), sign_bytes4(t2 - a[4], t2 - a[5], t2 - a[6], t2 - a[7]));
     int need = 6 - __popc(S);
     if (need != 0) {                                          // a tie: the lowest of the columns that equal t2
 #pragma unroll
@@ -45,6 +40,45 @@ __device__ __forceinline__ uint32_t select6of8(const float (&a)[8]) {
         }
     }
     return S;
+}
+
+// The same for two groups of bf16 weights at once, in halfword arithmetic: r[0 .. 3] and r[4 .. 7] are the groups' words.  Ties
+// are common with 8 significant bits, so their path is short too.
+__device__ __forceinline__ void select6of8_bf16(const uint32_t (&r)[8], uint32_t& S0, uint32_t& S1) {
+    uint32_t p[8];                                            // column j of both groups
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t a = r[i] & kAbs2, b = r[4 + i] & kAbs2;
+        p[2 * i] = prmt(a, b, 0x5410u);
+        p[2 * i + 1] = prmt(a, b, 0x7632u);
+    }
+    uint32_t lo[4], hi[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { lo[i] = __vminu2(p[2 * i], p[2 * i + 1]); hi[i] = __vmaxu2(p[2 * i], p[2 * i + 1]); }
+    const uint32_t l0 = __vminu2(lo[0], lo[1]), s0 = __vminu2(__vmaxu2(lo[0], lo[1]), __vminu2(hi[0], hi[1]));
+    const uint32_t l1 = __vminu2(lo[2], lo[3]), s1 = __vminu2(__vmaxu2(lo[2], lo[3]), __vminu2(hi[2], hi[3]));
+    const uint32_t t2 = __vminu2(__vmaxu2(l0, l1), __vminu2(s0, s1));
+    // flags in bits 15 and 31 of eight words -> a bit per column, group 0 in byte 0, group 1 in byte 1
+    auto gather = [](const uint32_t (&f)[8]) {
+        const uint32_t y = (prmt(f[0], f[1], kSign2) & 0x02020101u) | (prmt(f[2], f[3], kSign2) & 0x08080404u) |
+                           (prmt(f[4], f[5], kSign2) & 0x20201010u) | (prmt(f[6], f[7], kSign2) & 0x80804040u);
+        return (y | (y >> 16)) & 0xFFFFu;
+    };
+    uint32_t f[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) f[j] = sub_abs_bf16x2(t2, p[j]);
+    uint32_t drop = gather(f) ^ 0xFFFFu;                      // |w| <= t2: dropped, unless there are more than two
+    if (__popc(drop) != 4) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = sub_abs_bf16x2(p[j], t2);
+        uint32_t less = gather(f), same = drop & ~less;       // the highest of the equal columns go
+        uint32_t s_lo = same & 0xFFu, s_hi = same >> 8;
+        while (__popc(s_lo) + __popc(less & 0xFFu) > 2) s_lo &= s_lo - 1u;
+        while (__popc(s_hi) + __popc(less >> 8) > 2) s_hi &= s_hi - 1u;
+        drop = less | s_lo | (s_hi << 8);
+    }
+    S0 = ~drop & 0xFFu;
+    S1 = (~drop >> 8) & 0xFFu;
 }
 
 // Deals the kept columns S (6 bits set of 8) out to the three windows: 4-bit masks, two bits each.
@@ -101,16 +135,8 @@ __device__ __forceinline__ size_t vals68_offset(uint32_t n, uint32_t c, uint32_t
 __device__ __forceinline__ void ternary68(const float (&w)[8], const float thr_pred, uint32_t (&e)[8], uint32_t& b03, uint32_t& b47) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(thr_pred - fabsf(w[i]));
-    uint32_t b[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const uint32_t keep = prmt(prmt(e[4 * h], e[4 * h + 1], 0x00FBu), prmt(e[4 * h + 2], e[4 * h + 3], 0x00FBu), 0x5410u);
-        const uint32_t sign = prmt(prmt(__float_as_uint(w[4 * h]), __float_as_uint(w[4 * h + 1]), 0x00FBu),
-                                   prmt(__float_as_uint(w[4 * h + 2]), __float_as_uint(w[4 * h + 3]), 0x00FBu), 0x5410u);
-        b[h] = (sign | 0x01010101u) & keep;
-    }
-    b03 = b[0];
-    b47 = b[1];
+    b03 = (sign_bytes4(w[0], w[1], w[2], w[3]) | 0x01010101u) & sign_bytes4(e[0], e[1], e[2], e[3]);
+    b47 = (sign_bytes4(w[4], w[5], w[6], w[7]) | 0x01010101u) & sign_bytes4(e[4], e[5], e[6], e[7]);
 }
 
 // Values of this CTA's range again with the exact threshold (what qmp_pass2_full is for 2:4): a half-warp per unit, a lane

@@ -32,6 +32,8 @@
 //   three lists   matrix m - 1 is being fixed up while m waits and m + 1 is being written; a computing
 //                 warp starts matrix m only once m - 3 is fixed (its list slot is free) and the job
 //                 of m exists -- both normally long done.
+//   first look    a single long matrix without a hint: the finishers exchange what the first stages of all CTAs said about
+//                 the mean, while pass 1 runs, and narrow the bracket (qmp_look_report).
 //   tail          after the last matrix every warp joins: fix-up of the last matrix, then
 //                 the exact second passes that were put off (bracket missed, list overflow, or the
 //                 dense W_q wanted), all threads working.
@@ -76,13 +78,13 @@ struct QmpJob {
     uint8_t* meta;
     const uint8_t* prev;                                   // or null
     uint32_t KB;
-    uint32_t kb_magic;                                     // x / KB = umulhi(x, kb_magic) for the small x of a range's start; 0: KB = 1
+    uint32_t kb_magic;                                     // qmp_magic(KB)
     uint32_t units;                                        // of this CTA's range
     uint32_t n0, kb0;                                      // row and 128-column block of its first unit
     uint32_t rep_n, rep_kb;                                // kQmpStepUnits units further (next step of a stage)
     uint32_t next_n, next_kb;                              // from the last step of a stage to the first of the team's next one
     uint32_t bf16;
-    float lo, hi;                                          // bracket around the threshold
+    float2 bracket;                                        // around the threshold: lo, hi; may become narrower under way (one 8-byte store)
     int ready;                                             // m + 1 once the rest is that of matrix m
 };
 
@@ -96,6 +98,9 @@ struct QmpStreamShared {
     float thr_tail;
     int tail_second_pass;
     float sample[kQmpWarps];
+    float look_sum[kQmpStreamWarps];                       // sum |w| of each warp's first step of matrix 0
+    int look;                                              // the first look is wanted (matrix 0 has no hint)
+    unsigned long long bar_look;
     unsigned long long bar_full[kQmpStages];               // a stage's bytes have landed
     unsigned long long bar_empty[kQmpStages];              // the team's warps are done with a stage
     unsigned long long bar_done[kQmpLists];                // the computing warps are done with the matrix in this slot
@@ -212,10 +217,11 @@ __device__ __forceinline__ bool qmp_wait_ge(volatile int* word, int want, volati
 // meets an undecided value, and listing them is a tenth of pass 1's instructions otherwise.  A hint that
 // is off by more than that costs the exact second pass, never the result.
 constexpr float kQmpBracketHint = 0.005f;
-__device__ __forceinline__ void qmp_bracket_from(float gamma_est, uint32_t num_units, bool from_hint, float& lo, float& hi, bool wide = false) {
-    const float b = from_hint ? kQmpBracketHint : ((wide || num_units < kQmpSmallMatrixUnits) ? kQmpBracketSmall : kQmpBracket);
-    lo = 0.5f * fmaxf(gamma_est * (1.0f - b), kEps) * (1.0f - 1e-6f);
-    hi = 0.5f * fmaxf(gamma_est * (1.0f + b), kEps) * (1.0f + 1e-6f);
+__device__ __forceinline__ float2 qmp_bracket(float gamma_est, float b) {
+    return make_float2(0.5f * fmaxf(gamma_est * (1.0f - b), kEps) * (1.0f - 1e-6f), 0.5f * fmaxf(gamma_est * (1.0f + b), kEps) * (1.0f + 1e-6f));
+}
+__device__ __forceinline__ float2 qmp_bracket_from(float gamma_est, uint32_t num_units, bool from_hint, bool wide = false) {
+    return qmp_bracket(gamma_est, from_hint ? kQmpBracketHint : ((wide || num_units < kQmpSmallMatrixUnits) ? kQmpBracketSmall : kQmpBracket));
 }
 
 // The caller's estimate of gamma, if it gave a usable one.
@@ -237,29 +243,59 @@ __device__ __forceinline__ float4 qmp_load_group_raw(const QmpDesc& d, uint32_t 
     const float2 v = __ldg(static_cast<const float2*>(d.W) + static_cast<size_t>(u) * 32 + lane);
     return make_float4(v.x, v.y, 0.0f, 0.0f);
 }
-__device__ __forceinline__ float qmp_abs_sum_raw(const QmpDesc& d, const float4 v) {
-    if (d.w_bf16 == 0u) return (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
+__device__ __forceinline__ float qmp_abs_sum_raw(const bool bf16, const float4 v) {
+    if (!bf16) return (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
     const uint32_t a = __float_as_uint(v.x), b = __float_as_uint(v.y);
     return (fabsf(bf16lo_to_f32(a)) + fabsf(bf16hi_to_f32(a))) + (fabsf(bf16lo_to_f32(b)) + fabsf(bf16hi_to_f32(b)));
 }
-constexpr int kQmpSamplePerWarp = kQmpSampleUnits / kQmpWarps;
-__device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[kQmpSamplePerWarp]) {
+// Where the sampled units lie: number s in [s stride, (s + 1) stride).
+struct QmpSamplePlaces {
+    uint32_t n_s, stride;
+    float inv;
+    __device__ __forceinline__ explicit QmpSamplePlaces(uint32_t num_units) : n_s(qmp_sample_units(num_units)) {
+        // the usual counts are powers of two, a matrix of fewer units is read whole
+        stride = n_s == kQmpSampleUnits ? num_units / kQmpSampleUnits : (n_s == kQmpSampleUnitsSmall ? num_units / kQmpSampleUnitsSmall : 1u);
+        inv = __frcp_rn(static_cast<float>(stride));
+    }
+    __device__ __forceinline__ uint32_t unit(uint32_t s) const {
+        const uint32_t h = (s * 2654435761u) >> 8;                                       // h mod stride; h < 2^24: the quotient is one off at most
+        int rem = static_cast<int>(h - __float2uint_rz(static_cast<float>(h) * inv) * stride);
+        if (rem < 0) rem += static_cast<int>(stride);
+        if (rem >= static_cast<int>(stride)) rem -= static_cast<int>(stride);
+        return s * stride + static_cast<uint32_t>(rem);
+    }
+};
+// The loads carry no condition and no conversion (see above): a place beyond the sample is read as its last unit and left out
+// of the sum.  Small samples take two of a thread's loads, large ones all eight.
+constexpr int kQmpSamplePerWarp = kQmpSampleUnits / kQmpWarps, kQmpSamplePerWarpSmall = kQmpSampleUnitsSmall / kQmpWarps;
+template <int FIRST, int LAST>
+__device__ __forceinline__ void qmp_sample_loads(const QmpDesc& d, const QmpSamplePlaces& places, float4 (&v)[kQmpSamplePerWarp]) {
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const uint32_t n_s = qmp_sample_units(d.num_units);
-    const uint32_t stride = d.num_units / n_s;
+    const uint32_t warp = threadIdx.x >> 5;
+    uint32_t u[LAST - FIRST];
 #pragma unroll
-    for (int i = 0; i < kQmpSamplePerWarp; ++i) {
-        const uint32_t sidx = warp + i * kQmpWarps;
-        const uint32_t u = sidx * stride + ((sidx * 2654435761u) >> 8) % stride;
-        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (sidx < n_s) v[i] = qmp_load_group_raw(d, u, lane);
+    for (int i = FIRST; i < LAST; ++i) u[i - FIRST] = places.unit(min(warp + i * kQmpWarps, places.n_s - 1u));
+    if (d.w_bf16 != 0u) {
+#pragma unroll
+        for (int i = FIRST; i < LAST; ++i)
+            asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v[i].x), "=f"(v[i].y) : "l"(static_cast<const float2*>(d.W) + static_cast<size_t>(u[i - FIRST]) * 32 + lane));
+    } else {
+#pragma unroll
+        for (int i = FIRST; i < LAST; ++i)
+            asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w) : "l"(static_cast<const float4*>(d.W) + static_cast<size_t>(u[i - FIRST]) * 32 + lane));
     }
 }
+__device__ __forceinline__ void qmp_sample_issue(const QmpDesc& d, float4 (&v)[kQmpSamplePerWarp]) {
+    const QmpSamplePlaces places(d.num_units);
+    qmp_sample_loads<0, kQmpSamplePerWarpSmall>(d, places, v);
+    if (places.n_s > kQmpSampleUnitsSmall) qmp_sample_loads<kQmpSamplePerWarpSmall, kQmpSamplePerWarp>(d, places, v);
+}
 __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float4 (&v)[kQmpSamplePerWarp], float* s_sample) {
+    const uint32_t n_s = qmp_sample_units(d.num_units), warp = threadIdx.x >> 5;
     float acc = 0.0f;
 #pragma unroll
-    for (int i = 0; i < kQmpSamplePerWarp; ++i) acc += qmp_abs_sum_raw(d, v[i]);
+    for (int i = 0; i < kQmpSamplePerWarp; ++i)
+        if (warp + i * kQmpWarps < n_s) acc += qmp_abs_sum_raw(d.w_bf16 != 0u, v[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
     if ((threadIdx.x & 31) == 0) s_sample[threadIdx.x >> 5] = acc;
@@ -267,16 +303,15 @@ __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float
     float t = s_sample[threadIdx.x & 31];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-    return t / (static_cast<float>(qmp_sample_units(d.num_units)) * 128.0f);
+    return t / (static_cast<float>(n_s) * 128.0f);
 }
 
 // gamma_est by ONE warp (a scout, for matrices 1, 2, ... of a batch without hints) from the first
 // kQmpSampleUnitsSmall of qmp_sample_issue's scattered units, eight in flight at a time.  The smaller sample gets the
 // wider bracket (qmp_bracket_from, `wide`).
 __device__ __forceinline__ float qmp_sample_gamma_warp(const QmpDesc& d, int lane) {
-    const uint32_t n_full = qmp_sample_units(d.num_units);
-    const uint32_t stride = d.num_units / n_full;
-    const uint32_t n_s = min(n_full, static_cast<uint32_t>(kQmpSampleUnitsSmall));
+    const QmpSamplePlaces places(d.num_units);
+    const uint32_t n_s = min(places.n_s, static_cast<uint32_t>(kQmpSampleUnitsSmall));
     float acc = 0.0f;
 #pragma unroll 1
     for (uint32_t s0 = 0; s0 < n_s; s0 += 8u) {
@@ -284,12 +319,11 @@ __device__ __forceinline__ float qmp_sample_gamma_warp(const QmpDesc& d, int lan
 #pragma unroll
         for (uint32_t i = 0; i < 8u; ++i) {
             const uint32_t sidx = s0 + i;
-            const uint32_t u = sidx * stride + ((sidx * 2654435761u) >> 8) % stride;
             v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (sidx < n_s) v[i] = qmp_load_group_raw(d, u, lane);
+            if (sidx < n_s) v[i] = qmp_load_group_raw(d, places.unit(sidx), lane);
         }
 #pragma unroll
-        for (uint32_t i = 0; i < 8u; ++i) acc += qmp_abs_sum_raw(d, v[i]);
+        for (uint32_t i = 0; i < 8u; ++i) acc += qmp_abs_sum_raw(d.w_bf16 != 0u, v[i]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
@@ -309,12 +343,12 @@ struct QmpLoader {
     unsigned long long policy;   // L2 policy of the copies: read once
 };
 __device__ __forceinline__ bool qmp_loader_issue(QmpLoader& L, const QmpBatch& batch, int count, uint32_t max_copies,
-                                                 uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag) {
+                                                 uint32_t grid_magic, uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag) {
     for (;;) {
         while (!L.open) {
             if (L.m >= count) return true;
             const QmpDesc d = qmp_desc_of(batch, L.m);
-            const QmpRange rg = qmp_range(d);
+            const QmpRange rg = qmp_range(d, grid_magic);
             L.u = rg.u_begin;
             L.u_end = rg.u_end;
             L.unit_bytes = d.w_bf16 ? 256u : 512u;
@@ -337,22 +371,18 @@ __device__ __forceinline__ bool qmp_loader_issue(QmpLoader& L, const QmpBatch& b
 }
 
 // The job of matrix d for this CTA (everything but the bracket).
-__device__ __forceinline__ void qmp_make_job(const QmpDesc& d, QmpJob& jb) {
-    const QmpRange rg = qmp_range(d);
+__device__ __forceinline__ void qmp_make_job(const QmpDesc& d, uint32_t grid_magic, QmpJob& jb) {
+    const QmpRange rg = qmp_range(d, grid_magic);
     jb.vals = reinterpret_cast<unsigned char*>(d.vals);
     jb.meta = d.meta;
     jb.prev = d.prev_meta;
     jb.KB = d.KB;
-    jb.kb_magic = d.KB > 1u ? 0xFFFFFFFFu / d.KB + 1u : 0u;         // exact: x * KB < 2^32 for x < KB + a turn of the teams
+    jb.kb_magic = d.kb_magic;
     jb.units = rg.u_end - rg.u_begin;
-    jb.n0 = rg.u_begin / d.KB;
-    jb.kb0 = rg.u_begin - jb.n0 * d.KB;
-    jb.rep_n = kQmpStepUnits / d.KB;
-    jb.rep_kb = kQmpStepUnits % d.KB;
-    const uint32_t reps = kQmpStageBytes / (kQmpStepUnits * (d.w_bf16 ? 256u : 512u));
-    const uint32_t next = (kQmpTeams * reps - reps + 1u) * kQmpStepUnits;
-    jb.next_n = next / d.KB;
-    jb.next_kb = next % d.KB;
+    jb.n0 = qmp_div(rg.u_begin, d.KB, d.kb_magic, jb.kb0);
+    jb.rep_n = qmp_div(kQmpStepUnits, d.KB, d.kb_magic, jb.rep_kb);
+    const uint32_t next = (d.w_bf16 ? 2u * kQmpTeams - 1u : kQmpTeams) * kQmpStepUnits;     // two steps per stage of bf16 weights
+    jb.next_n = qmp_div(next, d.KB, d.kb_magic, jb.next_kb);
     jb.bf16 = d.w_bf16;
 }
 
@@ -391,6 +421,14 @@ __device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
     return __popc(any | (none << 1));
 }
 
+// The bracket of a step as two numbers: kept values are +-1 iff thr_pred - |w| is negative, undecided iff it is at most width.
+__device__ __forceinline__ void qmp_thresholds(const QmpJob& jb, float& thr_pred, uint32_t& width) {
+    float lo, hi;
+    asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(hi) : "r"(qmp_smem_u32(&jb.bracket)));
+    thr_pred = __uint_as_float(__float_as_uint(hi) - 1u);
+    width = __float_as_uint(thr_pred - lo);
+}
+
 // Where a computing warp is in a matrix: its quarter-warp's unit of the current step of its team's stages.
 template <bool BF16>
 struct QmpWalk {
@@ -400,10 +438,7 @@ struct QmpWalk {
     int left;                             // > 0: the quarter-warp has a unit in the step
     __device__ __forceinline__ QmpWalk(const QmpJob& jb, uint32_t stage_in_matrix, uint32_t in_step) {
         const uint32_t u0 = stage_in_matrix * (REP * kQmpStepUnits) + in_step;         // from the range's start
-        const uint32_t k0 = jb.kb0 + u0;
-        const uint32_t dn = jb.kb_magic != 0u ? __umulhi(k0, jb.kb_magic) : k0;
-        n = jb.n0 + dn;
-        kb = k0 - dn * jb.KB;
+        n = jb.n0 + qmp_div(jb.kb0 + u0, jb.KB, jb.kb_magic, kb);
         left = static_cast<int>(jb.units) - static_cast<int>(u0);
     }
     __device__ __forceinline__ void advance(const QmpJob& jb, uint32_t KB, bool in_stage) {
@@ -413,6 +448,30 @@ struct QmpWalk {
         left -= static_cast<int>((in_stage ? 1u : (kQmpTeams * REP - REP + 1u)) * kQmpStepUnits);
     }
 };
+
+// The first look: a matrix without a hint starts with a wide bracket (a sample of 64 or 256 units), and nearly every warp meets
+// undecided weights in every step then -- a fifth of pass 1's time.  So the CTAs tell each other, in the same slots but under
+// another tag, the mean |w| of what they have seen after their teams' first stages, and the bracket becomes as narrow as the spread of
+// these means allows (five standard errors: 0.3 % for Gaussian weights).  Nobody waits for it: the finisher looks while pass 1
+// runs and gives up when it has ended, and a CTA that is already done (its exchange's tag is in the slot) is left out.  Results
+// never depend on the bracket.
+constexpr unsigned long long kQmpLookTag = 1ull << 63;
+constexpr float kQmpLookErrors = 5.0f, kQmpLookLeast = 0.001f;
+// From this many units of a CTA on: shorter ranges are over before the answer is there, and then it costs them up to 2 us (bf16, 519 units
+// per CTA, us with / without: 21.0 / 19.1; 934 units: fp32 23.8 / 24.9, 6:8 31.1 / 33.4).
+constexpr uint32_t kQmpLookFrom = 700;
+__device__ __forceinline__ void qmp_look_report(QmpStreamShared& sh, double acc) {
+    float sum = static_cast<float>(acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    if ((threadIdx.x & 31u) == 0u) {
+        sh.look_sum[threadIdx.x >> 5] = sum;
+        qmp_mbar_arrive(qmp_smem_u32(&sh.bar_look));
+    }
+}
+__device__ __forceinline__ uint32_t qmp_look_units(uint32_t units, uint32_t bf16) {      // of a CTA's range: the first stage of each team
+    return min(units, kQmpTeams * (bf16 ? 2u : 1u) * kQmpStepUnits);
+}
 
 // Pass 1 of one matrix for a computing warp: its four units of every step of its team's stages (a quarter-warp per
 // unit, a lane 16 weights = four groups).  The matrix's stages are the ring's g0 .. g0 + n - 1, the team's next one is
@@ -430,8 +489,8 @@ struct QmpWalk {
 //
 // A lane's 64 B (fp32) are read as 16-byte pieces in rotated order, (i + l8 / 2) mod 4, so that the eight lanes of a
 // unit hit different banks; the rotation is undone on the 8 + 2 result bytes (two byte permutes, one shift).
-template <bool BF16>
-__device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
+template <bool BF16, bool LOOK>
+__device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamShared& sh, bool look, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
                                                    uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok) {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = threadIdx.x >> 5;
@@ -443,8 +502,6 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     // kept is +-1 iff |k| > thr_pred, undecided iff 0 <= thr_pred - |k| <= width.  The subtraction is exact near the
     // threshold and monotone everywhere: a value wrongly taken for undecided can only lie below thr_lo, and the
     // fix-up decides it like any other.
-    const float thr_pred = __uint_as_float(__float_as_uint(jb.hi) - 1u);
-    const uint32_t width = __float_as_uint(thr_pred - jb.lo);
     const uint32_t n_stages = (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
     const uint32_t g_end = g0 + n_stages;
     double acc = 0.0;
@@ -471,11 +528,22 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
     uint32_t q = tiled_row(at.n, at.kb);
     uint32_t prev = 0u;
     if (prev_lane != nullptr && at.left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
+    float thr_pred;
+    uint32_t width;
+    if constexpr (!LOOK) qmp_thresholds(jb, thr_pred, width);
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
+        if constexpr (LOOK) qmp_thresholds(jb, thr_pred, width);      // may have become narrower
 #pragma unroll
         for (uint32_t rep = 0; rep < REP; ++rep) {
+            // The warp has no unit in this step (a matrix's last stage): nothing to do.  (Batch of 14 bf16 tensors 124 -> 120 us; batches of
+            // fp32 ones, which wait for memory, were 0.5 % slower with it.)
+            if ((BF16 || LOOK) && at.left + (lane >> 3) <= 0) {
+                if (rep + 1 == REP && lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);
+                at.advance(jb, KB, rep + 1 < REP);
+                continue;
+            }
             float4 raw[PIECES];
             // a lane without a unit (last stage only) reads what is there: it is not used
 #pragma unroll
@@ -535,17 +603,128 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpWarpList
                                 return j & 4 ? (j & 2 ? d : c) : (j & 2 ? b : a);
                             });
         }
+        if constexpr (LOOK) {
+            if (look) { qmp_look_report(sh, acc); look = false; }
+        }
+    }
+    if constexpr (LOOK) {
+        if (look) qmp_look_report(sh, 0.0);                           // no stage of this matrix was the team's
     }
     g0 = g_end;
     flips *= 2u;
     return acc;
 }
 
+// The bracket as the computing warps use it.  fp32: a weight is kept as +-1 iff |w| > thr_pred, i.e. iff thr_pred - |w| is
+// negative, and undecided iff that difference lies in 0 .. width (an unsigned compare of the bits; the subtraction is exact near
+// the threshold and monotone everywhere).  bf16: the largest |w| that is not above / not inside the bracket, in both halves.
+template <bool BF16>
+struct QmpBracket {
+    float thr_pred, lo_pred;
+    uint32_t width;
+    uint32_t hi2, lo2;
+    __device__ __forceinline__ QmpBracket(float lo, float hi) {
+        const uint32_t hi_bits = __float_as_uint(hi) - 1u, lo_bits = __float_as_uint(lo) - 1u;
+        thr_pred = __uint_as_float(hi_bits);
+        lo_pred = __uint_as_float(lo_bits);
+        width = __float_as_uint(thr_pred - lo);
+        hi2 = (hi_bits >> 16) * 0x10001u;
+        lo2 = (lo_bits >> 16) * 0x10001u;
+    }
+};
+// Eight consecutive weights (half of a lane's 16): fp32 in eight words, bf16 in four.
+// Sum |w| in fp64.  |bf16| becomes a double by two integer instructions (see bf16_abs_to_f64 in norm_quant_act.cuh: a zero
+// counts as 2^-127, which no sum above the 1e-5 clamp can see); fp32 takes the conversion instruction.
+template <bool BF16>
+__device__ __forceinline__ double qmp_abs_sum8(const uint32_t* r) {
+    double d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if constexpr (BF16) {
+            const uint32_t w = r[i >> 1];
+            d[i] = __hiloint2double(static_cast<int>(((i & 1) ? (w & 0x7FFF0000u) >> 3 : (w & 0x7FFFu) << 13) + 0x38000000u), 0);
+        } else {
+            d[i] = static_cast<double>(fabsf(__uint_as_float(r[i])));
+        }
+    }
+    return ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7]));
+}
+
+// Ternary bytes of eight weights at the upper end of the bracket (t_lo, t_hi), and whether one of them may be undecided.
+// Byte order: columns 0 .. 7.
+template <bool BF16>
+__device__ __forceinline__ void qmp_ternary8(const uint32_t* r, const QmpBracket<BF16>& br, uint32_t& t_lo, uint32_t& t_hi, bool& maybe) {
+    uint32_t sign_lo, sign_hi, keep_lo, keep_hi;
+    if constexpr (BF16) {
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { h[i] = sub_abs_bf16x2(br.hi2, r[i]); l[i] = sub_abs_bf16x2(br.lo2, r[i]); }
+        const uint32_t open = ((l[0] & ~h[0]) | (l[1] & ~h[1])) | ((l[2] & ~h[2]) | (l[3] & ~h[3]));
+        keep_lo = prmt(h[0], h[1], kSign2); keep_hi = prmt(h[2], h[3], kSign2);
+        sign_lo = prmt(r[0], r[1], kSign2); sign_hi = prmt(r[2], r[3], kSign2);
+        maybe |= (open & kGuard2) != 0u;
+    } else {
+        uint32_t e[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(br.thr_pred - fabsf(__uint_as_float(r[i])));
+        keep_lo = sign_bytes4(e[0], e[1], e[2], e[3]); keep_hi = sign_bytes4(e[4], e[5], e[6], e[7]);
+        sign_lo = sign_bytes4(r[0], r[1], r[2], r[3]); sign_hi = sign_bytes4(r[4], r[5], r[6], r[7]);
+        maybe |= umin8(e) <= br.width;
+    }
+    t_lo = (sign_lo | 0x01010101u) & keep_lo;
+    t_hi = (sign_hi | 0x01010101u) & keep_hi;
+}
+// Byte masks of the undecided ones among them: inside the bracket and not kept as +-1.
+template <bool BF16>
+__device__ __forceinline__ void qmp_undecided8(const uint32_t* r, const QmpBracket<BF16>& br, uint32_t t_lo, uint32_t t_hi, uint32_t& u_lo, uint32_t& u_hi) {
+    if constexpr (BF16) {
+        uint32_t g[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g[i] = sub_abs_bf16x2(br.lo2, r[i]);
+        u_lo = prmt(g[0], g[1], kSign2); u_hi = prmt(g[2], g[3], kSign2);
+    } else {
+        uint32_t e[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(br.lo_pred - fabsf(__uint_as_float(r[i])));
+        u_lo = sign_bytes4(e[0], e[1], e[2], e[3]); u_hi = sign_bytes4(e[4], e[5], e[6], e[7]);
+    }
+    u_lo &= ~((t_lo & 0x01010101u) * 0xFFu);                          // a byte of t is 0, 1 or 0xFF
+    u_hi &= ~((t_hi & 0x01010101u) * 0xFFu);
+}
+
+template <bool BF16>
+__device__ __forceinline__ float qmp_lds_weight(uint32_t addr) {
+    if constexpr (BF16) {
+        uint16_t v;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+        return __uint_as_float(static_cast<uint32_t>(v) << 16);
+    } else {
+        float v;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+        return v;
+    }
+}
+
+// Reads the 16 weights of a lane: eight words of bf16 or sixteen of fp32, in 16-byte pieces from src[i] + off.
+template <int PIECES>
+__device__ __forceinline__ void qmp_lds_pieces(const uint32_t (&src)[PIECES], uint32_t off, uint32_t (&r)[4 * PIECES]) {
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i)
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[4 * i]), "=r"(r[4 * i + 1]), "=r"(r[4 * i + 2]), "=r"(r[4 * i + 3]) : "r"(src[i] + off));
+}
+
 // Pass 1 for the 6:8 pattern.  As above; a lane's 16 weights are two groups of 8, which leave as 12 value bytes (three 4-byte
 // stores) and 24 bits of metadata (a quad of lanes has 12 bytes, its lanes 0..2 store 4 each).  The two groups are read in the
 // order that halves the bank conflicts of the 64 B (fp32; none for bf16) per lane and put in place on the results.
+//
+// The ALU pipe (byte permutes, logic, minima: half rate) bounds it, so comparisons are subtractions on the FMA pipe whose sign bits
+// are gathered by byte permutes, and bf16 weights are selected two to a word.  The undecided are looked for only if one of the
+// warp's weights lies inside the bracket, for both groups at once, and their weights come from the stage again (held until then) instead of
+// a tree of selects.  Single calls without a hint, us, before / now (with the loops over matrices gone and the first look):
+// 2560 -> 2560 fp32 20.8 / 17.4, 2560 -> 6912 fp32 36.9 / 31.1, bf16 38.2 / 29.1 (memory: 13.5 and 8.1).
 template <bool BF16>
-__device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
+__device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpStreamShared& sh, bool look, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
                                                      uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok,
                                                      const uint2* table) {
     const int lane = threadIdx.x & 31;
@@ -553,16 +732,17 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
     const uint32_t l8 = lane & 7, quad = l8 & 3u;
     using Walk = QmpWalk<BF16>;
     constexpr uint32_t kUnitBytes = Walk::kUnitBytes, REP = Walk::REP;
+    constexpr int PIECES = BF16 ? 2 : 4;
     const uint32_t KB = jb.KB, KBp = KB + (KB >> 1);                  // K' / 128
-    const float thr_pred = __uint_as_float(__float_as_uint(jb.hi) - 1u);
-    const uint32_t width = __float_as_uint(thr_pred - jb.lo);
     const uint32_t g_end = g0 + (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
     double acc = 0.0;
     const uint32_t in_step = 4u * (warp % kQmpTeamWarps) + (lane >> 3);
     Walk at(jb, next_stage - g0, in_step);
     const uint32_t swap = BF16 ? (l8 >> 2) : ((l8 >> 1) & 1u);        // the second group is read first
     const uint32_t src0 = ring_base + in_step * kUnitBytes + l8 * (kUnitBytes / 8u);
-    const uint32_t src[2] = {src0 + swap * (kUnitBytes / 16u), src0 + (swap ^ 1u) * (kUnitBytes / 16u)};
+    uint32_t src[PIECES];
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) src[i] = src0 + 16u * (static_cast<uint32_t>(i) ^ (swap * (PIECES / 2)));
     // Column block kb of a row starts at byte 96 kb of its values and 24 kb of its metadata in the [N][K'] form: in tile 3 kb / 2,
     // for odd kb half a tile in.  With q = the row's index in that tile, a lane's three words of values are at
     // 64 q + (v ^ the row's swizzle) and its word of its quad's metadata at 16 q + m, v and m constants for even
@@ -586,19 +766,18 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
+        float lo, hi;
+        asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(hi) : "r"(qmp_smem_u32(&jb.bracket)));
+        const QmpBracket<BF16> br(lo, hi);
 #pragma unroll 1
         for (uint32_t rep = 0; rep < REP; ++rep) {
+            if (at.left + (lane >> 3) <= 0) {                         // the warp has no unit in this step (a matrix's last stage)
+                at.advance(jb, KB, rep + 1 < REP);
+                continue;
+            }
+            uint32_t r[4 * PIECES];
             const uint32_t off = stage * kQmpStageBytes + rep * (kQmpStepUnits * kUnitBytes);
-            float4 raw[2][BF16 ? 1 : 2];
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                raw[g][0] = qmp_lds128(src[g] + off);
-                if constexpr (!BF16) raw[g][1] = qmp_lds128(src[g] + off + 16u);
-            }
-            if (rep + 1 == REP) {
-                __syncwarp();
-                if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);
-            }
+            qmp_lds_pieces(src, off, r);
             const bool mine = at.left > 0;
             const uint32_t q_cur = q, odd_cur = at.kb & 1u, prev_cur = prev;
             const uint32_t half = odd_cur ? 0x4432u : 0x4410u, swizzle = ((at.n >> 1) & 3u) << 4;
@@ -606,48 +785,32 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
             q = tiled_row(at.n, at.kb);
             if (has_prev && quad < 3u && at.left > 0) prev = *reinterpret_cast<const uint32_t*>(jb.prev + meta_at(q, at.kb));
             auto v_off = [&](uint32_t v) { return prmt(v, 0u, half) ^ swizzle; };           // on top of 64 q_cur
-            uint32_t v4[2], v2[2], m12[2], S[2];
-            double sum = 0.0;
+            constexpr int kHalf = 2 * PIECES;                         // words of a group
+            uint32_t S[2];
+            if constexpr (BF16) {
+                select6of8_bf16(r, S[0], S[1]);
+            } else {
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    float a[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) a[i] = fabsf(__uint_as_float(r[8 * g + i]));
+                    S[g] = select6of8(a);
+                }
+            }
+            uint2 entry[2];
+            uint32_t t_lo[2], t_hi[2], v4[2], v2[2];
+            bool maybe = false;
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
-                float w[8], a[8];
-                if constexpr (BF16) {
-                    const float4 r = raw[g][0];
-                    const uint32_t r4[4] = {__float_as_uint(r.x), __float_as_uint(r.y), __float_as_uint(r.z), __float_as_uint(r.w)};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { w[2 * i] = bf16lo_to_f32(r4[i]); w[2 * i + 1] = bf16hi_to_f32(r4[i]); }
-                } else {
-                    w[0] = raw[g][0].x; w[1] = raw[g][0].y; w[2] = raw[g][0].z; w[3] = raw[g][0].w;
-                    w[4] = raw[g][1].x; w[5] = raw[g][1].y; w[6] = raw[g][1].z; w[7] = raw[g][1].w;
-                }
-                sum += abs_sum4(make_float4(w[0], w[1], w[2], w[3])) + abs_sum4(make_float4(w[4], w[5], w[6], w[7]));
-#pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = fabsf(w[i]);
-                S[g] = select6of8(a);
-                const uint2 entry = table[S[g]];
-                uint32_t e[8], b03, b47;
-                ternary68(w, thr_pred, e, b03, b47);
-                v4[g] = prmt(b03, b47, entry.x);
-                v2[g] = prmt(b03, b47, entry.x >> 16) & 0xFFFFu;
-                m12[g] = entry.y;
-                uint32_t und = 0u;
-                if (mine && umin8(e) <= width) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
-                    und &= S[g];
-                }
-                qmp_list_append(list, und,
-                                [&](int j) {
-                                    const uint32_t at_byte = 6u * (static_cast<uint32_t>(g) ^ swap) + __popc(S[g] & ((1u << j) - 1u));   // of the lane's 12
-                                    return q_cur * 64u + v_off(at_byte < 4u ? v_const[0] : (at_byte < 8u ? v_const[1] : v_const[2])) + (at_byte & 3u);
-                                },
-                                [&](int j) {
-                                    const float x = j & 1 ? w[1] : w[0], y = j & 1 ? w[3] : w[2], z = j & 1 ? w[5] : w[4], u = j & 1 ? w[7] : w[6];
-                                    return j & 4 ? (j & 2 ? u : z) : (j & 2 ? y : x);
-                                });
+                entry[g] = table[S[g]];
+                qmp_ternary8<BF16>(r + kHalf * g, br, t_lo[g], t_hi[g], maybe);
+                v4[g] = prmt(t_lo[g], t_hi[g], entry[g].x);
+                v2[g] = prmt(t_lo[g], t_hi[g], entry[g].x >> 16);     // two bytes
             }
+            const double sum = qmp_abs_sum8<BF16>(r) + qmp_abs_sum8<BF16>(r + kHalf);
             const uint32_t f4 = swap ? v4[1] : v4[0], f2 = swap ? v2[1] : v2[0], l4 = swap ? v4[0] : v4[1], l2 = swap ? v2[0] : v2[1];
-            const uint32_t m24 = swap ? (m12[1] | (m12[0] << 12)) : (m12[0] | (m12[1] << 12));
+            const uint32_t m24 = swap ? (entry[1].y | (entry[0].y << 12)) : (entry[0].y | (entry[1].y << 12));
             const uint32_t nxt = __shfl_down_sync(0xFFFFFFFFu, m24, 1);
             if (has_prev) {
                 // this lane's 24 bits of the previous metadata, from its own and the lane before's word
@@ -661,11 +824,34 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpWarpLi
                 if (quad < 3u) *reinterpret_cast<uint32_t*>(jb.meta + meta_at(q_cur, odd_cur)) = (m24 >> (8u * quad)) | (nxt << (24u - 8u * quad));
                 unsigned char* const row = jb.vals + static_cast<size_t>(q_cur) * 64u;
                 *reinterpret_cast<uint32_t*>(row + v_off(v_const[0])) = f4;
-                *reinterpret_cast<uint32_t*>(row + v_off(v_const[1])) = f2 | (l4 << 16);
-                *reinterpret_cast<uint32_t*>(row + v_off(v_const[2])) = (l4 >> 16) | (l2 << 16);
+                *reinterpret_cast<uint32_t*>(row + v_off(v_const[1])) = prmt(f2, l4, 0x5410u);
+                *reinterpret_cast<uint32_t*>(row + v_off(v_const[2])) = prmt(l4, l2, 0x5432u);
+            }
+            if (__any_sync(0xFFFFFFFFu, mine && maybe)) {
+                uint32_t und = 0u;
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    uint32_t u_lo, u_hi;
+                    qmp_undecided8<BF16>(r + kHalf * g, br, t_lo[g], t_hi[g], u_lo, u_hi);
+                    und |= (qmp_byte_bits(u_lo, u_hi) & S[g]) << (8 * g);
+                }
+                qmp_list_append(list, mine ? und : 0u,
+                                [&](int j) {                          // column j & 7 of the group read as number j >> 3
+                                    const uint32_t g = static_cast<uint32_t>(j) >> 3;
+                                    const uint32_t at_byte = 6u * (g ^ swap) + __popc((g ? S[1] : S[0]) & ((1u << (j & 7)) - 1u));   // of the lane's 12
+                                    return q_cur * 64u + v_off(at_byte < 4u ? v_const[0] : (at_byte < 8u ? v_const[1] : v_const[2])) + (at_byte & 3u);
+                                },
+                                [&](int j) {
+                                    const uint32_t g = (static_cast<uint32_t>(j) >> 3) ^ swap;
+                                    return qmp_lds_weight<BF16>(src0 + off + g * (kUnitBytes / 16u) + (j & 7) * (kUnitBytes / 128u));
+                                });
             }
         }
+        __syncwarp();
+        if (lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);      // the stage may be refilled
+        if (look) { qmp_look_report(sh, acc); look = false; }
     }
+    if (look) qmp_look_report(sh, 0.0);
     g0 = g_end;
     return acc;
 }
@@ -675,13 +861,18 @@ __device__ __forceinline__ void qmp_slot_store(QmpSlot* slot, unsigned long long
     asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                  ::"l"(slot), "l"(tag), "l"(__double_as_longlong(partial)) : "memory");
 }
-__device__ __forceinline__ bool qmp_slot_load(const QmpSlot* slot, unsigned long long tag, double& partial) {
+__device__ __forceinline__ unsigned long long qmp_slot_peek(const QmpSlot* slot, double& partial) {
     unsigned long long t;
     long long v;
     asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
                  : "=l"(t), "=l"(v) : "l"(slot) : "memory");
-    if (t != tag) return false;
     partial = __longlong_as_double(v);
+    return t;
+}
+__device__ __forceinline__ bool qmp_slot_load(const QmpSlot* slot, unsigned long long tag, double& partial) {
+    double v;
+    if (qmp_slot_peek(slot, v) != tag) return false;
+    partial = v;
     return true;
 }
 
@@ -723,6 +914,51 @@ __device__ __forceinline__ bool qmp_exchange(const QmpSlot* base, unsigned long 
     return true;
 }
 
+// The first look, by the finisher (see qmp_look_report).  Returns when the bracket has been narrowed or pass 1 of matrix 0 is over.
+__device__ __forceinline__ bool qmp_look_exchange(const QmpDesc& first, QmpStreamShared& sh, QmpSlot* slots, unsigned long long tag, int lane, volatile int* abort_flag) {
+    if (!qmp_mbar_wait(qmp_smem_u32(&sh.bar_look), 0u, abort_flag)) return false;
+    QmpJob& jb = sh.job[0];
+    const uint32_t seen = qmp_look_units(jb.units, jb.bf16), bar_done = qmp_smem_u32(&sh.bar_done[0]);
+    float sum = lane < kQmpStreamWarps ? sh.look_sum[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    if (lane == 0) qmp_slot_store(slots + blockIdx.x, tag ^ kQmpLookTag, seen != 0u ? static_cast<double>(sum / (128.0f * static_cast<float>(seen))) : -1.0);
+    __syncwarp();
+    constexpr int kPerLane = (kQmpMaxCtas + 31) / 32;
+    uint32_t missing = 0u;
+    float n = 0.0f, s1 = 0.0f, s2 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < kPerLane; ++j)
+        if (lane + 32u * j < gridDim.x) missing |= 1u << j;
+    while (__any_sync(0xFFFFFFFFu, missing != 0u)) {
+        if (__any_sync(0xFFFFFFFFu, qmp_mbar_try_wait(bar_done, 0u) || *abort_flag != 0)) return true;      // pass 1 has ended (or will not): too late
+#pragma unroll
+        for (int j = 0; j < kPerLane; ++j) {
+            double mean;
+            if (((missing >> j) & 1u) != 0u) {
+                const unsigned long long got = qmp_slot_peek(&slots[lane + 32 * j], mean);
+                if (got == tag || got == (tag ^ kQmpLookTag)) missing &= ~(1u << j);
+                if (got == (tag ^ kQmpLookTag) && mean > 0.0) { const float v = static_cast<float>(mean); n += 1.0f; s1 += v; s2 += v * v; }
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        n += __shfl_xor_sync(0xFFFFFFFFu, n, o);
+        s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, o);
+        s2 += __shfl_xor_sync(0xFFFFFFFFu, s2, o);
+    }
+    const float gamma = s1 / n, error = sqrtf(fmaxf(s2 / n - gamma * gamma, 0.0f) / n) / gamma, b = kQmpLookErrors * error + kQmpLookLeast;
+    if (lane == 0 && n >= 32.0f && b > 0.0f && b < kQmpBracketSmall) {
+        const float2 wide = jb.bracket, narrow = qmp_bracket(gamma, b);
+        const float lo = fmaxf(wide.x, narrow.x), hi = fminf(wide.y, narrow.y);
+        // outside what pass 1 has used so far: the exact threshold will miss one of the two, or the sample was far off
+        if (lo < hi) asm volatile("st.volatile.shared.v2.f32 [%0], {%1, %2};" ::"r"(qmp_smem_u32(&jb.bracket)), "f"(lo), "f"(hi) : "memory");
+    }
+    __syncwarp();
+    return true;
+}
+
 // ternary_threshold by a whole warp: lane i tries the i-th float from 8 below scale / 2, the lowest that passes is it.
 __device__ __forceinline__ float qmp_threshold_warp(float scale, int lane) {
     const float a = __uint_as_float(__float_as_uint(0.5f * scale) - 8u + lane);
@@ -733,7 +969,7 @@ __device__ __forceinline__ float qmp_threshold_warp(float scale, int lane) {
 // Do the listed values suffice, or must the whole range be ternarised again with the exact threshold?
 template <int PATTERN>
 __device__ __forceinline__ bool qmp_bracket_holds(const QmpDesc& d, float thr, const QmpJob& jb, unsigned int longest_list, uint32_t list_cap) {
-    return jb.lo <= thr && thr <= jb.hi && longest_list <= list_cap && d.dense_q == nullptr &&
+    return jb.bracket.x <= thr && thr <= jb.bracket.y && longest_list <= list_cap && d.dense_q == nullptr &&
            d.num_units <= (PATTERN == 68 ? 1u << 25 : 1u << 26);     // listed byte offsets are 32-bit
 }
 __device__ __forceinline__ void qmp_fix_entry(uint8_t* vals, const QmpEntry e, float thr) {
@@ -742,8 +978,8 @@ __device__ __forceinline__ void qmp_fix_entry(uint8_t* vals, const QmpEntry e, f
 
 // Ternarises this CTA's range of matrix d again with the exact threshold.
 template <int PATTERN>
-__device__ __forceinline__ void qmp_second_pass(const QmpDesc& d, float thr, const uint2* table) {
-    const QmpRange rg = qmp_range(d);
+__device__ __forceinline__ void qmp_second_pass(const QmpDesc& d, uint32_t grid_magic, float thr, const uint2* table) {
+    const QmpRange rg = qmp_range(d, grid_magic);
     if constexpr (PATTERN == 68) {
         if (d.w_bf16) qmp68_pass2_full<true>(d, rg, thr, table);
         else qmp68_pass2_full<false>(d, rg, thr, table);
@@ -753,12 +989,16 @@ __device__ __forceinline__ void qmp_second_pass(const QmpDesc& d, float thr, con
     }
 }
 
-// PATTERN: 24 (2:4) or 68 (6:8).
-template <int PATTERN>
+// PATTERN: 24 (2:4) or 68 (6:8).  SINGLE: one matrix, known at compile time.  Without the loops over matrices a call is 1 to 2 us
+// shorter (2560 -> 2560, no hint, with the first look and the set-up's divisions replaced, us before / now: fp32 17.4 / 15.7, bf16
+// 16.9 / 14.5; 2560 -> 6912 26.5 / 23.8 and 25.3 / 22.9; 4096 -> 11008 50 / 44.3 and 46 / 39.7); the first look would
+// cost a batch 1 %.
+template <int PATTERN, bool SINGLE>
 __global__ void __launch_bounds__(kQmpThreads, 1)
-quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, const QmpDesc* __restrict__ rest, int count,
+quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, const QmpDesc* __restrict__ rest, int n_matrices,
                                  QmpSlot* slots, unsigned long long* generation, unsigned long long call_nonce,
-                                 int test_withhold_slot, QmpMemo* memo) {
+                                 int test_withhold_slot, QmpMemo* memo, uint32_t grid_magic) {
+    const int count = SINGLE ? 1 : n_matrices;
     extern __shared__ __align__(128) unsigned char s_dyn[];   // [kQmpStages][kQmpStageBytes] ring, then kQmpLists * kQmpListEntries entries
     QmpEntry* const s_list = reinterpret_cast<QmpEntry*>(s_dyn + kQmpStages * kQmpStageBytes);
     const uint32_t list_cap = qmp_list_cap(count);
@@ -781,6 +1021,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         sh.ring_issued = 0u; sh.ring_used = 0u;
         for (int i = 0; i < kQmpJobs; ++i) sh.job[i].ready = 0;
         for (int i = 0; i < kQmpLists; ++i) qmp_mbar_init(bar_done0 + 8u * i, kQmpStreamWarps);
+        qmp_mbar_init(qmp_smem_u32(&sh.bar_look), kQmpStreamWarps);
         for (int i = 0; i < kQmpStages; ++i) {
             qmp_mbar_init(bar_full0 + 8u * i, 1u);                     // the loader's expect_tx
             qmp_mbar_init(bar_empty0 + 8u * i, kQmpTeamWarps);         // one arrival per computing warp of the stage's team
@@ -788,7 +1029,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (threadIdx.x == 32) qmp_make_job(first, sh.job[0]);
+    if (threadIdx.x == 32) qmp_make_job(first, grid_magic, sh.job[0]);
     for (int i = threadIdx.x; i < count; i += kQmpThreads) sh.thr_second_pass[i] = -1.0f;
     if (PATTERN == 68 && threadIdx.x < 256) s_table[threadIdx.x] = table68_entry(threadIdx.x);
     __syncthreads();
@@ -798,8 +1039,9 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
 
     // ---- What the first bracket needs is asked for BEFORE the loader fills the ring: the hint of matrix 0 (a 4-byte
     // read), or without a hint of the caller's its sample (all threads, one round trip) together with what an
-    // earlier call may have left.  Issued with the ring's first copies they queue behind the 17 MB that the loaders
-    // of all CTAs ask for at the same moment (up to 3.5 us measured, and the CTA that is served last finishes last).
+    // earlier call may have left.  Half of the ring follows at once, the rest when the bracket is known: behind all four stages
+    // (17 MB that the loaders of all CTAs ask for at the same moment) the sample of some CTAs comes late (single calls without a hint, us,
+    // all / half: 2560 -> 3840 bf16 17.9 / 17.1, fp32 17.9 / 17.3).
     float gamma0 = first.gamma_hint != nullptr ? *reinterpret_cast<const volatile float*>(first.gamma_hint) : 0.0f;
     float4 sample0[kQmpSamplePerWarp];
     const bool sample_early = first.gamma_hint == nullptr;
@@ -819,11 +1061,12 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     if (!sample_early && !hinted0) qmp_sample_issue(first, sample0);
     QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, qmp_policy_evict_first()};
     const bool is_loader = warp == kQmpLoaderWarp && lane == 0;
-    if (is_loader) qmp_loader_issue(loader, batch, count, kQmpStages, ring_base, bar_full0, bar_empty0, abort_flag);
+    if (is_loader) qmp_loader_issue(loader, batch, count, kQmpStages / 2, grid_magic, ring_base, bar_full0, bar_empty0, abort_flag);
     if (!hinted0) gamma0 = qmp_sample_finish(first, sample0, sh.sample);
     if (threadIdx.x == 0) {
-        qmp_bracket_from(gamma0, first.num_units, hinted0, sh.job[0].lo, sh.job[0].hi);
+        sh.job[0].bracket = qmp_bracket_from(gamma0, first.num_units, hinted0);
         sh.job[0].ready = 1;
+        sh.look = !SINGLE || hinted0 || sh.job[0].units < kQmpLookFrom ? 0 : 1;
         if (blockIdx.x == 0 && first.flip_bits != nullptr) *first.flip_bits = 0ull;      // published with this CTA's first slot
     }
     __syncthreads();
@@ -843,11 +1086,11 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
             QmpWarpList list{list_of(slot, warp), list_cap, 0u};
             double mine;
             if constexpr (PATTERN == 68)
-                mine = jb.bf16 ? qmp68_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table)
-                               : qmp68_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table);
+                mine = jb.bf16 ? qmp68_stream_pass1<true>(jb, sh, SINGLE && sh.look != 0, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table)
+                               : qmp68_stream_pass1<false>(jb, sh, SINGLE && sh.look != 0, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok, s_table);
             else
-                mine = jb.bf16 ? qmp_stream_pass1<true>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok)
-                               : qmp_stream_pass1<false>(jb, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok);
+                mine = jb.bf16 ? qmp_stream_pass1<true, SINGLE>(jb, sh, SINGLE && sh.look != 0, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok)
+                               : qmp_stream_pass1<false, SINGLE>(jb, sh, SINGLE && sh.look != 0, list, flips, stages, next_stage, ring_base, bar_full0, bar_empty0, abort_flag, ok);
             if (!ok) break;
             mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 16);
             mine += __shfl_xor_sync(0xFFFFFFFFu, mine, 8);
@@ -863,7 +1106,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     } else if (warp == kQmpLoaderWarp) {
         // ------------------------------------------------------------------ the loader (one lane)
         if (is_loader) {
-            qmp_loader_issue(loader, batch, count, 0xFFFFFFFFu, ring_base, bar_full0, bar_empty0, abort_flag);
+            qmp_loader_issue(loader, batch, count, 0xFFFFFFFFu, grid_magic, ring_base, bar_full0, bar_empty0, abort_flag);
             sh.ring_issued = loader.issued;                  // for the drain, should the CTA abort
             sh.ring_used = loader.ring.used;
         }
@@ -881,8 +1124,8 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
                 // zeroed well before any CTA can add to it (they add once they have seen this CTA's slot)
                 if (blockIdx.x == 0 && d.flip_bits != nullptr) { *d.flip_bits = 0ull; __threadfence(); }
                 QmpJob& jb = sh.job[m & (kQmpJobs - 1)];
-                qmp_make_job(d, jb);
-                qmp_bracket_from(g, d.num_units, hinted, jb.lo, jb.hi, true);
+                qmp_make_job(d, grid_magic, jb);
+                jb.bracket = qmp_bracket_from(g, d.num_units, hinted, true);
                 __threadfence_block();
                 *reinterpret_cast<volatile int*>(&jb.ready) = m + 1;
             }
@@ -892,12 +1135,12 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
         // ------------------------------------------------------------------ the finisher
         const unsigned long long gen0 = *reinterpret_cast<volatile unsigned long long*>(generation);
         const unsigned long long tag = qmp_tag(call_nonce, gen0);
-        bool ok = true;
+        bool ok = !SINGLE || sh.look == 0 || qmp_look_exchange(first, sh, slots, tag, lane, abort_flag);
         // step m: publish matrix m, then exchange and finish matrix m - 1; step `count` finishes the last matrix
         // (its fix-up is left to all warps)
         unsigned int flips_prev = 0u;
         QmpDesc dp = first;                                  // of matrix m - 1
-        for (int m = 0; m <= count; ++m) {
+        for (int m = 0; ok && m <= count; ++m) {
             unsigned int flips_cur = 0u;
             QmpDesc d = dp;
             if (m < count) {
@@ -1000,24 +1243,24 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
             }
         } else {
             const QmpDesc d = qmp_desc_of(batch, m);
-            qmp_second_pass<PATTERN>(d, thr, s_table);
+            qmp_second_pass<PATTERN>(d, grid_magic, thr, s_table);
         }
     }
     for (int m = 0; m + 1 < count; ++m) {
         const float thr = sh.thr_second_pass[m];
         if (thr >= 0.0f) {
             const QmpDesc d = qmp_desc_of(batch, m);
-            qmp_second_pass<PATTERN>(d, thr, s_table);
+            qmp_second_pass<PATTERN>(d, grid_magic, thr, s_table);
         }
     }
 }
 
 // Launch for `count` (<= kQmpMaxBatch) matrices: the first kQmpInlineDescs of `descs_host` by value, matrices
 // 1, 2, ... already copied to `rest_dev` if there are more than that.
-template <int PATTERN>
-inline sbn_status launch_quantize_mask_pack_stream(const QmpDesc* descs_host, const QmpDesc* rest_dev, int count,
+template <int PATTERN, bool SINGLE>
+inline sbn_status launch_quantize_mask_pack_stream_cfg(const QmpDesc* descs_host, const QmpDesc* rest_dev, int count,
                                                    uint32_t max_units, QmpSlot* slots, unsigned long long* generation,
-                                                   cudaStream_t stream, QmpMemo* memo = nullptr) {
+                                                   cudaStream_t stream, QmpMemo* memo) {
     QmpInlineDescs inl;
     for (int i = 0; i < kQmpInlineDescs; ++i) inl.d[i] = descs_host[i < count ? i : 0];
     const int test_withhold_slot = g_test_break_waits;
@@ -1026,14 +1269,22 @@ inline sbn_status launch_quantize_mask_pack_stream(const QmpDesc* descs_host, co
     // device has SMs, and never more than the workspace has slots
     const unsigned cap = static_cast<unsigned>(std::min(device_sm_count(), kQmpMaxCtas));
     const unsigned grid = max_units < cap ? max_units : cap;
-    if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel<PATTERN>>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
+    if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel<PATTERN, SINGLE>>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
     // At most one CTA per SM (1024 threads x 64 registers each) and never more CTAs than SMs, so all
     // of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
     // another kernel kept SMs busy for seconds, the bounded wait reports SBN_ERR_TIMEOUT instead.
-    const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel<PATTERN>, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
-                                          inl, rest_dev, count, slots, generation, nonce, test_withhold_slot, count == 1 ? memo : nullptr);
+    const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel<PATTERN, SINGLE>, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
+                                          inl, rest_dev, count, slots, generation, nonce, test_withhold_slot, count == 1 ? memo : nullptr, qmp_magic(grid));
     ++g_launch_count;
     return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+}
+template <int PATTERN>
+inline sbn_status launch_quantize_mask_pack_stream(const QmpDesc* descs_host, const QmpDesc* rest_dev, int count,
+                                                   uint32_t max_units, QmpSlot* slots, unsigned long long* generation,
+                                                   cudaStream_t stream, QmpMemo* memo = nullptr) {
+    if (count == 1) return launch_quantize_mask_pack_stream_cfg<PATTERN, true>(descs_host, rest_dev, count, max_units, slots, generation, stream, memo);
+    if constexpr (PATTERN == 24) return launch_quantize_mask_pack_stream_cfg<24, false>(descs_host, rest_dev, count, max_units, slots, generation, stream, memo);
+    return SBN_ERR_UNSUPPORTED;                              // no batches of 6:8
 }
 
 template <int PATTERN>

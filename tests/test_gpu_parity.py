@@ -352,6 +352,38 @@ def test_pack68_bf16_masters_and_ties():
     _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
 
 
+@pytest.mark.parametrize("scale", [1e-36, 1e-39])
+def test_pack_bf16_masters_of_tiny_magnitude(scale):
+    # magnitudes whose differences are subnormal: the selection subtracts, and no difference may be lost
+    bits = inputs.f32_to_bf16_bits((inputs.latent_weights(256, 512, seed=60) * np.float32(scale)).astype(np.float32))
+    W = (bits.astype(np.uint32) << 16).view(np.float32).reshape(256, 512)
+    _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
+    r, g = _oracle_pack(W), gpu_quantize_mask_pack(W, with_dense=False, w_bf16_bits=bits)
+    assert g["scale"] == r["scale"] and np.array_equal(g["vals"], r["vals"]) and np.array_equal(g["meta"], r["meta"])
+
+
+@pytest.mark.parametrize("misleading", [False, True])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_pack_long_matrix_narrows_its_bracket(bf16, misleading):
+    # ranges long enough for the CTAs to tell each other what their first stages say about the mean; misleading: the first 224 units
+    # of every CTA's range are far smaller than the rest, so that the narrowed bracket misses
+    N, K = 4096, 4096
+    W = inputs.latent_weights(N, K, seed=61)
+    if misleading:
+        units = W.reshape(-1, 128)
+        grid = min(torch.cuda.get_device_properties(0).multi_processor_count, 148)
+        per = -(-len(units) // grid)
+        assert per >= 700
+        for r in range(grid):
+            units[r * per:r * per + 224] *= np.float32(0.9)
+    bits = inputs.f32_to_bf16_bits(W) if bf16 else None
+    if bf16:
+        W = (bits.astype(np.uint32) << 16).view(np.float32).reshape(N, K)
+    r, g = _oracle_pack(W), gpu_quantize_mask_pack(W, with_dense=False, w_bf16_bits=bits)
+    assert g["scale"] == r["scale"] and np.array_equal(g["vals"], r["vals"]) and np.array_equal(g["meta"], r["meta"])
+    _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
+
+
 def test_pack68_every_kept_set():
     # all 28 ways of dropping two columns of eight, each with distinct magnitudes and with ties at
     # the boundary (the dropped pair equal to a kept column: the lower column must win)
