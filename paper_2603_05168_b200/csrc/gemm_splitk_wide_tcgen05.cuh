@@ -77,7 +77,7 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
     const uint32_t tmem_slot = bar_recv + 8;
 
     __shared__ int s_abort;
-    __shared__ float s_scale[128];                           // of the tokens this CTA finishes (c <= 128)
+    __shared__ float s_scale[256];                           // of the tokens this CTA finishes
     volatile int* abort_flag = &s_abort;
 
     const int warp = threadIdx.x >> 5;
@@ -288,7 +288,8 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     *reinterpret_cast<float4*>(static_cast<float*>(p.y) + o) = make_float4(v0, v1, v2, v3);
             }
         };
-        if (S == 2) finish(std::integral_constant<int, 2>{});
+        if (S == 1) finish(std::integral_constant<int, 1>{});
+        else if (S == 2) finish(std::integral_constant<int, 2>{});
         else if (S == 3) finish(std::integral_constant<int, 3>{});
         else if (S == 4) finish(std::integral_constant<int, 4>{});
         else finish(std::integral_constant<int, 0>{});

@@ -164,7 +164,7 @@ struct GemmPlan {
     bool pair;      // CTA-pair kernel (two M-tiles per CTA) or single-CTA tiles
     int bn;         // token tile
     int splits;     // split-K factor through global atomics (single-CTA kernel only)
-    int cluster;    // > 1: split-K inside clusters of this many CTAs (reduction in shared memory)
+    int cluster;    // > 1: split-K inside clusters of this many CTAs (reduction in shared memory); 1: the wide-tile kernel unsplit
     int mt = 2;     // CTA-pair kernel: M-tiles per CTA (2: 512-feature tiles; 1: 256-feature tiles, double-buffered accumulators)
 };
 static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool may_split = true);
@@ -245,6 +245,11 @@ static const PlanCosts kPlanCosts[2][2] = {                 // [sparse][fp32 out
       {4.6456, 0.2668, 0.03, 0.3028, -0.0285, 0.117, 0.0944, 0.0807},
       {5.1138, 0.2422, 0.2679, 0.126}, {5.9491, 0.2478, 0.3353, 0.1469}, {5.3549, 0.282, 2.349, 0.157}, {4.9998, 0.0107, 0.1749, 0.8473, 0.0446, 0.1231}, {2.7183, 0.0176, 0.233, 4.2553, 0.1481, 0.1171}}}};
 
+// Wide tiles, unsplit, dense: a + kb (c + u bn / 256 + z share) + sh share + tk tokens, share = of the SMs in use; c2, u2 as above.
+// [fp32 outputs].  Fitted the same way to 44 shapes, 26 token counts, against the other kernels' costs.
+struct WideOneCost { double a, c, u, c2, u2, sh, z, tk; };
+static const WideOneCost kWideOneCosts[2] = {{5.0092, 0.1812, 0.1058, 0.1353, 0.1165, 0.7654, 0.037, 0.0119}, {5.05, 0.1741, 0.116, 0.1386, 0.118, 1.025, 0.0223, 0.0102}};
+
 // Clusters of S with two CTAs per SM that were all resident at once; one more waited for a whole kernel lifetime (12288 -> 2304,
 // 128 tokens: 72 clusters of 4 19.5 us, other plans 13.1; clusters of 3: 88 were, 90 not always).
 constexpr int kNarrowClusters[5] = {0, 0, 148, 88, 70};
@@ -273,9 +278,10 @@ static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool 
         int S = -g_force_split_k;
         if (g_force_token_tile > 64) {                          // wide tiles: any width and cluster that fit
             const int bn = std::min(256, g_force_token_tile / 16 * 16);
+            const bool unsplit = S == 1;
             S = std::min(8, std::min(S, K / kBK));
             while (S > 1 && !wide_fits(bn, S)) --S;
-            if (S > 1) return GemmPlan{false, bn, 1, S};
+            if (S > 1 || unsplit) return GemmPlan{false, bn, 1, S};
         }
         S = S >= 8 ? 8 : (S >= 4 ? 4 : (S == 3 ? 3 : 2));
         while (S > 1 && S > K / kBK) --S;
@@ -313,6 +319,21 @@ static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool 
                 consider(GemmPlan{false, bn, 1, S}, cost.wide.a + q * c + cost.wide.e * tokens * (S - 1) / S +
                                                         (cost.wide.share + cost.wide.z * q) * rows * tt * S / kNumSMs);
             }
+        }
+    }
+    // The same kernel unsplit, dense weights, one tile per SM: its first stages hold weights before the dependency wait and it fetches two
+    // K-blocks with one instruction per operand, which the single-CTA kernel below does not (6912 -> 2560, 777 tokens, us: 24.8,
+    // here 22.5; 11008 -> 4096, 600 tokens 39.9 / 33.5; 2560 -> 2560 13.6 / 13.4).  Sparse weights: the pairs' instructions do more
+    // (2 to 3 % either way).
+    if (!sparse && T > 64 && T <= 2048) {
+        const WideOneCost& c = kWideOneCosts[out_wide];
+        const int fewest = (T + 255) / 256;
+        for (int tt = fewest; tt <= fewest + 5 && static_cast<long>(rows) * tt <= kNumSMs; ++tt) {
+            const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
+            if (bn * (tt - 1) >= T) continue;
+            const double share = static_cast<double>(rows) * tt / kNumSMs;
+            const double block = wide_group(sparse, bn) == 2 ? c.c2 + c.u2 * bn / 256 : c.c + c.u * bn / 256;
+            consider(GemmPlan{false, bn, 1, 1}, c.a + kb * (block + c.z * share) + c.sh * share + c.tk * std::min(bn, T));
         }
     }
     // Single-CTA tiles: one token tile in any number of waves, else up to two, with short K (1024 -> 2560: 15.0 us for 2048
@@ -497,7 +518,7 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
     p.w_vals = wvals; p.w_meta = sparse ? meta : nullptr; p.w_tile_bytes = sparse ? 8192 : 16384;
     p.test_skip_loads = g_test_break_waits;
 
-    if (plan.cluster > 1) {
+    if (plan.cluster >= 1) {
         p.k_splits = 1;
         if (bn > 64) {                                          // boxes of wide_group K-blocks
             const uint32_t G = static_cast<uint32_t>(wide_group(sparse, bn));
@@ -1047,7 +1068,7 @@ void sbn_plan_gemm(int sparse, int T, int N, int K, int* out4) {
     out4[0] = g.pair ? (g.mt == 1 ? 3 : 2) : (g.cluster > 1 ? 1 : 0);
     out4[1] = g.bn;
     out4[2] = g.splits;
-    out4[3] = g.cluster;
+    out4[3] = g.cluster > 1 ? g.cluster : 0;
 }
 
 sbn_status sbn_set_wait_test(int break_waits, unsigned long long wait_limit_us) {

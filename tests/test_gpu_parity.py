@@ -819,7 +819,8 @@ def test_gemm_parity_cluster_split_k(sparse, T, N, K, tile, cluster):
 # Wide token tiles split over clusters: one token in the last tile (CTAs that own none), unequal shares, tiles of the least
 # and the greatest width, K-blocks that do not divide by the cluster, one block per CTA, more blocks than stages.
 WIDE_CASES = [(81, 128, 512, 80, 4), (65, 256, 384, 80, 3), (201, 256, 1280, 112, 2), (256, 128, 1664, 256, 4), (255, 256, 2560, 256, 2),
-              (160, 128, 2176, 160, 3), (300, 128, 768, 208, 6), (97, 384, 256, 112, 2)]
+              (160, 128, 2176, 160, 3), (300, 128, 768, 208, 6), (97, 384, 256, 112, 2),
+              (81, 128, 128, 80, 1), (256, 256, 1664, 256, 1), (300, 128, 2560, 160, 1), (129, 384, 1152, 128, 1), (500, 128, 384, 176, 1)]
 
 
 @pytest.mark.parametrize("sparse", [True, False])
