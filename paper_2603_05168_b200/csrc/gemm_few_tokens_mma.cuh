@@ -77,6 +77,12 @@ __device__ __forceinline__ uint4 ldg_once(const uint8_t* p) {
     return v;
 }
 
+__device__ __forceinline__ uint32_t ldg_once_u32(const uint8_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
 // The warp's loads: blocks kb = warp, warp + W, ... of row groups blockIdx.x, + gridDim.x, ...  16 rows are contiguous in
 // every layout (1 KB of values, 256 B of metadata, 2 KB of dense weights) and repeat its swizzle.
 template <int WT, int W>
@@ -108,8 +114,8 @@ struct FewFetch {
                 b.w[1] = ldg_once(w + 512);
                 b.m = ldg_once(m);
             } else {
-                b.w[0] = __ldg(reinterpret_cast<const uint32_t*>(w));
-                b.w[1] = __ldg(reinterpret_cast<const uint32_t*>(w + 128));
+                b.w[0] = ldg_once_u32(w);
+                b.w[1] = ldg_once_u32(w + 128);
                 b.m = ldg_once(m);
             }
         }
@@ -124,6 +130,24 @@ struct FewFetch {
         }
     }
 };
+
+// The warp's next D blocks go to the L2 before the dependency wait (a lane per block): loaded after it, from memory, they were
+// another trip on the critical path.  Quantiser + GEMM in a decode loop, us, without / with: 6912 -> 2560 (seven blocks per warp, four
+// in registers) 1 token 6.05 / 5.77, dense 7.2 / 6.6; 4096 -> 11008 (two row groups per CTA) 8.25 / 8.15, dense 9.7 / 9.4.  All of the rest
+// at once is too much where memory is the limit (4096 -> 11008 8.5, dense 10.2), and very long rows lose by any of it (11008 -> 4096:
+// eleven blocks, 9.37 / 9.45 at 8 tokens, dense 11.5 / 11.7) -- unless they are packed and the memory has time (9.4 / 8.5).  Packed weights gain
+// a tenth everywhere, also where there is nothing to prefetch (2560 -> 2560 4.6 / 4.2): without a side effect here the compiler
+// expands the first blocks before it asks for the activations.
+template <int WT, int W, int D>
+__device__ __forceinline__ void few_prefetch_next(const FewParams& p, uint32_t lane, uint32_t warp, uint32_t rounds) {
+    if (lane >= D || (WT != kFewPacked && rounds > 2 * D)) return;
+    const uint32_t i = D + lane, nth = i / rounds, kb = warp + (i - nth * rounds) * W, group = blockIdx.x + nth * gridDim.x;
+    if (group >= static_cast<uint32_t>(p.N >> 4) || kb >= static_cast<uint32_t>(p.k_blocks)) return;
+    const size_t tile = static_cast<size_t>(group >> 3) * p.k_blocks + kb;
+    constexpr uint32_t kRows = WT == kFewDense ? 2048u : (WT == kFewSparse ? 1024u : 256u);       // bytes of 16 rows
+    prefetch_l2_bulk(p.vals + tile * (8u * kRows) + (group & 7u) * kRows, kRows);
+    if constexpr (WT != kFewDense) prefetch_l2_bulk(p.meta + tile * 2048 + (group & 7u) * 256u, 256u);
+}
 
 // The sparse operands of a block.  A lane's 32 columns are the groups G0 .. G7; the instruction of step s (0, 1) takes
 // {G[s], G[4 + s]} as its word for contraction positions 8 q .. and {G[2 + s], G[6 + s]} for 32 + 8 q .. .  On the
@@ -191,8 +215,9 @@ __device__ __forceinline__ void few_quantise(const uint4& lo, const uint4& hi, f
     out[3] = quant_pair2(hi.z, hi.w, s_x);
 }
 
-// NT groups of 8 tokens; W warps per CTA; D blocks of weights in flight per warp; MINB CTAs per SM (the register budget).
-template <int WT, int NT, int W, int D, int MINB, bool FUSED>
+// NT groups of 8 tokens; W warps per CTA; D blocks of weights in flight per warp; MINB CTAs per SM (the register budget); AHEAD: the
+// blocks after those go to the L2 early.
+template <int WT, int NT, int W, int D, int MINB, bool FUSED, bool AHEAD>
 __global__ void __launch_bounds__(32 * W, MINB)
 bitlinear_gemm_few_kernel(const FewParams p) {
     constexpr int kStride = 20;                                              // words between tokens of a warp's partial sums: no bank conflicts
@@ -211,6 +236,7 @@ bitlinear_gemm_few_kernel(const FewParams p) {
     FewBlock<WT> blk[D];
 #pragma unroll
     for (int j = 0; j < D; ++j) fetch.next(p, lane, blk[j]);
+    if constexpr (AHEAD) few_prefetch_next<WT, W, D>(p, lane, static_cast<uint32_t>(warp), static_cast<uint32_t>(rounds));
     pdl_wait();
 
     bool real[NT];                                                           // this lane's tokens exist
@@ -347,7 +373,13 @@ template <int WT, int NT, int W, int D, int MINB, bool FUSED>
 inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
     const int groups = p.N / 16, slots = device_sm_count() * MINB;
     ++g_launch_count;
-    return launch_kernel(bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED>, dim3(groups < slots ? groups : slots), dim3(32 * W), 0, stream, p);
+    // Where there is something to fetch; else for the sake of the order of the loads (see few_prefetch_next), which helps packed
+    // and, a little, int8-held 2:4 weights (2560 -> 2560 4.09 / 3.96) but not dense ones (2560 -> 3840, 8 tokens 4.75 / 4.95) nor the fused
+    // quantiser (2560 -> 3840 3.83 / 3.99).
+    const bool more = groups > slots || (p.k_blocks > W * D && p.k_blocks <= 2 * W * D);
+    const bool ahead = more || WT == kFewPacked || (WT == kFewSparse && !FUSED);
+    return launch_kernel(ahead ? bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, true> : bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, false>,
+                         dim3(groups < slots ? groups : slots), dim3(32 * W), 0, stream, p);
 }
 
 // Which calls run here, with what split.  All times in us for quantiser + GEMM in a decode loop (weights from HBM), this
