@@ -18,6 +18,7 @@
 #include "quantize_mask_pack_stream.cuh"
 #include "canonical_layout.cuh"
 #include "gemm_tcgen05.cuh"
+#include "quant_rows.cuh"
 #include "gemm_pair_tcgen05.cuh"
 #include "gemm_splitk_cluster_tcgen05.cuh"
 #include "gemm_splitk_wide_tcgen05.cuh"
@@ -782,7 +783,7 @@ sbn_status sbn_quant_act(const void* x_bf16, int T, int K, int8_t* xq, float* a_
     if (!x_bf16 || !xq || !a_scale) return SBN_ERR_NULL;
     if (T <= 0 || K <= 0 || K % kBK != 0 || K > (1 << 20)) return SBN_ERR_SHAPE;
     if (misaligned(x_bf16, 16) || misaligned(xq, 16) || misaligned(a_scale, 4)) return SBN_ERR_ALIGN;
-    return launch_quant_act(x_bf16, T, K, xq, a_scale, static_cast<cudaStream_t>(stream));
+    return quantise(x_bf16, T, K, xq, a_scale, static_cast<cudaStream_t>(stream));
 }
 
 sbn_status sbn_quant_act_expand68(const void* x_bf16, int T, int K, int8_t* xq, float* a_scale, void* stream) {
@@ -818,7 +819,7 @@ sbn_status sbn_norm_quant_act(const void* x_bf16, int T, int K, const float* gai
     if (!(eps >= 0.0f)) return SBN_ERR_SHAPE;
     if (misaligned(x_bf16, 16) || misaligned(xq, 16) || misaligned(a_scale, 4) || (gain && misaligned(gain, 16)))
         return SBN_ERR_ALIGN;
-    return launch_norm_quant_act(x_bf16, T, K, gain, eps, xq, a_scale, static_cast<cudaStream_t>(stream));
+    return normalise_and_quantise(x_bf16, T, K, gain, eps, xq, a_scale, static_cast<cudaStream_t>(stream));
 }
 
 sbn_status sbn_sparse_bitlinear(const int8_t* xq, const float* a_scale, int T, const int8_t* vals,

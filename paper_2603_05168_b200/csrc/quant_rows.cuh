@@ -1,0 +1,205 @@
+// The activation quantisers (quant_act.cuh, norm_quant_act.cuh) for many rows: a warp per row, rows through shared memory.
+//
+// With several warps per row the instructions of those kernels go into what every thread does once per row -- reductions,
+// two barriers, a square root and three divisions, about 200 instructions for 20 elements of a thread -- and
+// the next row's registers.  Here a warp owns a row: the per-row work is spread over K / 32 elements of a lane, nothing is shared
+// between warps, and a row arrives by a bulk copy into the warp's own piece of shared memory, which costs neither registers nor
+// issue slots.  Up to 32 warps, as many rows as fit in flight.  The row is read from shared memory once per step (squares, maximum,
+// codes); xn is computed again rather than kept.
+//
+// Measured in a chain of launches, us, those kernels / this one [HBM time of the bytes]: plain 4096 x 2560 7.7 / 7.2 [4.9], 4096 x
+// 3328 10.8 / 8.9 [6.3], 8192 x 4096 22.5 / 19.5 [15.6]; with norm and gain 2048 x 2560 8.2 / 6.8, 4096 x 2560 12.3 / 11.4, 8192 x
+// 2560 22.1 / 19.5 [9.7].  The norm is bound by its instructions (18 per element, before 26).  Two rows per warp (twice the
+// independent work, gains read once for both) were slower, two stages per warp too (half the warps).
+#pragma once
+
+#include "gemm_tcgen05.cuh"
+#include "norm_quant_act.cuh"
+
+namespace sbn {
+
+constexpr int kRowsMaxWarps = 32;
+constexpr int kRowsSmemBytes = 200 * 1024;
+// Never two CTAs on an SM: the ones that come early, while the kernel before still runs, crowd on the SMs that it has left and
+// the others stay idle (norm of 2048 x 2560 8.3 us, with one CTA per SM 6.9).
+constexpr int kRowsSmemLeast = 116 * 1024;
+
+__device__ __forceinline__ uint4 lds_vec(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+// Read once: the lines leave the L2 first (the codes written here are the next kernel's operand).
+__device__ __forceinline__ void bulk_load_row(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    unsigned long long policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    mbar_expect_tx(bar, bytes);
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
+}
+
+// Shared memory: gains [2][nvec] float4 (first halves of all vectors, then the second ones) when GAIN, then a row per warp.
+template <bool NORM, bool GAIN>
+__global__ void __launch_bounds__(32 * kRowsMaxWarps, 1)
+quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __restrict__ gain, float eps, double n, double inv_n,
+                  uint2* __restrict__ xq, float* __restrict__ a_scale) {
+    extern __shared__ __align__(128) uint8_t s_rows[];
+    __shared__ unsigned long long s_bar[kRowsMaxWarps];
+    __shared__ int s_abort;
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t row_bytes = static_cast<uint32_t>(nvec) * 16u;
+    const float4* const s_gain = reinterpret_cast<const float4*>(s_rows);
+    const uint32_t at = smem_u32(s_rows) + (GAIN ? 2u * row_bytes : 0u) + static_cast<uint32_t>(warp) * row_bytes;
+    const uint32_t bar = smem_u32(&s_bar[warp]);
+    const size_t tb8 = xq_tb8(T);
+    const int stride = gridDim.x * warps;
+    int row = blockIdx.x * warps + warp;
+
+    pdl_launch_dependents();
+    if (threadIdx.x == 0) s_abort = 0;
+    if (lane == 0u) {
+        mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    pdl_wait();
+    auto fetch = [&](int r) {
+        if (lane == 0u && r < T) bulk_load_row(at, x + static_cast<size_t>(r) * nvec, row_bytes, bar);
+    };
+    fetch(row);
+    if constexpr (GAIN) {
+        for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+            reinterpret_cast<float4*>(s_rows)[i] = __ldg(gain + 2 * i);
+            reinterpret_cast<float4*>(s_rows)[nvec + i] = __ldg(gain + 2 * i + 1);
+        }
+    }
+    __syncthreads();
+    for (uint32_t parity = 0u; row < T; parity ^= 1u, row += stride) {
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, &s_abort))) {
+            int keep_waiting = 0;                                               // the copy in flight must land before this CTA leaves
+            mbar_wait(bar, parity, &keep_waiting);
+            break;
+        }
+        float rinv = 1.0f, amax;
+        auto normalise = [&](const uint4& v, int idx, uint64_t (&o)[4]) {
+            const uint64_t r2 = pack_f32x2(rinv, rinv);
+            o[0] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.x), bf16hi_to_f32(v.x)), r2);
+            o[1] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.y), bf16hi_to_f32(v.y)), r2);
+            o[2] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.z), bf16hi_to_f32(v.z)), r2);
+            o[3] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.w), bf16hi_to_f32(v.w)), r2);
+            if constexpr (GAIN) {
+                const float4 a = s_gain[idx], b = s_gain[nvec + idx];
+                o[0] = mul_f32x2(o[0], pack_f32x2(a.x, a.y));
+                o[1] = mul_f32x2(o[1], pack_f32x2(a.z, a.w));
+                o[2] = mul_f32x2(o[2], pack_f32x2(b.x, b.y));
+                o[3] = mul_f32x2(o[3], pack_f32x2(b.z, b.w));
+            }
+        };
+        if constexpr (NORM) {
+            double s4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+            for (int idx = lane; idx < nvec; idx += 32) {
+                const uint4 v = lds_vec(at + 16u * idx);
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {                                   // exact product, one rounding in the add
+                    const double lo = bf16_abs_to_f64(w[j] & 0x7FFFu), hi = bf16_abs_to_f64((w[j] >> 16) & 0x7FFFu);
+                    s4[(2 * j) & 3] = __fma_rn(lo, lo, s4[(2 * j) & 3]);
+                    s4[(2 * j + 1) & 3] = __fma_rn(hi, hi, s4[(2 * j + 1) & 3]);
+                }
+            }
+            double ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
+            const double quot = ss * inv_n;                                     // ss / n, correctly rounded: see norm_quant_act.cuh
+            const float ms = static_cast<float>(__fma_rn(__fma_rn(-quot, n, ss), inv_n, quot));
+            rinv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(ms, eps)));
+            amax = 0.0f;
+#pragma unroll 4
+            for (int idx = lane; idx < nvec; idx += 32) {
+                uint64_t o[4];
+                normalise(lds_vec(at + 16u * idx), idx, o);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float lo, hi;
+                    unpack_f32x2(o[j], lo, hi);
+                    amax = max_abs3(amax, lo, hi);
+                }
+            }
+            amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax)));
+        } else {
+            uint32_t pm = 0u;
+#pragma unroll 4
+            for (int idx = lane; idx < nvec; idx += 32) pm = absmax8_packed(lds_vec(at + 16u * idx), pm);
+            amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, max(pm >> 16, pm & 0xFFFFu)) << 16);
+        }
+        const float d = fmaxf(amax, kEps);
+        const float s_x = __fdiv_rn(127.0f, d);
+        if (lane == 0u) a_scale[row] = __fdiv_rn(d, 127.0f);
+        const uint64_t s2 = pack_f32x2(s_x, s_x);
+#pragma unroll 4
+        for (int idx = lane; idx < nvec; idx += 32) {
+            const uint4 v = lds_vec(at + 16u * idx);
+            uint2 ov;
+            if constexpr (NORM) {
+                uint64_t o[4];
+                normalise(v, idx, o);
+                uint32_t q[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {                                   // rounding by adding 1.5 * 2^23: see norm_quant_act.cuh
+                    float lo, hi;
+                    unpack_f32x2(mul_f32x2(o[j], s2), lo, hi);
+                    q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
+                    q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
+                }
+                ov = make_uint2(low_bytes4(q[0], q[1], q[2], q[3]), low_bytes4(q[4], q[5], q[6], q[7]));
+            } else {
+                ov = make_uint2(quant_pair2(v.x, v.y, s_x), quant_pair2(v.z, v.w, s_x));
+            }
+            store_codes8<false>(xq, row, idx, tb8, ov);
+        }
+        if constexpr (NORM) {
+            if (fmaxf(d, rinv) == __int_as_float(0x7F800000)) odd_row_codes<32, false>(x, gain, rinv, row, nvec, lane, xq, tb8);
+        }
+        __syncwarp();                                                           // every lane has read the row
+        fetch(row + stride);
+    }
+}
+
+template <bool NORM, bool GAIN>
+static cudaError_t launch_quant_rows(const void* x, int T, int K, const float* gain, float eps, int8_t* xq, float* a_scale, cudaStream_t stream) {
+    auto kernel = quant_rows_kernel<NORM, GAIN>;
+    if (!ensure_dynamic_smem<quant_rows_kernel<NORM, GAIN>>(kRowsSmemBytes)) return cudaErrorUnknown;
+    const int row_bytes = 2 * K, gain_bytes = GAIN ? 4 * K : 0, sms = device_sm_count();
+    const int most = std::min(kRowsMaxWarps, (kRowsSmemBytes - gain_bytes) / row_bytes);
+    const int rounds = (T + sms * most - 1) / (sms * most), warps = (T + sms * rounds - 1) / (sms * rounds);     // the last round full
+    const int grid = std::min(sms, (T + warps - 1) / warps);
+    ++g_launch_count;
+    return launch_kernel(kernel, dim3(grid), dim3(32 * warps), static_cast<size_t>(std::max(kRowsSmemLeast, gain_bytes + warps * row_bytes)), stream,
+                         static_cast<const uint4*>(x), T, K / 8, reinterpret_cast<const float4*>(gain), eps, static_cast<double>(K), 1.0 / static_cast<double>(K),
+                         reinterpret_cast<uint2*>(xq), a_scale);
+}
+
+// Which calls run here.  Plain: from 13 rows per SM on (2560 columns, 1500 rows 3.8 us there, 4.0 here; 2048 rows 4.8 / 4.7), up to 5120
+// columns (8192 x 5120 26.1 / 24.1; 8192 x 6912 32.3 / 32.6: too few rows in flight).  With a norm earlier, 1280 to 3328 columns
+// (1000 x 2560 5.9 / 5.0; narrower rows have no advantage), wider ones only in great numbers (8192 x 4096 30.7 / 27.9, 4096 x 4096 16.7 / 18.8).
+// Not the expanded form of the 6:8 pattern (2048 x 2560 6.0 / 6.7).
+inline bool quant_rows_takes(bool norm, int T, int K) {
+    if (norm) return (K >= 1280 && K <= 3328 && T >= 1000) || (K > 3328 && K <= 5120 && T >= 7000);
+    return K >= 1024 && K <= 5120 && T >= 13 * kNumSMs;
+}
+
+inline sbn_status quantise(const void* x, int T, int K, int8_t* xq, float* a_scale, cudaStream_t stream) {
+    if (!quant_rows_takes(false, T, K)) return launch_quant_act(x, T, K, xq, a_scale, stream);
+    return launch_quant_rows<false, false>(x, T, K, nullptr, 0.0f, xq, a_scale, stream) == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+}
+inline sbn_status normalise_and_quantise(const void* x, int T, int K, const float* gain, float eps, int8_t* xq, float* a_scale, cudaStream_t stream) {
+    if (!quant_rows_takes(true, T, K)) return launch_norm_quant_act(x, T, K, gain, eps, xq, a_scale, stream);
+    const cudaError_t err = gain ? launch_quant_rows<true, true>(x, T, K, gain, eps, xq, a_scale, stream)
+                                 : launch_quant_rows<true, false>(x, T, K, gain, eps, xq, a_scale, stream);
+    return err == cudaSuccess ? SBN_OK : SBN_ERR_CUDA;
+}
+
+}  // namespace sbn

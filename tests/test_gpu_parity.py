@@ -93,6 +93,20 @@ def test_norm_quant_act_rows_per_cta(T, K):
     test_norm_quant_act_parity(T, K, True)
 
 
+# a warp per row: from the row counts where that begins, rows that leave the last round partly empty, columns that are no multiple
+# of 256 (the last vectors belong to half a warp), the narrowest and widest rows
+@pytest.mark.parametrize("T,K", [(1924, 1024), (1925, 1152), (2500, 2560), (1924, 5120)])
+def test_quant_act_warp_per_row(T, K):
+    test_quant_act_parity(T, K)
+
+
+@pytest.mark.parametrize("T,K", [(1000, 1280), (1001, 1408), (5000, 2560), (1000, 3328), (7000, 3456)])
+def test_norm_quant_act_warp_per_row(T, K):
+    for with_gain in (True, False):
+        test_norm_quant_act_parity(T, K, with_gain)
+    test_norm_quant_act_rows_that_overflow(T, K)
+
+
 # Finite inputs whose normalised row is not finite: no scale brings such a value into range, and its code is 127 (the saturated
 # end), as for every width of the kernel; with eps > 0 and finite products nothing changes.
 @pytest.mark.parametrize("T,K", [(5, 256), (5, 1280), (600, 1280), (600, 2560), (5, 4096), (600, 6912), (600, 11008), (5, 16384)])
