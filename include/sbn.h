@@ -126,7 +126,7 @@ size_t sbn_workspace_bytes(int op, int T, int N, int K);
  *              a speed-up for loops that re-pack the same buffers every step, never a change of the
  *              result; bytes that do not carry the tag are ignored
  * Residency rule (this call, the _bf16, _batched and _static_ws forms alike).  The kernel is one
- * persistent grid of at most one CTA per SM (1024 threads each) whose CTAs exchange their partial
+ * persistent grid of at most one CTA per SM (768 threads each) whose CTAs exchange their partial
  * sums through the workspace, so ALL of its CTAs must be resident at the same time.  On a GPU that
  * runs nothing else that is always so.  Two such calls that may overlap on the GPU (different
  * streams, no ordering between them) can each occupy part of the SMs and then wait for CTAs that

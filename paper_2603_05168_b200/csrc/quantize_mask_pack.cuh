@@ -4,7 +4,7 @@
 // gamma needs the whole matrix before any element can be rounded, but almost every element can be
 // rounded correctly from an ESTIMATE of gamma: W_q = sign(w) [ |w| >= thr(gamma) ] and only the
 // few |w| that lie within a few percent of thr depend on its exact value.  One persistent kernel
-// (one 1024-thread CTA per SM) therefore reads W ONCE, for one matrix or a batch of them.  This file
+// (one 768-thread CTA per SM) therefore reads W ONCE, for one matrix or a batch of them.  This file
 // holds the building blocks; the kernel runs the phases as one uninterrupted stream
 // (quantize_mask_pack_stream.cuh).  The phases:
 //
@@ -49,7 +49,7 @@
 
 namespace sbn {
 
-constexpr int kQmpThreads = 1024;
+constexpr int kQmpThreads = 768;
 constexpr int kQmpWarps = kQmpThreads / 32;
 constexpr int kQmpMaxCtas = kNumSMs;                       // one CTA per SM, all co-resident
 constexpr int kQmpSampleUnits = 256;                       // units in the gamma_est sample of a large matrix

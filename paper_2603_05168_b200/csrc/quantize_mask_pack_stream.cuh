@@ -7,25 +7,25 @@
 // matrix, a third of a batch of 2B-shaped matrices and more for small ones.  Here none of that stops
 // the stream:
 //
-//   warp 28       the loader: one lane copies the CTA's range of matrix 0, 1, 2, ... into a ring of shared-
-//                 memory stages (28 KB = 56 units of fp32 or 112 of bf16 weights each, four stages) with bulk
+//   warp 20       the loader: one lane copies the CTA's range of matrix 0, 1, 2, ... into a ring of shared-
+//                 memory stages (20 KB = 40 units of fp32 or 80 of bf16 weights each, six stages) with bulk
 //                 copies that count their bytes on a stage's `full` barrier; it refills a stage as soon as the
 //                 warps that use it have released it (`empty` barrier).  The loads cost no registers and no
 //                 issue slots, and run ahead across matrices.
-//   warps 0..27   pass 1 of matrix 0, 1, 2, ... back to back: two teams of 14 warps take the stages in turn
+//   warps 0..19   pass 1 of matrix 0, 1, 2, ... back to back: two teams of 10 warps take the stages in turn
 //                 (fixed order of additions: the partial sums are reproducible bit for bit); no CTA-wide barrier
 //                 between matrices.  A warp leaves its sum |W| and flip count of matrix m in shared memory and
 //                 arrives on the list slot's `done` barrier.  (Seven teams of four warps were tried, to keep more
 //                 warps busy while some are between two matrices: their 8 KB copies stream fp32 weights at
-//                 3.3 TB/s, 28 KB ones at 4.7.)
-//   warp 29       the finisher.  For matrix m, in this order:
-//                   wait until the 28 computing warps have arrived for m, add their sums in a fixed
+//                 3.3 TB/s, 20 KB ones and longer at 4.7.)
+//   warp 21       the finisher.  For matrix m, in this order:
+//                   wait until the 20 computing warps have arrived for m, add their sums in a fixed
 //                   order, publish {tag, partial} in the workspace;
 //                   exchange of matrix m - 1 (published by every CTA one matrix ago, so the slots are
 //                   there already), exact gamma, scale, threshold; fix-up of the listed values of
 //                   m - 1, or a note that m - 1 needs the exact second pass; its list becomes free.
 //                 All of it runs under pass 1 of the following matrices.
-//   warps 30, 31  the scouts take turns to prepare the matrices ahead: descriptor, what the computing warps need
+//   warps 22, 23  the scouts take turns to prepare the matrices ahead: descriptor, what the computing warps need
 //                 to know (`job`), bracket from the caller's hint or from a sample of the matrix.  Up to seven
 //                 matrices ahead, so neither is ever waited for.  When the finisher did this too it took 7 us per
 //                 matrix, and small matrices (1 us of streaming) waited for it.
@@ -46,13 +46,17 @@
 
 namespace sbn {
 
-constexpr int kQmpStreamWarps = 28;                        // 28 compute, then the loader, the finisher and two scouts
+// 20 compute, then the loader, the finisher and two scouts.  More warps (28, until the registers are used up at 64 per thread)
+// make this slower: pass 1 is bound by its instructions, and with 80 registers it has fewer of them.  28 warps and four stages
+// / 20 and six, us: one matrix 2560 -> 2560 fp32 15.7 / 14.9, bf16 14.7 / 13.6, 4096 -> 11008 bf16 39.8 / 39.0; 14 tensors with hints
+// fp32 133.7 / 130.3, bf16 122.1 / 114.4, without 156 / 147 and 152 / 141.  24 and 16 warps lie between.
+constexpr int kQmpStreamWarps = 20;
 constexpr int kQmpLoaderWarp = kQmpStreamWarps;
 constexpr int kQmpFinisherWarp = kQmpStreamWarps + 1;
 constexpr int kQmpScoutWarp = kQmpStreamWarps + 2;
 constexpr int kQmpScouts = kQmpWarps - kQmpScoutWarp;
 constexpr int kQmpLists = 3;
-constexpr int kQmpWarpListCap = 156;                       // undecided entries per computing warp and matrix, three lists in use
+constexpr int kQmpWarpListCap = 196;                       // undecided entries per computing warp and matrix, three lists in use
 constexpr int kQmpListEntries = kQmpStreamWarps * kQmpWarpListCap;
 // A launch of one or two matrices uses one or two of the three lists, each that much larger.
 __host__ __device__ inline uint32_t qmp_list_cap(int count) {
@@ -65,7 +69,7 @@ constexpr int kQmpStepUnits = 4 * kQmpTeamWarps;           // one unit per quart
 // Whole turns of the teams: a slot always belongs to the same team.  A team that comes to a slot's next use has then
 // itself seen the use before land, so the parity of the slot's barrier says which use it is.  (With slots that
 // wander from team to team a use could be taken for landed while the one before, another team's, was still on its way.)
-constexpr int kQmpStages = 2 * kQmpTeams;
+constexpr int kQmpStages = 3 * kQmpTeams;
 constexpr int kQmpStageBytes = kQmpStepUnits * 512;        // one step of fp32 units, or two of bf16 units
 constexpr int kQmpStreamSmemBytes = kQmpStages * kQmpStageBytes + kQmpLists * kQmpListEntries * 8;
 constexpr int kQmpMaxBatch = 512;                          // thresholds of put-off second passes live in shared memory
@@ -266,8 +270,8 @@ struct QmpSamplePlaces {
     }
 };
 // The loads carry no condition and no conversion (see above): a place beyond the sample is read as its last unit and left out
-// of the sum.  Small samples take two of a thread's loads, large ones all eight.
-constexpr int kQmpSamplePerWarp = kQmpSampleUnits / kQmpWarps, kQmpSamplePerWarpSmall = kQmpSampleUnitsSmall / kQmpWarps;
+// of the sum.  Small samples take three of a thread's loads, large ones all eleven.
+constexpr int kQmpSamplePerWarp = (kQmpSampleUnits + kQmpWarps - 1) / kQmpWarps, kQmpSamplePerWarpSmall = (kQmpSampleUnitsSmall + kQmpWarps - 1) / kQmpWarps;
 template <int FIRST, int LAST>
 __device__ __forceinline__ void qmp_sample_loads(const QmpDesc& d, const QmpSamplePlaces& places, float4 (&v)[kQmpSamplePerWarp]) {
     const int lane = threadIdx.x & 31;
@@ -300,7 +304,7 @@ __device__ __forceinline__ float qmp_sample_finish(const QmpDesc& d, const float
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
     if ((threadIdx.x & 31) == 0) s_sample[threadIdx.x >> 5] = acc;
     __syncthreads();
-    float t = s_sample[threadIdx.x & 31];
+    float t = (threadIdx.x & 31) < kQmpWarps ? s_sample[threadIdx.x & 31] : 0.0f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
     return t / (static_cast<float>(n_s) * 128.0f);
@@ -458,7 +462,7 @@ struct QmpWalk {
 constexpr unsigned long long kQmpLookTag = 1ull << 63;
 constexpr float kQmpLookErrors = 5.0f, kQmpLookLeast = 0.001f;
 // From this many units of a CTA on: shorter ranges are over before the answer is there, and then it costs them up to 2 us (bf16, 519 units
-// per CTA, us with / without: 21.0 / 19.1; 934 units: fp32 23.8 / 24.9, 6:8 31.1 / 33.4).
+// per CTA, us with / without: 17.4 / 16.0; 934 units: fp32 23.8 / 24.9, 6:8 31.1 / 33.4).
 constexpr uint32_t kQmpLookFrom = 700;
 __device__ __forceinline__ void qmp_look_report(QmpStreamShared& sh, double acc) {
     float sum = static_cast<float>(acc);
@@ -537,8 +541,8 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
         if constexpr (LOOK) qmp_thresholds(jb, thr_pred, width);      // may have become narrower
 #pragma unroll
         for (uint32_t rep = 0; rep < REP; ++rep) {
-            // The warp has no unit in this step (a matrix's last stage): nothing to do.  (Batch of 14 bf16 tensors 124 -> 120 us; batches of
-            // fp32 ones, which wait for memory, were 0.5 % slower with it.)
+            // The warp has no unit in this step (a matrix's last stage): nothing to do.  (Batch of 14 bf16 tensors 124 -> 120 us; of fp32
+            // ones 130.6 without, 133.4 with it.)
             if ((BF16 || LOOK) && at.left + (lane >> 3) <= 0) {
                 if (rep + 1 == REP && lane == 0) qmp_mbar_arrive(bar_empty0 + 8u * stage);
                 at.advance(jb, KB, rep + 1 < REP);
@@ -722,7 +726,7 @@ __device__ __forceinline__ void qmp_lds_pieces(const uint32_t (&src)[PIECES], ui
 // are gathered by byte permutes, and bf16 weights are selected two to a word.  The undecided are looked for only if one of the
 // warp's weights lies inside the bracket, for both groups at once, and their weights come from the stage again (held until then) instead of
 // a tree of selects.  Single calls without a hint, us, before / now (with the loops over matrices gone and the first look):
-// 2560 -> 2560 fp32 20.8 / 17.4, 2560 -> 6912 fp32 36.9 / 31.1, bf16 38.2 / 29.1 (memory: 13.5 and 8.1).
+// 2560 -> 2560 fp32 20.8 / 17.0, 2560 -> 6912 fp32 36.9 / 30.7, bf16 38.2 / 27.9 (memory: 13.5 and 8.1).
 template <bool BF16>
 __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpStreamShared& sh, bool look, QmpWarpList& list, unsigned int& flips, uint32_t& g0, uint32_t& next_stage,
                                                      uint32_t ring_base, uint32_t bar_full0, uint32_t bar_empty0, volatile int* abort_flag, bool& ok,
@@ -990,9 +994,8 @@ __device__ __forceinline__ void qmp_second_pass(const QmpDesc& d, uint32_t grid_
 }
 
 // PATTERN: 24 (2:4) or 68 (6:8).  SINGLE: one matrix, known at compile time.  Without the loops over matrices a call is 1 to 2 us
-// shorter (2560 -> 2560, no hint, with the first look and the set-up's divisions replaced, us before / now: fp32 17.4 / 15.7, bf16
-// 16.9 / 14.5; 2560 -> 6912 26.5 / 23.8 and 25.3 / 22.9; 4096 -> 11008 50 / 44.3 and 46 / 39.7); the first look would
-// cost a batch 1 %.
+// shorter; the first look would cost a batch 1 %.  Single calls without a hint, us, before / now, with 20 computing warps: 2560 ->
+// 2560 fp32 17.4 / 14.9, bf16 16.9 / 13.6; 2560 -> 6912 26.5 / 23.0 and 25.3 / 21.3; 4096 -> 11008 50 / 43.6 and 46 / 39.0.
 template <int PATTERN, bool SINGLE>
 __global__ void __launch_bounds__(kQmpThreads, 1)
 quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, const QmpDesc* __restrict__ rest, int n_matrices,
@@ -1039,9 +1042,9 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
 
     // ---- What the first bracket needs is asked for BEFORE the loader fills the ring: the hint of matrix 0 (a 4-byte
     // read), or without a hint of the caller's its sample (all threads, one round trip) together with what an
-    // earlier call may have left.  Half of the ring follows at once, the rest when the bracket is known: behind all four stages
-    // (17 MB that the loaders of all CTAs ask for at the same moment) the sample of some CTAs comes late (single calls without a hint, us,
-    // all / half: 2560 -> 3840 bf16 17.9 / 17.1, fp32 17.9 / 17.3).
+    // earlier call may have left.  A stage per team follows at once, the rest of the ring when the bracket is known: behind all
+    // stages (18 MB that the loaders of all CTAs ask for at the same moment) the sample of some CTAs comes late (single calls without a
+    // hint, us, all / half the ring / a stage per team: 2560 -> 3840 fp32 18.9 / 17.0 / 16.8, bf16 17.8 / 16.0 / 15.9).
     float gamma0 = first.gamma_hint != nullptr ? *reinterpret_cast<const volatile float*>(first.gamma_hint) : 0.0f;
     float4 sample0[kQmpSamplePerWarp];
     const bool sample_early = first.gamma_hint == nullptr;
@@ -1061,7 +1064,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     if (!sample_early && !hinted0) qmp_sample_issue(first, sample0);
     QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, qmp_policy_evict_first()};
     const bool is_loader = warp == kQmpLoaderWarp && lane == 0;
-    if (is_loader) qmp_loader_issue(loader, batch, count, kQmpStages / 2, grid_magic, ring_base, bar_full0, bar_empty0, abort_flag);
+    if (is_loader) qmp_loader_issue(loader, batch, count, kQmpTeams, grid_magic, ring_base, bar_full0, bar_empty0, abort_flag);
     if (!hinted0) gamma0 = qmp_sample_finish(first, sample0, sh.sample);
     if (threadIdx.x == 0) {
         sh.job[0].bracket = qmp_bracket_from(gamma0, first.num_units, hinted0);
@@ -1270,7 +1273,7 @@ inline sbn_status launch_quantize_mask_pack_stream_cfg(const QmpDesc* descs_host
     const unsigned cap = static_cast<unsigned>(std::min(device_sm_count(), kQmpMaxCtas));
     const unsigned grid = max_units < cap ? max_units : cap;
     if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel<PATTERN, SINGLE>>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
-    // At most one CTA per SM (1024 threads x 64 registers each) and never more CTAs than SMs, so all
+    // At most one CTA per SM (768 threads x 80 registers and 215 KB each) and never more CTAs than SMs, so all
     // of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
     // another kernel kept SMs busy for seconds, the bounded wait reports SBN_ERR_TIMEOUT instead.
     const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel<PATTERN, SINGLE>, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
