@@ -391,8 +391,9 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     for FUSED with K > 3072 (4096 -> 11008 10.0 against 9.5).
 //   9 to 16 tokens    only while two CTAs per SM take all row groups (4096 -> 11008 10.6 / 9.1: every CTA reads all activations,
 //                     the cluster kernel's 128-row tiles read them less often).  Packed weights then always (7B MLPs, whole pass,
-//                     47 / 52), int8-held ones up to K = 3328 (quantiser + GEMM at 16 tokens: 2560 -> 2560 4.85 / 5.12, 2560 -> 3840
-//                     4.97 / 5.18, 4096 -> 4096 5.95 / 5.74, 6912 -> 2560 7.6 / 6.7).  Dense: not
+//                     47 / 52), int8-held ones up to 12 tokens, beyond up to K = 4352 and for long rows of many groups (quantiser + GEMM,
+//                     9 tokens: 3584 -> 2560 5.0 / 6.1, 6912 -> 2560 6.9 / 7.2, 11008 -> 4096 9.7 / 10.9; 12: 9216 -> 2048 1 to 2 % slower, the worst; 16:
+//                     4096 -> 4096 5.6 / 6.0, 11008 -> 4096 10.2 / 10.6, but 6912 -> 2560 7.5 / 7.05).  Dense: not
 //                     (2B layers 63.5 / 59.3).  FUSED: not (6912 -> 2560 13.6 / 11.1).
 //   Not where a second round of CTAs would be barely filled: it costs as much as a full one, and the clusters have none.
 //                     Three CTAs per SM: int8-held 2:4 from K = 2560 on, a second round of up to a third (2560 -> 8192 6.6 / 5.7, 6912 -> 7424
@@ -405,7 +406,9 @@ inline bool few_wide(const FewParams& p) { return p.N / 16 > 2 * device_sm_count
 template <int WT, bool FUSED>
 inline bool few_takes(int T, int N, int K) {
     const double per_sm = static_cast<double>(N / 16) / device_sm_count();
-    if (T > 8) return T <= 16 && !FUSED && WT != kFewDense && per_sm <= 2.0 && (WT == kFewPacked || K <= 3328);
+    if (T > 8)
+        return T <= 16 && !FUSED && WT != kFewDense && per_sm <= 2.0 &&
+               (WT == kFewPacked || T <= 12 || K <= 4352 || (per_sm >= 1.7 && K >= 11008));
     if (FUSED && K > 3072)
         return !(per_sm > 2.0 && per_sm <= (T > 4 ? 3.25 : 3.0) && (K >= 6144 || (WT == kFewDense && T > 4 && K >= 4096)));
     if (WT == kFewDense) return !(per_sm > 3.0 && per_sm <= 3.7 && K >= 2560 && K <= 3584 && (!FUSED || T > 4));

@@ -247,6 +247,13 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
             for (int kb = kb0; kb < kb1; kb += G) {
                 if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { good = false; break; }
                 tcgen05_fence_after();
+                if constexpr (SPARSE) {
+                    // A copy occupies the tensor pipe as long as an MMA does (65 ns): one brings the metadata of both blocks of a stage
+                    const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(Cfg::META_COL0 + 4 * stage * G);
+                    const uint32_t e_addr = smem_e + stage * G * Cfg::E_BYTES;
+                    if constexpr (G == 2) tcgen05_cp_128x256b(e_tmem, make_smem_desc(e_addr, Cfg::E_BYTES, 128, kSwzNone));
+                    else tcgen05_cp_128x128b(e_tmem, make_smem_desc(e_addr, 128, 128, kSwzNone));
+                }
 #pragma unroll
                 for (int h = 0; h < G; ++h) {
                     if (h > 0 && kb + h >= kb1) break;
@@ -255,8 +262,6 @@ bitlinear_gemm_splitk_cluster_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     const uint32_t first = (kb + h == kb0) ? 0u : 1u;
                     if constexpr (SPARSE) {
                         const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(Cfg::META_COL0 + 4 * (stage * G + h));
-                        const uint64_t e_desc = make_smem_desc(smem_e + (stage * G + h) * Cfg::E_BYTES, 128, 128, kSwzNone);
-                        tcgen05_cp_128x128b(e_tmem, e_desc);
                         const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
                         const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
 #pragma unroll

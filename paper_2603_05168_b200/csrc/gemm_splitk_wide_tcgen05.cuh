@@ -177,6 +177,11 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { good = false; break; }
                 tcgen05_fence_after();
                 const uint32_t st = smem_base + stage * stage_bytes;
+                if constexpr (SPARSE) {                          // one copy for both blocks of a stage (see the narrow-tile kernel)
+                    const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(kWideMetaCol0 + 8 * stage);
+                    if constexpr (G == 2) tcgen05_cp_128x256b(e_tmem, make_smem_desc(st + G * A_BYTES, E_BYTES, 128, kSwzNone));
+                    else tcgen05_cp_128x128b(e_tmem, make_smem_desc(st + G * A_BYTES, 128, 128, kSwzNone));
+                }
 #pragma unroll
                 for (int h = 0; h < G; ++h) {
                     if (h > 0 && kb + h >= kb1) break;
@@ -186,7 +191,6 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
                     const uint64_t b_desc = make_smem_desc(b_addr, 16, 1024, kSwz128);
                     if constexpr (SPARSE) {
                         const uint32_t e_tmem = tmem_base + static_cast<uint32_t>(kWideMetaCol0 + 8 * stage + 4 * h);
-                        tcgen05_cp_128x128b(e_tmem, make_smem_desc(st + G * A_BYTES + h * E_BYTES, 128, 128, kSwzNone));
                         const uint64_t a_desc = make_smem_desc(a_addr, 16, 512, kSwz64);
 #pragma unroll
                         for (int j = 0; j < kBK / 64; ++j)

@@ -160,6 +160,10 @@ __device__ __forceinline__ void tcgen05_commit(uint32_t bar) {
 __device__ __forceinline__ void tcgen05_cp_128x128b(uint32_t taddr, uint64_t sdesc) {
     asm volatile("tcgen05.cp.cta_group::1.128x128b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
 }
+// 128 lanes x 32 B: two 16 B-wide source blocks (LBO apart) land in 8 consecutive TMEM columns.
+__device__ __forceinline__ void tcgen05_cp_128x256b(uint32_t taddr, uint64_t sdesc) {
+    asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
+}
 __device__ __forceinline__ void mma_i8_dense(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                              uint32_t idesc, uint32_t accumulate) {
     asm volatile(
