@@ -388,7 +388,8 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     4096 -> 11008 7.8 / 8.5, 11008 -> 4096 8.4 / 10.6.
 //                     With more row groups than two CTAs per SM take at once, three CTAs per SM with fewer blocks in flight
 //                     each (4.6 against 5.4 for 2560 -> 6912; but 6.4 against 5.7 for 6912 -> 2560, which fits two).  Not
-//                     for FUSED with K > 3072 (4096 -> 11008 10.0 against 9.5).
+//                     for FUSED with K > 3072 (4096 -> 11008 10.0 against 9.5).  Dense weights of long rows already from one and a half
+//                     groups per SM on (11008 -> 4096 11.5 / 10.85; 6912 -> 2560, fewer groups, 6.6 / 7.2).
 //   9 to 16 tokens    only while two CTAs per SM take all row groups (4096 -> 11008 10.6 / 9.1: every CTA reads all activations,
 //                     the cluster kernel's 128-row tiles read them less often).  Packed weights then always (7B MLPs, whole pass,
 //                     47 / 52), int8-held ones up to 12 tokens, beyond up to K = 4352 and for long rows of many groups (quantiser + GEMM,
@@ -422,7 +423,8 @@ inline sbn_status launch_few(const FewParams& p, cudaStream_t stream) {
     if (p.T > 8) {
         if constexpr (FUSED || WT == kFewDense) return SBN_ERR_UNSUPPORTED;  // not reached: few_takes()
         else err = launch_few_cfg<WT, 2, 8, 2, 2, false>(p, stream);
-    } else if (few_wide(p) && !(FUSED && p.k_blocks > 24)) {
+    } else if ((few_wide(p) && !(FUSED && p.k_blocks > 24)) ||
+               (WT == kFewDense && !FUSED && 2 * (p.N / 16) >= 3 * device_sm_count() && p.k_blocks >= 32)) {
         err = launch_few_cfg<WT, 1, 8, 2, 3, FUSED>(p, stream);
     } else {
         err = launch_few_cfg<WT, 1, 8, 4, 2, FUSED>(p, stream);
