@@ -236,6 +236,9 @@ bitlinear_gemm_few_kernel(const FewParams p) {
     FewBlock<WT> blk[D];
 #pragma unroll
     for (int j = 0; j < D; ++j) fetch.next(p, lane, blk[j]);
+    if constexpr (FUSED) {                                                   // the activations too: a warp per token
+        if (lane == 0u && warp < p.T) prefetch_l2_bulk(p.x_bf16 + static_cast<size_t>(warp) * (p.k_blocks * 16), static_cast<uint32_t>(p.k_blocks) * 256u);
+    }
     if constexpr (AHEAD) few_prefetch_next<WT, W, D>(p, lane, static_cast<uint32_t>(warp), static_cast<uint32_t>(rounds));
     pdl_wait();
 
@@ -392,9 +395,9 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //                     groups per SM on (11008 -> 4096 11.5 / 10.85; 6912 -> 2560, fewer groups, 6.6 / 7.2).
 //   9 to 16 tokens    only while two CTAs per SM take all row groups (4096 -> 11008 10.6 / 9.1: every CTA reads all activations,
 //                     the cluster kernel's 128-row tiles read them less often).  Packed weights then always (7B MLPs, whole pass,
-//                     47 / 52), int8-held ones up to 12 tokens, beyond up to K = 4352 and for long rows of many groups (quantiser + GEMM,
+//                     47 / 52), int8-held ones up to 12 tokens, beyond up to K = 4352 (quantiser + GEMM,
 //                     9 tokens: 3584 -> 2560 5.0 / 6.1, 6912 -> 2560 6.9 / 7.2, 11008 -> 4096 9.7 / 10.9; 12: 9216 -> 2048 1 to 2 % slower, the worst; 16:
-//                     4096 -> 4096 5.6 / 6.0, 11008 -> 4096 10.2 / 10.6, but 6912 -> 2560 7.5 / 7.05).  Dense: not
+//                     4096 -> 4096 5.6 / 6.0, but 6912 -> 2560 7.5 / 7.05; two 7B MLPs, whole pass, 44.5 / 41.8).  Dense: not
 //                     (2B layers 63.5 / 59.3).  FUSED: not (6912 -> 2560 13.6 / 11.1).
 //   Not where a second round of CTAs would be barely filled: it costs as much as a full one, and the clusters have none.
 //                     Three CTAs per SM: int8-held 2:4 from K = 2560 on, a second round of up to a third (2560 -> 8192 6.6 / 5.7, 6912 -> 7424
@@ -409,7 +412,7 @@ inline bool few_takes(int T, int N, int K) {
     const double per_sm = static_cast<double>(N / 16) / device_sm_count();
     if (T > 8)
         return T <= 16 && !FUSED && WT != kFewDense && per_sm <= 2.0 &&
-               (WT == kFewPacked || T <= 12 || K <= 4352 || (per_sm >= 1.7 && K >= 11008));
+               (WT == kFewPacked || T <= 12 || K <= 4352);
     if (FUSED && K > 3072)
         return !(per_sm > 2.0 && per_sm <= (T > 4 ? 3.25 : 3.0) && (K >= 6144 || (WT == kFewDense && T > 4 && K >= 4096)));
     if (WT == kFewDense) return !(per_sm > 3.0 && per_sm <= 3.7 && K >= 2560 && K <= 3584 && (!FUSED || T > 4));

@@ -101,11 +101,16 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
     const int iters = (T + row_stride - 1) / row_stride;        // same for every thread of the CTA
 
     pdl_launch_dependents();             // the next kernel may become resident (and fetch weights) right away
+    uint4 cur[VPT], nxt[VPT];
+    int row = blockIdx.x * ROWS + r;
+    // the first row and the gains go to the L2 while the kernel before finishes (see quant_act.cuh)
+    if (row < T && g * 8 < nvec) prefetch_l2_line(x + static_cast<size_t>(row) * nvec + g * 8);
+    if (GAIN) {
+        for (int i = threadIdx.x; i * 4 < nvec; i += kActThreads) prefetch_l2_line(gain + 8 * i);
+    }
     pdl_wait();
 
     // the first row is on its way before the gains are fetched (one after the other they were two trips to memory)
-    uint4 cur[VPT], nxt[VPT];
-    int row = blockIdx.x * ROWS + r;
 #pragma unroll
     for (int i = 0; i < VPT; ++i) {
         const int idx = g + i * G;

@@ -64,6 +64,10 @@ quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
+    if (lane == 0u && row < T) prefetch_l2_bulk(x + static_cast<size_t>(row) * nvec, row_bytes);       // see quant_act.cuh
+    if constexpr (GAIN) {
+        for (int i = threadIdx.x; i * 4 < nvec; i += blockDim.x) prefetch_l2_line(gain + 8 * i);
+    }
     pdl_wait();
     auto fetch = [&](int r) {
         if (lane == 0u && r < T) bulk_load_row(at, x + static_cast<size_t>(r) * nvec, row_bytes, bar);

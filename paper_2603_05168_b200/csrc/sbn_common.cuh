@@ -126,6 +126,10 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
     return launch_kernel_cluster(kernel, grid, block, smem, stream, 0u, std::forward<Args>(args)...);
 }
 
+// Ask the L2 for the line at p, before the dependency wait: the L2 is the point of coherence, so nothing can go stale,
+// whoever writes the line in the meantime.
+__device__ __forceinline__ void prefetch_l2_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Ask the L2 to fetch [p, p + bytes) (a multiple of 16 B) -- issued by one thread, no destination.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
