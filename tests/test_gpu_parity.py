@@ -366,10 +366,10 @@ def test_pack68_bf16_masters_and_ties():
     _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
 
 
-@pytest.mark.parametrize("scale", [1e-36, 1e-39])
+@pytest.mark.parametrize("scale", [1e-36, 1e-38, 1e-39])
 def test_pack_bf16_masters_of_tiny_magnitude(scale):
     # magnitudes whose differences are subnormal: the selection subtracts, and no difference may be lost
-    bits = inputs.f32_to_bf16_bits((inputs.latent_weights(256, 512, seed=60) * np.float32(scale)).astype(np.float32))
+    bits = inputs.f32_to_bf16_bits((inputs.latent_weights(256, 512, seed=61) * np.float32(scale)).astype(np.float32))
     W = (bits.astype(np.uint32) << 16).view(np.float32).reshape(256, 512)
     _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
     r, g = _oracle_pack(W), gpu_quantize_mask_pack(W, with_dense=False, w_bf16_bits=bits)
