@@ -16,7 +16,8 @@
 // 4096 x 6912 26.8 [13.2], 8192 x 4096 29.7 [15.6], 8192 x 11008 76 [42] -- bound by the instructions, 22.7 per element
 // (73 % of the issue slots busy); the plain quantiser (7.4, 16.3, 21.8, 49) needs fewer.  Squares through the conversion instruction, gains
 // fetched before the row, a division for the mean and a clamp: 2.21, 2.10, 3.14, 12.0, 28.2, 31.6 and 82.  One or two
-// warps per row without the prefetch of the next row were slower: 15.7, 31.7, 36.6, 90.
+// warps per row without the prefetch of the next row were slower: 15.7, 31.7, 36.6, 90.  Many rows of up to 5120 columns go to
+// quant_rows.cuh.
 #pragma once
 
 #include "quant_act.cuh"
