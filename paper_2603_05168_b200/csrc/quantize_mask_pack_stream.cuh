@@ -638,7 +638,8 @@ struct QmpBracket {
 };
 // Eight consecutive weights (half of a lane's 16): fp32 in eight words, bf16 in four.
 // Sum |w| in fp64.  |bf16| becomes a double by two integer instructions (see bf16_abs_to_f64 in norm_quant_act.cuh: a zero
-// counts as 2^-127, which no sum above the 1e-5 clamp can see); fp32 takes the conversion instruction.
+// counts as 2^-127, which no sum above the 1e-5 clamp can see; the sums of a lane that saw an infinity or a NaN are taken again, below);
+// fp32 takes the conversion instruction.
 template <bool BF16>
 __device__ __forceinline__ double qmp_abs_sum8(const uint32_t* r) {
     double d[8];
@@ -652,6 +653,23 @@ __device__ __forceinline__ double qmp_abs_sum8(const uint32_t* r) {
         }
     }
     return ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7]));
+}
+
+// A lane's 16 bf16 weights as fp32 weights of the same values are selected and summed: for infinities and NaN, whose exponent field
+// qmp_abs_sum8 takes for 2^128 (and select6of8_bf16 orders by their bits), so that a diverged run shows in the scale.
+__device__ __forceinline__ void select_and_sum_as_f32(const uint32_t (&r)[8], uint32_t (&S)[2], double& sum) {
+    sum = 0.0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        float a[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t w = r[4 * g + (i >> 1)];
+            a[i] = fabsf((i & 1) ? bf16hi_to_f32(w) : bf16lo_to_f32(w));
+            sum += static_cast<double>(a[i]);
+        }
+        S[g] = select6of8(a);
+    }
 }
 
 // Ternary bytes of eight weights at the upper end of the bracket (t_lo, t_hi), and whether one of them may be undecided.
@@ -791,8 +809,10 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpStream
             auto v_off = [&](uint32_t v) { return prmt(v, 0u, half) ^ swizzle; };           // on top of 64 q_cur
             constexpr int kHalf = 2 * PIECES;                         // words of a group
             uint32_t S[2];
+            double sum = qmp_abs_sum8<BF16>(r) + qmp_abs_sum8<BF16>(r + kHalf);
             if constexpr (BF16) {
                 select6of8_bf16(r, S[0], S[1]);
+                if (__double2hiint(sum) >= 0x47F00000) select_and_sum_as_f32(r, S, sum);      // 2^128 or more
             } else {
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
@@ -812,7 +832,6 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpStream
                 v4[g] = prmt(t_lo[g], t_hi[g], entry[g].x);
                 v2[g] = prmt(t_lo[g], t_hi[g], entry[g].x >> 16);     // two bytes
             }
-            const double sum = qmp_abs_sum8<BF16>(r) + qmp_abs_sum8<BF16>(r + kHalf);
             const uint32_t f4 = swap ? v4[1] : v4[0], f2 = swap ? v2[1] : v2[0], l4 = swap ? v4[0] : v4[1], l2 = swap ? v2[0] : v2[1];
             const uint32_t m24 = swap ? (entry[1].y | (entry[0].y << 12)) : (entry[0].y | (entry[1].y << 12));
             const uint32_t nxt = __shfl_down_sync(0xFFFFFFFFu, m24, 1);

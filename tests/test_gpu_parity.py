@@ -376,6 +376,24 @@ def test_pack_bf16_masters_of_tiny_magnitude(scale):
     assert g["scale"] == r["scale"] and np.array_equal(g["vals"], r["vals"]) and np.array_equal(g["meta"], r["meta"])
 
 
+@pytest.mark.parametrize("N,K", [(256, 512), (4096, 4096)])      # 4096 rows: the CTAs exchange what they have seen under way
+@pytest.mark.parametrize("special", [(0x7F80,), (0xFF80,), (0x7FC0,), (0x7F80, 0xFFC0, 0xFF80), (0x7F7F, 0xFF7F)])
+def test_pack68_bf16_masters_show_what_is_not_finite(special, N, K):
+    # bf16 masters with infinities, NaN or the largest finite magnitude give what fp32 masters of the same values do: an infinite weight
+    # makes the scale infinite
+    bits = inputs.f32_to_bf16_bits(inputs.latent_weights(N, K, seed=62)).reshape(N, K)
+    for i, v in enumerate(special):
+        bits.reshape(-1)[(104729 * (i + 1)) % bits.size] = v
+        bits[5 + i, 8:16] = v                                  # a whole group
+        bits[N - 1, K - 9 + i] = v
+    W = (bits.astype(np.uint32) << 16).view(np.float32).reshape(N, K)
+    f, g = gpu_quantize_mask_pack68(W), gpu_quantize_mask_pack68(W, w_bf16_bits=bits)
+    assert f["scale"].view(np.uint32) == g["scale"].view(np.uint32)
+    assert np.array_equal(f["vals"], g["vals"]) and np.array_equal(f["meta"], g["meta"])
+    mean = np.abs(W.astype(np.float64)).mean()
+    assert np.isnan(mean) or g["scale"] == np.float32(mean)
+
+
 @pytest.mark.parametrize("misleading", [False, True])
 @pytest.mark.parametrize("bf16", [False, True])
 def test_pack_long_matrix_narrows_its_bracket(bf16, misleading):
