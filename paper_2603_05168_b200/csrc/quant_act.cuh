@@ -92,11 +92,18 @@ __device__ __forceinline__ void store_codes8(uint2* __restrict__ xq, int t, int 
     }
 }
 
+// The maximum of a row of nvec vectors is taken over this many parts; blocks of 32 vectors belong to them in turn.  Within a part the
+// largest bit pattern is the maximum, so that a NaN takes the part over; over the parts it is fmaxf, which ignores such a part.
+// Finite rows do not depend on it, but a row with a NaN must not get other codes in a call with more or fewer rows: all kernels that
+// take a row length use the same number.
+__host__ __device__ constexpr int row_parts(int nvec) { return nvec <= 32 * 2 ? 1 : (nvec <= 64 * 2 ? 2 : (nvec <= 128 * 3 ? 4 : 8)); }
+
 // G threads per token row, VPT 16-byte vectors per thread (G * VPT >= K / 8).  Persistent CTAs:
 // every row group walks over rows with a grid-sized stride and loads its NEXT row while it reduces,
 // rounds and stores the current one, so each SM always has loads in flight (a non-pipelined
 // version of this kernel was latency-bound at a third of the HBM rate).
-template <int G, int VPT, bool EXPAND68 = false>
+// PARTS: see row_parts; warps w, w + PARTS, ... of a row belong to one part.
+template <int G, int VPT, bool EXPAND68 = false, int PARTS = (G + 31) / 32>
 __global__ void __launch_bounds__(kActThreads, (VPT <= 4) ? 3 : 2)
 quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, uint2* __restrict__ xq,
                  float* __restrict__ a_scale) {
@@ -142,10 +149,13 @@ quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, uint2* __restrict
             if ((threadIdx.x & 31) == 0) sm[warp] = amax;
             __syncthreads();
             const int w0 = (r * G) >> 5;
-            float m = sm[w0];
 #pragma unroll
-            for (int w = 1; w < WARPS_PER_ROW; ++w) m = fmaxf(m, sm[w0 + w]);
-            amax = m;
+            for (int p = 0; p < PARTS; ++p) {
+                uint32_t m = __float_as_uint(sm[w0 + p]);
+#pragma unroll
+                for (int w = p + PARTS; w < WARPS_PER_ROW; w += PARTS) m = max(m, __float_as_uint(sm[w0 + w]));
+                amax = p == 0 ? __uint_as_float(m) : fmaxf(amax, __uint_as_float(m));
+            }
         }
         if (row < T) {
             const float d = fmaxf(amax, kEps);
@@ -200,13 +210,13 @@ quant_act_long_row_kernel(const uint4* __restrict__ x, int T, int nvec, uint2* _
     }
 }
 
-template <int G, int VPT, bool EXPAND68>
+template <int G, int VPT, bool EXPAND68, int PARTS = (G + 31) / 32>
 static void launch_quant_act_cfg(const uint4* x, int T, int nvec, uint2* q, float* a_scale, cudaStream_t stream) {
     constexpr int rows = kActThreads / G;
     const int ctas_per_sm = (VPT <= 4) ? 3 : 2;
     int grid = (T + rows - 1) / rows;
     if (grid > kNumSMs * ctas_per_sm) grid = kNumSMs * ctas_per_sm;
-    launch_kernel(quant_act_kernel<G, VPT, EXPAND68>, dim3(grid), dim3(kActThreads), 0, stream, x, T, nvec, q, a_scale);
+    launch_kernel(quant_act_kernel<G, VPT, EXPAND68, PARTS>, dim3(grid), dim3(kActThreads), 0, stream, x, T, nvec, q, a_scale);
 }
 
 template <bool EXPAND68 = false>
@@ -217,7 +227,7 @@ inline sbn_status launch_quant_act(const void* x_bf16, int T, int K, int8_t* xq,
     uint2* q = reinterpret_cast<uint2*>(xq);
     // Few rows: a whole CTA each (16 x 2560 1.30 us, 1.12; with the GEMM after it 2560 -> 3840 4.85 / 4.58; at 148 rows 7.95 / 8.4: a CTA on
     // every SM keeps the GEMM's out).  Else the smallest group that keeps <= 3 (then 4, 6, 8) vectors per thread.
-    if (T <= 100 && nvec > 128 && nvec <= 256 * 2) launch_quant_act_cfg<256, 2, EXPAND68>(x, T, nvec, q, a_scale, stream);
+    if (T <= 100 && nvec > 64 * 2 && nvec <= 128 * 3) launch_quant_act_cfg<256, 2, EXPAND68, row_parts(128 * 3)>(x, T, nvec, q, a_scale, stream);
     else if (nvec <= 32 * 2) launch_quant_act_cfg<32, 2, EXPAND68>(x, T, nvec, q, a_scale, stream);
     else if (nvec <= 64 * 2) launch_quant_act_cfg<64, 2, EXPAND68>(x, T, nvec, q, a_scale, stream);
     else if (nvec <= 128 * 2) launch_quant_act_cfg<128, 2, EXPAND68>(x, T, nvec, q, a_scale, stream);

@@ -138,6 +138,17 @@ quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __
 #pragma unroll 4
             for (int idx = lane; idx < nvec; idx += 32) pm = absmax8_packed(lds_vec(at + 16u * idx), pm);
             amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, max(pm >> 16, pm & 0xFFFFu)) << 16);
+            if (__float_as_uint(amax) > 0x7F800000u) {                          // a NaN: part by part (see row_parts)
+                const int parts = row_parts(nvec);
+                amax = 0.0f;
+#pragma unroll 1
+                for (int p = 0; p < parts; ++p) {
+                    pm = 0u;
+#pragma unroll 1
+                    for (int idx = 32 * p + lane; idx < nvec; idx += 32 * parts) pm = absmax8_packed(lds_vec(at + 16u * idx), pm);
+                    amax = fmaxf(amax, __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, max(pm >> 16, pm & 0xFFFFu)) << 16));
+                }
+            }
         }
         const float d = fmaxf(amax, kEps);
         const float s_x = __fdiv_rn(127.0f, d);

@@ -107,6 +107,30 @@ def test_norm_quant_act_warp_per_row(T, K):
     test_norm_quant_act_rows_that_overflow(T, K)
 
 
+# What a row becomes does not depend on how many rows the call has, non-finite rows included: row counts on both sides of where other
+# kernels begin, every number of warps that a row of that length can have
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("K", [1024, 1152, 2560, 3072, 4096, 5120])
+def test_rows_do_not_depend_on_their_number(K, norm):
+    T, parts = 7040, [16, 101, 963, 1000, 1960, 3000]
+    bits = inputs.activations_bf16(T, K, seed=K).reshape(T, K)
+    rng = np.random.default_rng(K)
+    for t in range(0, T, 5):                                    # an infinity or a NaN or two in every fifth row, anywhere
+        for v in rng.choice([0x7F80, 0xFF80, 0x7FC0, 0xFFC1, 0x7F7F], size=1 + t % 2):
+            bits[t, rng.integers(K)] = v
+    bits[3, :] = 0x7FC0
+    quantise = gpu_norm_quant_act if norm else gpu_quant_act
+    xq, s = quantise(bits)
+    xq, s = xq_to_numpy(xq, T, K), s.cpu().numpy()
+    begin = 0
+    for n in parts:
+        q, t = quantise(bits[begin:begin + n])
+        assert np.array_equal(xq_to_numpy(q, n, K), xq[begin:begin + n]), n
+        assert np.array_equal(t.cpu().numpy().view(np.uint32), s[begin:begin + n].view(np.uint32)), n
+        begin += n
+    assert begin == T
+
+
 # Finite inputs whose normalised row is not finite: no scale brings such a value into range, and its code is 127 (the saturated
 # end), as for every width of the kernel; with eps > 0 and finite products nothing changes.
 @pytest.mark.parametrize("T,K", [(5, 256), (5, 1280), (600, 1280), (600, 2560), (5, 4096), (600, 6912), (600, 11008), (5, 16384)])
