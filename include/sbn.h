@@ -435,8 +435,8 @@ const char *sbn_status_string(sbn_status s);
  * 256 dense; with split_k = 1 its variant with one M-tile per CTA) and the backward GEMMs with tiles of 128 (BN <= 128) or
  * 256 columns.  split_k: 0 = automatic; k > 0 = split K k ways through int32 atomics in the
  * workspace (single-CTA kernel); -2, -3, -4, -8 = split K inside thread-block clusters of that many
- * CTAs (token tile 64, or 32 if token_tile says so; a token_tile above 64 selects the wide-tile kernel with that width,
- * a multiple of 16 up to 256, and clusters of 2 to 8, or -1: unsplit; no workspace; -2, -3, -4 also set the
+ * CTAs (token tile 64, or 32 if token_tile says so; a token_tile of 80 or more selects the wide-tile kernel with that width,
+ * rounded down to a multiple of 16, up to 256, and clusters of 2 to 8, or -1: unsplit; no workspace; -2, -3, -4 also set the
  * cluster size of sbn_sparse_bitlinear_packed and of the sbn_quant_act_*bitlinear kernels).  Results do not depend on
  * it. */
 void sbn_set_gemm_tuning(int token_tile, int split_k);

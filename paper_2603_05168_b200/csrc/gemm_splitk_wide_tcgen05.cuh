@@ -32,6 +32,7 @@ namespace sbn {
 constexpr int kWideEpiWarps = 8;
 constexpr int kWideThreads = 32 * (2 + kWideEpiWarps);
 constexpr int kWideMaxStages = 8;
+constexpr int kWideMinBn = 80;                              // narrower tiles belong to the narrow-tile kernel
 constexpr int kWideDataBytes = 224 * 1024;                  // stages, then P and the receive area
 constexpr int kWideSmemBytes = 1024 + kWideDataBytes + kBarrierBytes;
 static_assert(kWideSmemBytes + 1024 + 64 <= 232448, "shared memory overflow");

@@ -277,7 +277,7 @@ static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool 
     }
     if (g_force_split_k < 0) {                                  // diagnostics: cluster split-K as told
         int S = -g_force_split_k;
-        if (g_force_token_tile > 64) {                          // wide tiles: any width and cluster that fit
+        if (g_force_token_tile >= kWideMinBn) {                 // wide tiles: any width and cluster that fit
             const int bn = std::min(256, g_force_token_tile / 16 * 16);
             const bool unsplit = S == 1;
             S = std::min(8, std::min(S, K / kBK));
@@ -310,7 +310,7 @@ static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool 
     if (T > 64 && T <= 2048) {
         const int fewest = (T + 255) / 256;
         for (int tt = fewest; tt <= fewest + (T > 512 ? 4 : 2); ++tt) {
-            const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
+            const int bn = std::max(kWideMinBn, ((T + tt - 1) / tt + 15) / 16 * 16);
             if (bn * (tt - 1) >= T) continue;
             const int tokens = std::min(bn, T);
             const double c = wide_group(sparse, bn) == 2 ? cost.wide.c2 + cost.wide.u2 * bn / 256 : cost.wide.c + cost.wide.u * bn / 256;
@@ -330,7 +330,7 @@ static GemmPlan plan_gemm(bool sparse, bool out_wide, int T, int N, int K, bool 
         const WideOneCost& c = kWideOneCosts[out_wide];
         const int fewest = (T + 255) / 256;
         for (int tt = fewest; tt <= fewest + 5 && static_cast<long>(rows) * tt <= kNumSMs; ++tt) {
-            const int bn = std::max(80, ((T + tt - 1) / tt + 15) / 16 * 16);
+            const int bn = std::max(kWideMinBn, ((T + tt - 1) / tt + 15) / 16 * 16);
             if (bn * (tt - 1) >= T) continue;
             const double share = static_cast<double>(rows) * tt / kNumSMs;
             const double block = wide_group(sparse, bn) == 2 ? c.c2 + c.u2 * bn / 256 : c.c + c.u * bn / 256;
@@ -520,8 +520,11 @@ static sbn_status run_gemm(bool sparse, const int8_t* xq, const float* a_scale, 
     p.test_skip_loads = g_test_break_waits;
 
     if (plan.cluster >= 1) {
+        // the cluster sizes that the kernels have code for; another would write to CTAs that do not exist
+        const bool wide = bn >= kWideMinBn;
+        if (wide ? plan.cluster > 8 : (plan.cluster != 2 && plan.cluster != 3 && plan.cluster != 4 && plan.cluster != 8)) return SBN_ERR_UNSUPPORTED;
         p.k_splits = 1;
-        if (bn > 64) {                                          // boxes of wide_group K-blocks
+        if (wide) {                                             // boxes of wide_group K-blocks
             const uint32_t G = static_cast<uint32_t>(wide_group(sparse, bn));
             ok = (sparse ? encode_flat_1k(&ta, wvals, NK / 2, 8 * G) && encode_flat_1k(&te, meta, NK / 8, 2 * G) : encode_flat_1k(&ta, wvals, NK, 16 * G)) &&
                  (G == 1 || encode_3d_1k(&tb, xq, xq_tb8(T), static_cast<uint64_t>(K) / kBK, static_cast<uint32_t>(bn / 8), G));   // G = 1: tb as it is

@@ -284,6 +284,27 @@ def test_plans_never_ask_for_more_clusters_than_fit(L):
     assert len(seen) >= 9                                             # tiles, both pairs, every cluster size in both widths
 
 
+def test_forced_cluster_plans_are_ones_that_a_kernel_has(L):
+    """Whatever sbn_set_gemm_tuning is given: narrow tiles have code for clusters of 2, 3, 4 and 8 CTAs only (5 to 7, or 1, would
+    address CTAs that do not exist), wide tiles are at least 80 tokens wide."""
+    from paper_2603_05168_b200 import binding as b
+    try:
+        for tile in [*range(32, 100), 128, 255, 256, 300]:
+            for split in range(-9, 0):
+                for sparse, T, N, K in [(True, 72, 256, 2560), (False, 300, 384, 1024), (True, 9, 128, 256), (False, 100, 128, 128)]:
+                    b.sbn_set_gemm_tuning(tile, split)
+                    kernel, bn, _, cluster = plan = b.sbn_plan_gemm(sparse, T, N, K)
+                    assert bn % 16 == 0 and cluster <= max(1, K // 128), (tile, split, plan)
+                    if kernel == 1:
+                        assert cluster in (2, 3, 4, 8) if bn <= 64 else 2 <= cluster <= 8, (tile, split, plan)
+                        assert bn in (32, 64) or bn >= 80, (tile, split, plan)
+                    if 64 < tile < 80 and K >= 256:                   # rounds down to 64, a narrow tile
+                        b.sbn_set_gemm_tuning(64, split)
+                        assert plan == b.sbn_plan_gemm(sparse, T, N, K), (tile, split)
+    finally:
+        b.sbn_set_gemm_tuning(0, 0)
+
+
 def test_wide_matrices_run_on_pairs_and_long_dense_rows_may_split(L):
     from paper_2603_05168_b200 import binding as b
     assert b.sbn_plan_gemm(True, 16, 20480, 4096)[0] in (2, 3)        # 160 row tiles: more than the clusters have places
