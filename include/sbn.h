@@ -463,7 +463,8 @@ void sbn_set_gemm_probe(int flags);
  * whenever sbn_set_gemm_tuning or sbn_set_wait_test is in force; most calls of up to 8 tokens, and some sparse ones of up
  * to 16, run the register-fed few-token kernel instead.
  * out4[0] = kernel (0 single-CTA tiles, 1 cluster split-K, 2 CTA pair with 512-feature tiles, 3 CTA
- * pair with 256-feature tiles and double-buffered accumulators), out4[1] = tokens per tile,
+ * pair with 256-feature tiles and double-buffered accumulators, 4 the wide-tile kernel of 1 unsplit:
+ * dense weights, one tile per SM at most), out4[1] = tokens per tile,
  * out4[2] = split-K factor through global memory (1 = none), out4[3] = cluster size (0 = none).
  * All zero for an illegal shape. */
 void sbn_plan_gemm(int sparse, int T, int N, int K, int *out4);

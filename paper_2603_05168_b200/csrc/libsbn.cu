@@ -1069,7 +1069,7 @@ void sbn_plan_gemm(int sparse, int T, int N, int K, int* out4) {
     out4[0] = out4[1] = out4[2] = out4[3] = 0;
     if (T <= 0 || N <= 0 || K <= 0 || N % kBM != 0 || K % kBK != 0) return;
     const GemmPlan g = plan_gemm(sparse != 0, false, T, N, K);
-    out4[0] = g.pair ? (g.mt == 1 ? 3 : 2) : (g.cluster > 1 ? 1 : 0);
+    out4[0] = g.pair ? (g.mt == 1 ? 3 : 2) : (g.cluster > 1 ? 1 : (g.cluster == 1 ? 4 : 0));
     out4[1] = g.bn;
     out4[2] = g.splits;
     out4[3] = g.cluster > 1 ? g.cluster : 0;

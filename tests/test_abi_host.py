@@ -284,6 +284,25 @@ def test_plans_never_ask_for_more_clusters_than_fit(L):
     assert len(seen) >= 9                                             # tiles, both pairs, every cluster size in both widths
 
 
+def test_unsplit_wide_tiles_are_reported_and_at_most_one_per_sm(L):
+    import random
+    from paper_2603_05168_b200 import binding as b
+    rng = random.Random(4)
+    assert b.sbn_plan_gemm(False, 600, 4096, 11008)[0] == 4
+    n = 0
+    for _ in range(5000):
+        T, N, K = round(2 ** rng.uniform(6, 11.5)), 128 * round(2 ** rng.uniform(0, 7)), 128 * round(2 ** rng.uniform(1, 7.5))
+        assert b.sbn_plan_gemm(True, T, N, K)[0] != 4                 # dense weights only
+        kernel, bn, split, cluster = b.sbn_plan_gemm(False, T, N, K)
+        if kernel == 0:
+            assert bn in (64, 128, 256), (T, N, K)                    # the widths that the single-CTA kernel has
+        if kernel == 4:
+            n += 1
+            assert 80 <= bn <= 256 and bn % 16 == 0 and (split, cluster) == (1, 0)
+            assert 64 < T <= 2048 and N // 128 * -(-T // bn) <= 148, (T, N, K)
+    assert n > 100
+
+
 def test_forced_cluster_plans_are_ones_that_a_kernel_has(L):
     """Whatever sbn_set_gemm_tuning is given: narrow tiles have code for clusters of 2, 3, 4 and 8 CTAs only (5 to 7, or 1, would
     address CTAs that do not exist), wide tiles are at least 80 tokens wide."""
