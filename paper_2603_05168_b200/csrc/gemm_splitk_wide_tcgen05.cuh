@@ -36,6 +36,11 @@ constexpr int kWideMinBn = 80;                              // narrower tiles be
 constexpr int kWideDataBytes = 224 * 1024;                  // stages, then P and the receive area
 constexpr int kWideSmemBytes = 1024 + kWideDataBytes + kBarrierBytes;
 static_assert(kWideSmemBytes + 1024 + 64 <= 232448, "shared memory overflow");
+// A CTA of the activation quantiser (1 KB that the system takes, 128 B) fits beside one of these to the byte: in a chain of quantisers
+// and GEMMs the next quantiser is then resident before this kernel ends.  With 512 B more here every such GEMM took 0.4 to
+// 0.7 us longer (dense 2560 -> 2560, 256 tokens 8.5 / 9.2; 2560 -> 3840 9.3 / 9.7; 6912 -> 2560 sparse, 201 tokens 10.6 / 10.9).
+constexpr int kWideStaticSmemBytes = 640;                   // what ptxas reports for this kernel
+static_assert(kWideSmemBytes + kWideStaticSmemBytes + 1024 + (1024 + 128) <= 228 * 1024, "the quantiser no longer fits beside");
 constexpr uint32_t kWideTmemCols = 512;                     // accumulator up to 256, metadata above it
 constexpr int kWideMetaCol0 = 256;
 
@@ -78,7 +83,7 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
     const uint32_t tmem_slot = bar_recv + 8;
 
     __shared__ int s_abort;
-    __shared__ float s_scale[256];                           // of the tokens this CTA finishes
+    __shared__ float s_scale_split[128];                     // of the tokens this CTA finishes, S > 1 (at most 128 then)
     volatile int* abort_flag = &s_abort;
 
     const int warp = threadIdx.x >> 5;
@@ -224,8 +229,12 @@ bitlinear_gemm_splitk_wide_kernel(const __grid_constant__ CUtensorMap tmap_a,
 #pragma unroll
             for (int j = 0; j < 4; ++j) bias[j] = __ldg(p.bias + n4 + j);
         }
-        if (e < my_tokens) s_scale[e] = __fmul_rn(__ldg(p.w_scale), __ldg(p.a_scale + t0 + my0 + e));
+        // unsplit: up to 256 scales, at the end of the area that the stages leave once the MMAs are done (P needs at most 128 KB of it)
+        float* const s_scale = S == 1 ? reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)) + kWideDataBytes) - 256 : s_scale_split;
+        const float scale = e < my_tokens ? __fmul_rn(__ldg(p.w_scale), __ldg(p.a_scale + t0 + my0 + e)) : 0.0f;
+        if (S > 1 && e < my_tokens) s_scale[e] = scale;
         bool ok = mbar_wait(bar_acc_full, 0u, abort_flag);
+        if (S == 1 && ok) s_scale[e] = scale;
         tcgen05_fence_after();
         cluster_wait();                                      // all peers have started, their barriers exist
         if (ok && e < S) mbar_arrive_cluster(map_to_cta(bar_ready, static_cast<uint32_t>(e)));

@@ -918,6 +918,23 @@ def test_gemm_bias_and_bf16_output(sparse):
     assert np.abs(got_bits - ref_bits).max() <= 1
 
 
+@pytest.mark.parametrize("T,N,K", [(200, 6272, 1280), (777, 1664, 1280), (2000, 1920, 6912)])
+def test_gemm_dense_plan_of_unsplit_wide_tiles(T, N, K):
+    # the library's own choice: accumulators against a product in fp64 (exact), outputs bit for bit in the documented order of roundings
+    assert b.sbn_plan_gemm(False, T, N, K)[0] == 4
+    g = gpu_quantize_mask_pack(inputs.latent_weights(N, K, seed=T))
+    xq, a_scale = gpu_quant_act(inputs.activations_bf16(T, K, seed=T + 1, token_lognormal_sigma=0.5))
+    codes = dev(xq_to_numpy(xq, T, K)).double()
+    acc_ref = (codes @ dev(g["dense_q"]).double().T).to(torch.int32)
+    bias = torch.randn(N, device="cuda", generator=torch.Generator("cuda").manual_seed(K))
+    y_ref = acc_ref.float() * (a_scale * g["dev"]["w_scale"])[:, None]
+    for out_dtype, with_bias, want_acc in [(torch.float32, True, True), (torch.float32, False, False), (torch.bfloat16, True, False)]:
+        y, acc = gpu_gemm(False, xq, a_scale, g["dev"], out_dtype=out_dtype, bias=bias if with_bias else None, want_acc=want_acc)
+        if want_acc:
+            assert torch.equal(acc, acc_ref)
+        assert torch.equal(y, (y_ref + bias if with_bias else y_ref).to(out_dtype))
+
+
 def test_exact_integer_layer_on_gpu():
     # integer activations and ternary weights: no quantisation error anywhere, acc is the exact
     # integer product and sparse == dense when the pruned entries are zeros
