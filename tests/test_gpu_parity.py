@@ -377,6 +377,14 @@ def _assert_pack68(W, g):
     return r
 
 
+def _masters(W, bf16):
+    """(W, the bf16 bit patterns or None): the weights as fp32 masters, or rounded to bf16 ones of the same values."""
+    if not bf16:
+        return W, None
+    bits = inputs.f32_to_bf16_bits(W).reshape(W.shape)
+    return (bits.astype(np.uint32) << 16).view(np.float32).reshape(W.shape), bits
+
+
 @pytest.mark.parametrize("N,K,seed", [(128, 256, 50), (256, 512, 51), (384, 2560, 52), (128, 6912, 53), (2048, 2560, 54),
                                       (640, 1280, 55)])
 def test_pack68_parity(N, K, seed):
@@ -418,29 +426,49 @@ def test_pack68_bf16_masters_show_what_is_not_finite(special, N, K):
     assert np.isnan(mean) or g["scale"] == np.float32(mean)
 
 
-@pytest.mark.parametrize("misleading", [False, True])
+def _first_look(W, bf16):
+    """What a single call without a hint does to its bracket around the mean |w| while it runs, on the host: (the sample's bracket,
+    the bracket from the means that the CTAs have seen after their teams' first stages)."""
+    units = np.abs(W.reshape(-1, 128).astype(np.float64))
+    grid = min(torch.cuda.get_device_properties(0).multi_processor_count, 148)
+    per = -(-len(units) // grid)
+    assert per >= 700 and len(units) < 1 << 18                  # long enough for it; the sample of 64 units
+    s = np.arange(64, dtype=np.uint64)
+    stride = len(units) // 64
+    sample = units[(s * stride + (((s * 2654435761) & 0xFFFFFFFF) >> np.uint64(8)) % stride).astype(np.int64)].mean()
+    seen = min(per, 160 if bf16 else 80)                        # two teams' stages of 20 KB
+    means = np.array([units[r * per:min(len(units), r * per + seen)].mean() for r in range(grid) if r * per < len(units)])
+    b = 5.0 * means.std() / np.sqrt(len(means)) / means.mean() + 0.001
+    assert b < 0.04
+    return (sample * 0.96, sample * 1.04), (means.mean() * (1.0 - b), means.mean() * (1.0 + b))
+
+
+# factor: the first 224 units of every CTA's range are smaller than the rest by this
+@pytest.mark.parametrize("factor,narrows,holds", [(1.0, True, True), (0.98, True, False), (0.9, False, False)])
 @pytest.mark.parametrize("bf16", [False, True])
-def test_pack_long_matrix_narrows_its_bracket(bf16, misleading):
-    # ranges long enough for the CTAs to tell each other what their first stages say about the mean; misleading: the first 224 units
-    # of every CTA's range are far smaller than the rest, so that the narrowed bracket misses
+def test_pack_long_matrix_narrows_its_bracket(bf16, factor, narrows, holds):
+    # ranges long enough for the CTAs to tell each other what their first stages say about the mean: the narrowed bracket holds, or it
+    # misses the mean (values decided with the wide bracket before it, the exact second pass after it), or it lies outside the sample's
     N, K = 4096, 4096
     W = inputs.latent_weights(N, K, seed=61)
-    if misleading:
-        units = W.reshape(-1, 128)
-        grid = min(torch.cuda.get_device_properties(0).multi_processor_count, 148)
-        per = -(-len(units) // grid)
-        assert per >= 700
-        for r in range(grid):
-            units[r * per:r * per + 224] *= np.float32(0.9)
-    bits = inputs.f32_to_bf16_bits(W) if bf16 else None
-    if bf16:
-        W = (bits.astype(np.uint32) << 16).view(np.float32).reshape(N, K)
+    units = W.reshape(-1, 128)
+    grid = min(torch.cuda.get_device_properties(0).multi_processor_count, 148)
+    per = -(-len(units) // grid)
+    for r in range(grid):
+        units[r * per:r * per + 224] *= np.float32(factor)
+    W, bits = _masters(W, bf16)
+    wide, narrow = _first_look(W, bf16)
+    lo, hi = max(wide[0], narrow[0]), min(wide[1], narrow[1])
+    mean = np.abs(W.astype(np.float64)).mean()
+    assert wide[0] < mean < wide[1]
+    assert (lo < hi) == narrows and (not narrows or (lo < mean < hi) == holds)
     r, g = _oracle_pack(W), gpu_quantize_mask_pack(W, with_dense=False, w_bf16_bits=bits)
     assert g["scale"] == r["scale"] and np.array_equal(g["vals"], r["vals"]) and np.array_equal(g["meta"], r["meta"])
     _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
 
 
-def test_pack68_every_kept_set():
+@pytest.mark.parametrize("bf16", [False, True])
+def test_pack68_every_kept_set(bf16):
     # all 28 ways of dropping two columns of eight, each with distinct magnitudes and with ties at
     # the boundary (the dropped pair equal to a kept column: the lower column must win)
     N, K = 128, 256
@@ -459,17 +487,20 @@ def test_pack68_every_kept_set():
         grp[idx + 56, :, j] = np.float32(-0.75)
     W[120, :] = 0.0                                           # all-zero groups: columns 0..5 kept
     W[121, :] = 0.3
-    _assert_pack68(W, gpu_quantize_mask_pack68(W))
+    W, bits = _masters(W, bf16)
+    _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
 
 
-def test_pack68_misleading_sample_and_list_overflow():
+@pytest.mark.parametrize("bf16", [False, True])
+def test_pack68_misleading_sample_and_list_overflow(bf16):
     N, K = 1024, 2560
     W = inputs.latent_weights(N, K, seed=58)
     KB = K // 128
     for u in _sampled_units(N, K):
         n, kb = divmod(int(u), KB)
         W[n, kb * 128:(kb + 1) * 128] *= np.float32(1e-3)
-    _assert_pack68(W, gpu_quantize_mask_pack68(W))
+    W, bits = _masters(W, bf16)
+    _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
     # nearly every kept value within 1 % of the rounding threshold: the list overflows
     rng = np.random.default_rng(59)
     a = np.float32(0.01)
@@ -479,35 +510,39 @@ def test_pack68_misleading_sample_and_list_overflow():
     heavy = (np.arange(G) % 16) == 0
     # mean |w| must come out near 2a for thr = scale / 2 to sit at a: heavy groups carry the rest
     groups[heavy] *= np.float32(17.0)
-    W = groups.reshape(N, K)
-    r = _assert_pack68(W, gpu_quantize_mask_pack68(W))
+    W, bits = _masters(groups.reshape(N, K), bf16)
+    r = _assert_pack68(W, gpu_quantize_mask_pack68(W, w_bf16_bits=bits))
     frac = np.count_nonzero(r["w_eff"]) / (0.75 * r["w_eff"].size)
     assert 0.2 < frac < 0.9, "the construction should split the kept values"
     # a short list (small matrix): the fix-up route
-    _assert_pack68(W[:256, :512].copy(), gpu_quantize_mask_pack68(W[:256, :512].copy()))
+    small = None if bits is None else bits[:256, :512].copy()
+    _assert_pack68(W[:256, :512].copy(), gpu_quantize_mask_pack68(W[:256, :512].copy(), w_bf16_bits=small))
 
 
-def test_pack68_degenerate_scales():
-    Z = np.zeros((128, 256), np.float32)
-    g = gpu_quantize_mask_pack68(Z)
+@pytest.mark.parametrize("bf16", [False, True])
+def test_pack68_degenerate_scales(bf16):
+    Z, bits = _masters(np.zeros((128, 256), np.float32), bf16)
+    g = gpu_quantize_mask_pack68(Z, w_bf16_bits=bits)
     assert g["scale"] == np.float32(1e-5)
     _assert_pack68(Z, g)
-    tiny = np.full((128, 256), 7e-6, np.float32)
-    _assert_pack68(tiny, gpu_quantize_mask_pack68(tiny))
+    tiny, bits = _masters(np.full((128, 256), 7e-6, np.float32), bf16)
+    _assert_pack68(tiny, gpu_quantize_mask_pack68(tiny, w_bf16_bits=bits))
 
 
+@pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("in_place", [False, True])
-def test_pack68_flip_count(in_place):
+def test_pack68_flip_count(in_place, bf16):
     W = inputs.latent_weights(256, 2560, seed=60)
-    Wp = inputs.perturb_weights(W, seed=61, sigma=1e-4)
-    g0 = gpu_quantize_mask_pack68(W)
+    Wp, bits_p = _masters(inputs.perturb_weights(W, seed=61, sigma=1e-4), bf16)
+    W, bits = _masters(W, bf16)
+    g0 = gpu_quantize_mask_pack68(W, w_bf16_bits=bits)
     r0 = _assert_pack68(W, g0)
-    g1 = gpu_quantize_mask_pack68(Wp, prev_meta=g0["meta"], in_place=in_place)
+    g1 = gpu_quantize_mask_pack68(Wp, prev_meta=g0["meta"], in_place=in_place, w_bf16_bits=bits_p)
     r1 = _assert_pack68(Wp, g1)
     expected = oracle.flip_count(r0["mask"], r1["mask"])
     assert expected > 0
     assert g1["flips"] == expected
-    assert gpu_quantize_mask_pack68(W, prev_meta=g0["meta"])["flips"] == 0
+    assert gpu_quantize_mask_pack68(W, prev_meta=g0["meta"], w_bf16_bits=bits)["flips"] == 0
 
 
 def test_pack68_rejects_what_it_cannot_do():
@@ -1189,11 +1224,11 @@ def test_tile_canonical_round_trip_and_gemm():
 
 
 # ---- a captured pack call replayed on changed weights ---------------------------------------------------
-def test_quantize_mask_pack_graph_replay_on_changed_weights():
+@pytest.mark.parametrize("N,K", [(2560, 2560), (4096, 4096)])    # 4096 rows: the CTAs also exchange what they have seen under way
+def test_quantize_mask_pack_graph_replay_on_changed_weights(N, K):
     # A launch captured in a CUDA graph carries the same host-side nonce at every replay; the slots
     # of the previous replay must still not be taken for this replay's partial sums.  Replays on
     # weights of very different scale: a stale partial sum would give a wrong gamma.
-    N, K = 2560, 2560
     Ws = [inputs.latent_weights(N, K, seed=130 + i, sigma=0.02 * (3 ** i)) for i in range(3)]
     refs = [_oracle_pack(W) for W in Ws]
     Wd = dev(Ws[0])
@@ -1249,10 +1284,10 @@ def test_gemm_wait_runs_out_and_the_library_recovers(name, T, N, K, tuning, spar
     assert np.array_equal(acc.cpu().numpy(), acc_ref)
 
 
-def test_pack_wait_runs_out_and_the_library_recovers():
+@pytest.mark.parametrize("N,K", [(512, 2560), (4096, 4096)])     # 4096 rows: the CTAs also exchange what they have seen under way
+def test_pack_wait_runs_out_and_the_library_recovers(N, K):
     # one CTA of the pack kernel withholds its partial sum: every CTA's bounded wait for that slot runs
     # out, all of them return, the status word says SBN_ERR_TIMEOUT; the next call is exact
-    N, K = 512, 2560
     W = inputs.latent_weights(N, K, seed=150)
     r = _oracle_pack(W)
     b.sbn_check_status()
