@@ -137,7 +137,8 @@ struct FewFetch {
 // at once is too much where memory is the limit (4096 -> 11008 8.5, dense 10.2), and very long rows lose by any of it (11008 -> 4096:
 // eleven blocks, 9.37 / 9.45 at 8 tokens, dense 11.5 / 11.7) -- unless they are packed and the memory has time (9.4 / 8.5).  Packed weights gain
 // a tenth everywhere, also where there is nothing to prefetch (2560 -> 2560 4.6 / 4.2): without a side effect here the compiler
-// expands the first blocks before it asks for the activations.
+// expands the first blocks before it asks for the activations.  (It does so too behind an empty asm that takes the blocks' registers
+// after the activations' loads: 2560 -> 2560 4.4, 4096 -> 4096 5.2 / 4.4.)
 template <int WT, int W, int D>
 __device__ __forceinline__ void few_prefetch_next(const FewParams& p, uint32_t lane, uint32_t warp, uint32_t rounds) {
     if (lane >= D || (WT != kFewPacked && rounds > 2 * D)) return;
@@ -371,17 +372,32 @@ bitlinear_gemm_few_kernel(const FewParams p) {
     }
 }
 
+// Does the early fetch of the next blocks pay?  Not without any (groups and blocks per warp that the first D do not cover, or
+// more than the next D do).  FUSED, three CTAs per SM, where the first row group's activations are still to be quantised: not while a warp
+// has one block per row group (K = 640 to 1024: 1 to 5 % slower); int8-held 2:4 not beyond 1.9 groups per place (2048 -> 14336 6.5 /
+// 6.7 us), nor 1.25 with K > 2048 (3072 -> 12288 8.5 / 8.8; 2560 -> 7680 6.1 / 5.9); dense, K of about 1280 to 2048, only beyond 1.3
+// (2048 -> 8704 5.3 / 5.6; 2048 -> 16384 8.2 / 7.7, 2560 -> 7680 6.4 / 5.9).
+template <int WT, bool FUSED, int W, int D, int MINB>
+inline bool few_ahead(int k_blocks, int groups, int slots) {
+    if (groups <= slots && (k_blocks <= W * D || k_blocks > 2 * W * D)) return false;
+    if (!FUSED || MINB < 3) return true;
+    const double per_place = static_cast<double>(groups) / slots;
+    if (k_blocks <= W) return false;
+    if (WT == kFewSparse) return per_place <= (k_blocks <= 2 * W ? 1.9 : 1.25);
+    return k_blocks <= 10 || k_blocks > 2 * W || per_place > 1.3;
+}
+
 template <int WT, int NT, int W, int D, int MINB, bool FUSED>
 inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
     const int groups = p.N / 16, slots = device_sm_count() * MINB;
     ++g_launch_count;
-    // Where there is something to fetch; else for the sake of the order of the loads (see few_prefetch_next), which helps packed
-    // and, a little, int8-held 2:4 weights (2560 -> 2560 4.09 / 3.96) but not dense ones (2560 -> 3840, 8 tokens 4.75 / 4.95) nor the fused
-    // quantiser (2560 -> 3840 3.83 / 3.99).
-    const bool more = groups > slots || (p.k_blocks > W * D && p.k_blocks <= 2 * W * D);
-    const bool ahead = more || WT == kFewPacked || (WT == kFewSparse && !FUSED);
-    return launch_kernel(ahead ? bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, true> : bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, false>,
-                         dim3(groups < slots ? groups : slots), dim3(32 * W), 0, stream, p);
+    auto kernel = bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, true>;
+    // 2:4 weights always, for the sake of the order of the loads (see few_prefetch_next), which helps packed and, a little, int8-held ones
+    // (2560 -> 2560 4.09 / 3.96) but not dense ones (2560 -> 3840, 8 tokens 4.75 / 4.95) nor the fused quantiser (2560 -> 3840 3.83 / 3.99).
+    if constexpr (WT == kFewDense || FUSED) {
+        if (!few_ahead<WT, FUSED, W, D, MINB>(p.k_blocks, groups, slots)) kernel = bitlinear_gemm_few_kernel<WT, NT, W, D, MINB, FUSED, false>;
+    }
+    return launch_kernel(kernel, dim3(groups < slots ? groups : slots), dim3(32 * W), 0, stream, p);
 }
 
 // Which calls run here, with what split.  All times in us for quantiser + GEMM in a decode loop (weights from HBM), this
