@@ -57,6 +57,62 @@ __device__ __forceinline__ double bf16_abs_to_f64(uint32_t abs15) {
     return __hiloint2double(static_cast<int>((abs15 << 13) + 0x38000000u), 0);
 }
 
+// The arithmetic that every form of the kernel shares, 8 columns (a vector) at a time.
+// Adds the squares in fp64, four chains so that the adds overlap: exact products, one rounding in the add.
+__device__ __forceinline__ void add_squares8(const uint4& v, double (&s4)[4]) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const double lo = bf16_abs_to_f64(w[j] & 0x7FFFu), hi = bf16_abs_to_f64((w[j] >> 16) & 0x7FFFu);
+        s4[(2 * j) & 3] = __fma_rn(lo, lo, s4[(2 * j) & 3]);
+        s4[(2 * j + 1) & 3] = __fma_rn(hi, hi, s4[(2 * j + 1) & 3]);
+    }
+}
+// r from the sum of squares.  ss / n, correctly rounded, from the rounded reciprocal: quotient, exact remainder, correction
+// (Markstein's theorem for division with a correctly rounded reciprocal).
+__device__ __forceinline__ float norm_factor(double ss, double n, double inv_n, float eps) {
+    const double quot = ss * inv_n;
+    const float ms = static_cast<float>(__fma_rn(__fma_rn(-quot, n, ss), inv_n, quot));
+    return __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(ms, eps)));
+}
+// xn = (x * r) * g with packed fp32x2 multiplies: both factors of all pairs, then the gains.
+__device__ __forceinline__ void normalise8(const uint4& v, uint64_t r2, uint64_t (&out)[4]) {
+    out[0] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.x), bf16hi_to_f32(v.x)), r2);
+    out[1] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.y), bf16hi_to_f32(v.y)), r2);
+    out[2] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.z), bf16hi_to_f32(v.z)), r2);
+    out[3] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.w), bf16hi_to_f32(v.w)), r2);
+}
+__device__ __forceinline__ void apply_gain8(const float4& a, const float4& b, uint64_t (&out)[4]) {
+    out[0] = mul_f32x2(out[0], pack_f32x2(a.x, a.y));
+    out[1] = mul_f32x2(out[1], pack_f32x2(a.z, a.w));
+    out[2] = mul_f32x2(out[2], pack_f32x2(b.x, b.y));
+    out[3] = mul_f32x2(out[3], pack_f32x2(b.z, b.w));
+}
+__device__ __forceinline__ float max_abs8(const uint64_t (&xn)[4], float m) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float lo, hi;
+        unpack_f32x2(xn[j], lo, hi);
+        m = max_abs3(m, lo, hi);
+    }
+    return m;
+}
+// rint(xn * s_x): multiply, then add 1.5 * 2^23 -- the adder's round-to-nearest-even IS the rounding of the method, and the
+// integer is left in the low mantissa bits.  The adds are scalar: a packed multiply followed by a packed add came out with ONE
+// rounding (a fused multiply-add), which breaks exact ties such as 63.5.  The method's clamp cannot act: |xn| <= d (finite), so
+// |xn * s_x| <= 127 (1 + 2^-23) and rounds to at most 127.  The code is the low byte; the lowest column is the lowest byte of .x.
+__device__ __forceinline__ uint2 round_codes8(const uint64_t (&xn)[4], uint64_t s2) {
+    uint32_t q[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float lo, hi;
+        unpack_f32x2(mul_f32x2(xn[j], s2), lo, hi);
+        q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
+        q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
+    }
+    return make_uint2(low_bytes4(q[0], q[1], q[2], q[3]), low_bytes4(q[4], q[5], q[6], q[7]));
+}
+
 // Codes of a finite row whose xn is not finite: mean square 0 with eps = 0 (rinv infinite), or a gain that takes xn out of range
 // (s_x = 0).  The product is NaN where xn is infinite or NaN: code 127, as a saturating conversion gives; else 0.  The row is read
 // again and its codes stored over the ones before: a call that is never made, 1 % of the kernel's time on average (5 % for 8192 rows
@@ -142,17 +198,9 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
             nxt[i] = (row_n < T && idx < nvec) ? __ldg(x + static_cast<size_t>(row_n) * nvec + idx) : make_uint4(0u, 0u, 0u, 0u);
         }
         // ---- mean square
-        double s4[4] = {0.0, 0.0, 0.0, 0.0};                      // four chains: the adds overlap
+        double s4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-        for (int i = 0; i < VPT; ++i) {
-            const uint32_t w[4] = {cur[i].x, cur[i].y, cur[i].z, cur[i].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {                                   // exact product, one rounding in the add
-                const double lo = bf16_abs_to_f64(w[j] & 0x7FFFu), hi = bf16_abs_to_f64((w[j] >> 16) & 0x7FFFu);
-                s4[(2 * j) & 3] = __fma_rn(lo, lo, s4[(2 * j) & 3]);
-                s4[(2 * j + 1) & 3] = __fma_rn(hi, hi, s4[(2 * j + 1) & 3]);
-            }
-        }
+        for (int i = 0; i < VPT; ++i) add_squares8(cur[i], s4);
         double ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
@@ -165,29 +213,18 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
             for (int w = 0; w < WARPS_PER_ROW; ++w) t += sm[w0 + w];
             ss = t;
         }
-        // ss / n, correctly rounded, from the rounded reciprocal: quotient, exact remainder, correction (Markstein's theorem
-        // for division with a correctly rounded reciprocal)
-        const double quot = ss * inv_n;
-        const float ms = static_cast<float>(__fma_rn(__fma_rn(-quot, n, ss), inv_n, quot));
-        const float rinv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(ms, eps)));
-        // ---- xn = (x * r) * g with packed fp32x2 multiplies, and max |xn|.  Up to four vectors per
-        // thread the fp32 xn stays in registers for the rounding; longer rows recompute it.
+        const float rinv = norm_factor(ss, n, inv_n, eps);
+        // ---- xn and max |xn|.  Up to four vectors per thread the fp32 xn stays in registers for the rounding; longer rows recompute it.
         constexpr bool KEEP = VPT <= 4;
         const uint64_t r2 = pack_f32x2(rinv, rinv);
         uint64_t xn2[KEEP ? VPT : 1][4];
         float amax = 0.0f;
         auto normalise = [&](const uint4& v, int i, uint64_t (&out)[4]) {
             const int idx = g + i * G;
-            out[0] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.x), bf16hi_to_f32(v.x)), r2);
-            out[1] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.y), bf16hi_to_f32(v.y)), r2);
-            out[2] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.z), bf16hi_to_f32(v.z)), r2);
-            out[3] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.w), bf16hi_to_f32(v.w)), r2);
+            normalise8(v, r2, out);
             if (GAIN && idx < nvec) {
                 const float4 a = GAIN_REGS ? gain_r[GAIN_REGS ? i : 0][0] : s_gain[idx], b = GAIN_REGS ? gain_r[GAIN_REGS ? i : 0][1] : s_gain[nvec + idx];
-                out[0] = mul_f32x2(out[0], pack_f32x2(a.x, a.y));
-                out[1] = mul_f32x2(out[1], pack_f32x2(a.z, a.w));
-                out[2] = mul_f32x2(out[2], pack_f32x2(b.x, b.y));
-                out[3] = mul_f32x2(out[3], pack_f32x2(b.z, b.w));
+                apply_gain8(a, b, out);
             }
         };
 #pragma unroll
@@ -195,12 +232,7 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
             uint64_t tmp[4];
             uint64_t (&o)[4] = KEEP ? xn2[KEEP ? i : 0] : tmp;
             normalise(cur[i], i, o);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float lo, hi;
-                unpack_f32x2(o[j], lo, hi);
-                amax = max_abs3(amax, lo, hi);
-            }
+            amax = max_abs8(o, amax);
         }
         // bit patterns of non-negative floats order like integers: one redux instruction per warp
         amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax)));
@@ -225,24 +257,7 @@ norm_quant_act_kernel(const uint4* __restrict__ x, int T, int nvec, const float4
                     uint64_t tmp[4];
                     if constexpr (!KEEP) normalise(cur[i], i, tmp);
                     const uint64_t (&o)[4] = KEEP ? xn2[KEEP ? i : 0] : tmp;
-                    uint32_t q[8];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        // rint(xn * s_x) for two values: multiply, then add 1.5 * 2^23 -- the adder's round-to-nearest-even
-                        // IS the rounding of the method, and the integer is left in the low mantissa bits.  The
-                        // adds are scalar: a packed multiply followed by a packed add came out with ONE
-                        // rounding (a fused multiply-add), which breaks exact ties such as 63.5.
-                        float lo, hi;
-                        unpack_f32x2(mul_f32x2(o[j], s2), lo, hi);
-                        q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
-                        q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
-                    }
-                    // The method's clamp cannot act: |xn| <= d (finite), so |xn * s_x| <= 127 (1 + 2^-23) and rounds to at most 127.  The
-                    // code is the low byte.
-                    uint2 ov;                                      // lowest column in the lowest byte
-                    ov.x = low_bytes4(q[0], q[1], q[2], q[3]);
-                    ov.y = low_bytes4(q[4], q[5], q[6], q[7]);
-                    store_codes8<EXPAND68>(xq, row, idx, tb8, ov);     // plain, or expanded for the 6:8 pattern
+                    store_codes8<EXPAND68>(xq, row, idx, tb8, round_codes8(o, s2));     // plain, or expanded for the 6:8 pattern
                 }
             }
             if (fmaxf(d, rinv) == __int_as_float(0x7F800000))              // for the whole group of threads, so for whole warps

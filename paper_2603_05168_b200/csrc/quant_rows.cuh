@@ -29,14 +29,6 @@ __device__ __forceinline__ uint4 lds_vec(uint32_t addr) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
 }
-// Read once: the lines leave the L2 first (the codes written here are the next kernel's operand).
-__device__ __forceinline__ void bulk_load_row(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    unsigned long long policy;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-    mbar_expect_tx(bar, bytes);
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
-}
 
 // Shared memory: gains [2][nvec] float4 (first halves of all vectors, then the second ones) when GAIN, then a row per warp.
 template <bool NORM, bool GAIN>
@@ -70,7 +62,10 @@ quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __
     }
     pdl_wait();
     auto fetch = [&](int r) {
-        if (lane == 0u && r < T) bulk_load_row(at, x + static_cast<size_t>(r) * nvec, row_bytes, bar);
+        if (lane == 0u && r < T) {
+            mbar_expect_tx(bar, row_bytes);
+            bulk_load_once(at, x + static_cast<size_t>(r) * nvec, row_bytes, bar, l2_policy_evict_first());
+        }
     };
     fetch(row);
     if constexpr (GAIN) {
@@ -88,49 +83,23 @@ quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __
         }
         float rinv = 1.0f, amax;
         auto normalise = [&](const uint4& v, int idx, uint64_t (&o)[4]) {
-            const uint64_t r2 = pack_f32x2(rinv, rinv);
-            o[0] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.x), bf16hi_to_f32(v.x)), r2);
-            o[1] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.y), bf16hi_to_f32(v.y)), r2);
-            o[2] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.z), bf16hi_to_f32(v.z)), r2);
-            o[3] = mul_f32x2(pack_f32x2(bf16lo_to_f32(v.w), bf16hi_to_f32(v.w)), r2);
-            if constexpr (GAIN) {
-                const float4 a = s_gain[idx], b = s_gain[nvec + idx];
-                o[0] = mul_f32x2(o[0], pack_f32x2(a.x, a.y));
-                o[1] = mul_f32x2(o[1], pack_f32x2(a.z, a.w));
-                o[2] = mul_f32x2(o[2], pack_f32x2(b.x, b.y));
-                o[3] = mul_f32x2(o[3], pack_f32x2(b.z, b.w));
-            }
+            normalise8(v, pack_f32x2(rinv, rinv), o);
+            if constexpr (GAIN) apply_gain8(s_gain[idx], s_gain[nvec + idx], o);
         };
         if constexpr (NORM) {
             double s4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
-            for (int idx = lane; idx < nvec; idx += 32) {
-                const uint4 v = lds_vec(at + 16u * idx);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {                                   // exact product, one rounding in the add
-                    const double lo = bf16_abs_to_f64(w[j] & 0x7FFFu), hi = bf16_abs_to_f64((w[j] >> 16) & 0x7FFFu);
-                    s4[(2 * j) & 3] = __fma_rn(lo, lo, s4[(2 * j) & 3]);
-                    s4[(2 * j + 1) & 3] = __fma_rn(hi, hi, s4[(2 * j + 1) & 3]);
-                }
-            }
+            for (int idx = lane; idx < nvec; idx += 32) add_squares8(lds_vec(at + 16u * idx), s4);
             double ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
-            const double quot = ss * inv_n;                                     // ss / n, correctly rounded: see norm_quant_act.cuh
-            const float ms = static_cast<float>(__fma_rn(__fma_rn(-quot, n, ss), inv_n, quot));
-            rinv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(ms, eps)));
+            rinv = norm_factor(ss, n, inv_n, eps);
             amax = 0.0f;
 #pragma unroll 4
             for (int idx = lane; idx < nvec; idx += 32) {
                 uint64_t o[4];
                 normalise(lds_vec(at + 16u * idx), idx, o);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float lo, hi;
-                    unpack_f32x2(o[j], lo, hi);
-                    amax = max_abs3(amax, lo, hi);
-                }
+                amax = max_abs8(o, amax);
             }
             amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(amax)));
         } else {
@@ -161,15 +130,7 @@ quant_rows_kernel(const uint4* __restrict__ x, int T, int nvec, const float4* __
             if constexpr (NORM) {
                 uint64_t o[4];
                 normalise(v, idx, o);
-                uint32_t q[8];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {                                   // rounding by adding 1.5 * 2^23: see norm_quant_act.cuh
-                    float lo, hi;
-                    unpack_f32x2(mul_f32x2(o[j], s2), lo, hi);
-                    q[2 * j] = __float_as_uint(__fadd_rn(lo, 12582912.0f));
-                    q[2 * j + 1] = __float_as_uint(__fadd_rn(hi, 12582912.0f));
-                }
-                ov = make_uint2(low_bytes4(q[0], q[1], q[2], q[3]), low_bytes4(q[4], q[5], q[6], q[7]));
+                ov = round_codes8(o, s2);
             } else {
                 ov = make_uint2(quant_pair2(v.x, v.y, s_x), quant_pair2(v.z, v.w, s_x));
             }

@@ -154,18 +154,6 @@ __device__ __forceinline__ bool qmp_mbar_wait(uint32_t bar, uint32_t parity, vol
     }
     return true;
 }
-// The copies of data that is read once (the master weights of pass 1) carry an L2 policy: the lines are the first to leave the
-// L2 again, so the stream does not push out what the kernels after this one will read (the packed weights
-// this kernel writes, the activations).
-__device__ __forceinline__ unsigned long long qmp_policy_evict_first() {
-    unsigned long long pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void qmp_bulk_load_once(uint32_t smem_dst, const void* gmem_src, uint32_t bytes, uint32_t bar, unsigned long long policy) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-                 ::"r"(smem_dst), "l"(gmem_src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
-}
 __device__ __forceinline__ float4 qmp_lds128(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
@@ -239,7 +227,7 @@ __device__ __forceinline__ bool qmp_hint(const QmpDesc& d, float& g) {
 // gamma_est of the first matrix: mean |w| over qmp_sample_units units scattered over it (the same units in every
 // CTA; a multiplicative hash keeps them off any row / column-block period).  In two halves, so that something can
 // be started between asking for the sample and using it: all of a thread's sample loads are issued (into v), later
-// they are added up over the CTA -- one barrier, after which every warp adds the 32 partial sums itself.
+// they are added up over the CTA -- one barrier, after which every warp adds the partial sums of all warps itself.
 // The values stay as loaded (bf16: two words) until they are added up: a conversion next to the load makes every
 // load of a thread wait for the one before (64 trips in a row, 60 us, for a warp's sample of a bf16 matrix).
 __device__ __forceinline__ float4 qmp_load_group_raw(const QmpDesc& d, uint32_t u, int lane) {
@@ -365,7 +353,7 @@ __device__ __forceinline__ bool qmp_loader_issue(QmpLoader& L, const QmpBatch& b
         const uint32_t units = min(L.u_end - L.u, static_cast<uint32_t>(kQmpStageBytes) / L.unit_bytes);
         const uint32_t bytes = units * L.unit_bytes;
         qmp_mbar_expect_tx(bar_full0 + 8u * L.ring.stage(), bytes);
-        qmp_bulk_load_once(ring_base + L.ring.stage() * kQmpStageBytes, L.W + static_cast<size_t>(L.u) * L.unit_bytes, bytes, bar_full0 + 8u * L.ring.stage(),
+        bulk_load_once(ring_base + L.ring.stage() * kQmpStageBytes, L.W + static_cast<size_t>(L.u) * L.unit_bytes, bytes, bar_full0 + 8u * L.ring.stage(),
                            L.policy);
         ++L.issued;
         L.ring.advance();
@@ -425,13 +413,26 @@ __device__ __forceinline__ uint32_t qmp_flip_pairs(uint32_t x) {
     return __popc(any | (none << 1));
 }
 
-// The bracket of a step as two numbers: kept values are +-1 iff thr_pred - |w| is negative, undecided iff it is at most width.
-__device__ __forceinline__ void qmp_thresholds(const QmpJob& jb, float& thr_pred, uint32_t& width) {
-    float lo, hi;
-    asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(hi) : "r"(qmp_smem_u32(&jb.bracket)));
-    thr_pred = __uint_as_float(__float_as_uint(hi) - 1u);
-    width = __float_as_uint(thr_pred - lo);
-}
+// The bracket as the computing warps use it.  fp32: a weight is kept as +-1 iff |w| > thr_pred, i.e. iff thr_pred - |w| is
+// negative, and undecided iff that difference lies in 0 .. width (an unsigned compare of the bits; the subtraction is exact near
+// the threshold and monotone everywhere: a value wrongly taken for undecided can only lie below the bracket, and the fix-up decides it
+// like any other).  bf16 in halfword arithmetic: the largest |w| that is not above / not inside the bracket, in both halves.
+template <bool BF16>
+struct QmpBracket {
+    float thr_pred, lo_pred;
+    uint32_t width;
+    uint32_t hi2, lo2;
+    __device__ __forceinline__ explicit QmpBracket(const QmpJob& jb) {
+        float lo, hi;
+        asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(hi) : "r"(qmp_smem_u32(&jb.bracket)));
+        const uint32_t hi_bits = __float_as_uint(hi) - 1u, lo_bits = __float_as_uint(lo) - 1u;
+        thr_pred = __uint_as_float(hi_bits);
+        lo_pred = __uint_as_float(lo_bits);
+        width = __float_as_uint(thr_pred - lo);
+        hi2 = (hi_bits >> 16) * 0x10001u;
+        lo2 = (lo_bits >> 16) * 0x10001u;
+    }
+};
 
 // Where a computing warp is in a matrix: its quarter-warp's unit of the current step of its team's stages.
 template <bool BF16>
@@ -503,9 +504,6 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
     constexpr uint32_t kUnitBytes = Walk::kUnitBytes, REP = Walk::REP;
     constexpr int PIECES = BF16 ? 2 : 4;                              // 16-byte pieces per lane
     const uint32_t KB = jb.KB;
-    // kept is +-1 iff |k| > thr_pred, undecided iff 0 <= thr_pred - |k| <= width.  The subtraction is exact near the
-    // threshold and monotone everywhere: a value wrongly taken for undecided can only lie below thr_lo, and the
-    // fix-up decides it like any other.
     const uint32_t n_stages = (jb.units + REP * kQmpStepUnits - 1u) / (REP * kQmpStepUnits);
     const uint32_t g_end = g0 + n_stages;
     double acc = 0.0;
@@ -532,13 +530,11 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
     uint32_t q = tiled_row(at.n, at.kb);
     uint32_t prev = 0u;
     if (prev_lane != nullptr && at.left > 0) prev = *reinterpret_cast<const uint16_t*>(prev_lane + static_cast<size_t>(q) * 16u);
-    float thr_pred;
-    uint32_t width;
-    if constexpr (!LOOK) qmp_thresholds(jb, thr_pred, width);
+    QmpBracket<false> br(jb);                                         // (bf16 weights are fp32 by then)
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
-        if constexpr (LOOK) qmp_thresholds(jb, thr_pred, width);      // may have become narrower
+        if constexpr (LOOK) br = QmpBracket<false>(jb);               // may have become narrower
 #pragma unroll
         for (uint32_t rep = 0; rep < REP; ++rep) {
             // The warp has no unit in this step (a matrix's last stage): nothing to do.  (Batch of 14 bf16 tensors 124 -> 120 us; of fp32
@@ -581,14 +577,12 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
             const uint32_t word = ((nibbles * 0x10001u) >> (16u - 4u * rot)) & 0xFFFFu;        // nibble i to its place, (i + rot) mod 4
             uint32_t e[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(thr_pred - fabsf(k[i]));
+            for (int i = 0; i < 8; ++i) e[i] = __float_as_uint(br.thr_pred - fabsf(k[i]));
             uint32_t t[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint32_t keep = prmt(prmt(e[4 * h], e[4 * h + 1], 0x00FBu), prmt(e[4 * h + 2], e[4 * h + 3], 0x00FBu), 0x5410u);
-                const uint32_t sign = prmt(prmt(__float_as_uint(k[4 * h]), __float_as_uint(k[4 * h + 1]), 0x00FBu),
-                                           prmt(__float_as_uint(k[4 * h + 2]), __float_as_uint(k[4 * h + 3]), 0x00FBu), 0x5410u);
-                t[h] = (sign | 0x01010101u) & keep;
+                const uint32_t keep = sign_bytes4(e[4 * h], e[4 * h + 1], e[4 * h + 2], e[4 * h + 3]);
+                t[h] = (sign_bytes4(k[4 * h], k[4 * h + 1], k[4 * h + 2], k[4 * h + 3]) | 0x01010101u) & keep;
             }
             uint32_t und = 0u;
             if (mine) {
@@ -596,9 +590,9 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
                 *reinterpret_cast<uint16_t*>(meta_lane + static_cast<size_t>(q_cur) * 16u) = static_cast<uint16_t>(word);
                 *reinterpret_cast<uint2*>(jb.vals + static_cast<size_t>(v8) * 8u) = make_uint2(prmt(t[0], t[1], sel_lo), prmt(t[0], t[1], sel_hi));
                 if (prev_lane != nullptr) flips += qmp_flip_pairs(word ^ prev_cur);
-                if (umin8(e) <= width) {
+                if (umin8(e) <= br.width) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) und |= e[i] <= width ? 1u << i : 0u;
+                    for (int i = 0; i < 8; ++i) und |= e[i] <= br.width ? 1u << i : 0u;
                 }
             }
             qmp_list_append(list, und, [&](int j) { return v8 * 8u + 2u * (((j >> 1) + rot) & 3u) + (j & 1u); },
@@ -619,23 +613,6 @@ __device__ __forceinline__ double qmp_stream_pass1(const QmpJob& jb, QmpStreamSh
     return acc;
 }
 
-// The bracket as the computing warps use it.  fp32: a weight is kept as +-1 iff |w| > thr_pred, i.e. iff thr_pred - |w| is
-// negative, and undecided iff that difference lies in 0 .. width (an unsigned compare of the bits; the subtraction is exact near
-// the threshold and monotone everywhere).  bf16: the largest |w| that is not above / not inside the bracket, in both halves.
-template <bool BF16>
-struct QmpBracket {
-    float thr_pred, lo_pred;
-    uint32_t width;
-    uint32_t hi2, lo2;
-    __device__ __forceinline__ QmpBracket(float lo, float hi) {
-        const uint32_t hi_bits = __float_as_uint(hi) - 1u, lo_bits = __float_as_uint(lo) - 1u;
-        thr_pred = __uint_as_float(hi_bits);
-        lo_pred = __uint_as_float(lo_bits);
-        width = __float_as_uint(thr_pred - lo);
-        hi2 = (hi_bits >> 16) * 0x10001u;
-        lo2 = (lo_bits >> 16) * 0x10001u;
-    }
-};
 // Eight consecutive weights (half of a lane's 16): fp32 in eight words, bf16 in four.
 // Sum |w| in fp64.  |bf16| becomes a double by two integer instructions (see bf16_abs_to_f64 in norm_quant_act.cuh: a zero
 // counts as 2^-127, which no sum above the 1e-5 clamp can see; the sums of a lane that saw an infinity or a NaN are taken again, below);
@@ -788,9 +765,7 @@ __device__ __forceinline__ double qmp68_stream_pass1(const QmpJob& jb, QmpStream
     for (; next_stage < g_end; next_stage += kQmpTeams) {
         const uint32_t use = next_stage / kQmpStages, stage = next_stage - use * kQmpStages;
         if (!qmp_mbar_wait(bar_full0 + 8u * stage, use & 1u, abort_flag)) { ok = false; break; }
-        float lo, hi;
-        asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(hi) : "r"(qmp_smem_u32(&jb.bracket)));
-        const QmpBracket<BF16> br(lo, hi);
+        const QmpBracket<BF16> br(jb);                                // may have become narrower
 #pragma unroll 1
         for (uint32_t rep = 0; rep < REP; ++rep) {
             if (at.left + (lane >> 3) <= 0) {                         // the warp has no unit in this step (a matrix's last stage)
@@ -1081,7 +1056,7 @@ quantize_mask_pack_stream_kernel(const __grid_constant__ QmpInlineDescs inl, con
     }
     const bool hinted0 = qmp_hint_usable(gamma0);
     if (!sample_early && !hinted0) qmp_sample_issue(first, sample0);
-    QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, qmp_policy_evict_first()};
+    QmpLoader loader{0, 0u, 0u, 0u, nullptr, false, QmpRing{0u}, 0u, l2_policy_evict_first()};
     const bool is_loader = warp == kQmpLoaderWarp && lane == 0;
     if (is_loader) qmp_loader_issue(loader, batch, count, kQmpTeams, grid_magic, ring_base, bar_full0, bar_empty0, abort_flag);
     if (!hinted0) gamma0 = qmp_sample_finish(first, sample0, sh.sample);
@@ -1292,8 +1267,8 @@ inline sbn_status launch_quantize_mask_pack_stream_cfg(const QmpDesc* descs_host
     const unsigned cap = static_cast<unsigned>(std::min(device_sm_count(), kQmpMaxCtas));
     const unsigned grid = max_units < cap ? max_units : cap;
     if (!ensure_dynamic_smem<quantize_mask_pack_stream_kernel<PATTERN, SINGLE>>(kQmpStreamSmemBytes)) return SBN_ERR_CUDA;
-    // At most one CTA per SM (768 threads x 80 registers and 215 KB each) and never more CTAs than SMs, so all
-    // of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
+    // At most one CTA per SM (kQmpThreads threads of up to 80 registers; kQmpStreamSmemBytes and a few KB more of shared memory) and
+    // never more CTAs than SMs, so all of them become resident as soon as the SMs are free and the exchange cannot deadlock; if
     // another kernel kept SMs busy for seconds, the bounded wait reports SBN_ERR_TIMEOUT instead.
     const cudaError_t err = launch_kernel(quantize_mask_pack_stream_kernel<PATTERN, SINGLE>, dim3(grid), dim3(kQmpThreads), kQmpStreamSmemBytes, stream,
                                           inl, rest_dev, count, slots, generation, nonce, test_withhold_slot, count == 1 ? memo : nullptr, qmp_magic(grid));
