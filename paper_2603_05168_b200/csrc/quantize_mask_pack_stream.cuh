@@ -462,8 +462,9 @@ struct QmpWalk {
 // never depend on the bracket.
 constexpr unsigned long long kQmpLookTag = 1ull << 63;
 constexpr float kQmpLookErrors = 5.0f, kQmpLookLeast = 0.001f;
-// From this many units of a CTA on: shorter ranges are over before the answer is there, and then it costs them up to 2 us (bf16, 519 units
-// per CTA, us with / without: 17.4 / 16.0; 934 units: fp32 23.8 / 24.9, 6:8 31.1 / 33.4).
+// From this many units of a CTA on: shorter ranges are over before the answer is there.  With it / without, 21 sizes, light and heavy tails:
+// 2:4 346 units fp32 1.09, 519 bf16 1.06, 606 1.00 to 1.02, 692 0.98 to 1.00, 934 0.95 to 0.98, 1384 0.92 to 0.94; 6:8 519 0.97 to 0.99, 692 0.95 to 0.98,
+// 934 0.92 to 0.94 (2560 -> 6912 6:8 fp32 33.4 / 31.1 us).
 constexpr uint32_t kQmpLookFrom = 700;
 __device__ __forceinline__ void qmp_look_report(QmpStreamShared& sh, double acc) {
     float sum = static_cast<float>(acc);
