@@ -411,7 +411,7 @@ inline cudaError_t launch_few_cfg(const FewParams& p, cudaStream_t stream) {
 //   9 to 16 tokens    only while two CTAs per SM take all row groups (4096 -> 11008 10.6 / 9.1: every CTA reads all activations,
 //                     the cluster kernel's 128-row tiles read them less often).  Packed weights then always (7B MLPs, whole pass,
 //                     47 / 52), int8-held ones up to 12 tokens, beyond up to K = 4352 (quantiser + GEMM,
-//                     9 tokens: 3584 -> 2560 5.0 / 6.1, 6912 -> 2560 6.9 / 7.2, 11008 -> 4096 9.7 / 10.9; 12: 9216 -> 2048 1 to 2 % slower, the worst; 16:
+//                     9 tokens: 3584 -> 2560 4.4 / 5.3, 6912 -> 2560 6.5 / 6.6, 11008 -> 4096 9.3 / 10.4; 12: 11008 -> 2048 8.93 / 8.97, the least gain of 28 shapes; 16:
 //                     4096 -> 4096 5.6 / 6.0, but 6912 -> 2560 7.5 / 7.05; two 7B MLPs, whole pass, 44.5 / 41.8).  Dense: not
 //                     (2B layers 63.5 / 59.3).  FUSED: not (6912 -> 2560 13.6 / 11.1).
 //   Not where a second round of CTAs would be barely filled: it costs as much as a full one, and the clusters have none.
