@@ -1433,11 +1433,12 @@ def test_quantize_mask_pack_68_starts_from_a_sample():
 # ---- the register-fed few-token kernel -----------------------------------------------------------------------------
 @pytest.mark.parametrize("T,N,K", [(1, 128, 128), (8, 128, 256), (3, 256, 1152), (5, 4864, 384), (1, 4864, 3328), (9, 640, 1408),
                                    (16, 2560, 256), (16, 128, 128), (5, 7296, 1152), (8, 7296, 2176), (3, 5120, 3328),
-                                   (12, 256, 6912), (16, 256, 4352), (2, 128, 8320)])
+                                   (12, 256, 6912), (16, 256, 4352), (2, 128, 8320), (5, 7296, 896), (3, 7296, 1536), (1, 9216, 2304)])
 def test_few_token_kernel_all_forms(T, N, K):
     # one token and the last of each group of 8; fewer 128-column blocks than warps, a last round that leaves warps without
     # a block; CTAs with a second row group (7296 / 16 = 456 of them on 444 places, in one and in more rounds over K; fused with
-    # K > 3072: 304 and 320 on 296); rows long enough for the early fetch of the next blocks, too long for it.  Accumulators exact, outputs as everywhere.
+    # K > 3072: 304 and 320 on 296); rows long enough for the early fetch of the next blocks, too long for it; fused calls with a second row
+    # group that leave it out (one block per warp; dense, twelve blocks; 2:4, 576 groups on 444 places).  Accumulators exact, outputs as everywhere.
     W = inputs.latent_weights(N, K, seed=200 + T)
     bits = inputs.activations_bf16(T, K, seed=300 + K, token_lognormal_sigma=0.5)
     bias = np.random.default_rng(N).standard_normal(N).astype(np.float32)
